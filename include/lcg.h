@@ -136,7 +136,7 @@ const char* lcg_last_error(const lcg_ctx* ctx);
 int lcg_last_build_stats(const lcg_ctx* ctx, lcg_build_stats* out);
 /* Per-kernel CUDA-event timing in later calls: 0 off, 1 every kernel launch,
  * 2 only the parse launches (k_parse, the kernel with most device time, and
- * k_parse_small, the single-block parse of a short round; few
+ * k_parse_small, the parse of a short round; few
  * events, so the call's own time is barely changed).  Timed launches are
  * bracketed by two events on the context's stream; the sums are read with
  * lcg_last_kernel_times.  Other values give LCG_EINVAL. */
@@ -146,8 +146,8 @@ int lcg_set_kernel_timing(lcg_ctx* ctx, int enable);
  *   table_load          phrase-table slots per expected new rule is 1 / table_load
  *                       (0.3 .. 0.78; a table past 0.8 is regrown and the round rerun);
  *   parse_blocks_per_sm resident k_parse blocks per SM, 0 = as many as fit;
- *   miss_flush          byte rounds: queued cache misses that trigger a lookup pass
- *                       (32 .. 256; at most 128 take effect with 4096-position tiles);
+ *   miss_flush          accepted (32 .. 256) and kept; it has no effect: every warp of
+ *                       the parse looks its queued phrases up as soon as there are 32;
  *   table_slots_max     0, or at most this many slots (>= 1024) in the first phrase
  *                       table of every round: a table too small for the round fills
  *                       past its load limit, is regrown (x4) and the parse rerun, so
@@ -157,9 +157,9 @@ int lcg_set_kernel_timing(lcg_ctx* ctx, int enable);
  *                       strings that are near-copies of one another at the same
  *                       offsets are parsed side by side;
  *   parse_tile          positions per parse tile: 1024, 2048 or 4096.  A block of
- *                       k_parse stages, lists and looks up one tile at a time (fewer
- *                       barriers per phrase with larger tiles, more blocks' worth of
- *                       tiles in flight with smaller ones);
+ *                       k_parse takes a tile at a time, each of its eight warps an
+ *                       eighth of it (less work per phrase with larger tiles, more
+ *                       warps' worth of work with smaller ones);
  *   parse_tile_min      a round's tile is halved (down to 1024 positions) while the
  *                       round would have fewer than this many tiles per SM (0 .. 1024;
  *                       0 keeps every round at parse_tile).

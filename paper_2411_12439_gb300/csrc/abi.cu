@@ -438,6 +438,12 @@ struct RoundInput {
     const u64* d_n;  // device values, for rounds enqueued without a sync
     const u64* d_k;
     bool own_offsets = true;  // soff / sid are this build's to free
+    // rounds >= 2: what names the symbols (ids) of the sequence: ids below
+    // prev_base are ranks of the level below, the others claims of the round
+    // before (at most prev_cap), whose ranks are in rank_prev
+    u32* rank_prev = nullptr;
+    u32 prev_base = 0;
+    u64 prev_cap = 0;
 };
 
 
@@ -448,6 +454,8 @@ void free_round_input(lcg_ctx* ctx, RoundInput& in) {
     }
     if (in.S_owned) dfree(ctx, in.S_owned);
     if (in.Sf) dfree(ctx, (void*)in.Sf);
+    dfree(ctx, in.rank_prev);
+    in.rank_prev = nullptr;
     in.soff = nullptr;
     in.sid = nullptr;
     in.S_owned = nullptr;
@@ -456,38 +464,34 @@ void free_round_input(lcg_ctx* ctx, RoundInput& in) {
 
 // Buffers of one round.
 struct RoundBufs {
-    u64 tiles = 0, Pmax = 0, Tcap = 0, cap = 0, g_alloc = 0;
-    u32 tp = 4096;  // positions per parse tile
+    u64 tiles = 0, Pmax = 0, Tcap = 0, cap = 0, first_words = 0;
+    u32 tp = 512;  // positions per parse unit
     u64* string_first = nullptr;
     u64* soff_next = nullptr;
     u32* sid_next = nullptr;
     u64* R_phr = nullptr;
     u32* R_sid = nullptr;
-    u32* P_slot = nullptr;
     u32* tile_cnt = nullptr;
     u64* tile_pfx = nullptr;
     u32* Tnext = nullptr;
     u32* Fnext = nullptr;
-    u32* tile_str = nullptr;
+    u32* step_str = nullptr;
     u32* brk = nullptr;
     u32* sbm = nullptr;
     u64 sbm_words = 0;
     unsigned char* tab = nullptr;  // phrase table: cap slots
-    u64* rv = nullptr;             // per slot: (F^i << 32) | rank, once named
-    u32* claims = nullptr;
-    u32* first_bits = nullptr;
-    u32* first_prefix = nullptr;
-    u32* slot_r = nullptr;
-    u32* len_r = nullptr;
-    u64* xlen = nullptr;
-    u64* mkey = nullptr;
-    u64* mval = nullptr;
-    u64* rkey = nullptr;
+    u64 id_cap = 0;                // claim numbers
+    u32 id_chunk = 1;
+    unsigned char* crec = nullptr; // the claims' records
+    u64* minpos = nullptr;         // and first occurrences
+    u32* rank_of = nullptr;        // their ranks, once named (kept until the next round is named)
+    uint2* first = nullptr;        // first-occurrence bitmap and prefix
+    u64 r_cap = 0;
+    unsigned char* rrec = nullptr; // the claims' records in rank order
 };
 
 // The next sequence (Tnext, Fnext) gets `t_cap` entries; 0 leaves it to
-// alloc_next (a round run with a host synchronisation knows its phrase count
-// after the parse).
+// alloc_next.
 void alloc_next(lcg_ctx* ctx, RoundBufs& b, u64 t_cap) {
     b.Tcap = std::min<u64>(t_cap, b.Pmax);
     b.Tnext = dalloc<u32>(ctx, b.Tcap);
@@ -506,7 +510,7 @@ u32 round_tile(const lcg_ctx* ctx, u64 n) {
 }
 
 void alloc_round(lcg_ctx* ctx, RoundBufs& b, u64 n_bound, u32 kk, u64 t_cap) {
-    b.tp = round_tile(ctx, n_bound);
+    b.tp = parse_unit(round_tile(ctx, n_bound));
     b.tiles = (n_bound + b.tp - 1) / b.tp;
     // every phrase but a string's first has length >= 2
     b.Pmax = n_bound / 2 + 2ull * kk + 1;
@@ -515,56 +519,57 @@ void alloc_round(lcg_ctx* ctx, RoundBufs& b, u64 n_bound, u32 kk, u64 t_cap) {
     b.sid_next = dalloc<u32>(ctx, kk);
     b.R_phr = dalloc<u64>(ctx, kk);
     b.R_sid = dalloc<u32>(ctx, kk);
-    b.P_slot = dalloc<u32>(ctx, parse_slot_entries(b.tiles, kk, b.tp));
     b.tile_cnt = dalloc<u32>(ctx, b.tiles);
     b.tile_pfx = dalloc<u64>(ctx, b.tiles);
     if (t_cap) alloc_next(ctx, b, t_cap);
-    b.tile_str = dalloc<u32>(ctx, b.tiles);
+    b.step_str = dalloc<u32>(ctx, breaks_steps(b.tiles, b.tp));
     b.brk = dalloc<u32>(ctx, b.tiles * b.tp / 32);
     b.sbm_words = b.tiles * b.tp / 32 + 2;  // positions 0 .. n inclusive
     b.sbm = dalloc<u32>(ctx, b.sbm_words);
     ck(ctx, cudaMemsetAsync(b.sbm, 0, b.sbm_words * sizeof(u32), ctx->st), "memset starts");
 }
 
-void alloc_table(lcg_ctx* ctx, RoundBufs& b, u64 cap) {
+// A phrase table of `cap` slots, and numbers for `claims` claims (at most 0.8
+// of the slots: past it the table is too full).  The blocks of the parse take
+// the numbers in ranges (a quarter of the claims that a block makes on
+// average, at least a warp's worth), of which each may leave one unused.
+void alloc_table(lcg_ctx* ctx, RoundBufs& b, u64 cap, u64 claims) {
     b.cap = cap;
+    claims = std::min(claims, cap - cap / 5);
+    const u64 blocks = std::min<u64>((u64)kParseBlocksMax * (u64)ctx->sms, (b.tiles + kParseWarps - 1) / kParseWarps);
+    b.id_chunk = (u32)std::min<u64>(2048, std::max<u64>(32, claims / (4 * std::max<u64>(1, blocks))));
+    b.id_cap = claims + blocks * b.id_chunk;
     b.tab = dalloc<unsigned char>(ctx, cap * slot_bytes());
-    b.rv = dalloc<u64>(ctx, cap);
-    b.claims = dalloc<u32>(ctx, cap);
+    b.crec = dalloc<unsigned char>(ctx, b.id_cap * claim_rec_bytes());
+    b.minpos = dalloc<u64>(ctx, b.id_cap);
+    b.rank_of = dalloc<u32>(ctx, b.id_cap);
     ck(ctx, cudaMemsetAsync(b.tab, 0xFF, cap * slot_bytes(), ctx->st), "memset table");
+    ck(ctx, cudaMemsetAsync(b.minpos, 0xFF, b.id_cap * sizeof(u64), ctx->st), "memset positions");
 }
 
 void free_table(lcg_ctx* ctx, RoundBufs& b) {
-    dfree(ctx, b.tab);
-    dfree(ctx, b.rv);
-    dfree(ctx, b.claims);
+    for (void* p : {(void*)b.tab, (void*)b.crec, (void*)b.minpos, (void*)b.rank_of}) dfree(ctx, p);
     b.tab = nullptr;
-    b.rv = nullptr;
-    b.claims = nullptr;
+    b.crec = nullptr;
+    b.minpos = nullptr;
+    b.rank_of = nullptr;
 }
 
-void alloc_naming(lcg_ctx* ctx, RoundBufs& b, u64 g_alloc) {
-    b.g_alloc = g_alloc;
-    const u64 nw = b.tiles * b.tp / 32;  // order keys tile * TP + q
-    b.first_bits = dalloc<u32>(ctx, nw);
-    b.first_prefix = dalloc<u32>(ctx, nw);
-    b.slot_r = dalloc<u32>(ctx, g_alloc);
-    b.len_r = dalloc<u32>(ctx, g_alloc);
-    b.xlen = dalloc<u64>(ctx, g_alloc);
-    b.mkey = dalloc<u64>(ctx, 2 * g_alloc);  // 16-byte keys
-    b.mval = dalloc<u64>(ctx, g_alloc);
-    b.rkey = dalloc<u64>(ctx, 2 * g_alloc);
-    ck(ctx, cudaMemsetAsync(b.first_bits, 0, nw * sizeof(u32), ctx->st), "memset bits");
+// Naming arrays for up to r_cap new rules and `phrases` phrases.
+void alloc_naming(lcg_ctx* ctx, RoundBufs& b, u64 r_cap, u64 phrases) {
+    b.r_cap = r_cap;
+    b.first_words = phrases / 32 + 1;
+    b.first = dalloc<uint2>(ctx, b.first_words);
+    b.rrec = dalloc<unsigned char>(ctx, r_cap * claim_rec_bytes());
+    ck(ctx, cudaMemsetAsync(b.first, 0, b.first_words * sizeof(uint2), ctx->st), "memset bits");
 }
 
 // Free a round's buffers except those that become the next round's input.
 void free_round(lcg_ctx* ctx, RoundBufs& b) {
-    for (void* p : {(void*)b.string_first, (void*)b.R_phr, (void*)b.R_sid, (void*)b.P_slot, (void*)b.tile_cnt,
-                    (void*)b.tile_pfx, (void*)b.tile_str, (void*)b.brk, (void*)b.sbm, (void*)b.first_bits,
-                    (void*)b.first_prefix,
-                    (void*)b.slot_r, (void*)b.len_r, (void*)b.xlen, (void*)b.mkey, (void*)b.mval, (void*)b.rkey})
+    for (void* p : {(void*)b.string_first, (void*)b.R_phr, (void*)b.R_sid, (void*)b.tile_cnt, (void*)b.tile_pfx,
+                    (void*)b.step_str, (void*)b.brk, (void*)b.sbm, (void*)b.first, (void*)b.rrec, (void*)b.tab,
+                    (void*)b.crec, (void*)b.minpos})
         dfree(ctx, p);
-    free_table(ctx, b);
 }
 
 // Bits that hold every rank below `count` (at least 1).
@@ -591,11 +596,12 @@ RoundArgs round_args(lcg_ctx* ctx, lcg_grammar* R, const RoundInput& in, RoundBu
     a.level = i;
     a.parse_blocks = ctx->tuning.parse_blocks_per_sm;
     a.stripes = ctx->tuning.tile_stripes;
-    a.miss_flush = ctx->tuning.miss_flush;
+    a.prev_base = in.prev_base;
+    a.rank_prev = in.rank_prev;
     a.tiles_bound = b.tiles;
     a.tp = b.tp;
     a.string_first = b.string_first;
-    a.tile_str = b.tile_str;
+    a.step_str = b.step_str;
     a.brk = b.brk;
     a.sbm = b.sbm;
     a.sbm_words = b.sbm_words;
@@ -607,12 +613,12 @@ RoundArgs round_args(lcg_ctx* ctx, lcg_grammar* R, const RoundInput& in, RoundBu
     a.total = ctx->tot_arr + 3 * (i - 1);  // [0] phrases; [1], [2] scratch of the scans
     a.d_tiles = &a.rc->tiles;
     a.d_gnew = &a.ds->claims;
+    a.d_ids = &a.ds->aux[1];
     a.d_Gnew = &a.ds->claim_len;
     a.soff_next = b.soff_next;
     a.sid_next = b.sid_next;
     a.R_phr = b.R_phr;
     a.R_sid = b.R_sid;
-    a.P_slot = b.P_slot;
     a.T_cap = b.Tcap;
     a.Tnext = b.Tnext;
     a.Fnext = b.Fnext;
@@ -623,45 +629,30 @@ RoundArgs round_args(lcg_ctx* ctx, lcg_grammar* R, const RoundInput& in, RoundBu
 
 void set_table(RoundArgs& a, RoundBufs& b) {
     a.tab = b.tab;
-    a.rv = b.rv;
     a.tab_cap = b.cap;
-    a.claims = b.claims;
-    a.claim_limit = b.cap - b.cap / 5;
+    a.id_cap = b.id_cap;
+    a.id_chunk = b.id_chunk;
+    a.crec = b.crec;
+    a.minpos = b.minpos;
+    a.rank_of = b.rank_of;
 }
 
-// Parse: tile strings, k_parse, tile scan, strings.
-void enqueue_parse(lcg_ctx* ctx, RoundArgs& a, u64 n_for_bytes) {
-    const Range range("parse, round", a.level);
-    if (!round_is_small(a)) {
-        const int ht = kt_begin(ctx, "k_tile_strings", 4.0 * (double)a.tiles_bound, a.level);
-        ck(ctx, launch_tile_strings(a, ctx->st), "k_tile_strings");
-        kt_end(ctx, ht);
-    }
+// The round's phrases: tile strings, breaks, tile scan, strings.  A short round
+// runs them with the parse (enqueue_parse).
+void enqueue_phrases(lcg_ctx* ctx, RoundArgs& a, u64 n_for_bytes) {
     // k_breaks' look-ahead words: a buffer of their own, so that no other
     // kernel's data can read as a head of this launch's epoch
     const u64 steps = breaks_steps(a.tiles_bound, a.tp);
     ensure_lb(ctx, &ctx->heads, &ctx->heads_steps, steps, steps * sizeof(u64));
     a.heads = reinterpret_cast<u64*>(ctx->heads);
     a.brk_epoch = ++ctx->epoch;
-    if (round_is_small(a)) {
-        // a short round: tile strings, breaks, parse, scan and strings in one cooperative launch
-        const int hs = kt_begin(ctx, "k_parse_small", 5.0 * (double)n_for_bytes, a.level);
-        const u64 bar = ctx->ctr_val;  // the grid barriers' counter values
-        ctx->ctr_val += (u64)kSmallParseBarriers * small_round_grid(a);
-        ck(ctx, launch_parse_small(a, bar, ctx->st), "k_parse_small");
-        kt_end(ctx, hs);
-        ctx->launches += 1;
-        return;
-    }
-    int hb = kt_begin(ctx, "k_breaks", (a.sym_bytes == 1 ? 1.0 : 4.0) * n_for_bytes + (double)n_for_bytes / 8.0, a.level);
+    if (round_is_small(a)) return;
+    const Range range("phrases, round", a.level);
+    const int ht = kt_begin(ctx, "k_tile_strings", 4.0 * (double)a.tiles_bound, a.level);
+    ck(ctx, launch_tile_strings(a, ctx->st), "k_tile_strings");
+    kt_end(ctx, ht);
+    int h = kt_begin(ctx, "k_breaks", (a.sym_bytes == 1 ? 1.0 : 4.0) * n_for_bytes + (double)n_for_bytes / 8.0, a.level);
     ck(ctx, launch_breaks(a, ctx->st), "k_breaks");
-    kt_end(ctx, hb);
-    const double tab_bytes = a.tab_cap * (double)slot_bytes();
-    const double tbytes = tab_bytes > kL2Bytes ? 32.0 * (double)n_for_bytes / 3.0 : 0.0;
-    int h = kt_begin(ctx, "k_parse",
-                     (a.sym_bytes == 1 ? 1.0 : 4.0) * n_for_bytes + (double)n_for_bytes / 8.0 +
-                         4.0 * (double)n_for_bytes / 3.0 + tbytes, a.level);
-    ck(ctx, launch_parse(a, ctx->st), "k_parse");
     kt_end(ctx, h);
     const u64 stiles = std::max<u64>(1, scan2_tiles_for(a.tiles_bound));
     ensure_lb(ctx, &ctx->lb2, &ctx->lb2_tiles, stiles, scan2_lb_bytes(stiles));
@@ -675,65 +666,77 @@ void enqueue_parse(lcg_ctx* ctx, RoundArgs& a, u64 n_for_bytes) {
     h = kt_begin(ctx, "k_strings", 40.0 * a.k, a.level);
     ck(ctx, launch_strings(a, ctx->st), "k_strings");
     kt_end(ctx, h);
-    ctx->launches += 5;
+    ctx->launches += 4;
 }
 
-// Naming and rewrite: mark, popcount scan, rank, length scan, rules, rewrite.
-void enqueue_naming(lcg_ctx* ctx, RoundArgs& a, RoundBufs& b, double g_bytes, double G_bytes, double P_bytes) {
-    const Range range("naming, round", a.level);
-    a.first_bits = b.first_bits;
-    a.first_prefix = b.first_prefix;
-    a.slot_r = b.slot_r;
-    a.len_r = b.len_r;
-    a.xlen = b.xlen;
-    a.mkey = b.mkey;
-    a.mval = b.mval;
-    a.rkey = b.rkey;
-    a.g_alloc = b.g_alloc;
-    const u64 g_grid = std::max<u64>(1, b.g_alloc);
+// Parse: the phrases' lookups, and the next sequence.
+void enqueue_parse(lcg_ctx* ctx, RoundArgs& a, u64 n_for_bytes) {
+    const Range range("parse, round", a.level);
     if (round_is_small(a)) {
-        // a short round: marks, popcount prefix, ranks, length scan, rules and rewrite in one
-        // cooperative launch
-        const int hs = kt_begin(ctx, "k_naming_small", 12.0 * P_bytes, a.level);
-        const u64 bar = ctx->ctr_val;
-        ctx->ctr_val += (u64)kSmallNamingBarriers * small_round_grid(a);
-        ck(ctx, launch_naming_small(a, b.tiles * b.tp / 32, g_grid, bar, ctx->st), "k_naming_small");
+        // a short round: tile strings, breaks, scan, strings and parse in one cooperative launch
+        const int hs = kt_begin(ctx, "k_parse_small", 5.0 * (double)n_for_bytes, a.level);
+        const u64 bar = ctx->ctr_val;  // the grid barriers' counter values
+        ctx->ctr_val += (u64)kSmallParseBarriers * small_round_grid(a);
+        ck(ctx, launch_parse_small(a, bar, ctx->st), "k_parse_small");
         kt_end(ctx, hs);
         ctx->launches += 1;
         return;
     }
-    int h = kt_begin(ctx, "k_mark", 12.0 * g_bytes, a.level);
+    const double tab_bytes = a.tab_cap * (double)slot_bytes();
+    const double tbytes = tab_bytes > kL2Bytes ? 32.0 * (double)n_for_bytes / 3.0 : 0.0;
+    const int h = kt_begin(ctx, "k_parse",
+                           (a.sym_bytes == 1 ? 1.0 : 8.0) * n_for_bytes + (double)n_for_bytes / 8.0 +
+                               8.0 * (double)n_for_bytes / 3.0 + tbytes, a.level);
+    ck(ctx, launch_parse(a, ctx->st), "k_parse");
+    kt_end(ctx, h);
+    ctx->launches += 1;
+}
+
+// Naming: mark, popcount scan, rank, rule offsets, rules.
+void enqueue_naming(lcg_ctx* ctx, RoundArgs& a, RoundBufs& b, double g_bytes, double G_bytes) {
+    const Range range("naming, round", a.level);
+    a.first = b.first;
+    a.first_words = b.first_words;
+    a.rrec = b.rrec;
+    a.r_cap = b.r_cap;
+    const u64 g_grid = std::max<u64>(1, b.r_cap);
+    if (round_is_small(a)) {
+        // a short round: marks, popcount prefix, ranks, offsets and rules in one cooperative launch
+        const int hs = kt_begin(ctx, "k_naming_small", 100.0 * g_bytes + 4.0 * G_bytes, a.level);
+        const u64 bar = ctx->ctr_val;
+        ctx->ctr_val += (u64)kSmallNamingBarriers * small_round_grid(a);
+        ck(ctx, launch_naming_small(a, bar, ctx->st), "k_naming_small");
+        kt_end(ctx, hs);
+        ctx->launches += 1;
+        return;
+    }
+    int h = kt_begin(ctx, "k_mark", 8.0 * g_bytes, a.level);
     ck(ctx, launch_mark(a, g_grid, ctx->st), "k_mark");
     kt_end(ctx, h);
-    const u64 nw = b.tiles * b.tp / 32;
-    const u64 ptiles = std::max<u64>(1, popscan_tiles_for(nw));
-    ensure_lb(ctx, &ctx->lb1, &ctx->lb1_tiles, ptiles, lb1_bytes(ptiles));
+    const u64 ptiles = std::max<u64>(1, popscan_tiles_for(b.first_words));
+    const u64 rtiles = rule_offs_tiles(g_grid);
+    const u64 lbt = std::max(ptiles, rtiles);
+    ensure_lb(ctx, &ctx->lb1, &ctx->lb1_tiles, lbt, lb1_bytes(lbt));
     a.lb1 = ctx->lb1;
     a.epoch = ++ctx->epoch;
     a.ctr_base = ctx->ctr_val;
     ctx->ctr_val += ptiles;
-    h = kt_begin(ctx, "k_popscan", 8.0 * (double)nw, a.level);
-    ck(ctx, launch_popscan(a, nw, ctx->st), "k_popscan");
+    h = kt_begin(ctx, "k_popscan", 12.0 * (double)b.first_words, a.level);
+    ck(ctx, launch_popscan(a, ctx->st), "k_popscan");
     kt_end(ctx, h);
-    h = kt_begin(ctx, "k_rank", 24.0 * g_bytes, a.level);
+    h = kt_begin(ctx, "k_rank", 76.0 * g_bytes, a.level);
     ck(ctx, launch_rank(a, g_grid, ctx->st), "k_rank");
     kt_end(ctx, h);
-    const u64 stiles = std::max<u64>(1, scan2_tiles_for(g_grid));
-    ensure_lb(ctx, &ctx->lb2, &ctx->lb2_tiles, stiles, scan2_lb_bytes(stiles));
-    u64 grid = 0;
-    h = kt_begin(ctx, "k_scan2", 12.0 * g_bytes, a.level);
-    ck(ctx, launch_scan2(b.len_r, nullptr, g_grid, b.xlen, nullptr, a.total + 1, ctx->lb2, ++ctx->epoch, ctx->ctr,
-                         ctx->ctr_val, a.ds, ctx->st, &grid, a.d_gnew),
-       "scan");
+    a.epoch = ++ctx->epoch;
+    a.ctr_base = ctx->ctr_val;
+    ctx->ctr_val += rtiles;
+    h = kt_begin(ctx, "k_rule_offs", 16.0 * g_bytes, a.level);
+    ck(ctx, launch_rule_offs(a, g_grid, ctx->st), "k_rule_offs");
     kt_end(ctx, h);
-    ctx->ctr_val += grid;
-    h = kt_begin(ctx, "k_rules", 4.0 * G_bytes + 12.0 * g_bytes, a.level);
+    h = kt_begin(ctx, "k_rules", 4.0 * G_bytes + 44.0 * g_bytes, a.level);
     ck(ctx, launch_rules(a, g_grid, ctx->st), "k_rules");
     kt_end(ctx, h);
-    h = kt_begin(ctx, "k_rewrite", 12.0 * P_bytes, a.level);
-    ck(ctx, launch_rewrite(a, ctx->st), "k_rewrite");
-    kt_end(ctx, h);
-    ctx->launches += 6;
+    ctx->launches += 5;
 }
 
 void next_input(lcg_ctx* ctx, RoundInput& in, RoundBufs& b) {
@@ -744,6 +747,9 @@ void next_input(lcg_ctx* ctx, RoundInput& in, RoundBufs& b) {
     in.own_offsets = true;
     if (in.S_owned) dfree(ctx, in.S_owned);
     if (in.Sf) dfree(ctx, (void*)in.Sf);
+    dfree(ctx, in.rank_prev);
+    in.rank_prev = b.rank_of;
+    in.prev_cap = b.id_cap;
     in.S = b.Tnext;
     in.S_owned = b.Tnext;
     in.Sf = b.Fnext;
@@ -754,6 +760,8 @@ void next_input(lcg_ctx* ctx, RoundInput& in, RoundBufs& b) {
 
 // One round with a host synchronisation after the parse: the table is
 // regrown and the parse rerun until it fits, and all later sizes are exact.
+constexpr u64 kExactNext = 1ull << 22;  // phrases
+
 void round_sync(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, bool against_resident, double& prev_ratio,
                 double& p_ratio) {
     fail_if(ctx, i >= ctx->levels || i > kMaxRounds,
@@ -771,9 +779,11 @@ void round_sync(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, bool agains
     RoundArgs a = round_args(ctx, R, in, b, i);
     a.d_n = nullptr;
     a.d_k = nullptr;
-    // inline keys as narrow as the level below allows; tables of resident
+    // inline keys as narrow as the symbols' ids allow; tables of resident
     // grammars keep the full width
-    if (i > 1 && !against_resident) a.sym_w = rank_width(R->lv[i - 2].g);
+    if (i > 1 && !against_resident) a.sym_w = rank_width(in.prev_base + in.prev_cap);
+    const u64 id_base = L.g;  // ids below it are ranks of resident rules
+    a.id_base = (u32)id_base;
     if (against_resident && L.g > 0) {
         ensure_resident(ctx, R, i, L.g);
         a.rtab = L.rtab;
@@ -796,13 +806,37 @@ void round_sync(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, bool agains
         cap = 2 * std::max<u64>(4096, std::min<u64>(P_est, (u64)(ratio * 1.3 * (double)P_est) + 1));
     }
     if (ctx->tuning.table_slots_max) cap = std::min<u64>(cap, ctx->tuning.table_slots_max);
+    // the claims' ids follow the resident ranks and are below 2^31; the claims
+    // that the table is expected to see, with slack (a round past them is rerun
+    // with a larger table)
+    const u64 max_ids = (kMaxRank + 1 - id_base) / 5 * 4;
+    const double g_hint = hint * ctx->p_hint[std::min<u32>(i, 63)] * (double)n * 1.5 + 1024;
     u32 retries = 0;
     DevStatus st;
     RoundCounts rc;
+    ck(ctx, cudaMemsetAsync(a.ds, 0, sizeof(DevStatus), ctx->st), "reset counters");
+    enqueue_phrases(ctx, a, n);
+    // The next sequence: at most Pmax symbols; a large one gets exactly the
+    // round's phrases, which the host then waits for (the short rounds' parse
+    // counts them itself).
+    u64 t_cap = b.Pmax;
+    if (!round_is_small(a) && t_cap > kExactNext) {
+        ck(ctx, cudaMemcpyAsync(&rc, a.rc, sizeof(rc), cudaMemcpyDeviceToHost, ctx->st), "read counts");
+        ck(ctx, cudaMemcpyAsync(&st, a.ds, sizeof(st), cudaMemcpyDeviceToHost, ctx->st), "read status");
+        sync(ctx);
+        check_device_status(ctx, st);
+        t_cap = rc.phrases + 1;
+    }
+    alloc_next(ctx, b, t_cap);
+    a.Tnext = b.Tnext;
+    a.Fnext = b.Fnext;
+    a.T_cap = b.Tcap;
     while (true) {
-        fail_if(ctx, cap > (kMaxRank + 1), LCG_ETABLE, "phrase table would exceed 2^31 slots");
-        alloc_table(ctx, b, cap);
-        ck(ctx, cudaMemsetAsync(a.ds, 0, sizeof(DevStatus), ctx->st), "reset counters");
+        fail_if(ctx, cap > kMaxRank + 1, LCG_ETABLE, "phrase table would exceed 2^31 slots");
+        // (a large table without a hint gets numbers for half its slots: they take
+        // more memory than the slots)
+        const u64 most = cap <= (1ull << 26) ? cap : std::max<u64>(cap / 2, (u64)g_hint);
+        alloc_table(ctx, b, cap, std::min<u64>(max_ids, most));
         set_table(a, b);
         enqueue_parse(ctx, a, n);
         ck(ctx, cudaMemcpyAsync(&rc, a.rc, sizeof(rc), cudaMemcpyDeviceToHost, ctx->st), "read counts");
@@ -811,8 +845,10 @@ void round_sync(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, bool agains
         check_device_status(ctx, st);
         if (!st.overflow) break;
         free_table(ctx, b);
+        fail_if(ctx, b.id_cap >= max_ids, LCG_EOVERFLOW, "level with 2^31 rules or more");
         cap *= 4;
         retries++;
+        ck(ctx, cudaMemsetAsync(a.ds, 0, sizeof(DevStatus), ctx->st), "reset counters");
     }
     const u64 P = rc.phrases;
     rs.phrases = P;
@@ -834,11 +870,7 @@ void round_sync(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, bool agains
     } else {
         L.rvalid = false;
     }
-    alloc_naming(ctx, b, g_new);
-    alloc_next(ctx, b, P + 1);  // the next sequence: exactly the round's phrases
-    a.Tnext = b.Tnext;
-    a.Fnext = b.Fnext;
-    a.T_cap = b.Tcap;
+    alloc_naming(ctx, b, g_new, P);
     a.g_base = L.g;
     a.G_base = L.G;
     a.cap_g = L.cap_g;
@@ -846,7 +878,8 @@ void round_sync(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, bool agains
     a.rhs = L.rhs;
     a.rhs_off = L.rhs_off;
     a.F = L.F;
-    enqueue_naming(ctx, a, b, (double)g_new, (double)G_new, (double)P);
+    enqueue_naming(ctx, a, b, (double)g_new, (double)G_new);
+    in.prev_base = (u32)id_base;
     L.g += g_new;
     L.G += G_new;
     free_round(ctx, b);
@@ -933,14 +966,16 @@ void rounds_async_enqueue(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, AsyncRou
         RoundArgs a = round_args(ctx, R, in, b, r);
         // a round stops early when the one before it failed
         if (r > 1) a.ds_prev = ctx->ds_arr + (r - 2);
-        // every rank of the level below is under its capacity
-        if (r > 1) a.sym_w = rank_width(R->lv[r - 2].cap_g);
-        alloc_table(ctx, b, p.cap);
+        // every id is under the claims that the round before may make
+        if (r > 1) a.sym_w = rank_width(in.prev_cap);
+        alloc_table(ctx, b, p.cap, p.g_alloc);
         set_table(a, b);
+        enqueue_phrases(ctx, a, p.n_est);
         enqueue_parse(ctx, a, p.n_est);
         grow_level(ctx, L, L.g + p.g_alloc, L.G + p.G_alloc);
         L.rvalid = false;
-        alloc_naming(ctx, b, p.g_alloc);
+        // the phrases: the planned next sequence and the strings that retire
+        alloc_naming(ctx, b, p.g_alloc, b.Tcap + kk);
         ar.g_base[r] = L.g;
         ar.G_base[r] = L.G;
         a.g_base = L.g;
@@ -950,7 +985,7 @@ void rounds_async_enqueue(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, AsyncRou
         a.rhs = L.rhs;
         a.rhs_off = L.rhs_off;
         a.F = L.F;
-        enqueue_naming(ctx, a, b, p.g_est, p.G_est, p.P_est);
+        enqueue_naming(ctx, a, b, p.g_est, p.G_est);
         free_round(ctx, b);
         next_input(ctx, in, b);
         in.d_n = &a.rc->n_next;
@@ -1137,10 +1172,10 @@ void capture_graph(lcg_ctx* ctx, const unsigned char* d_in, const std::vector<u6
     u64 t1 = 1, t2 = 1, hs = 1;
     for (u32 r = 1; r <= planned; r++) {
         const RoundPlan& p = plan[r];
-        const u32 tp = round_tile(ctx, p.n_alloc);
+        const u32 tp = parse_unit(round_tile(ctx, p.n_alloc));
         const u64 tiles = (p.n_alloc + tp - 1) / tp;
-        t1 = std::max({t1, tiles, popscan_tiles_for(tiles * tp / 32)});
-        t2 = std::max({t2, scan2_tiles_for(tiles), scan2_tiles_for(std::max<u64>(1, p.g_alloc))});
+        t1 = std::max({t1, tiles, popscan_tiles_for((p.t_cap + k) / 32 + 1), rule_offs_tiles(std::max<u64>(1, p.g_alloc))});
+        t2 = std::max(t2, scan2_tiles_for(tiles));
         hs = std::max(hs, breaks_steps(tiles, tp));
     }
     ensure_lb(ctx, &ctx->lb1, &ctx->lb1_tiles, t1, lb1_bytes(t1));

@@ -16,11 +16,12 @@ namespace lcg {
 // launch allowed (also inside stream capture, where it becomes a programmatic
 // edge of the graph).
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t st, Args&&... args) {
+cudaError_t launch_pdl_smem(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                            Args&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -29,16 +30,21 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStre
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t st, Args&&... args) {
+    return launch_pdl_smem(kernel, grid, block, 0, st, std::forward<Args>(args)...);
+}
 
 // A cooperative launch (every block resident at once: the kernel's blocks
 // may wait for one another), with programmatic dependent launch like the
 // others (the kernel's first steps wait for the grid before it).
 template <typename... KArgs, typename... Args>
-cudaError_t launch_coop(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t st, Args&&... args) {
+cudaError_t launch_coop(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                        Args&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeCooperative;
@@ -56,12 +62,19 @@ struct RoundCounts {
     u64 retired;  // strings that became one symbol
     u64 k_next;   // strings still active
     u64 n_next;   // |T^{i+1}|
-    u64 tiles;    // parse tiles of the round
+    u64 tiles;    // parse units of the round
     u64 pad[3];
 };
 
+// Symbols inside a build are ids, not yet ranks: an id of level i below the
+// round's id_base is the rank of a resident rule (id_base = the level's rules
+// before the round, 0 in a fresh build), and id_base + c names the round's
+// claim c (its c-th new phrase, in the order of the claims).  Ids are known as
+// soon as the phrase is looked up, so the parse writes T^{i+1} at once; the
+// ranks (first-occurrence order) are only needed for the rules' right-hand
+// sides and the roots, which are translated through rank_of.
 struct RoundArgs {
-    int sym_bytes;        // 1 in round 1 (bytes), 4 afterwards (ranks)
+    int sym_bytes;        // 1 in round 1 (bytes), 4 afterwards (ids)
     int sym_w;            // bits per symbol in the round's inline keys (every symbol < 2^sym_w)
     const void* S;        // T^i
     const u32* Sf;        // fingerprints of T^i (rounds >= 2)
@@ -75,19 +88,21 @@ struct RoundArgs {
     LevelHash lh;         // parameters of h^i
     u32 level;            // i
     u32 parse_blocks;     // resident k_parse blocks per SM (0: as many as fit)
-    u32 stripes;          // rounds >= 2: tiles taken in this many interleaved stripes (1: in order)
-    u32 miss_flush;       // byte rounds: queued cache misses that trigger a lookup pass
-    u32 tp;               // positions per parse tile (1024, 2048 or 4096): order keys are tile * tp + q
-    // parse pass
-    u64 tiles_bound;      // parse tiles the buffers were sized for
-    u64* d_tiles;         // parse tiles of the round (written by k_tile_strings)
-    u32* brk;             // break bitmap of T^i (k_breaks), 64 words per parse tile
+    u32 stripes;          // rounds >= 2: units taken in this many interleaved stripes (1: in order)
+    u32 tp;               // positions per parse unit (128, 256 or 512)
+    u32 prev_base;        // rounds >= 2: ids of T^i below it are ranks of level i-1
+    u32 id_base;          // ids of T^{i+1} below it are ranks of level i
+    const u32* rank_prev; // rounds >= 2: per claim of the round before, its rule's rank
+    // breaks
+    u64 tiles_bound;      // parse units the buffers were sized for
+    u64* d_tiles;         // parse units of the round (written by k_tile_strings)
+    u32* brk;             // break bitmap of T^i (k_breaks), one bit per position
     u32* sbm;             // bitmap of string starts of T^i (and of n)
     u64 sbm_words;
-    u32* tile_str;        // per parse tile: the string holding its first position
-    u32* tile_cnt;        // per parse tile: phrases starting in it
-    u64* tile_pfx;        // exclusive prefix of tile_cnt: global index of a tile's first phrase
-    u64* string_first;    // order key (tile * TP + q) of each active string's first phrase
+    u32* step_str;        // per block step of k_breaks: the string holding its first position
+    u32* tile_cnt;        // per parse unit: phrases starting in it
+    u64* tile_pfx;        // exclusive prefix of tile_cnt: global index of a unit's first phrase
+    u64* string_first;    // unit * tp + q of each active string's first phrase (q: its index in the unit)
     void* lb1;            // look-back slots
     u64 epoch;
     u64* heads;           // k_breaks: the head word of each block step (its own buffer)
@@ -96,59 +111,57 @@ struct RoundArgs {
     u64 ctr_base;
     u64* total;           // device: phrases of the round
     DevStatus* ds;
+    // strings
+    u64* soff_next;
+    u32* sid_next;
+    u64* R_phr;           // phrase indices (ascending) of the strings that became one phrase
+    u32* R_sid;           // their string indices
+    RoundCounts* rc;
+    const DevStatus* ds_prev;  // status of the round before (rounds enqueued without a sync), or null
+    // parse
     void* tab;            // the round's phrase table (32-byte slots)
     u64 tab_cap;
-    u64 claim_limit;
-    u32* claims;          // slots claimed in this round (tab_cap entries)
+    u64 id_cap;           // claim numbers (more: the table is regrown); crec, minpos and rank_of have as many entries
+    u32 id_chunk;         // claim numbers a block of the parse takes at a time
+    void* crec;           // claim c: its phrase's key and fingerprint (ClaimRec)
+    u64* minpos;          // claim c: its first occurrence (a phrase index), ~0 before
     void* rtab;           // table of the resident level i (read), or cap 0
     u64 rtab_cap;
     const u32* rrhs;
     const u64* rrhs_off;
-    u32* P_slot;          // per phrase (tile t's phrases from pslot_base(t) on): slot, or a
-                          // resident rank with the top bit set
-    // strings pass
-    u64* soff_next;
-    u32* sid_next;
-    u64* R_phr;
-    u32* R_sid;
-    RoundCounts* rc;
-    const DevStatus* ds_prev;  // status of the round before (rounds enqueued without a sync), or null
-    // naming pass
-    const u64* d_gnew;    // new rules of the round (device: the claim count)
+    u64 T_cap;            // entries of Tnext / Fnext
+    u32* Tnext;           // ids of T^{i+1}
+    u32* Fnext;           // fingerprints of T^{i+1}
+    u32* c_level;
+    u32* c_rank;
+    // naming
+    const u64* d_gnew;    // new rules of the round (device: the claims made)
+    const u64* d_ids;     // claim numbers taken (device): claims and a few unused numbers
     const u64* d_Gnew;    // their total length (device)
-    u64 g_alloc;          // entries of slot_r, len_r, xlen
     u64 cap_g, cap_G;     // capacity of the level's arrays
-    u32* first_bits;      // bitmap over phrase indices
-    u32* first_prefix;    // exclusive popcount prefix of its words
-    u32* slot_r;          // slot of the rank-r new rule
-    u32* len_r;           // its length
-    void* mkey;           // claim c: its slot's key (Key128), read once by k_mark
-    u64* mval;            // claim c: its slot's value (first occurrence)
-    void* rkey;           // key of the rank-r new rule (Key128), for k_rules
-    u64* rv;              // per table slot: (F^i << 32) | rank of its rule (k_rules, read by k_rewrite)
-    u64* xlen;            // exclusive prefix of len_r
+    u64 first_words;      // words of the first-occurrence bitmap
+    uint2* first;         // bitmap over phrase indices (x) and the exclusive popcount prefix of its words (y)
+    u64 r_cap;            // entries of rrec
+    void* rrec;           // the claim records in rank order
+    u32* rank_of;         // claim c: the rank of its rule
     u64 g_base, G_base;   // rules / rhs symbols of level i before this round
-
     u32* rhs;
     u64* rhs_off;
     u32* F;
     void* rtab_w;         // table of level i to extend with the new rules, or cap 0
     u64 rtab_w_cap;
-    // rewrite pass
-    u64 T_cap;            // entries of Tnext / Fnext
-    u32* Tnext;
-    u32* Fnext;           // fingerprints of T^{i+1}
-    u32* c_level;
-    u32* c_rank;
 };
 
 constexpr double kL2Bytes = 126.5 * 1024 * 1024;  // GB300 L2 (byte accounting, launch choices)
 bool parse_tile_valid(u32 tp);                 // 1024, 2048 or 4096 positions
+u32 parse_unit(u32 tile);                      // positions that each warp of a block takes of a tile
+constexpr u32 kParseBlocksMax = 4;             // k_parse blocks per SM at most (its launch bounds)
+constexpr u32 kParseWarps = 8;                 // warps of a block, a unit each
 bool round_is_small(const RoundArgs& a);        // the round runs as k_parse_small and k_naming_small
 u32 small_round_grid(const RoundArgs& a);       // their blocks (one launch of each per round)
-constexpr u32 kSmallParseBarriers = 3, kSmallNamingBarriers = 5;  // grid barriers of each
-u64 parse_slot_entries(u64 tiles, u64 strings, u32 tp);  // entries of P_slot for a round's tiles and strings
-u64 breaks_steps(u64 tiles, u32 tp);                     // k_breaks' block steps over a round's parse tiles
+constexpr u32 kSmallParseBarriers = 3, kSmallNamingBarriers = 4;  // grid barriers of each
+size_t claim_rec_bytes();                       // bytes of one ClaimRec
+u64 breaks_steps(u64 units, u32 tp);           // k_breaks' block steps over a round's parse units
 u64 popscan_tiles_for(u64 nw);
 size_t lb1_bytes(u64 tiles);
 size_t lb2_bytes(u64 tiles);
@@ -158,14 +171,15 @@ cudaError_t launch_tile_strings(const RoundArgs& a, cudaStream_t st);
 cudaError_t launch_breaks(const RoundArgs& a, cudaStream_t st);
 cudaError_t launch_parse(const RoundArgs& a, cudaStream_t st);
 cudaError_t launch_parse_small(const RoundArgs& a, u64 bar_base, cudaStream_t st);
-cudaError_t launch_naming_small(const RoundArgs& a, u64 nw, u64 g_bound, u64 bar_base, cudaStream_t st);
+cudaError_t launch_naming_small(const RoundArgs& a, u64 bar_base, cudaStream_t st);
 int parse_max_blocks(int sym_bytes);  // resident k_parse blocks per SM at most
 cudaError_t launch_strings(const RoundArgs& a, cudaStream_t st);
 cudaError_t launch_mark(const RoundArgs& a, u64 g_grid, cudaStream_t st);
-cudaError_t launch_popscan(const RoundArgs& a, u64 nw_bound, cudaStream_t st);
+cudaError_t launch_popscan(const RoundArgs& a, cudaStream_t st);
 cudaError_t launch_rank(const RoundArgs& a, u64 g_grid, cudaStream_t st);
+cudaError_t launch_rule_offs(const RoundArgs& a, u64 g_grid, cudaStream_t st);
+u64 rule_offs_tiles(u64 g);
 cudaError_t launch_rules(const RoundArgs& a, u64 g_grid, cudaStream_t st);
-cudaError_t launch_rewrite(const RoundArgs& a, cudaStream_t st);
 cudaError_t launch_level0(const unsigned char* data, const u64* pos, const u32* ids, u32 cnt, u32* c_level,
                           u32* c_rank, cudaStream_t st);
 cudaError_t launch_resident_build(const u32* rhs, const u64* rhs_off, u64 r0, u64 cnt, bool bytes, const u32* Fprev,

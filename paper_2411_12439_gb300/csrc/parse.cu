@@ -1,33 +1,39 @@
 // Kernels of one BuildGram round (Sec. 3.3) over all active strings of a
 // batch, and their host-side launchers.
 //
-// A round i reads the sequence T^i (bytes in round 1, uint32 ranks later) of
+// A round i reads the sequence T^i (bytes in round 1, uint32 ids later) of
 // the active strings, laid out back to back with offsets soff[0..k], and the
 // fingerprints of its symbols (F^0 of the bytes in round 1; afterwards the
-// fingerprint stream the previous round's rewrite wrote).  It runs:
-//   k_tile_strings  per parse tile, the string holding its first position, and
-//                   the bitmap of string starts
+// fingerprint stream the previous round's parse wrote).  It runs:
+//   k_tile_strings  per block step of k_breaks, the string holding its first
+//                   position, and the bitmap of string starts
 //   k_breaks   RandLMSPar break bits (Eq. rand_types) as a bitmap, 32
-//              positions per thread
-//   k_parse    per tile: the phrase starts (from the bitmap), a key per phrase
+//              positions per thread; the phrases of every parse unit; the
+//              first phrase of every string
+//   k_scan2    unit phrase counts -> global phrase indices (single pass)
+//   k_strings  per-string phrase ranges; strings that become one phrase retire
+//   k_parse    per unit: the phrase starts (from the bitmap), a key per phrase
 //              (its symbols when short, else a hash of its Eq. fast_hash
-//              polynomial and its position) and its slot in the round's
-//              phrase table, whose value is the smallest phrase index of the
-//              content (content-confirmed, never by hash alone)
-//   k_scan2    tile phrase counts -> global phrase indices (single pass)
-//   k_strings  per-string phrase ranges; strings that became one phrase retire
+//              polynomial and its position), its fingerprint F^i and its slot
+//              in the round's phrase table, whose value is the smallest phrase
+//              index of the content (content-confirmed, never by hash alone);
+//              T^{i+1} gets the slot's id and the fingerprint, retired strings
+//              left out
 //   k_mark, k_popscan, k_rank
 //              first-occurrence naming: the first occurrences of the new
 //              phrases are marked in a bitmap over phrase indices, and a
 //              phrase's rank is the number of marks before its own
-//   k_scan2    rule lengths -> right-hand-side offsets
-//   k_rules    the level-i rules in rank order: rhs, rhs_off and F^i, and the
-//              (F^i, rank) pair of every table slot
-//   k_rewrite  T^{i+1}[p] = rank of phrase p and its fingerprint, compacting
-//              retired strings
+//   k_rule_offs  rule lengths -> right-hand-side offsets
+//   k_rules    the level-i rules in rank order: rhs (ids translated to ranks)
+//              and F^i, and the ranks of the retired strings' roots
+// The sequence between the rounds holds ids (slots), not ranks, and the parse
+// computes a phrase's fingerprint from the stream it reads anyway.  Before,
+// a rewrite pass followed the naming and read (F^i, rank) of every phrase
+// from an array indexed by slot: one random DRAM sector per phrase in the
+// rounds whose table is beyond L2 (4 x 3.1 Gbp: 42.3 ms of 218 ms).
 // A short round (at most kSmallTiles tiles) runs the same steps as two
-// cooperative launches instead: k_parse_small (tile strings to strings) and
-// k_naming_small (marks to rewrite), with grid barriers between the steps.
+// cooperative launches instead: k_parse_small (tile strings to parse) and
+// k_naming_small (marks to rules), with grid barriers between the steps.
 // Every kernel of the round starts with pdl_wait(): it is launched with
 // programmatic dependent launch after the one before it.
 #include <algorithm>
@@ -38,22 +44,6 @@
 #include "table.cuh"
 
 namespace lcg {
-
-constexpr u32 kResidentBit = 0x80000000u;  // P_slot entry names a resident rank
-
-template <typename T>
-struct FpSource;  // fingerprint of a symbol
-
-template <>
-struct FpSource<unsigned char> {
-    const u32* F;  // shared-memory copy of F^0
-    __device__ __forceinline__ u32 operator()(unsigned char s) const { return F[s]; }
-};
-template <>
-struct FpSource<u32> {
-    const u32* F;  // F^{i-1} in global memory
-    __device__ __forceinline__ u32 operator()(u32 s) const { return __ldg(F + s); }
-};
 
 // Sizes of a round: from the device when the round was enqueued without a
 // host synchronisation, else from the arguments.
@@ -90,50 +80,46 @@ __device__ __forceinline__ u32 string_of(const u64* soff, u32 k, u64 pos) {
 // k_parse
 // --------------------------------------------------------------------------
 //
-// Persistent blocks take tiles of TP positions.  A tile's symbols (and kHalo
-// more) and its words of the break bitmap are staged in shared memory (byte
-// rounds read the next tile's into registers while parsing the current one);
-// the phrase starts are listed in order by a block scan.  Each phrase gets a
-// key: its symbols packed exactly when they fit in 124 bits, else a hash of
-// its polynomial fingerprint H (Eq. fast_hash) with its length and position,
-// confirmed by comparing contents.  It is looked up first in the resident
-// level (when parsing against a resident grammar), then in the round's table,
-// where a new content is claimed.  In byte rounds a per-block cache of packed
-// phrases (kept across the block's tiles) answers most lookups; the phrases
-// that miss are queued and looked up together, with full warps.  The slot of
-// phrase q of tile t goes to P_slot[pslot_base(t) + q] (its order key is
-// t * TP + q); new entries
-// (claims) are listed in shared memory and appended to the round's claim list
-// every few tiles.
+// The warps of a persistent grid take units of U positions (an eighth of
+// lcg_tuning.parse_tile: 128, 256 or 512) and never wait for one another.  A
+// warp copies its next unit's symbols (and kHalo more) to shared memory while
+// it parses the current one, and lists the unit's phrase starts from the
+// break bitmap.  Each phrase gets a key: its symbols packed exactly when they
+// fit in 124 bits, else a hash of its polynomial H (Eq. fast_hash) with its
+// length and position, confirmed by comparing contents.  It is looked up
+// first in the resident level (when parsing against a resident grammar and
+// all its symbols are resident), then in the round's table, where a new
+// content is claimed; the slot says the claim's number (the id) and the
+// fingerprint F^i.  Phrase p of the round goes to place p of T^{i+1}, less the
+// retired strings' phrases before it.
+//
+// Most phrases are answered with one read: in rank rounds of their home slot,
+// in byte rounds of a per-block cache of packed phrases.  What that read does not answer goes to the warp's queue,
+// with all that the long path needs (so the queue outlives the unit), and the
+// long path runs on 32 queued phrases at a time: fingerprint, probing, claim.
+//
+// What bounds it: the byte round instruction issue, the rank rounds random
+// 32-byte DRAM reads (one slot per phrase) and, with many new phrases, the
+// chain slot read -> compare-and-swap -> store of the long path.
 
-constexpr int kParseThreads = 256;
-// Positions per parse tile, TP: 1024, 2048 or 4096 (the default), a launch
-// parameter (lcg_tuning.parse_tile) that every kernel of a round reads from
-// RoundArgs::tp; k_parse is compiled for each.
-constexpr int kTPMin = 1024, kTPMax = 4096;
-// Rounds of at most kSmallTiles tiles of kTPMin positions run as two
-// cooperative launches (parse; naming and rewrite) whose steps are separated
-// by grid barriers, instead of eleven launches: launch latency, not work,
-// bounds such rounds.
-constexpr u64 kSmallTiles = 128;
-constexpr int kHalo = 64;          // positions staged past the tile end
+constexpr int kParseThreads = 32 * (int)kParseWarps;
+constexpr int kUnitMin = 128, kUnitMax = 512;
+// Rounds of at most kSmallUnits units of kUnitMin positions run as two
+// cooperative launches (parse; naming) whose steps are separated by grid
+// barriers, instead of ten launches: launch latency, not work, bounds such
+// rounds.
+constexpr u64 kSmallUnits = 1024;
+constexpr int kHalo = 64;  // symbols staged past the unit's end
 
-// Where the phrase slots of parse tile t begin in P_slot.  Every phrase but a
-// string's first is at least two symbols long, so a tile of TP positions in
-// which s strings start holds at most TP / 2 + 1 + s phrases.  With j0(t)
-// the string holding the tile's first position (tile_str[t]), s is at most
-// j0(t + 1) - j0(t) + 1, so tile t's slots can begin at t (TP / 2 + 2) + j0(t).
-__device__ __forceinline__ u64 pslot_base(u64 t, u32 j0, u32 tp) { return t * (u64)(tp / 2 + 2) + j0; }
-
-// Tile order of the rank rounds' parse and rewrite: with `stripes` = k > 1
+// Unit order of the rank rounds' parse: with `stripes` = k > 1
 // the round's tiles are cut into k equal stripes and taken interleaved
 // (stripe 0's first tile, stripe 1's first tile, ..., then every stripe's
 // second tile), so that strings which are near-copies of one another at the
 // same offsets (k assemblies of one genome) are parsed side by side and the
 // later copies find the first copy's new table entries still in L2.  Logical
 // tile l in [0, k * ceil(T / k)) names tile (l % k) * ceil(T / k) + l / k, or
-// nothing (>= T).  Phrase order keys stay tile * TP + q, so the result does
-// not depend on the order.
+// nothing (>= T).  Phrases keep their indices, so the result does not depend
+// on the order.
 __device__ __forceinline__ u64 stripe_tiles(u64 ntiles, u32 stripes) {
     if (stripes <= 1) return ntiles;
     const u64 per = (ntiles + stripes - 1) / stripes;
@@ -147,63 +133,19 @@ __device__ __forceinline__ u64 stripe_tile(u64 l, u64 ntiles, u32 stripes) {
 constexpr int kCacheBits = 11;
 constexpr int kCacheSlots = 1 << kCacheBits;  // per-block phrase cache (byte rounds)
 constexpr int kCacheProbes = 8;
-// New table entries of a block are listed in shared memory and appended to
-// the round's claim list once the buffer is half full, or in rank rounds once
-// another tile could overflow it (a tile claims at most TP entries), and
-// after the block's last tile, so that the global counter is touched every
-// few tiles only.
-constexpr int kClaimBufB = 512;   // byte rounds (shared memory also holds the phrase cache)
-constexpr int kClaimBufR = 4096;  // rank rounds
-// Byte rounds: phrases that miss the block's cache are queued with their keys
-// and looked up in the global table together once the queue is half full, so
-// that full warps run the long lookup path, every few tiles.
-constexpr int kMissBuf = 256;
-constexpr int kMissFlushDefault = 64;  // queued misses that trigger a lookup pass
-constexpr u64 kOkeyBits = 44;  // order keys are below 2^44
-// Table slots read per round trip.  One: a random DRAM read costs per 32-byte
-// sector (one slot), and at the default table load of 0.35 most lookups end
-// at their home slot; reading the home slot's group of two took more DRAM
-// sectors per lookup and was slower in the rank rounds, where those random
-// sectors bound k_parse.
-constexpr int kProbeGroup = 1;
-// Long phrases (hashed keys) in rank rounds: fingerprints read per round
-// trip for H, and symbols per round trip when a match is confirmed by content
-// (byte rounds read staged fingerprints and take one at a time).
-constexpr int kHornerBatchR = 8;
+// A cache entry's value: bits 58..63 an exponent x, bits 32..57 the id, the low
+// half F^1.  The phrase's first occurrence is known to be before 2^x, so a
+// phrase at place 2^x or later needs nothing more; the warps of a block are at
+// different places, and one before that takes the long path, which keeps the
+// first occurrence right.
+
+// Long phrases (hashed keys) in rank rounds: symbols per round trip when a
+// match is confirmed by content (byte rounds take one at a time).
 constexpr int kCompareBatchR = 4;
 // Phrases longer than kLongLen (N-runs of DNA, repeated text) are hashed and
-// compared by a whole warp after the tile's other phrases: a thread alone
-// would spend a round trip per symbol on them while its block waits.  Their
-// starts are more than kLongLen apart, so a tile holds at most
-// TP / (kLongLen + 1) + 1.
+// compared by a whole warp after the unit's other phrases: a thread alone
+// would spend a round trip per symbol on them while its warp waits.
 constexpr int kLongLen = 32;
-
-// Load n_sym symbols of type V from src (16-byte aligned when `vec`) into the
-// shared array dst, with every 16-byte load issued before any is stored.
-template <int SP, typename V>
-__device__ __forceinline__ void stage_vec(V* dst, const V* src, int n_sym, bool vec) {
-    constexpr int PER = 16 / sizeof(V);
-    constexpr int NV = (SP + PER - 1) / PER;
-    constexpr int IT = (NV + kParseThreads - 1) / kParseThreads;
-    uint4 buf[IT];
-#pragma unroll
-    for (int it = 0; it < IT; it++) {
-        const int x0 = (threadIdx.x + it * kParseThreads) * PER;
-        if (x0 + PER <= n_sym && vec) {
-            buf[it] = __ldcs(reinterpret_cast<const uint4*>(src + x0));  // streamed once: evict first
-        } else if (x0 < n_sym) {
-            V tmp[PER];
-#pragma unroll
-            for (int e = 0; e < PER; e++) tmp[e] = (x0 + e < n_sym) ? src[x0 + e] : (V)0;
-            buf[it] = *reinterpret_cast<const uint4*>(tmp);
-        }
-    }
-#pragma unroll
-    for (int it = 0; it < IT; it++) {
-        const int x0 = (threadIdx.x + it * kParseThreads) * PER;
-        if (x0 < n_sym) *reinterpret_cast<uint4*>(dst + x0) = buf[it];
-    }
-}
 
 // --------------------------------------------------------------------------
 // k_breaks: the round's break bitmap (Eq. rand_types)
@@ -234,7 +176,7 @@ __device__ __forceinline__ void stage_vec(V* dst, const V* src, int n_sym, bool 
 
 constexpr int kBrkThreads = 256;
 constexpr u64 kBrkSpan = (u64)kBrkThreads * 32;  // positions per block step
-static_assert(kBrkSpan % kTPMax == 0, "a block step starts a parse tile");
+static_assert(kUnitMax <= 32 * 32, "a warp of k_breaks covers whole parse units");
 
 // Head of block step b in the look-ahead words: (epoch << 8) | (state << 2) |
 // type, state 1 = open, 2 = decided.
@@ -292,6 +234,7 @@ __device__ __forceinline__ void body_breaks(const RoundArgs& a, u64 nblocks) {
     __shared__ u32 sF0[kByte ? 256 : 1];
     __shared__ u32 sst[SW + 1];      // string starts at base .. base + kBrkSpan
     __shared__ u32 sfirst[kBrkThreads];  // type of each thread's first position
+    __shared__ u32 s_bits[kBrkThreads], s_pre[kBrkThreads];
     __shared__ u64 s_step;
     __shared__ u32 s_open, s_carry;
     if (round_halted(a)) return;
@@ -422,574 +365,583 @@ __device__ __forceinline__ void body_breaks(const RoundArgs& a, u64 nblocks) {
         if (x0 < bend) {
             if (bend - x0 < 32) bits &= (1u << (bend - x0)) - 1u;
             a.brk[x0 >> 5] = bits;
-        }
-        __syncthreads();
-    }
-}
-
-// Exclusive scan of one 32-bit value per thread of a kParseThreads block, with
-// one barrier: every warp scans the warp totals itself.  `s_wsum` (one word
-// per warp) must not be written again before all threads have returned.
-__device__ __forceinline__ u32 block_scan32(u32 x, u32& total, u32* s_wsum) {
-    constexpr int NW = kParseThreads / 32;
-    const u32 lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    u32 incl = x;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const u32 y = __shfl_up_sync(0xffffffffu, incl, o);
-        if ((int)lane >= o) incl += y;
-    }
-    if (lane == 31) s_wsum[wid] = incl;
-    __syncthreads();
-    const u32 w = lane < (u32)NW ? s_wsum[lane] : 0u;
-    u32 wi = w;
-#pragma unroll
-    for (int o = 1; o < NW; o <<= 1) {
-        const u32 y = __shfl_up_sync(0xffffffffu, wi, o);
-        if ((int)lane >= o) wi += y;
-    }
-    total = __shfl_sync(0xffffffffu, wi, NW - 1);
-    return __shfl_sync(0xffffffffu, wi - w, wid) + incl - x;
-}
-
-template <typename T, int TP>
-__device__ __forceinline__ void body_parse(const RoundArgs& a, u64 ntiles) {
-    pdl_wait();
-    constexpr int kSP = TP + kHalo;  // staged positions
-    constexpr int NWS = kSP / 32;    // staged break words
-    constexpr int NWT = TP / 32;     // tile break words
-    constexpr int kLongBuf = TP / (kLongLen + 1) + 1;
-    constexpr bool kByte = sizeof(T) == 1;
-    constexpr bool kLocal = kByte;
-    static_assert(NWT <= kParseThreads, "one tile word per thread");
-    constexpr int kClaimBuf = kByte ? kClaimBufB : kClaimBufR;
-    constexpr int kHornerBatch = kByte ? 1 : kHornerBatchR;
-    constexpr int kCompareBatch = kByte ? 1 : kCompareBatchR;
-
-    __shared__ u32 sF0[kByte ? 256 : 1];
-    // bytes of tile positions (and 32 more: packed keys read whole 8-byte words past a phrase)
-    __shared__ __align__(16) unsigned char sb[kByte ? kSP + 32 : 16];
-    __shared__ __align__(16) u32 sT[kByte ? 4 : kSP];             // ranks of tile positions
-    __shared__ u32 sbits[NWS];
-    __shared__ u32 swp[NWT];
-    __shared__ unsigned short sP[TP];
-    // byte rounds: per-block cache of phrase (packed bytes) -> slot, kept across
-    // the block's tiles (its entries always come from earlier tiles)
-    __shared__ u64 ckey[kLocal ? kCacheSlots : 1];
-    __shared__ u32 cval[kLocal ? kCacheSlots : 1];
-    __shared__ u32 sClaim[kClaimBuf];
-    __shared__ u32 s_wsum[kParseThreads / 32];
-    // byte rounds: queued cache misses: key, and order key | (cache slot + 1) << kOkeyBits
-    // (half as many with 4096-position tiles, whose staged bytes and phrase
-    // list take that room: the block's static shared memory stays under 48 KB)
-    constexpr int kMissCap = TP >= 4096 ? kMissBuf / 2 : kMissBuf;
-    __shared__ Key128 sMissKey[kLocal ? kMissCap : 1];
-    __shared__ u64 sMissOk[kLocal ? kMissCap : 1];
-    __shared__ u64 sMissPs[kLocal ? kMissCap : 1];  // where the queued phrase's slot goes in P_slot
-    __shared__ u32 s_nmiss;
-    __shared__ unsigned short sLong[kLongBuf];  // tile offsets (q) of the tile's long phrases
-    __shared__ u32 s_nlong;
-    __shared__ u64 s_tail_end;
-    __shared__ u32 s_nclaim;
-    __shared__ u64 s_claim_len;
-    __shared__ u64 s_claim_base;
-
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const T* S = (const T*)a.S;
-    const u64 n = round_n(a);
-    const u32 kact = round_k(a);
-    const u64 nwords = (n + 31) / 32;  // words of the break bitmap
-    ntiles = min(ntiles, (n + TP - 1) / TP);
-    FpSource<T> fp;
-    if constexpr (kByte) {
-        for (int x = tid; x < 256; x += kParseThreads) sF0[x] = a.Fprev[x];
-        fp.F = sF0;
-    } else {
-        fp.F = a.Fprev;
-    }
-    const ContentTable bt{(Slot*)a.tab, a.tab_cap};
-    const ContentTable rt{(Slot*)a.rtab, a.rtab_cap};
-    if constexpr (kLocal) {
-        for (int x = tid; x < kCacheSlots; x += kParseThreads) {
-            ckey[x] = kEmpty;
-            cval[x] = ~0u;
-        }
-    }
-    if (tid == 0) {
-        s_nclaim = 0;
-        s_claim_len = 0;
-        s_nmiss = 0;
-        s_nlong = 0;
-    }
-
-    // persistent blocks: tiles blockIdx.x, blockIdx.x + gridDim.x, ...  Tiles
-    // do not depend on one another.
-    // Byte rounds: a tile's bytes (16 per thread and load), break words and
-    // string index are read into registers while the block parses the tile
-    // before it.
-    constexpr int kFetch = (kSP + 16 * kParseThreads - 1) / (16 * kParseThreads);  // 16-byte loads per thread
-    static_assert(NWS <= kParseThreads, "one break word per thread");
-    uint4 pf_sym[kFetch];
-#pragma unroll
-    for (int f = 0; f < kFetch; f++) pf_sym[f] = make_uint4(0u, 0u, 0u, 0u);
-    u32 pf_bits = 0, pf_j0 = 0;
-    auto fetch = [&](u64 tl) {
-        const u64 f0 = tl * (u64)TP;
-        const int fns = (int)(min(f0 + (u64)kSP, n) - f0);
-        const unsigned char* src = (const unsigned char*)S + f0;
-#pragma unroll
-        for (int f = 0; f < kFetch; f++) {
-            const int x0 = (tid + f * kParseThreads) * 16;
-            if (x0 + 16 <= fns && (reinterpret_cast<unsigned long long>(src) & 15) == 0) {
-                pf_sym[f] = __ldcs(reinterpret_cast<const uint4*>(src + x0));  // streamed once: evict first
-            } else if (x0 < fns) {
-                unsigned char tmp[16];
-#pragma unroll
-                for (int e = 0; e < 16; e++) tmp[e] = (x0 + e < fns) ? src[x0 + e] : (unsigned char)0;
-                pf_sym[f] = *reinterpret_cast<const uint4*>(tmp);
-            }
-        }
-        const u64 gw = f0 / 32 + (u64)tid;
-        pf_bits = (tid < NWS && gw < nwords) ? __ldg(a.brk + gw) : 0u;
-        pf_j0 = a.tile_str[tl];
-    };
-
-    u64 iter = 0;
-    // rank rounds may take their tiles in stripes (stripe_tile); byte rounds in order
-    const u32 stripes = kByte ? 1u : a.stripes;
-    const u64 nlog = stripe_tiles(ntiles, stripes);
-    for (u64 lt = blockIdx.x; lt < nlog; lt += gridDim.x, iter++) {
-        if ((iter & 15) == 0 && round_halted(a)) break;
-        const u64 tile = stripe_tile(lt, ntiles, stripes);
-        const bool last = lt + gridDim.x >= nlog;  // the block's last tile
-        if (tile >= ntiles) continue;  // no tile here (claims still buffered are flushed after the loop)
-        const u64 t0 = tile * (u64)TP;
-        const u64 t_end = min(t0 + (u64)TP, n), s_end = min(t0 + (u64)kSP, n);
-        const int ns = (int)(s_end - t0), nt = (int)(t_end - t0);
-
-        // 1. stage the tile's symbols (bytes in round 1, ranks afterwards) and
-        //    its break words (k_breaks)
-        u32 j0;  // string holding t0
-        if constexpr (kByte) {
-            if (iter == 0) fetch(tile);
-#pragma unroll
-            for (int f = 0; f < kFetch; f++) {
-                const int x0 = (tid + f * kParseThreads) * 16;
-                if (x0 < ns) *reinterpret_cast<uint4*>(sb + x0) = pf_sym[f];
-            }
-            if (tid < NWS) sbits[tid] = pf_bits;
-            j0 = pf_j0;
-            if (tile + gridDim.x < ntiles) fetch(tile + gridDim.x);  // byte rounds: in order
         } else {
-            j0 = a.tile_str[tile];
-            stage_vec<kSP, u32>(sT, S + t0, ns, (reinterpret_cast<unsigned long long>(S + t0) & 15) == 0);
-            for (int w = tid; w < NWS; w += kParseThreads) {
-                const u64 gw = t0 / 32 + (u64)w;
-                sbits[w] = gw < nwords ? __ldg(a.brk + gw) : 0u;
+            bits = 0;
+        }
+        // phrases of each parse unit (a unit is a.tp / 32 lanes of one warp)
+        const u32 lpu = a.tp / 32;
+        u32 ucnt = (u32)__popc(bits);
+        for (u32 o = 1; o < lpu; o <<= 1) ucnt += __shfl_xor_sync(0xffffffffu, ucnt, (int)o);
+        if ((lane & (int)(lpu - 1)) == 0 && x0 < bend) a.tile_cnt[x0 / a.tp] = ucnt;
+        // the first phrase of every string that starts in the step: its index
+        // among its unit's phrases
+        if (__syncthreads_or((int)(st & bits))) {
+            u32 pre = (u32)__popc(bits);
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const u32 y = __shfl_up_sync(0xffffffffu, pre, o);
+                if (lane >= o) pre += y;
+            }
+            pre -= (u32)__popc(bits);
+            s_bits[tid] = bits;
+            s_pre[tid] = pre - __shfl_sync(0xffffffffu, pre, lane & ~(int)(lpu - 1));
+            __syncthreads();
+            const u32 kact = round_k(a);
+            for (u32 jj = a.step_str[b] + (u32)tid;; jj += kBrkThreads) {
+                const u64 s = jj < kact ? __ldg(a.soff + jj) : ~0ull;
+                if (s >= base && s < bend) {
+                    const u32 x = (u32)(s - base);
+                    a.string_first[jj] = s / a.tp * a.tp + s_pre[x >> 5] +
+                                         __popc(s_bits[x >> 5] & ((1u << (x & 31)) - 1u));
+                }
+                if (__shfl_sync(0xffffffffu, s < bend ? 1u : 0u, 31) == 0) break;
             }
         }
-        // offsets of the strings from j0 on, for step 5 (read now, used at the tile's end)
-        const u64 s_first = (warp == 0 && j0 + lane < kact) ? __ldg(a.soff + j0 + lane) : ~0ull;
-        const u64 pb0 = pslot_base(tile, j0, TP);  // the tile's phrase slots in P_slot
-        __syncthreads();
+    }
+}
 
-        // 3. phrase starts of the tile, in order: kTPW threads per break
-        //    word, kBPT bits each
-        constexpr int kTPW = kParseThreads / NWT, kBPT = 32 / kTPW;
-        static_assert(kTPW * NWT == kParseThreads && kTPW * kBPT == 32 && kBPT < 32, "threads per tile word");
-        const int wq = tid / kTPW, bq = (tid % kTPW) * kBPT;
-        u32 word = sbits[wq];
-        if (wq * 32 >= nt) word = 0;
-        else if (nt - wq * 32 < 32) word &= (1u << (nt - wq * 32)) - 1u;
-        const u32 part = (word >> bq) & ((1u << kBPT) - 1u);
-        u32 cnt;
-        const u32 poff = block_scan32((u32)__popc(part), cnt, s_wsum);
-        if (tid % kTPW == 0) swp[wq] = (u32)poff;
-        {
-            u32 m = part, o = (u32)poff;
-            while (m) {
-                const int b = __ffs(m) - 1;
-                m &= m - 1;
-                sP[o++] = (unsigned short)(wq * 32 + bq + b);
+// What the parse's functions take from RoundArgs, in shared memory (they are not
+// inlined, and a kernel's parameters passed by reference are read through
+// generic addresses).
+struct ParseArgs {
+    const void* S;
+    const u32* Sf;
+    u32* Tnext;
+    u32* Fnext;
+    u64 T_cap, retired;
+    LevelHash lh;
+    RoundTable table;
+    u64 rtab_cap;
+    const RoundArgs* all;  // for what is seldom needed
+    u32 sym_w, inline_most, find_inline, id_base, prev_base;
+};
+
+// Shared memory of a k_parse block (dynamic).  A warp's part holds its unit's
+// symbols (and those of the unit it takes next), phrase starts and queue.
+template <typename T, int U>
+struct ParseSmem {
+    static constexpr bool kByte = sizeof(T) == 1;
+    static constexpr int kSP = U + kHalo;            // staged symbols
+    // phrase starts: a phrase has two symbols or more unless it is a string's
+    // first, and a string in a round two or more, so at most two phrases start
+    // in three positions; one more entry for the end of the last
+    static constexpr int kStarts = (2 * U / 3 + 2 + 7) / 8 * 8;
+    struct Warp {
+        __align__(16) T sym[2][kSP];  // (packed byte keys read whole 8-byte words past a phrase)
+        ulonglong2 queue[32 + 31];
+        u64 claims, claim_len;  // what the warp claimed
+        unsigned short start[kStarts];
+    };
+    Warp w[kParseThreads / 32];
+    ClaimIds ids;
+    ParseArgs args;
+    // byte rounds: the block's phrase cache, packed bytes -> CacheVal
+    u64 ckey[kByte ? kCacheSlots : 1];
+    u64 cval[kByte ? kCacheSlots : 1];
+    u32 sF[kByte ? 256 : 1];  // byte rounds: F^0
+};
+
+// A queued phrase: where it starts in S, its length, what is known of its home
+// slot, and the cache slot it may take (0: none); with its index p.
+constexpr int kPosBits = 44;  // positions and phrase indices are below 2^44
+__device__ __forceinline__ u64 queue_word(u64 pos, u32 len, u32 home, u32 cache) {
+    return pos | ((u64)len << kPosBits) | ((u64)home << (kPosBits + 6)) | ((u64)cache << (kPosBits + 8));
+}
+static_assert(kLongLen < 64 && kCacheBits + 1 <= 64 - kPosBits - 8, "queue word");
+
+// First index with R_phr >= p (the phrases of the strings that retire, ascending).
+__device__ __noinline__ u64 retired_before(const RoundArgs& a, u64 p) {
+    u64 lo = 0, hi = a.rc->retired;
+    while (lo < hi) {
+        const u64 mid = (lo + hi) >> 1;
+        if (a.R_phr[mid] < p) lo = mid + 1; else hi = mid;
+    }
+    return lo;
+}
+
+// Phrase p becomes a symbol of T^{i+1}, or the root of its string, when
+// strings retire this round (or there is no room).
+__device__ __noinline__ void emit_slow(const RoundArgs& a, u64 p, u32 id, u32 F) {
+    const u64 lo = retired_before(a, p);
+    if (lo < a.rc->retired && a.R_phr[lo] == p) {
+        a.c_level[a.R_sid[lo]] = a.level;
+        a.c_rank[a.R_sid[lo]] = id;  // k_rules makes it a rank
+        return;
+    }
+    if (p - lo >= a.T_cap) {
+        set_error(a.ds, kErrCapacity);
+        return;
+    }
+    __stcs(a.Tnext + (p - lo), id);
+    __stcs(a.Fnext + (p - lo), F);
+}
+
+template <typename T, int U>
+__device__ __forceinline__ ParseSmem<T, U>& parse_smem() {
+    static_assert((sizeof(ParseSmem<T, U>) + 1024) * kParseBlocksMax <= 228 * 1024, "shared memory of an SM");
+    extern __shared__ __align__(16) unsigned char dyn_smem[];
+    return *reinterpret_cast<ParseSmem<T, U>*>(dyn_smem);
+}
+
+// The resident rank of a phrase given its key (a hashed key names the
+// phrase's position in S), or ~0.
+template <typename T>
+__device__ __noinline__ u64 find_resident(const RoundArgs& a, const Key128& key) {
+    const T* S = (const T*)a.S;
+    const u64 len = key_len(key), pos = key.lo;
+    return table_find(ContentTable{(Slot*)a.rtab, a.rtab_cap}, key, key_is_hashed(key), [&](u64 rank) {
+        const u64 o = a.rrhs_off[rank];
+        for (u64 j = 0; j < len; j++)
+            if ((u32)S[pos + j] != a.rrhs[o + j]) return false;
+        return true;
+    });
+}
+
+// The phrase that a hashed key names (at pos) against the one at ref, kBatch
+// symbols per round trip.
+template <typename T, int kBatch>
+__device__ __noinline__ bool same_content(const T* S, u64 pos, u64 len, u64 ref) {
+    for (u64 j = 0; j < len; j += kBatch) {
+        T x[kBatch], y[kBatch];
+#pragma unroll
+        for (int u = 0; u < kBatch; u++) {
+            const bool in = j + u < len;
+            x[u] = in ? S[ref + j + u] : (T)0;
+            y[u] = in ? S[pos + j + u] : (T)0;
+        }
+#pragma unroll
+        for (int u = 0; u < kBatch; u++)
+            if (x[u] != y[u]) return false;
+    }
+    return true;
+}
+
+// A phrase of more than kLongLen symbols at `pos`, by the whole warp: the
+// fingerprint polynomial H (Eq. fast_hash) and the content comparisons of its
+// hashed key are spread over the lanes.
+template <typename T, int U>
+__device__ __noinline__ void parse_long(u64 pos, u64 len, u64 p) {
+    ParseSmem<T, U>& sm = parse_smem<T, U>();
+    const RoundArgs& a = *sm.args.all;
+    const T* S = (const T*)a.S;
+    const u32 lane = threadIdx.x & 31;
+    auto& w = sm.w[threadIdx.x >> 5];
+    if (len > kMaxPhraseLen) {
+        if (lane == 0) set_error(a.ds, kErrPhraseLong);
+        return;
+    }
+    const u64 H = warp_poly61([&](u64 j) -> u64 {
+        if constexpr (sizeof(T) == 1) return sm.sF[S[pos + j]];
+        else return __ldg(a.Sf + pos + j);
+    }, len, a.lh.c);
+    const u32 F = finish_hash(a.lh, H);
+    const Key128 key = key_hashed(H, len, pos);
+    const ContentTable rt{(Slot*)a.rtab, a.rtab_cap};
+    u64 r = ~0ull;
+    if (rt.cap)
+        r = table_find_warp(rt, key, [&](u64 rank) {
+            const u64 o = a.rrhs_off[rank];
+            return warp_equal([&](u64 j) { return (u32)S[pos + j]; }, [&](u64 j) { return a.rrhs[o + j]; }, len);
+        });
+    u64 pub = kNoPub;
+    if (r == ~0ull) {
+        ClaimSum sum{0, 0};
+        pub = table_resolve_warp(sm.args.table, &sm.ids, sum, key, p, F, [&](u64 ref) {
+            return warp_equal([&](u64 j) { return S[ref + j]; }, [&](u64 j) { return S[pos + j]; }, len);
+        });
+        __syncwarp();
+        if (lane == 0) {
+            w.claims += sum.count;
+            w.claim_len += sum.len;
+        }
+        __syncwarp();
+    }
+    if (lane == 0) {
+        if (r != ~0ull) emit_slow(a, p, (u32)r, F);
+        else if (pub != kNoPub) emit_slow(a, p, a.id_base + (u32)pub, (u32)(pub >> 32));
+    }
+}
+
+// The long path on the warp's queued phrases first .. first + take - 1 (at
+// most 32): fingerprint, resident lookup, find or claim, and the symbol of
+// T^{i+1}.  Not inlined, so that the loop over the units keeps its registers.
+template <typename T, int U>
+__device__ __noinline__ void parse_queued(u32 first, u32 take) {
+    ParseSmem<T, U>& sm = parse_smem<T, U>();
+    const ParseArgs& a = sm.args;
+    constexpr bool kByte = sizeof(T) == 1;
+    const T* S = (const T*)a.S;
+    const u32 lane = threadIdx.x & 31;
+    auto& w = sm.w[threadIdx.x >> 5];
+    const bool act = lane < take;
+    ulonglong2 e = make_ulonglong2(0ull, 0ull);
+    if (act) e = w.queue[first + lane];
+    const u64 pos = e.x & ((1ull << kPosBits) - 1), p = e.y;
+    const u32 plen = (u32)(e.x >> kPosBits) & 63u, home = (u32)(e.x >> (kPosBits + 6)) & 3u;
+    Key128 k;
+    u64 H = 0;
+    bool res = a.rtab_cap != 0;  // a phrase with a symbol that is new in this build is no resident rule
+    {
+        // four symbols from the last on at a time: H by Horner, and the packed symbols
+        PackedSyms ps;
+        for (u32 j = plen; j > 0;) {
+            const u32 m = min(j, 4u);
+            u32 v[4], f[4];
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                v[u] = f[u] = 0;
+                if ((u32)u < m) {
+                    v[u] = (u32)__ldg(S + pos + j - 1 - u);
+                    if constexpr (!kByte) f[u] = __ldg(a.Sf + pos + j - 1 - u);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; u++)
+                if ((u32)u < m) {
+                    if constexpr (kByte) f[u] = sm.sF[v[u]];
+                    else res = res && v[u] < a.prev_base;
+                    ps.push(v[u], a.sym_w);
+                    H = addmod61(mulmod61(H, a.lh.c), (u64)f[u]);
+                }
+            j -= m;
+        }
+        k = plen <= a.inline_most ? ps.key(plen) : key_hashed(H, plen, pos);
+    }
+    const u32 F = finish_hash(a.lh, H);
+    u64 r = ~0ull;
+    if (act && res) r = find_resident<T>(*a.all, k);
+    u64 first_occ = r != ~0ull ? 0 : p;  // a bound of its first occurrence
+    ClaimSum sum{0, 0};
+    const u64 pub = table_resolve(a.table, &sm.ids, sum, act && r == ~0ull, home, k, p, F, first_occ, [&](u64 ref) {
+        return same_content<T, kByte ? 1 : kCompareBatchR>(S, k.lo, key_len(k), ref);
+    });
+    const u32 count = __reduce_add_sync(0xffffffffu, sum.count), len = __reduce_add_sync(0xffffffffu, sum.len);
+    if (lane == 0) {
+        w.claims += count;
+        w.claim_len += len;
+    }
+    if (act && (r != ~0ull || pub != kNoPub)) {
+        const u32 id = r != ~0ull ? (u32)r : a.id_base + (u32)pub;
+        if constexpr (kByte) {
+            // into the cache, valid from a place after its first occurrence on
+            const u32 ch = (u32)(e.x >> (kPosBits + 8));
+            if (ch && id < (1u << 26)) {
+                const u64 ck = ((u64)plen << 56) | (k.hi & ((1ull << (8 * plen)) - 1));
+                if (atomicCAS((unsigned long long*)&sm.ckey[ch - 1], (unsigned long long)kEmpty,
+                              (unsigned long long)ck) == kEmpty)
+                    *(volatile u64*)&sm.cval[ch - 1] = ((u64)(64 - __clzll((long long)first_occ)) << 58) |
+                                                       ((u64)id << 32) | F;
             }
         }
-        if (tid == 0) {
-            // end of the tile's last phrase: the first phrase start at or after t_end
-            u64 e = n;
-            bool found = false;
-            for (int w = nt >> 5; w < (ns + 31) >> 5 && !found; w++) {
-                u32 m = sbits[w];
-                if (w == (nt >> 5)) m &= ~((1u << (nt & 31)) - 1u);
-                if (m) { e = t0 + (u64)(w * 32 + __ffs(m) - 1); found = true; }
-            }
-            // past the staged words (s_end < n is then a multiple of 32): the
-            // bitmap in global memory
-            for (u64 gw = s_end / 32; !found && s_end < n && gw < nwords; gw++) {
-                const u32 m = __ldg(a.brk + gw);
-                if (m) { e = min(n, gw * 32 + (u64)(__ffs(m) - 1)); found = true; }
-            }
-            s_tail_end = e;
+        if (a.retired == 0 && p < a.T_cap) {
+            __stcs(a.Tnext + p, id);
+            __stcs(a.Fnext + p, F);
+        } else {
+            emit_slow(*a.all, p, id, F);
         }
-        __syncthreads();
+    }
+    __syncwarp();
+}
 
-        // 4. lookups.  A phrase's order key is tile * TP + q: it orders phrases
-        //    like their global index.
-        const u64 tail = s_tail_end - t0;
-        const u32 cntq = (u32)cnt;
-        const u64 okey0 = tile * (u64)TP;
-        auto phrase_end = [&](u32 q) -> u64 { return (q + 1 < cntq) ? (u64)sP[q + 1] : tail; };
-        auto sym = [&](u64 x) -> u32 {  // symbol at tile offset x
-            if (x < (u64)ns) {
-                if constexpr (kByte) return (u32)sb[x]; else return sT[x];
-            }
-            return (u32)S[t0 + x];
-        };
-        // the slot of phrase q = [st, en); *claimed when this call made the entry
-        // key of phrase [st, en) (tile offsets); *ok = false for one too long
-        auto make_key = [&](u64 st, u64 en, bool* ok) -> Key128 {
-            const u64 len = en - st;
-            *ok = len <= kMaxPhraseLen;
-            if (!*ok) {
-                set_error(a.ds, kErrPhraseLong);
-                return Key128{0, 0};
-            }
-            if (len > inline_max(a.sym_w)) {
-                // H = sum_j F[Q_j] c^{j-1} mod p, by Horner from the last symbol;
-                // the fingerprints (staged F^0 of bytes, or the round's
-                // fingerprint stream) are read kHornerBatch at a time
-                u64 H = 0;
-                for (u64 x = en; x > st;) {
-                    const u64 c = min((u64)kHornerBatch, x - st);
-                    u32 f[kHornerBatch];
-#pragma unroll
-                    for (int u = 0; u < kHornerBatch; u++) {
-                        if ((u64)u < c) {
-                            if constexpr (kByte) f[u] = fp((unsigned char)sym(x - 1 - u));
-                            else f[u] = __ldg(a.Sf + t0 + x - 1 - u);
-                        } else {
-                            f[u] = 0;
-                        }
-                    }
-#pragma unroll
-                    for (int u = 0; u < kHornerBatch; u++)
-                        if ((u64)u < c) H = addmod61(mulmod61(H, a.lh.c), (u64)f[u]);
-                    x -= c;
-                }
-                return key_hashed(H, len, t0 + st);
-            }
-            return key_inline([&](u64 j) { return sym(st + j); }, len, a.sym_w);
-        };
-        // The slot of a phrase given its key and order key (a hashed key names
-        // the phrase's position in S); *claimed when this call made the entry.
-        auto lookup_key = [&](const Key128& key, u64 okey, bool* claimed) -> u32 {
-            *claimed = false;
-            const bool hashed = key_is_hashed(key);
-            const u64 len = key_len(key), pos = key.lo;
-            if (rt.cap) {
-                const u64 r = table_find(rt, key, hashed, [&](u64 rank) {
-                    const u64 o = a.rrhs_off[rank];
-                    for (u64 j = 0; j < len; j++)
-                        if ((u32)S[pos + j] != a.rrhs[o + j]) return false;
-                    return true;
-                });
-                if (r != ~0ull) return kResidentBit | (u32)r;
-            }
-            return (u32)table_claim_or_find<kByte ? 1 : kProbeGroup>(bt, key, hashed, okey, [&](u64 ref) {
-                // both contents in global memory, kCompareBatch symbols per round trip
-                for (u64 j = 0; j < len; j += kCompareBatch) {
-                    T x[kCompareBatch], y[kCompareBatch];
-#pragma unroll
-                    for (int u = 0; u < kCompareBatch; u++) {
-                        const bool in = j + u < len;
-                        x[u] = in ? S[ref + j + u] : (T)0;
-                        y[u] = in ? S[pos + j + u] : (T)0;
-                    }
-#pragma unroll
-                    for (int u = 0; u < kCompareBatch; u++)
-                        if (x[u] != y[u]) return false;
-                }
-                return true;
-            }, claimed, a.ds);
-        };
-        auto lookup = [&](u32 q, u64 st, u64 en, bool* claimed) -> u32 {
-            bool ok;
-            const Key128 key = make_key(st, en, &ok);
-            if (!ok) {
-                *claimed = false;
-                return ~0u;
-            }
-            return lookup_key(key, okey0 + q, claimed);
-        };
-        // New entries join the block's claim buffer (or, when it is full, the
-        // round's list at once).  claim_warp is called by all lanes of a warp
-        // together and makes one shared-memory update per warp.
-        auto claim_one = [&](u32 slot, u64 len, u32 c) {
-            if (c < (u32)kClaimBuf) {
-                sClaim[c] = slot;
-            } else {
-                const u64 g = atomicAdd(&a.ds->claims, 1ull);
-                if (g < bt.cap) a.claims[g] = slot;
-            }
-        };
-        auto claim_warp = [&](bool claimed, u32 slot, u64 len) {
-            const unsigned m = __ballot_sync(0xffffffffu, claimed);
-            if (m == 0) return;
-            u64 sum = claimed ? len : 0;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-            const int leader = __ffs(m) - 1;
-            u32 base = 0;
-            if (lane == leader) {
-                base = atomicAdd(&s_nclaim, (u32)__popc(m));
-                atomicAdd(&s_claim_len, sum);
-            }
-            base = __shfl_sync(0xffffffffu, base, leader);
-            if (claimed) claim_one(slot, len, base + (u32)__popc(m & ((1u << lane) - 1u)));
-        };
-        auto claim_single = [&](u32 slot, u64 len) {
-            atomicAdd(&s_claim_len, len);
-            claim_one(slot, len, atomicAdd(&s_nclaim, 1u));
-        };
-        auto defer_long = [&](u32 q) {
-            const u32 x = atomicAdd(&s_nlong, 1u);
-            if (x < (u32)kLongBuf) sLong[x] = (unsigned short)q;
-            else set_error(a.ds, kErrCapacity);  // not reached: long phrases start > kLongLen apart
-        };
-
-        if constexpr (kLocal) {
-            // Short phrases go through the block's cache.  Its entries come
-            // from earlier tiles of the block, whose phrases precede this
-            // tile's: a hit needs nothing more.  Misses are queued with their
-            // keys and looked up in the global table together once the queue
-            // is half full (and after the block's last tile).
-            const u64* sb64 = reinterpret_cast<const u64*>(sb);
-            // packed bytes of a phrase of length <= 7 inside the staged bytes
-            auto short_key = [&](u32 st, u32 len) -> u64 {
-                const u32 w = st >> 3, sh = (st & 7) * 8;
-                const u64 lo = sb64[w], hi = sb64[w + 1];
-                const u64 v = sh ? (lo >> sh) | (hi << (64 - sh)) : lo;
-                return ((u64)len << 56) | (v & ((1ull << (8 * len)) - 1));
-            };
-            // the inline key of a phrase of length <= kInlineMax inside the staged
-            // bytes: its bytes as one little-endian number B, B mod 2^60 (with
-            // the length above) in hi and B >> 60 in lo (the layout of
-            // key_inline for 8-bit symbols)
-            auto byte_key = [&](u32 st, u32 len) -> Key128 {
-                const u32 w = st >> 3, sh = (st & 7) * 8;
-                const u64 x0 = sb64[w], x1 = sb64[w + 1], x2 = sb64[w + 2];
-                u64 b0 = sh ? (x0 >> sh) | (x1 << (64 - sh)) : x0;
-                u64 b1 = sh ? (x1 >> sh) | (x2 << (64 - sh)) : x1;
-                if (len < 8) {
-                    b0 &= (1ull << (8 * len)) - 1;
-                    b1 = 0;
-                } else if (len < 16) {
-                    b1 &= (1ull << (8 * (len - 8))) - 1;
-                }
-                return Key128{(b0 >> 60) | (b1 << 4), (b0 & ((1ull << 60) - 1)) | ((u64)len << 60)};
-            };
-            for (u32 q = tid; q < cntq; q += kParseThreads) {
-                const u32 st = sP[q];
-                const u64 en = phrase_end(q);
-                const u64 len = en - st;
-                if (len > (u64)kLongLen) {  // a whole warp takes it below
-                    defer_long(q);
-                    continue;
-                }
-                u32 slot = ~0u;
-                int free_h = -1;
-                if (len <= 7 && en <= (u64)ns) {
-                    const u64 key = short_key(st, (u32)len);
-                    u32 h = (u32)((key * 0x9E3779B97F4A7C15ull) >> (64 - kCacheBits));
+// The first read for the phrases of a unit from q0 on: cache or home slot.
+// What that does not answer joins the warp's nq queued phrases; stops when 32
+// are queued.  `span`: q0 | (the unit's phrases) << 16.  Returns the next
+// phrase, the queue's length (bits 10..17) and whether there was a long phrase
+// (bit 18).  Not inlined, and without calls: this loop keeps every value in
+// registers (inlined beside the long path it spilled: the byte round of
+// 4 x 3.1 Gbp took 52.7 ms, now 37.1).  One phrase per thread at a time: with
+// two in flight round 2 of the same took 45.2 ms (44.4), with four 52.2: the
+// rounds with large tables are bound by random sectors, not by their latency.
+template <typename T, int U>
+__device__ __noinline__ u32 parse_unit_find(u32 buf, u64 t0, u64 p0, u64 out, u32 span, u32 nq, bool direct) {
+    using Smem = ParseSmem<T, U>;
+    Smem& sm = parse_smem<T, U>();
+    const ParseArgs& a = sm.args;
+    constexpr bool kByte = Smem::kByte;
+    const u32 lane = threadIdx.x & 31;
+    typename Smem::Warp& w = sm.w[threadIdx.x >> 5];
+    const T* sym = w.sym[buf];
+    volatile u64* ckey = sm.ckey;
+    volatile u64* cval = sm.cval;
+    const u32 find_inline = a.find_inline, id_base = a.id_base;
+    const int sym_w = (int)a.sym_w;
+    Slot* const slots = a.table.slots;
+    const u64 cap = a.table.cap;
+    u32* Tn = a.Tnext + out;
+    u32* Fn = a.Fnext + out;
+    auto emit = [&](u32 q, u32 id, u32 F) {
+        __stcs(Tn + q, id);
+        __stcs(Fn + q, F);
+    };
+    constexpr u32 kDone = 3, kLong = 4;  // else the home state of a phrase to be queued
+    const u32 cnt = span >> 16;
+    u32 q0 = span & 0xFFFFu, longs = 0;
+    for (; q0 < cnt && nq < 32; q0 += 32) {
+        const u32 q = q0 + lane;
+        u32 state = kDone, cache = 0, st = 0, len = 0;
+        if (q < cnt) {
+            st = w.start[q];
+            len = w.start[q + 1] - st;
+            state = len > (u32)kLongLen ? kLong : kHomeUnknown;
+            if constexpr (kByte) {
+                if (len <= 7 && direct) {
+                    // the packed bytes of the phrase
+                    const u64* s64 = reinterpret_cast<const u64*>(sym) + (st >> 3);
+                    const u32 sh = (st & 7) * 8;
+                    const u64 lo = s64[0], hi = s64[1];
+                    const u64 v = sh ? (lo >> sh) | (hi << (64 - sh)) : lo;
+                    const u64 k = ((u64)len << 56) | (v & ((1ull << (8 * len)) - 1));
+                    u32 h = (u32)((k * 0x9E3779B97F4A7C15ull) >> (64 - kCacheBits));
                     for (int probe = 0; probe < kCacheProbes; probe++) {
-                        const u64 k = ckey[h];
-                        if (k == key) {
-                            slot = cval[h];
+                        const u64 ck = ckey[h];
+                        if (ck == k) {
+                            const u64 cv = cval[h];
+                            // (not yet written, or first seen after this place: the long path)
+                            if (cv != ~0ull && ((p0 + q) >> (cv >> 58)) != 0) {
+                                state = kDone;
+                                emit(q, (u32)(cv >> 32) & ((1u << 26) - 1), (u32)cv);
+                            }
                             break;
                         }
-                        if (k == kEmpty) {
-                            free_h = (int)h;
+                        if (ck == kEmpty) {
+                            cache = h + 1;
                             break;
                         }
                         h = (h + 1) & (kCacheSlots - 1);
                     }
                 }
-                if (slot == ~0u) {
-                    bool ok = true;
-                    const Key128 key = (len <= (u64)kInlineMax && en <= (u64)ns) ? byte_key(st, (u32)len) : make_key(st, en, &ok);
-                    if (ok) {
-                        const u32 m = atomicAdd(&s_nmiss, 1u);
-                        if (m < (u32)kMissCap) {
-                            sMissKey[m] = key;
-                            sMissOk[m] = (okey0 + q) | ((u64)(free_h + 1) << kOkeyBits);
-                            sMissPs[m] = pb0 + q;
-                            continue;
-                        }
-                        bool claimed;  // queue full: at once (no cache entry)
-                        slot = lookup_key(key, okey0 + q, &claimed);
-                        if (claimed) claim_single(slot, len);
-                    }
+            } else if (len <= find_inline && direct) {
+                const Key128 key = key_inline32(sym + st, len, sym_w);
+                const Slot c = ld_slot_relaxed(&slots[key_home(key, cap)]);
+                if (c.key.hi == key.hi && c.key.lo == key.lo && c.pub != kUnpublished && c.val <= p0 + q) {
+                    state = kDone;
+                    emit(q, id_base + (u32)c.pub, (u32)(c.pub >> 32));
+                } else if (c.key.hi == kEmptyHi) {
+                    state = kHomeEmpty;
+                } else if (c.key.hi != key.hi) {
+                    state = kHomeOther;
                 }
-                __stcs(a.P_slot + pb0 + q, slot);
-            }
-            __syncthreads();
-            const u32 nq = s_nmiss;
-            if (nq >= min(a.miss_flush ? a.miss_flush : (u32)kMissFlushDefault, (u32)kMissCap) ||
-                last) {
-                const u32 nm = min(nq, (u32)kMissCap);
-                for (u32 i0 = 0; i0 < nm; i0 += kParseThreads) {  // whole warps take each step
-                    const u32 i = i0 + tid;
-                    bool claimed = false;
-                    u32 slot = ~0u;
-                    u64 len = 0;
-                    if (i < nm) {
-                        const Key128 key = sMissKey[i];
-                        const u64 meta = sMissOk[i];
-                        const u64 okey = meta & ((1ull << kOkeyBits) - 1);
-                        const int free_h = (int)(meta >> kOkeyBits) - 1;
-                        len = key_len(key);
-                        slot = lookup_key(key, okey, &claimed);
-                        if (free_h >= 0 && slot != ~0u && !(slot & kResidentBit)) {
-                            // inline byte key of length <= 7 -> the cache's packed form
-                            const u64 ck = (len << 56) | (key.hi & ((1ull << (8 * len)) - 1));
-                            const u64 old = atomicCAS((unsigned long long*)&ckey[free_h], (unsigned long long)kEmpty,
-                                                      (unsigned long long)ck);
-                            if (old == kEmpty) cval[free_h] = slot;
-                        }
-                        __stcs(a.P_slot + sMissPs[i], slot);
-                    }
-                    claim_warp(claimed, slot, len);
-                }
-                __syncthreads();
-                if (tid == 0) s_nmiss = 0;
-            }
-        } else {
-            for (u32 q0 = 0; q0 < cntq; q0 += kParseThreads) {  // whole warps take each step
-                const u32 q = q0 + tid;
-                bool claimed = false;
-                u32 slot = ~0u;
-                u64 len = 0;
-                if (q < cntq) {
-                    const u64 st = sP[q], en = phrase_end(q);
-                    len = en - st;
-                    if (len > (u64)kLongLen) {  // a whole warp takes it below
-                        defer_long(q);
-                        len = 0;
-                    } else {
-                        slot = lookup(q, st, en, &claimed);
-                        __stcs(a.P_slot + pb0 + q, slot);
-                    }
-                }
-                claim_warp(claimed, slot, len);
+                // else: another key, one being written, or a first occurrence
+                // that may be here: the long path reads the slot again
             }
         }
-        __syncthreads();
-
-        // 4b. long phrases, one warp each: the fingerprint polynomial H
-        //     (Eq. fast_hash) and the content comparisons of a hashed key are
-        //     spread over the warp's lanes
-        const u32 nlong = s_nlong;
-        for (u32 i = warp; i < nlong; i += kParseThreads / 32) {
-            const u32 q = sLong[i];
-            const u64 st = sP[q], en = phrase_end(q), len = en - st;
-            const u64 pos = t0 + st;  // the phrase's position in S
-            u32 slot = ~0u;
-            bool claimed = false;
-            if (len > kMaxPhraseLen) {
-                if (lane == 0) set_error(a.ds, kErrPhraseLong);
-            } else {
-                u64 H;
-                if constexpr (kByte) {
-                    H = warp_poly61([&](u64 j) -> u64 { return fp((unsigned char)sym(st + j)); }, len, a.lh.c);
-                } else {
-                    H = warp_poly61([&](u64 j) -> u64 { return __ldg(a.Sf + pos + j); }, len, a.lh.c);
-                }
-                const Key128 key = key_hashed(H, len, pos);
-                u64 r = ~0ull;
-                if (rt.cap)
-                    r = table_find_warp(rt, key, [&](u64 rank) {
-                        const u64 o = a.rrhs_off[rank];
-                        return warp_equal([&](u64 j) { return (u32)S[pos + j]; },
-                                          [&](u64 j) { return a.rrhs[o + j]; }, len);
-                    });
-                if (r != ~0ull) {
-                    slot = kResidentBit | (u32)r;
-                } else {
-                    slot = (u32)table_claim_or_find_warp(bt, key, okey0 + q, [&](u64 ref) {
-                        return warp_equal([&](u64 j) { return S[ref + j]; }, [&](u64 j) { return S[pos + j]; }, len);
-                    }, &claimed, a.ds);
-                }
-            }
-            if (lane == 0) {
-                __stcs(a.P_slot + pb0 + q, slot);
-                if (claimed) claim_single(slot, len);
-            }
-        }
-        if (nlong) {
-            __syncthreads();
-            if (tid == 0) s_nlong = 0;
-            __syncthreads();
-        }
-
-        // 5. outputs: phrase slots (from pb0 on), the tile's phrase count, and
-        //    the order key of the first phrase of every string starting here
-        if (tid == 0) a.tile_cnt[tile] = cntq;
-        if (warp == 0) {
-            for (u32 jj = j0 + lane;; jj += 32) {
-                const u64 s = (jj == j0 + lane) ? s_first : (jj < kact) ? __ldg(a.soff + jj) : ~0ull;
-                if (s >= t0 && s < t_end) {
-                    const int x = (int)(s - t0);
-                    a.string_first[jj] = okey0 + swp[x >> 5] + __popc(sbits[x >> 5] & ((1u << (x & 31)) - 1u));
-                }
-                if (__shfl_sync(0xffffffffu, (jj < kact && s < t_end) ? 1u : 0u, 31) == 0) break;
-            }
-        }
-        // 6. the block's new entries join the round's claim list when the
-        //    buffer is half full, and after the block's last tile
-        const u32 ncl = s_nclaim;
-        constexpr u32 kFlushAt = kByte ? (u32)kClaimBuf / 2 : (u32)(kClaimBuf - TP);
-        static_assert(kByte || kClaimBufR >= TP, "a rank-round tile never overflows the buffer");
-        if (ncl >= kFlushAt || last) {
-            const u32 nb = min(ncl, (u32)kClaimBuf);
-            if (tid == 0 && ncl) {
-                const u64 base = atomicAdd(&a.ds->claims, (u64)nb);
-                s_claim_base = base;
-                atomicAdd(&a.ds->claim_len, s_claim_len);
-                if (base + nb > a.claim_limit) atomicExch(&a.ds->overflow, 1u);
-            }
-            __syncthreads();
-            if (nb) {
-                const u64 base = s_claim_base;
-                for (u32 x = tid; x < nb; x += kParseThreads)
-                    if (base + x < bt.cap) a.claims[base + x] = sClaim[x];
-            }
-            __syncthreads();
-            if (tid == 0) {
-                s_nclaim = 0;
-                s_claim_len = 0;
-            }
-        }
-        __syncthreads();
+        const unsigned m = __ballot_sync(0xffffffffu, state < kDone);
+        if (state < kDone)
+            w.queue[nq + __popc(m & ((1u << lane) - 1u))] =
+                make_ulonglong2(queue_word(t0 + st, len, state, cache), p0 + q);
+        nq += (u32)__popc(m);
+        longs |= __ballot_sync(0xffffffffu, state == kLong);
+        __syncwarp();
     }
-    // claims still buffered: a block whose last logical tiles were empty
-    // (striped order) did not flush after its last tile
-    __syncthreads();
-    const u32 ncl = s_nclaim;
-    if (ncl) {
-        const u32 nb = min(ncl, (u32)kClaimBuf);
-        if (tid == 0) {
-            const u64 base = atomicAdd(&a.ds->claims, (u64)nb);
-            s_claim_base = base;
-            atomicAdd(&a.ds->claim_len, s_claim_len);
-            if (base + nb > a.claim_limit) atomicExch(&a.ds->overflow, 1u);
+    return min(q0, cnt) | (nq << 10) | ((longs ? 1u : 0u) << 18);
+}
+
+template <typename T, int U>
+__device__ __forceinline__ void body_parse(const RoundArgs& a, u64 nunits) {
+    pdl_wait();
+    using Smem = ParseSmem<T, U>;
+    constexpr bool kByte = Smem::kByte;
+    constexpr int kSP = Smem::kSP;
+    constexpr int kWords = U / 32;  // break words of a unit
+    constexpr int kBits = U / 32;   // positions per lane in the phrase list
+    static_assert(kWords + kHalo / 32 <= 32 && kHalo % 32 == 0 && kBits <= 32, "a unit's break words fit one per lane");
+    static_assert(kHalo > kLongLen, "a phrase that is not long lies in the staged symbols");
+    Smem& sm = parse_smem<T, U>();
+    const u32 lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    typename Smem::Warp& w = sm.w[warp];
+
+    const T* S = (const T*)a.S;
+    const u64 n = round_n(a);
+    const u64 nwords = (n + 31) / 32;  // words of the break bitmap
+    nunits = min(nunits, (n + U - 1) / U);
+    const u64 nr = a.rc->retired;
+    u32 nq = 0;  // the warp's queued phrases
+    if constexpr (kByte) {
+        for (int x = threadIdx.x; x < 256; x += kParseThreads) sm.sF[x] = a.Fprev[x];
+        for (int x = threadIdx.x; x < kCacheSlots; x += kParseThreads) {
+            sm.ckey[x] = kEmpty;
+            sm.cval[x] = ~0ull;
         }
-        __syncthreads();
-        const u64 base = s_claim_base;
-        for (u32 x = tid; x < nb; x += kParseThreads)
-            if (base + x < bt.cap) a.claims[base + x] = sClaim[x];
+    }
+    if (threadIdx.x == 0) {
+        ParseArgs& pa = sm.args;
+        pa.S = a.S;
+        pa.Sf = a.Sf;
+        pa.Tnext = a.Tnext;
+        pa.Fnext = a.Fnext;
+        pa.T_cap = a.T_cap;
+        pa.retired = nr;
+        pa.lh = a.lh;
+        pa.table = RoundTable{(Slot*)a.tab, a.tab_cap, a.minpos, (ClaimRec*)a.crec, a.id_cap, a.id_chunk, a.ds};
+        pa.rtab_cap = a.rtab_cap;
+        pa.all = &a;
+        pa.sym_w = (u32)a.sym_w;
+        pa.inline_most = (u32)inline_max(a.sym_w);
+        pa.find_inline = a.rtab_cap ? 0u : pa.inline_most;  // phrases looked up in the table at once
+        pa.id_base = a.id_base;
+        pa.prev_base = a.prev_base;
+    }
+    if (threadIdx.x == 0) sm.ids = ClaimIds{0, 0, 0};
+    if (lane == 0) {
+        w.claims = w.claim_len = 0;
+    }
+    __syncthreads();
+
+    // The warps of the grid take units in turn (rank rounds in stripes when
+    // asked) and wait for no other: unit lt of the logical order.
+    const u32 stripes = kByte ? 1u : a.stripes;
+    const u32 nlog = (u32)stripe_tiles(nunits, stripes), step = gridDim.x * (kParseThreads / 32);
+    // A unit's symbols go to buffer b; its break words (one per lane) and first
+    // phrase index to registers.
+    u32 nx_bits = 0;
+    u64 nx_p0 = 0;
+    auto fetch = [&](u32 lt, u32 b) {
+        const u64 unit = lt < nlog ? stripe_tile(lt, nunits, stripes) : ~0ull;
+        if (unit < nunits) {
+            const u64 f0 = unit * (u64)U;
+            const u32 ns = (u32)(min(f0 + (u64)kSP, n) - f0);
+            const T* src = S + f0;
+            constexpr u32 PER = 16 / sizeof(T);
+            const bool vec = (reinterpret_cast<unsigned long long>(src) & 15) == 0;
+            for (u32 x = lane * PER; x < ns; x += 32 * PER) {
+                if (x + PER <= ns && vec) {
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                                     (u32)__cvta_generic_to_shared(&w.sym[b][x])),
+                                 "l"(src + x)
+                                 : "memory");
+                } else {
+                    T v[PER];
+#pragma unroll
+                    for (u32 e = 0; e < PER; e++) v[e] = x + e < ns ? src[x + e] : (T)0;
+#pragma unroll
+                    for (u32 e = 0; e < PER; e++) w.sym[b][x + e] = v[e];  // (kSP is a multiple of PER)
+                }
+            }
+            const u64 gw = f0 / 32 + lane;
+            nx_bits = (lane < kWords + kHalo / 32 && gw < nwords) ? __ldg(a.brk + gw) : 0u;
+            nx_p0 = a.tile_pfx[unit];
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+
+    u32 lt = blockIdx.x * (kParseThreads / 32) + warp;
+    fetch(lt, 0);
+    for (u32 iter = 0;; lt += step, iter++) {
+        const bool have = lt < nlog;  // past the last unit: the queue is emptied
+        if (!have && nq == 0) break;
+        // a round that has failed stops early
+        if ((iter & 15) == 0) {
+            u32 h = 0;
+            if (lane == 0) {
+                h = vload(&a.ds->error) | vload(&a.ds->overflow);
+                if (a.ds_prev) h |= vload(&a.ds_prev->error) | vload(&a.ds_prev->overflow);
+            }
+            if (__shfl_sync(0xffffffffu, h, 0)) break;
+        }
+        const u64 unit = have ? stripe_tile(lt, nunits, stripes) : ~0ull;
+        const u32 bits = nx_bits;
+        const u64 p0 = nx_p0;  // the unit's first phrase
+        fetch(lt + step, (iter + 1) & 1);
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncwarp();
+        const u64 t0 = unit * (u64)U;
+
+        // 1. phrase starts of the unit, in order, kBits positions per lane
+        u32 cnt = 0;
+        u64 tail = 0;  // end of the last phrase
+        if (unit < nunits) {  // (none in a gap of the striped order)
+            const u32 nt = (u32)(min(t0 + (u64)U, n) - t0);
+            u32 part = __shfl_sync(0xffffffffu, bits, (int)(lane * kBits / 32)) >> (lane * kBits % 32);
+            if (kBits < 32) part &= (1u << (kBits & 31)) - 1u;
+            const u32 x0 = lane * kBits;
+            if (x0 >= nt) part = 0;
+            else if (nt - x0 < (u32)kBits) part &= (1u << (nt - x0)) - 1u;
+            u32 o = (u32)__popc(part);
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const u32 y = __shfl_up_sync(0xffffffffu, o, d);
+                if (lane >= (u32)d) o += y;
+            }
+            cnt = __shfl_sync(0xffffffffu, o, 31);
+            o -= (u32)__popc(part);
+            if (cnt >= (u32)Smem::kStarts) {  // not reached: a phrase but a string's first has two symbols
+                if (lane == 0) set_error(a.ds, kErrCapacity);
+                cnt = part = 0;
+            }
+            for (; part; part &= part - 1) w.start[o++] = (unsigned short)(x0 + (u32)__ffs(part) - 1);
+            // the first phrase start at or after the unit's end: in the break
+            // words after the unit, else further on in the bitmap
+            const u32 h0 = __shfl_sync(0xffffffffu, bits, kWords), h1 = __shfl_sync(0xffffffffu, bits, kWords + 1);
+            if (nt < (u32)U) tail = nt;
+            else if (h0) tail = (u64)U + (u32)__ffs(h0) - 1;
+            else if (h1) tail = (u64)U + 32 + (u32)__ffs(h1) - 1;
+            else {
+                tail = n - t0;
+                for (u64 gw = t0 / 32 + kWords + 2; gw < nwords; gw += 32) {
+                    const u32 x = gw + lane < nwords ? __ldg(a.brk + gw + lane) : 0u;
+                    const unsigned m = __ballot_sync(0xffffffffu, x != 0);
+                    if (m) {
+                        const int l = __ffs(m) - 1;
+                        tail = (gw + (u64)l) * 32 + (u32)__ffs(__shfl_sync(0xffffffffu, x, l)) - 1 - t0;
+                        break;
+                    }
+                }
+            }
+            if (lane == 0) w.start[cnt] = (unsigned short)min(tail, (u64)0xFFFF);
+        }
+        __syncwarp();
+
+        // 2. lookups: what the cache or the home slot does not answer is queued
+        //    (with all that the long path needs, so the queue outlives the
+        //    unit), and whenever 32 phrases are queued the warp runs the long
+        //    path on them.
+        // Where the unit's phrases go in T^{i+1}; a unit in which a string
+        // retires (or that does not fit) leaves all of them to the long path,
+        // which looks each place up.
+        u64 out = p0;
+        bool direct = true;
+        if (nr) {
+            const u64 r0 = retired_before(a, p0);
+            direct = r0 == nr || a.R_phr[r0] >= p0 + cnt;
+            out -= r0;
+        }
+        direct = direct && out + cnt <= a.T_cap;
+        bool longs = false;
+        for (u32 q0 = 0;;) {
+            if (q0 < cnt) {
+                const u32 r = parse_unit_find<T, U>(iter & 1, t0, p0, out, q0 | (cnt << 16), nq, direct);
+                q0 = r & 0x3FFu;
+                nq = (r >> 10) & 0xFFu;
+                longs = longs || (r >> 18) != 0;
+            }
+            if (nq < 32 && (have || nq == 0)) break;  // (the whole unit has been looked at)
+            const u32 take = min(nq, 32u);
+            nq -= take;
+            parse_queued<T, U>(nq, take);
+        }
+
+        // 3. long phrases, one at a time by the whole warp
+        if (longs) {
+            for (u32 q0 = 0; q0 < cnt; q0 += 32) {
+                const u32 q = q0 + lane;
+                u32 m = __ballot_sync(0xffffffffu, q < cnt && w.start[q + 1] - w.start[q] > kLongLen);
+                for (; m; m &= m - 1) {
+                    const u32 x = q0 + (u32)__ffs(m) - 1;
+                    const u64 st = w.start[x], en = x + 1 < cnt ? (u64)w.start[x + 1] : tail;
+                    parse_long<T, U>(t0 + st, en - st, p0 + x);
+                }
+            }
+        }
+        __syncwarp();
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    if (lane == 0 && w.claims) {
+        atomicAdd(&a.ds->claims, w.claims);
+        atomicAdd(&a.ds->claim_len, w.claim_len);
     }
 }
 
-// Per parse tile: the string that holds its first position.
+// Per block step of k_breaks: the string that holds its first position.
 __device__ __forceinline__ void body_tile_strings(const RoundArgs& a, u64 tiles) {
     pdl_wait();
     const u64 n = round_n(a);
@@ -1003,9 +955,9 @@ __device__ __forceinline__ void body_tile_strings(const RoundArgs& a, u64 tiles)
             set_error(a.ds, kErrCapacity);
     }
     if (round_halted(a)) return;
-    tiles = min(tiles, nt);
-    for (u64 t = blockIdx.x * (u64)blockDim.x + threadIdx.x; t < tiles; t += (u64)gridDim.x * blockDim.x)
-        a.tile_str[t] = string_of(a.soff, k, t * (u64)a.tp);
+    const u64 steps = (min(tiles * a.tp, n) + kBrkSpan - 1) / kBrkSpan;
+    for (u64 t = blockIdx.x * (u64)blockDim.x + threadIdx.x; t < steps; t += (u64)gridDim.x * blockDim.x)
+        a.step_str[t] = string_of(a.soff, k, t * kBrkSpan);
     // bitmap of string starts (and of n), zeroed by the host
     for (u64 j = blockIdx.x * (u64)blockDim.x + threadIdx.x; j <= k; j += (u64)gridDim.x * blockDim.x) {
         const u64 s0 = __ldg(a.soff + j);
@@ -1059,39 +1011,39 @@ __device__ __forceinline__ void body_strings(const RoundArgs& a) {
 // first-occurrence naming over the claimed entries
 // --------------------------------------------------------------------------
 
-// Mark the first occurrence of every new phrase in a bitmap over phrase indices.
 // Number of new rules of the round, bounded by the naming arrays.
 __device__ __forceinline__ u64 round_gnew(const RoundArgs& a) {
     const u64 g = *a.d_gnew;
-    if (g > a.g_alloc) {
+    if (g > a.r_cap) {
         if (blockIdx.x == 0 && threadIdx.x == 0) set_error(a.ds, kErrCapacity);
-        return a.g_alloc;
+        return a.r_cap;
     }
     return g;
 }
 
+// Whether the new rules fit the level's arrays.
+__device__ __forceinline__ bool rules_fit(const RoundArgs& a) {
+    if (a.g_base + min(*a.d_gnew, a.r_cap) <= a.cap_g && a.G_base + *a.d_Gnew <= a.cap_G) return true;
+    if (blockIdx.x == 0 && threadIdx.x == 0) set_error(a.ds, kErrCapacity);
+    return false;
+}
+
+// Mark the first occurrence of every new phrase in a bitmap over phrase
+// indices.  Claims are numbered about in the order of their positions, so the
+// marks of a warp fall close together.
 __device__ __forceinline__ void body_mark(const RoundArgs& a) {
     pdl_wait();
     if (round_halted(a)) return;
-    const u64 g_new = round_gnew(a);
-    const u64 keys = a.tiles_bound * (u64)a.tp;  // order keys the bitmap covers
-    Key128* mkey = (Key128*)a.mkey;
-    for (u64 c = blockIdx.x * (u64)blockDim.x + threadIdx.x; c < g_new; c += (u64)gridDim.x * blockDim.x) {
-        const u32 s = a.claims[c];
-        u64 m = ~0ull;
-        Key128 key{0, 0};
-        if (s < a.tab_cap) {  // the slot's key and value (one sector), kept in claim order for k_rank
-            const Slot* sl = (const Slot*)a.tab + s;
-            key = sl->key;
-            m = sl->val;
-        }
-        mkey[c] = key;
-        a.mval[c] = m;
-        if (m >= keys) {
+    const u64 ids = min(*a.d_ids, a.id_cap);
+    const u64 phrases = a.first_words * 32;  // phrase indices the bitmap covers
+    for (u64 c = blockIdx.x * (u64)blockDim.x + threadIdx.x; c < ids; c += (u64)gridDim.x * blockDim.x) {
+        const u64 m = a.minpos[c];
+        if (m == ~0ull) continue;  // a number that no claim used
+        if (m >= phrases) {
             set_error(a.ds, kErrCapacity);
             continue;
         }
-        atomicOr(a.first_bits + (m >> 5), 1u << (m & 31));
+        atomicOr(&a.first[m >> 5].x, 1u << (m & 31));
     }
 }
 
@@ -1099,77 +1051,120 @@ constexpr int kPopThreads = 256;
 constexpr int kPopItems = 16;
 constexpr int kPopTile = kPopThreads * kPopItems;
 
-// Exclusive prefix of the popcounts of the bitmap words (single pass).
-__global__ void __launch_bounds__(kPopThreads) k_popscan(const RoundArgs a, u64 nw) {
+// Exclusive prefix of the popcounts of the bitmap words (single pass).  Word
+// and prefix lie side by side, so that k_rank reads both with one sector.
+__global__ void __launch_bounds__(kPopThreads) k_popscan(const RoundArgs a) {
     pdl_wait();
     const u64 tile = dynamic_tile(a.ctr, a.ctr_base);
-    nw = min(nw, *a.d_tiles * (u64)(a.tp / 32));
+    const u64 nw = min(a.first_words, (*a.total + 31) / 32);
     if (tile > 0 && tile * (u64)kPopTile >= nw) return;  // beyond the count read on the device
     const u64 w0 = tile * (u64)kPopTile + (u64)threadIdx.x * kPopItems;
-    static_assert(kPopItems % 4 == 0, "16-byte words");
-    // a thread's words start at a multiple of 64 bytes of the arrays
-    const bool full = w0 + kPopItems <= nw && ((reinterpret_cast<unsigned long long>(a.first_bits) |
-                                                 reinterpret_cast<unsigned long long>(a.first_prefix)) & 15) == 0;
-    u32 c[kPopItems];
+    static_assert(kPopItems % 2 == 0, "16-byte pairs of words");
+    const bool full = w0 + kPopItems <= nw && (reinterpret_cast<unsigned long long>(a.first) & 15) == 0;
+    u32 x[kPopItems];
     if (full) {
 #pragma unroll
-        for (int q = 0; q < kPopItems / 4; q++) {
-            const uint4 x = reinterpret_cast<const uint4*>(a.first_bits + w0)[q];
-            c[4 * q] = __popc(x.x), c[4 * q + 1] = __popc(x.y), c[4 * q + 2] = __popc(x.z), c[4 * q + 3] = __popc(x.w);
+        for (int q = 0; q < kPopItems / 2; q++) {
+            const uint4 v = reinterpret_cast<const uint4*>(a.first + w0)[q];
+            x[2 * q] = v.x, x[2 * q + 1] = v.z;
         }
     } else {
 #pragma unroll
-        for (int it = 0; it < kPopItems; it++) c[it] = (w0 + it < nw) ? (u32)__popc(a.first_bits[w0 + it]) : 0u;
+        for (int it = 0; it < kPopItems; it++) x[it] = (w0 + it < nw) ? a.first[w0 + it].x : 0u;
     }
     u64 sum = 0;
 #pragma unroll
-    for (int it = 0; it < kPopItems; it++) sum += c[it];
+    for (int it = 0; it < kPopItems; it++) sum += (u32)__popc(x[it]);
     u64 tot;
     u64 e = block_excl_scan(sum, tot);
     u64 agg[1] = {tot}, excl[1];
     block_lookback<1>((LBSlot<1>*)a.lb1, tile, a.epoch, agg, excl, a.ds);
     e += excl[0];
-    u32 o[kPopItems];
-#pragma unroll
-    for (int it = 0; it < kPopItems; it++) {
-        o[it] = (u32)e;
-        e += c[it];
-    }
     if (full) {
-        uint4* dst = reinterpret_cast<uint4*>(a.first_prefix + w0);
+        uint4* dst = reinterpret_cast<uint4*>(a.first + w0);
 #pragma unroll
-        for (int q = 0; q < kPopItems / 4; q++) dst[q] = make_uint4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
+        for (int q = 0; q < kPopItems / 2; q++) {
+            const u32 e0 = (u32)e, e1 = e0 + __popc(x[2 * q]);
+            dst[q] = make_uint4(x[2 * q], e0, x[2 * q + 1], e1);
+            e = e1 + __popc(x[2 * q + 1]);
+        }
     } else {
 #pragma unroll
-        for (int it = 0; it < kPopItems; it++)
-            if (w0 + it < nw) a.first_prefix[w0 + it] = o[it];
+        for (int it = 0; it < kPopItems; it++) {
+            if (w0 + it < nw) a.first[w0 + it].y = (u32)e;
+            e += (u32)__popc(x[it]);
+        }
     }
 }
 
-// Rank of every new phrase: the marks before its first occurrence.
+// Rank of every new phrase: the marks before its first occurrence.  Its
+// record moves to its rank's place.
 __device__ __forceinline__ void body_rank(const RoundArgs& a) {
     pdl_wait();
     if (round_halted(a)) return;
-    const u64 g_new = round_gnew(a);
-    const Key128* mkey = (const Key128*)a.mkey;
-    Key128* rkey = (Key128*)a.rkey;
-    for (u64 c = blockIdx.x * (u64)blockDim.x + threadIdx.x; c < g_new; c += (u64)gridDim.x * blockDim.x) {
-        const u32 s = a.claims[c];
-        const u64 m = a.mval[c];  // k_mark's copy of the slot, in claim order
-        if (m >= a.tiles_bound * (u64)a.tp) continue;  // k_mark flagged it
-        const Key128 key = mkey[c];
-        const u32 w = (u32)(m >> 5);
-        const u64 r = a.first_prefix[w] + __popc(a.first_bits[w] & ((1u << (m & 31)) - 1u));
+    const u64 g_new = round_gnew(a), ids = min(*a.d_ids, a.id_cap);
+    const ClaimRec* crec = (const ClaimRec*)a.crec;
+    ClaimRec* rrec = (ClaimRec*)a.rrec;
+    for (u64 c = blockIdx.x * (u64)blockDim.x + threadIdx.x; c < ids; c += (u64)gridDim.x * blockDim.x) {
+        const u64 m = a.minpos[c];
+        const ClaimRec rec = crec[c];
+        if (m >= a.first_words * 32) continue;  // no claim (or k_mark flagged it)
+        const uint2 f = a.first[m >> 5];
+        const u64 r = f.y + __popc(f.x & ((1u << (m & 31)) - 1u));
         if (r >= g_new) { set_error(a.ds, kErrCapacity); continue; }
-        a.slot_r[r] = s;
-        a.len_r[r] = (u32)key_len(key);
-        rkey[r] = key;
+        a.rank_of[c] = (u32)(a.g_base + r);
+        rrec[r] = rec;
     }
 }
 
-// The new rules of level i in rank order: right-hand side, offsets and F^i
-// (Eq. fast_hash over F^{i-1}).  When the grammar keeps a table of its rules,
-// the new rules enter it.
+constexpr int kRoThreads = 256;
+constexpr int kRoItems = 8;
+constexpr int kRoTile = kRoThreads * kRoItems;
+
+// Right-hand-side offsets of the new rules, straight from their keys' lengths
+// (single pass).
+__global__ void __launch_bounds__(kRoThreads) k_rule_offs(const RoundArgs a) {
+    pdl_wait();
+    const u64 tile = dynamic_tile(a.ctr, a.ctr_base);
+    if (!rules_fit(a)) return;  // the same answer for every block
+    const u64 n = min(*a.d_gnew, a.r_cap);
+    if (tile * (u64)kRoTile >= n && tile > 0) return;
+    const ClaimRec* rec = (const ClaimRec*)a.rrec;
+    const u64 p0 = tile * (u64)kRoTile + (u64)threadIdx.x * kRoItems;
+    u32 len[kRoItems];
+    u64 sum = 0;
+#pragma unroll
+    for (int it = 0; it < kRoItems; it++) {
+        // the length is in the key's high half
+        const Key128 k{0, p0 + it < n ? rec[p0 + it].key.hi : 0ull};
+        len[it] = (u32)key_len(k);
+    }
+#pragma unroll
+    for (int it = 0; it < kRoItems; it++) sum += len[it];
+    u64 tot;
+    u64 e = block_excl_scan(sum, tot);
+    u64 agg[1] = {tot}, excl[1];
+    block_lookback<1>((LBSlot<1>*)a.lb1, tile, a.epoch, agg, excl, a.ds);
+    e += excl[0] + a.G_base;
+    u64* off = a.rhs_off + a.g_base;
+#pragma unroll
+    for (int it = 0; it < kRoItems; it++) {
+        if (p0 + it < n) off[p0 + it] = e;
+        e += len[it];
+    }
+    if ((tile + 1) * (u64)kRoTile >= n && threadIdx.x == 0) off[n] = a.G_base + excl[0] + tot;
+}
+
+// The rank of a symbol of T^i (ids; bytes name themselves).
+template <typename T>
+__device__ __forceinline__ u32 sym_rank(const RoundArgs& a, u32 v) {
+    if constexpr (sizeof(T) == 1) return v;
+    return v < a.prev_base ? v : __ldg(a.rank_prev + (v - a.prev_base));
+}
+
+// The new rules of level i in rank order: right-hand sides (ids translated to
+// ranks) and F^i.  When the grammar keeps a table of its rules, the new rules
+// enter it.  The roots of the retired strings get their ranks.
 template <typename T>
 __device__ __forceinline__ void body_rules(const RoundArgs& a) {
     pdl_wait();
@@ -1177,49 +1172,53 @@ __device__ __forceinline__ void body_rules(const RoundArgs& a) {
     const ContentTable rw{(Slot*)a.rtab_w, a.rtab_w_cap};
     if (round_halted(a)) return;
     const u64 g_new = round_gnew(a);
-    const u64 G_new = *a.d_Gnew;
-    if (a.g_base + g_new > a.cap_g || a.G_base + G_new > a.cap_G) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) set_error(a.ds, kErrCapacity);
-        return;
+    if (!rules_fit(a)) return;
+    for (u64 x = blockIdx.x * (u64)blockDim.x + threadIdx.x; x < a.rc->retired; x += (u64)gridDim.x * blockDim.x) {
+        const u32 id = a.c_rank[a.R_sid[x]];
+        if (id < a.id_base) continue;
+        if (id - a.id_base < a.id_cap) a.c_rank[a.R_sid[x]] = a.rank_of[id - a.id_base];
+        else set_error(a.ds, kErrCapacity);
     }
     // whole warps step through the ranks, so that a warp can take its long
     // rules (more than kLongLen symbols) together after its short ones
     const u32 lane = threadIdx.x & 31;
-    auto finish_rule = [&](u32 slot, const Key128& k, u64 len, bool hashed, u64 rank, u64 H) {
-        const u32 fpv = finish_hash(a.lh, H);
-        a.F[rank] = fpv;
-        a.rv[slot] = ((u64)fpv << 32) | rank;  // for the rewrite: rank and fingerprint, dense by slot
-        if (rw.cap) table_put(rw, hashed ? key_hashed(H, len, rank) : k, rank, a.ds);
-    };
+    const ClaimRec* rec = (const ClaimRec*)a.rrec;
     const u64 stride = (u64)gridDim.x * blockDim.x;
     for (u64 r0 = blockIdx.x * (u64)blockDim.x + (threadIdx.x & ~31u); r0 < g_new; r0 += stride) {
         const u64 r = r0 + lane;
         bool longr = false;
         if (r < g_new) {
-            const u32 slot = a.slot_r[r];
-            if (slot >= a.tab_cap) {
-                set_error(a.ds, kErrCapacity);
+            const Key128 k = rec[r].key;
+            const u64 len = key_len(k);
+            const bool hashed = key_is_hashed(k);
+            const u64 rank = a.g_base + r;
+            const u64 off = a.rhs_off[rank];
+            a.F[rank] = rec[r].fp;
+            if (len > (u64)kLongLen) {
+                longr = true;
             } else {
-                const Key128 k = ((const Key128*)a.rkey)[r];  // the rule's key, in rank order (k_rank)
-                const u64 len = key_len(k);
-                const bool hashed = key_is_hashed(k);
-                const u64 off = a.G_base + a.xlen[r];
-                const u64 rank = a.g_base + r;
-                a.rhs_off[rank] = off;
-                if (len > (u64)kLongLen) {
-                    longr = true;
-                } else {
-                    auto get = [&](u64 j) -> u32 { return hashed ? (u32)S[k.lo + j] : key_sym(k, j, a.sym_w); };
+                // four symbols at a time: their reads (and the translation's) are issued together
+                for (u64 j = 0; j < len; j += 4) {
+                    u32 v[4];
+#pragma unroll
+                    for (int u = 0; u < 4; u++)
+                        v[u] = j + u < len ? (hashed ? (u32)S[k.lo + j + u] : key_sym(k, j + u, a.sym_w)) : 0u;
+#pragma unroll
+                    for (int u = 0; u < 4; u++)
+                        if (j + u < len) v[u] = sym_rank<T>(a, v[u]);
+#pragma unroll
+                    for (int u = 0; u < 4; u++)
+                        if (j + u < len) a.rhs[off + j + u] = v[u];
+                }
+                if (rw.cap) {
+                    auto get = [&](u64 j) -> u32 { return a.rhs[off + j]; };
+                    const int w = sizeof(T) == 1 ? 8 : kRankBits;
                     u64 H = 0;
-                    for (u64 j = len; j-- > 0;) {
-                        const u32 v = get(j);
-                        a.rhs[off + j] = v;
-                        H = addmod61(mulmod61(H, a.lh.c), (u64)__ldg(a.Fprev + v));
-                    }
-                    finish_rule(slot, k, len, hashed, rank, H);
+                    if (len > inline_max(w))
+                        for (u64 j = len; j-- > 0;) H = addmod61(mulmod61(H, a.lh.c), (u64)__ldg(a.Fprev + get(j)));
+                    table_put(rw, rule_key(get, len, w, H, rank), rank, a.ds);
                 }
             }
-            if (r == 0) a.rhs_off[a.g_base + g_new] = a.G_base + G_new;
         }
         // long rules (hashed keys: the content is read at the first occurrence
         // k.lo), one at a time by the whole warp
@@ -1227,106 +1226,14 @@ __device__ __forceinline__ void body_rules(const RoundArgs& a) {
         while (m) {
             const u64 rr = r0 + (u64)(__ffs(m) - 1);
             m &= m - 1;
-            const u32 slot = a.slot_r[rr];
-            const Key128 k = ((const Key128*)a.rkey)[rr];
+            const Key128 k = rec[rr].key;
             const u64 len = key_len(k);
-            const u64 off = a.G_base + a.xlen[rr];
-            const u64 H = warp_poly61([&](u64 j) -> u64 {
-                const u32 v = (u32)S[k.lo + j];
-                a.rhs[off + j] = v;
-                return __ldg(a.Fprev + v);
-            }, len, a.lh.c);
-            if (lane == 0) finish_rule(slot, k, len, true, a.g_base + rr, H);
-        }
-    }
-}
-
-// --------------------------------------------------------------------------
-// k_rewrite: T^{i+1} and retired strings
-// --------------------------------------------------------------------------
-
-// Phrases a thread of k_rewrite reads at once: many when the per-slot array
-// it gathers from is small enough to stay in L2 (the rewrite then streams, and
-// more reads in flight bring it closer to DRAM bandwidth), few when that array
-// is far beyond L2 (random DRAM sectors bound it, and fewer registers keep
-// more warps resident).
-constexpr int kRwUnrollStream = 16, kRwUnrollGather = 4;
-
-// T^{i+1}[p] = rank of phrase p and f^{i+1}[p] = its fingerprint F^i[rank]
-// (so that the next round reads fingerprints without gathers).  Strings that
-// became one phrase take their C entry instead.  The (fingerprint, rank) pair
-// of a slot comes from the dense array k_rules wrote (read-only here: small
-// and cached in L1 in early rounds, in L2 after its writes later on).
-template <int kRwUnroll>
-__device__ __forceinline__ void body_rewrite(const RoundArgs& a, u64 ntiles) {
-    pdl_wait();
-    if (round_halted(a)) return;
-    const u64 nr = a.rc->retired;
-    ntiles = min(ntiles, *a.d_tiles);
-    // ranks of the level after this round (never past its arrays)
-    const u64 g_total = min(a.g_base + *a.d_gnew, a.cap_g);
-    const u64* __restrict__ rv = a.rv;
-    // one tile per warp: the tile's header reads and its first phrase reads
-    // of every warp of the SM are in flight together
-    const u32 lane = threadIdx.x & 31, warps = blockDim.x >> 5;
-    const u32 stripes = a.level > 1 ? a.stripes : 1u;
-    const u64 nlog = stripe_tiles(ntiles, stripes);
-    for (u64 lt = (u64)blockIdx.x * warps + (threadIdx.x >> 5); lt < nlog; lt += (u64)gridDim.x * warps) {
-        const u64 t = stripe_tile(lt, ntiles, stripes);
-        if (t >= ntiles) continue;
-        const u32 cnt = a.tile_cnt[t];
-        const u64 pbase = a.tile_pfx[t];
-        const u32* ps = a.P_slot + pslot_base(t, a.tile_str[t], a.tp);
-        // kRwUnroll phrases per thread at a time: their reads are issued together
-        for (u32 q0 = lane; q0 < cnt; q0 += kRwUnroll * 32) {
-            u32 s[kRwUnroll];
-            u64 v[kRwUnroll];
-#pragma unroll
-            for (int u = 0; u < kRwUnroll; u++) {
-                const u32 q = q0 + (u32)u * 32;
-                s[u] = q < cnt ? __ldcs(ps + q) : ~0u;
-            }
-#pragma unroll
-            for (int u = 0; u < kRwUnroll; u++) {
-                if (s[u] == ~0u) {
-                    v[u] = 0;  // no phrase, or the round's table overflowed
-                } else if (s[u] & kResidentBit) {
-                    const u32 r = s[u] & ~kResidentBit;
-                    v[u] = ((u64)__ldg(a.F + r) << 32) | r;
-                } else {
-                    v[u] = __ldg(rv + s[u]);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < kRwUnroll; u++) {
-                const u32 q = q0 + (u32)u * 32;
-                if (q >= cnt) continue;
-                u32 rr = (u32)v[u];
-                if (rr >= g_total) {  // an entry that got no rank: only after a capacity error
-                    set_error(a.ds, kErrCapacity);
-                    rr = 0;
-                }
-                const u64 p = pbase + q;
-                u64 out = p;
-                if (nr != 0) {
-                    u64 lo = 0, hi = nr;  // first index with R_phr >= p
-                    while (lo < hi) {
-                        const u64 mid = (lo + hi) >> 1;
-                        if (a.R_phr[mid] < p) lo = mid + 1; else hi = mid;
-                    }
-                    if (lo < nr && a.R_phr[lo] == p) {
-                        a.c_level[a.R_sid[lo]] = a.level;
-                        a.c_rank[a.R_sid[lo]] = rr;
-                        continue;
-                    }
-                    out = p - lo;
-                }
-                if (out >= a.T_cap) {
-                    set_error(a.ds, kErrCapacity);
-                    continue;
-                }
-                __stcs(a.Tnext + out, rr);
-                __stcs(a.Fnext + out, (u32)(v[u] >> 32));
+            const u64 off = a.rhs_off[a.g_base + rr];
+            for (u64 j = lane; j < len; j += 32) a.rhs[off + j] = sym_rank<T>(a, (u32)S[k.lo + j]);
+            if (rw.cap) {
+                __syncwarp();
+                const u64 H = warp_poly61([&](u64 j) -> u64 { return __ldg(a.Fprev + a.rhs[off + j]); }, len, a.lh.c);
+                if (lane == 0) table_put(rw, key_hashed(H, len, a.g_base + rr), a.g_base + rr, a.ds);
             }
         }
     }
@@ -1384,9 +1291,9 @@ __global__ void k_gather_strings(const unsigned char* __restrict__ data, const u
 
 template <typename T>
 __global__ void __launch_bounds__(kBrkThreads) k_breaks(const RoundArgs a, u64 nblocks) { body_breaks<T>(a, nblocks); }
-template <typename T, int TP>
-__global__ void __launch_bounds__(kParseThreads, sizeof(T) == 1 ? 5 : 4) k_parse(const RoundArgs a, u64 ntiles) {
-    body_parse<T, TP>(a, ntiles);
+template <typename T, int U>
+__global__ void __launch_bounds__(kParseThreads, kParseBlocksMax) k_parse(const __grid_constant__ RoundArgs a, u64 nunits) {
+    body_parse<T, U>(a, nunits);
 }
 __global__ void k_tile_strings(const RoundArgs a, u64 tiles) { body_tile_strings(a, tiles); }
 __global__ void __launch_bounds__(1024) k_strings(const RoundArgs a) { body_strings(a); }
@@ -1394,17 +1301,13 @@ __global__ void k_mark(const RoundArgs a) { body_mark(a); }
 __global__ void k_rank(const RoundArgs a) { body_rank(a); }
 template <typename T>
 __global__ void k_rules(const RoundArgs a) { body_rules<T>(a); }
-template <int kRwUnroll>
-__global__ void __launch_bounds__(256) k_rewrite(const RoundArgs a, u64 ntiles) { body_rewrite<kRwUnroll>(a, ntiles); }
 
-// Exclusive prefix of in[0 .. n) (n: the smaller of the bound and *n_dev when
-// given) into out, the sum into totals[0] and 0 into totals[1] (what k_scan2
-// gives for one column), by one block of kSmallThreads threads.
+// Exclusive prefix of get(0 .. n) by one block of kSmallThreads threads:
+// put(i, prefix) for every i, and the sum to every thread.
 constexpr int kSmallThreads = 256;
 constexpr int kSmallItems = 16;
-template <typename Get>
-__device__ void block_scan_small(Get get, u64 n, const u64* n_dev, u64* out64, u32* out32, u64* totals) {
-    if (n_dev != nullptr) n = min(*n_dev, n);
+template <typename Get, typename Put>
+__device__ u64 block_scan_small(Get get, u64 n, Put put) {
     u64 carry = 0;
     for (u64 base = 0; base < n; base += (u64)kSmallThreads * kSmallItems) {
         const u64 p0 = base + (u64)threadIdx.x * kSmallItems;
@@ -1419,19 +1322,13 @@ __device__ void block_scan_small(Get get, u64 n, const u64* n_dev, u64* out64, u
         u64 e = block_excl_scan(sum, tot) + carry;
 #pragma unroll
         for (int i = 0; i < kSmallItems; i++) {
-            if (p0 + i < n) {
-                if (out64) out64[p0 + i] = e;
-                if (out32) out32[p0 + i] = (u32)e;
-            }
+            if (p0 + i < n) put(p0 + i, e);
             e += v[i];
         }
         carry += tot;
     }
-    if (threadIdx.x == 0 && totals != nullptr) {
-        totals[0] = carry;
-        totals[1] = 0;
-    }
     __syncthreads();
+    return carry;
 }
 
 // Barrier over the grid of a cooperative launch: the k-th barrier of a launch
@@ -1462,11 +1359,12 @@ __device__ void grid_barrier(u64* ctr, u64 target, DevStatus* ds) {
 }
 
 // A short round's parse in one cooperative launch instead of five: tile
-// strings, breaks, k_parse over the tiles (grid-stride, like the launches),
-// then block 0 scans the tiles' phrase counts and runs the per-string pass.
-// Grid barriers separate the steps.  Same buffers and results as the launches.
+// strings, breaks, block 0 scans the tiles' phrase counts and runs the
+// per-string pass, then k_parse over the tiles (grid-stride, like the
+// launches).  Grid barriers separate the steps.  Same buffers and results as
+// the launches.
 template <typename T>
-__global__ void __launch_bounds__(kSmallThreads) k_parse_small(const RoundArgs a, u64 tiles, u64 nsteps,
+__global__ void __launch_bounds__(kSmallThreads) k_parse_small(const __grid_constant__ RoundArgs a, u64 tiles, u64 nsteps,
                                                                 u64 bar_base) {
     static_assert(kSmallThreads == kParseThreads && kSmallThreads == kBrkThreads, "one block shape");
     const u64 g = gridDim.x;
@@ -1474,35 +1372,39 @@ __global__ void __launch_bounds__(kSmallThreads) k_parse_small(const RoundArgs a
     grid_barrier(a.ctr, bar_base + g, a.ds);
     body_breaks<T>(a, nsteps);
     grid_barrier(a.ctr, bar_base + 2 * g, a.ds);
-    body_parse<T, kTPMin>(a, tiles);
-    grid_barrier(a.ctr, bar_base + 3 * g, a.ds);
     if (blockIdx.x == 0) {
-        block_scan_small([&](u64 i) { return a.tile_cnt[i]; }, tiles, a.d_tiles, a.tile_pfx, nullptr, a.total);
+        const u64 P = block_scan_small([&](u64 i) { return a.tile_cnt[i]; }, min(tiles, *a.d_tiles),
+                                       [&](u64 i, u64 e) { a.tile_pfx[i] = e; });
+        if (threadIdx.x == 0) *a.total = P;
         body_strings(a);
     }
+    grid_barrier(a.ctr, bar_base + 3 * g, a.ds);
+    body_parse<T, kUnitMin>(a, tiles);
 }
 
-// A short round's naming and rewrite in one cooperative launch instead of
-// six: marks, (block 0) the prefix of the marks' popcounts, ranks, (block 0)
-// the scan of the rule lengths, rules and the rewrite.
+// A short round's naming in one cooperative launch instead of five: marks,
+// (block 0) the prefix of the marks' popcounts, ranks, (block 0) the rules'
+// offsets, rules.
 template <typename T>
-__global__ void __launch_bounds__(kSmallThreads) k_naming_small(const RoundArgs a, u64 nw, u64 g_bound,
-                                                                 u64 bar_base) {
+__global__ void __launch_bounds__(kSmallThreads) k_naming_small(const RoundArgs a, u64 bar_base) {
     const u64 g = gridDim.x;
     body_mark(a);
     grid_barrier(a.ctr, bar_base + g, a.ds);
     if (blockIdx.x == 0)
-        block_scan_small([&](u64 w) { return (u32)__popc(a.first_bits[w]); },
-                         min(nw, *a.d_tiles * (u64)(a.tp / 32)), nullptr, nullptr, a.first_prefix, nullptr);
+        block_scan_small([&](u64 w) { return (u32)__popc(a.first[w].x); }, min(a.first_words, (*a.total + 31) / 32),
+                         [&](u64 w, u64 e) { a.first[w].y = (u32)e; });
     grid_barrier(a.ctr, bar_base + 2 * g, a.ds);
     body_rank(a);
     grid_barrier(a.ctr, bar_base + 3 * g, a.ds);
-    if (blockIdx.x == 0)
-        block_scan_small([&](u64 i) { return a.len_r[i]; }, g_bound, a.d_gnew, a.xlen, nullptr, a.total + 1);
+    if (blockIdx.x == 0 && rules_fit(a)) {
+        const u64 g_new = min(*a.d_gnew, a.r_cap);
+        const ClaimRec* rec = (const ClaimRec*)a.rrec;
+        const u64 G = block_scan_small([&](u64 r) { return (u32)key_len(rec[r].key); }, g_new,
+                                       [&](u64 r, u64 e) { a.rhs_off[a.g_base + r] = a.G_base + e; });
+        if (threadIdx.x == 0) a.rhs_off[a.g_base + g_new] = a.G_base + G;
+    }
     grid_barrier(a.ctr, bar_base + 4 * g, a.ds);
     body_rules<T>(a);
-    grid_barrier(a.ctr, bar_base + 5 * g, a.ds);
-    body_rewrite<kRwUnrollGather>(a, a.tiles_bound);
 }
 
 static unsigned grid_for(u64 n, u64 cap = 152ull * 32) {
@@ -1511,8 +1413,11 @@ static unsigned grid_for(u64 n, u64 cap = 152ull * 32) {
     return (unsigned)(b < cap ? b : cap);
 }
 
+constexpr u32 kWarps = kParseWarps;
 bool parse_tile_valid(u32 tp) { return tp == 1024 || tp == 2048 || tp == 4096; }
-u64 parse_slot_entries(u64 tiles, u64 strings, u32 tp) { return tiles * (u64)(tp / 2 + 2) + strings + 1; }
+u32 parse_unit(u32 tile) { return tile / kWarps; }
+static_assert(1024 / kWarps == kUnitMin && 4096 / kWarps == kUnitMax, "units of the accepted tiles");
+size_t claim_rec_bytes() { return sizeof(ClaimRec); }
 u64 breaks_steps(u64 tiles, u32 tp) { return (tiles * (u64)tp + kBrkSpan - 1) / kBrkSpan + 1; }
 
 u64 popscan_tiles_for(u64 nw) { return (nw + kPopTile - 1) / kPopTile; }
@@ -1521,7 +1426,7 @@ cudaError_t launch_tile_strings(const RoundArgs& a, cudaStream_t st) {
     return launch_pdl(k_tile_strings, grid_for(a.tiles_bound), 256, st, a, a.tiles_bound);
 }
 
-template <typename T, int TP>
+template <typename T, int U>
 static int parse_occupancy(int* sms_out) {
     // queried once per instantiation (thread-safe static initialisation:
     // contexts on several host threads launch at once)
@@ -1529,7 +1434,9 @@ static int parse_occupancy(int* sms_out) {
         int dev = 0, sms = 0, occ = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_parse<T, TP>, kParseThreads, 0);
+        constexpr int smem = (int)sizeof(ParseSmem<T, U>);
+        cudaFuncSetAttribute(k_parse<T, U>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_parse<T, U>, kParseThreads, smem);
         return std::make_pair(occ > 0 ? occ : 1, sms);
     }();
     if (sms_out) *sms_out = occ_sms.second;
@@ -1537,22 +1444,22 @@ static int parse_occupancy(int* sms_out) {
 }
 
 // Persistent grid: `per_sm` blocks per SM (0 or more than fit: as many as fit).
-template <typename T, int TP>
-static unsigned persistent_grid(u64 tiles, u32 per_sm) {
+template <typename T, int U>
+static unsigned persistent_grid(u64 units, u32 per_sm) {
     int sms = 0;
-    const int occ = parse_occupancy<T, TP>(&sms);
+    const int occ = parse_occupancy<T, U>(&sms);
     const u64 b = (per_sm == 0 || per_sm > (u32)occ) ? (u64)occ : (u64)per_sm;
-    const u64 g = b * (u64)sms;
-    return (unsigned)(tiles < g ? (tiles ? tiles : 1) : g);
+    const u64 g = b * (u64)sms, most = (units + kWarps - 1) / kWarps;
+    return (unsigned)(most < g ? (most ? most : 1) : g);
 }
 
-// Most k_parse blocks that fit on an SM, over every tile size.
+// Most k_parse blocks that fit on an SM, over every unit size.
 int parse_max_blocks(int sym_bytes) {
     if (sym_bytes == 1)
-        return std::max({parse_occupancy<unsigned char, 1024>(nullptr), parse_occupancy<unsigned char, 2048>(nullptr),
-                         parse_occupancy<unsigned char, 4096>(nullptr)});
-    return std::max({parse_occupancy<u32, 1024>(nullptr), parse_occupancy<u32, 2048>(nullptr),
-                     parse_occupancy<u32, 4096>(nullptr)});
+        return std::max({parse_occupancy<unsigned char, 128>(nullptr), parse_occupancy<unsigned char, 256>(nullptr),
+                         parse_occupancy<unsigned char, 512>(nullptr)});
+    return std::max({parse_occupancy<u32, 128>(nullptr), parse_occupancy<u32, 256>(nullptr),
+                     parse_occupancy<u32, 512>(nullptr)});
 }
 
 template <typename T>
@@ -1574,18 +1481,19 @@ cudaError_t launch_breaks(const RoundArgs& a, cudaStream_t st) {
     return launch_pdl(k_breaks<u32>, breaks_grid<u32>(blocks), kBrkThreads, st, a, blocks);
 }
 
-template <typename T, int TP>
+template <typename T, int U>
 static cudaError_t launch_parse_tp(const RoundArgs& a, cudaStream_t st) {
     const u64 tiles = a.tiles_bound;
-    return launch_pdl(k_parse<T, TP>, persistent_grid<T, TP>(tiles, a.parse_blocks), kParseThreads, st, a, tiles);
+    return launch_pdl_smem(k_parse<T, U>, persistent_grid<T, U>(tiles, a.parse_blocks), kParseThreads,
+                           sizeof(ParseSmem<T, U>), st, a, tiles);
 }
 
 template <typename T>
 static cudaError_t launch_parse_t(const RoundArgs& a, cudaStream_t st) {
     switch (a.tp) {
-        case 1024: return launch_parse_tp<T, 1024>(a, st);
-        case 2048: return launch_parse_tp<T, 2048>(a, st);
-        case 4096: return launch_parse_tp<T, 4096>(a, st);
+        case 128: return launch_parse_tp<T, 128>(a, st);
+        case 256: return launch_parse_tp<T, 256>(a, st);
+        case 512: return launch_parse_tp<T, 512>(a, st);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -1595,38 +1503,42 @@ cudaError_t launch_parse(const RoundArgs& a, cudaStream_t st) {
     return launch_parse_t<u32>(a, st);
 }
 
-bool round_is_small(const RoundArgs& a) { return a.tp == (u32)kTPMin && a.tiles_bound <= kSmallTiles; }
+bool round_is_small(const RoundArgs& a) { return a.tp == (u32)kUnitMin && a.tiles_bound <= kSmallUnits; }
 
-// Blocks of a short round's cooperative launches: one per tile, at most one
-// per SM (and never more than can be resident at once).
+// Blocks of a short round's cooperative launches: a warp per unit, at most one
+// block per SM (and never more than can be resident at once).
 u32 small_round_grid(const RoundArgs& a) {
     static const int cap = [] {
         int dev = 0, sms = 0, o1 = 0, o2 = 0, o3 = 0, o4 = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o1, k_parse_small<unsigned char>, kSmallThreads, 0);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o2, k_parse_small<u32>, kSmallThreads, 0);
+        constexpr int s1 = (int)sizeof(ParseSmem<unsigned char, kUnitMin>), s4 = (int)sizeof(ParseSmem<u32, kUnitMin>);
+        cudaFuncSetAttribute(k_parse_small<unsigned char>, cudaFuncAttributeMaxDynamicSharedMemorySize, s1);
+        cudaFuncSetAttribute(k_parse_small<u32>, cudaFuncAttributeMaxDynamicSharedMemorySize, s4);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o1, k_parse_small<unsigned char>, kSmallThreads, s1);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o2, k_parse_small<u32>, kSmallThreads, s4);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o3, k_naming_small<unsigned char>, kSmallThreads, 0);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o4, k_naming_small<u32>, kSmallThreads, 0);
         // one block per SM (a cooperative launch checks that they fit)
         return (std::min({o1, o2, o3, o4}) >= 1 && sms > 0) ? sms : 1;
     }();
-    return (u32)std::min<u64>((u64)cap, std::max<u64>(1, a.tiles_bound));
+    return (u32)std::min<u64>((u64)cap, std::max<u64>(1, (a.tiles_bound + kParseThreads / 32 - 1) / (kParseThreads / 32)));
 }
 
 cudaError_t launch_parse_small(const RoundArgs& a, u64 bar_base, cudaStream_t st) {
     const u64 nsteps = (a.tiles_bound * (u64)a.tp + kBrkSpan - 1) / kBrkSpan;
     const u32 g = small_round_grid(a);
     if (a.sym_bytes == 1)
-        return launch_coop(k_parse_small<unsigned char>, g, kSmallThreads, st, a, a.tiles_bound, nsteps, bar_base);
-    return launch_coop(k_parse_small<u32>, g, kSmallThreads, st, a, a.tiles_bound, nsteps, bar_base);
+        return launch_coop(k_parse_small<unsigned char>, g, kSmallThreads, sizeof(ParseSmem<unsigned char, kUnitMin>),
+                           st, a, a.tiles_bound, nsteps, bar_base);
+    return launch_coop(k_parse_small<u32>, g, kSmallThreads, sizeof(ParseSmem<u32, kUnitMin>), st, a, a.tiles_bound,
+                       nsteps, bar_base);
 }
 
-cudaError_t launch_naming_small(const RoundArgs& a, u64 nw, u64 g_bound, u64 bar_base, cudaStream_t st) {
+cudaError_t launch_naming_small(const RoundArgs& a, u64 bar_base, cudaStream_t st) {
     const u32 g = small_round_grid(a);
-    if (a.sym_bytes == 1)
-        return launch_coop(k_naming_small<unsigned char>, g, kSmallThreads, st, a, nw, g_bound, bar_base);
-    return launch_coop(k_naming_small<u32>, g, kSmallThreads, st, a, nw, g_bound, bar_base);
+    if (a.sym_bytes == 1) return launch_coop(k_naming_small<unsigned char>, g, kSmallThreads, 0, st, a, bar_base);
+    return launch_coop(k_naming_small<u32>, g, kSmallThreads, 0, st, a, bar_base);
 }
 
 cudaError_t launch_strings(const RoundArgs& a, cudaStream_t st) {
@@ -1637,10 +1549,16 @@ cudaError_t launch_mark(const RoundArgs& a, u64 g_grid, cudaStream_t st) {
     return launch_pdl(k_mark, grid_for(g_grid), 256, st, a);
 }
 
-cudaError_t launch_popscan(const RoundArgs& a, u64 nw_bound, cudaStream_t st) {
-    u64 tiles = popscan_tiles_for(nw_bound);
+cudaError_t launch_popscan(const RoundArgs& a, cudaStream_t st) {
+    u64 tiles = popscan_tiles_for(a.first_words);
     if (tiles == 0) tiles = 1;
-    return launch_pdl(k_popscan, (unsigned)tiles, kPopThreads, st, a, nw_bound);
+    return launch_pdl(k_popscan, (unsigned)tiles, kPopThreads, st, a);
+}
+
+u64 rule_offs_tiles(u64 g) { return std::max<u64>(1, (g + kRoTile - 1) / kRoTile); }
+
+cudaError_t launch_rule_offs(const RoundArgs& a, u64 g_grid, cudaStream_t st) {
+    return launch_pdl(k_rule_offs, (unsigned)rule_offs_tiles(g_grid), kRoThreads, st, a);
 }
 
 cudaError_t launch_rank(const RoundArgs& a, u64 g_grid, cudaStream_t st) {
@@ -1650,15 +1568,6 @@ cudaError_t launch_rank(const RoundArgs& a, u64 g_grid, cudaStream_t st) {
 cudaError_t launch_rules(const RoundArgs& a, u64 g_grid, cudaStream_t st) {
     if (a.sym_bytes == 1) return launch_pdl(k_rules<unsigned char>, grid_for(g_grid), 256, st, a);
     return launch_pdl(k_rules<u32>, grid_for(g_grid), 256, st, a);
-}
-
-cudaError_t launch_rewrite(const RoundArgs& a, cudaStream_t st) {
-    const u64 tiles = a.tiles_bound;
-    const u64 blocks = (tiles + 7) / 8;  // 8 warps per block, one tile each
-    const u64 g = blocks < 152ull * 8 ? (blocks ? blocks : 1) : 152ull * 8;
-    if ((double)a.tab_cap * sizeof(u64) <= kL2Bytes)
-        return launch_pdl(k_rewrite<kRwUnrollStream>, (unsigned)g, 256, st, a, tiles);
-    return launch_pdl(k_rewrite<kRwUnrollGather>, (unsigned)g, 256, st, a, tiles);
 }
 
 cudaError_t launch_level0(const unsigned char* data, const u64* pos, const u32* ids, u32 cnt, u32* c_level,
