@@ -52,6 +52,29 @@ __device__ __forceinline__ u64 powmod61(u64 c, u64 e) {
     return r;
 }
 
+// A sum of products v * w mod p with v < 2^32 and w < p, without a reduction
+// per term: v * w = (v * w_lo) + (v * w_hi) 2^32, collected as a0 + a1 2^32.
+// Up to 8 terms fit (a0 < 2^35; v * w_hi + 2^32 < 2^61, so a1 < 2^64); fold()
+// then reduces what was collected and adds it to the sum.  About 8
+// instructions a term, against 25 of a Horner step with mulmod61.
+struct PolySum {
+    u64 a0 = 0, a1 = 0, h = 0;
+    __device__ __forceinline__ void add(u32 v, u64 w) {
+        const u64 p0 = (u64)v * (u32)w;
+        a1 += (u64)v * (u32)(w >> 32);
+        a1 += p0 >> 32;
+        a0 += (u32)p0;
+    }
+    __device__ __forceinline__ void fold() {
+        // a1 2^32 = (a1 >> 29) 2^61 + (a1 mod 2^29) 2^32, and 2^61 = 1 (mod p)
+        u64 r = a0 + (a1 >> 29) + ((a1 & ((1ull << 29) - 1)) << 32);  // < 2^61 + 2^36
+        r = (r & kP61) + (r >> 61);
+        r = r >= kP61 ? r - kP61 : r;
+        h = addmod61(h, r);
+        a0 = a1 = 0;
+    }
+};
+
 // H = sum_{j < len} v(j) c^j mod p (the polynomial of Eq. fast_hash), by a
 // whole warp: every lane calls it with the same len and c.  Lane l takes the
 // terms j = l, l + 32, ...: h_l = sum_k v(32k + l) (c^32)^k by Horner over

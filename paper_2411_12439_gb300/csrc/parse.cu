@@ -133,6 +133,11 @@ __device__ __forceinline__ u64 stripe_tile(u64 l, u64 ntiles, u32 stripes) {
 constexpr int kCacheBits = 11;
 constexpr int kCacheSlots = 1 << kCacheBits;  // per-block phrase cache (byte rounds)
 constexpr int kCacheProbes = 8;
+// Byte rounds: so many misses among a warp's 32 phrases are looked up in the table
+// at once (text, whose phrases are too many for the cache); fewer go to the
+// queue, where a full warp takes the long path.  Round 1 of 32 x 2 MB of text:
+// 1.06 ms with the queue alone, 0.72 ms with 8 to 16 here, 0.84 ms with 24.
+constexpr int kByteFind = 16;
 // A cache entry's value: bits 58..63 an exponent x, bits 32..57 the id, the low
 // half F^1.  The phrase's first occurrence is known to be before 2^x, so a
 // phrase at place 2^x or later needs nothing more; the warps of a block are at
@@ -408,7 +413,7 @@ struct ParseArgs {
     const u32* Sf;
     u32* Tnext;
     u32* Fnext;
-    u64 T_cap, retired;
+    u64 n, T_cap, retired;
     LevelHash lh;
     RoundTable table;
     u64 rtab_cap;
@@ -439,6 +444,7 @@ struct ParseSmem {
     u64 ckey[kByte ? kCacheSlots : 1];
     u64 cval[kByte ? kCacheSlots : 1];
     u32 sF[kByte ? 256 : 1];  // byte rounds: F^0
+    u64 cpow[kLongLen];       // c^j mod p
 };
 
 // A queued phrase: where it starts in S, its length, what is known of its home
@@ -516,6 +522,38 @@ __device__ __noinline__ bool same_content(const T* S, u64 pos, u64 len, u64 ref)
     return true;
 }
 
+// The inline key of a phrase of len <= kInlineMax bytes at offset st of the
+// 8-byte words s64: its bytes as one little-endian number B, B mod 2^60 (with
+// the length above) in hi and B >> 60 in lo (the layout of key_inline for
+// 8-bit symbols).
+__device__ __forceinline__ Key128 byte_key_of(u64 b0, u64 b1, u32 len) {
+    if (len < 8) {
+        b0 &= (1ull << (8 * len)) - 1;
+        b1 = 0;
+    } else if (len < 16) {
+        b1 &= (1ull << (8 * (len - 8))) - 1;
+    }
+    return Key128{(b0 >> 60) | (b1 << 4), (b0 & ((1ull << 60) - 1)) | ((u64)len << 60)};
+}
+__device__ __forceinline__ Key128 byte_key(const u64* s64, u32 st, u32 len) {
+    const u32 sh = (st & 7) * 8;
+    s64 += st >> 3;
+    const u64 x0 = s64[0], x1 = s64[1], x2 = s64[2];
+    return byte_key_of(sh ? (x0 >> sh) | (x1 << (64 - sh)) : x0, sh ? (x1 >> sh) | (x2 << (64 - sh)) : x1, len);
+}
+
+// Byte rounds: a phrase found or claimed enters the cache at its free place
+// `cache` - 1 (0: none; then it is not short either), valid from a place
+// after its first occurrence (at or before `first`) on.
+template <int U>
+__device__ __forceinline__ void cache_put(u32 cache, const Key128& key, u32 len, u32 id, u32 F, u64 first) {
+    ParseSmem<unsigned char, U>& sm = parse_smem<unsigned char, U>();
+    if (cache == 0 || id >= (1u << 26)) return;
+    const u64 ck = ((u64)len << 56) | (key.hi & ((1ull << (8 * len)) - 1));
+    if (atomicCAS((unsigned long long*)&sm.ckey[cache - 1], (unsigned long long)kEmpty, (unsigned long long)ck) == kEmpty)
+        *(volatile u64*)&sm.cval[cache - 1] = ((u64)(64 - __clzll((long long)first)) << 58) | ((u64)id << 32) | F;
+}
+
 // A phrase of more than kLongLen symbols at `pos`, by the whole warp: the
 // fingerprint polynomial H (Eq. fast_hash) and the content comparisons of its
 // hashed key are spread over the lanes.
@@ -581,9 +619,39 @@ __device__ __noinline__ void parse_queued(u32 first, u32 take) {
     Key128 k;
     u64 H = 0;
     bool res = a.rtab_cap != 0;  // a phrase with a symbol that is new in this build is no resident rule
-    {
-        // four symbols from the last on at a time: H by Horner, and the packed symbols
+    if constexpr (kByte) {
+        // up to 16 bytes with three aligned 8-byte reads
+        const u64 adr = reinterpret_cast<unsigned long long>(S + pos);
+        const bool words = plen <= 16 && pos >= 8 && pos + 24 <= a.n;
+        u64 b0 = 0, b1 = 0;
+        if (words) {
+            const u64* q = reinterpret_cast<const u64*>(adr & ~7ull);
+            const u32 sh = (u32)(adr & 7) * 8;
+            const u64 x0 = __ldg(q), x1 = __ldg(q + 1), x2 = __ldg(q + 2);
+            b0 = sh ? (x0 >> sh) | (x1 << (64 - sh)) : x0;
+            b1 = sh ? (x1 >> sh) | (x2 << (64 - sh)) : x1;
+        } else if (plen <= 16) {
+            for (u32 j = 0; j < plen; j++) {
+                const u64 x = (u64)S[pos + j] << (8 * (j & 7));
+                if (j < 8) b0 |= x; else b1 |= x;
+            }
+        }
+        PolySum ps;
+        for (u32 j = 0; j < plen;) {
+            const u64 x = j < 8 ? b0 : b1;
+            const u32 end = min(plen, j + 8);
+            for (u32 sh = 0; j < end; j++, sh += 8) {
+                const u32 v = plen <= 16 ? (u32)(x >> sh) & 0xFFu : (u32)S[pos + j];
+                ps.add(sm.sF[v], sm.cpow[j]);
+            }
+            ps.fold();
+        }
+        H = ps.h;
+        k = plen <= (u32)kInlineMax ? byte_key_of(b0, b1, plen) : key_hashed(H, plen, pos);
+    } else {
+        // four symbols from the last on at a time: H, and the packed symbols
         PackedSyms ps;
+        PolySum poly;
         for (u32 j = plen; j > 0;) {
             const u32 m = min(j, 4u);
             u32 v[4], f[4];
@@ -592,19 +660,20 @@ __device__ __noinline__ void parse_queued(u32 first, u32 take) {
                 v[u] = f[u] = 0;
                 if ((u32)u < m) {
                     v[u] = (u32)__ldg(S + pos + j - 1 - u);
-                    if constexpr (!kByte) f[u] = __ldg(a.Sf + pos + j - 1 - u);
+                    f[u] = __ldg(a.Sf + pos + j - 1 - u);
                 }
             }
 #pragma unroll
             for (int u = 0; u < 4; u++)
                 if ((u32)u < m) {
-                    if constexpr (kByte) f[u] = sm.sF[v[u]];
-                    else res = res && v[u] < a.prev_base;
+                    res = res && v[u] < a.prev_base;
                     ps.push(v[u], a.sym_w);
-                    H = addmod61(mulmod61(H, a.lh.c), (u64)f[u]);
+                    poly.add(f[u], sm.cpow[j - 1 - u]);
                 }
+            poly.fold();
             j -= m;
         }
+        H = poly.h;
         k = plen <= a.inline_most ? ps.key(plen) : key_hashed(H, plen, pos);
     }
     const u32 F = finish_hash(a.lh, H);
@@ -623,15 +692,7 @@ __device__ __noinline__ void parse_queued(u32 first, u32 take) {
     if (act && (r != ~0ull || pub != kNoPub)) {
         const u32 id = r != ~0ull ? (u32)r : a.id_base + (u32)pub;
         if constexpr (kByte) {
-            // into the cache, valid from a place after its first occurrence on
-            const u32 ch = (u32)(e.x >> (kPosBits + 8));
-            if (ch && id < (1u << 26)) {
-                const u64 ck = ((u64)plen << 56) | (k.hi & ((1ull << (8 * plen)) - 1));
-                if (atomicCAS((unsigned long long*)&sm.ckey[ch - 1], (unsigned long long)kEmpty,
-                              (unsigned long long)ck) == kEmpty)
-                    *(volatile u64*)&sm.cval[ch - 1] = ((u64)(64 - __clzll((long long)first_occ)) << 58) |
-                                                       ((u64)id << 32) | F;
-            }
+            cache_put<U>((u32)(e.x >> (kPosBits + 8)), k, plen, id, F, first_occ);
         }
         if (a.retired == 0 && p < a.T_cap) {
             __stcs(a.Tnext + p, id);
@@ -710,22 +771,34 @@ __device__ __noinline__ u32 parse_unit_find(u32 buf, u64 t0, u64 p0, u64 out, u3
                         h = (h + 1) & (kCacheSlots - 1);
                     }
                 }
-            } else if (len <= find_inline && direct) {
-                const Key128 key = key_inline32(sym + st, len, sym_w);
-                const Slot c = ld_slot_relaxed(&slots[key_home(key, cap)]);
-                if (c.key.hi == key.hi && c.key.lo == key.lo && c.pub != kUnpublished && c.val <= p0 + q) {
-                    state = kDone;
-                    emit(q, id_base + (u32)c.pub, (u32)(c.pub >> 32));
-                } else if (c.key.hi == kEmptyHi) {
-                    state = kHomeEmpty;
-                } else if (c.key.hi != key.hi) {
-                    state = kHomeOther;
-                }
-                // else: another key, one being written, or a first occurrence
-                // that may be here: the long path reads the slot again
             }
         }
-        const unsigned m = __ballot_sync(0xffffffffu, state < kDone);
+        // the home slot: every phrase in rank rounds, in byte rounds when enough
+        // lanes of the warp missed the cache
+        auto look = [&]() {
+            const Key128 key = kByte ? byte_key(reinterpret_cast<const u64*>(sym), st, len)
+                                     : key_inline32(reinterpret_cast<const u32*>(sym) + st, len, sym_w);
+            const Slot c = ld_slot_relaxed(&slots[key_home(key, cap)]);
+            if (c.key.hi == key.hi && c.key.lo == key.lo && c.pub != kUnpublished && c.val <= p0 + q) {
+                const u32 id = id_base + (u32)c.pub, F = (u32)(c.pub >> 32);
+                state = kDone;
+                emit(q, id, F);
+                if constexpr (kByte) cache_put<U>(cache, key, len, id, F, c.val);
+            } else if (c.key.hi == kEmptyHi) {
+                state = kHomeEmpty;
+            } else if (c.key.hi != key.hi) {
+                state = kHomeOther;
+            }
+            // else: another key, one being written, or a first occurrence
+            // that may be here: the long path reads the slot again
+        };
+        if constexpr (!kByte)
+            if (state == kHomeUnknown && len <= find_inline && direct) look();
+        unsigned m = __ballot_sync(0xffffffffu, state < kDone);
+        if (kByte && __popc(m) >= kByteFind) {
+            if (state == kHomeUnknown && len <= find_inline && direct) look();
+            m = __ballot_sync(0xffffffffu, state < kDone);
+        }
         if (state < kDone)
             w.queue[nq + __popc(m & ((1u << lane) - 1u))] =
                 make_ulonglong2(queue_word(t0 + st, len, state, cache), p0 + q);
@@ -769,6 +842,7 @@ __device__ __forceinline__ void body_parse(const RoundArgs& a, u64 nunits) {
         pa.Sf = a.Sf;
         pa.Tnext = a.Tnext;
         pa.Fnext = a.Fnext;
+        pa.n = n;
         pa.T_cap = a.T_cap;
         pa.retired = nr;
         pa.lh = a.lh;
@@ -781,6 +855,7 @@ __device__ __forceinline__ void body_parse(const RoundArgs& a, u64 nunits) {
         pa.id_base = a.id_base;
         pa.prev_base = a.prev_base;
     }
+    if (threadIdx.x < (u32)kLongLen) sm.cpow[threadIdx.x] = powmod61(a.lh.c, threadIdx.x);
     if (threadIdx.x == 0) sm.ids = ClaimIds{0, 0, 0};
     if (lane == 0) {
         w.claims = w.claim_len = 0;
