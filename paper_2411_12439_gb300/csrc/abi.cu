@@ -34,6 +34,7 @@ struct Level {
     void* rtab = nullptr;      // table over the rules (for parses against this grammar and merges)
     u64 rcap = 0;
     bool rvalid = false;
+    bool shared_rules = false, shared_rhs = false;  // rhs_off and F, rhs: parts of one of the grammar's slabs
 };
 
 }  // namespace
@@ -47,6 +48,7 @@ struct lcg_grammar {
     u32 k = 0, cap_k = 0;
     u32* c_level = nullptr;
     u32* c_rank = nullptr;
+    std::vector<void*> slabs;  // allocations that hold the arrays of several levels
 };
 
 namespace {
@@ -103,6 +105,7 @@ struct lcg_ctx {
         double bytes;
         u32 round;  // BuildGram round of a parse launch, else 0
         bool graph;  // the events belong to a captured graph
+        bool part = false;  // a further round of the launch before: no events, no time of its own
     };
     std::vector<KRec> krecs;
     std::vector<cudaEvent_t> evpool;
@@ -168,7 +171,7 @@ cudaError_t record_event(lcg_ctx* ctx, cudaEvent_t e) {
 
 void kt_reset(lcg_ctx* ctx) {
     for (auto& r : ctx->krecs) {
-        if (r.graph) continue;  // recorded by a graph's event nodes: the graph owns them
+        if (r.graph || r.part) continue;  // recorded by a graph's event nodes: the graph owns them
         ctx->evpool.push_back(r.a);
         ctx->evpool.push_back(r.b);
     }
@@ -192,13 +195,27 @@ void kt_end(lcg_ctx* ctx, int h) {
     if (h >= 0) ck(ctx, record_event(ctx, ctx->krecs[h].b), "cudaEventRecord");
 }
 
+// The launch of record h runs `more` further rounds: a record without a time
+// for each of them.
+void kt_parts(lcg_ctx* ctx, int h, u32 more) {
+    if (h < 0) return;
+    for (u32 x = 1; x <= more; x++) {
+        const lcg_ctx::KRec& r = ctx->krecs[h];
+        ctx->krecs.push_back(lcg_ctx::KRec{r.name, nullptr, nullptr, 0.0, r.round + x, false, true});
+    }
+}
+
 // After the call's last synchronisation: sum the times per kernel kind.
 void kt_collect(lcg_ctx* ctx) {
     ctx->ktimes.clear();
     ctx->klaunches.clear();
     for (auto& r : ctx->krecs) {
         float ms = 0.f;
-        ck(ctx, cudaEventElapsedTime(&ms, r.a, r.b), "cudaEventElapsedTime");
+        if (r.part) {
+            if (r.round > ctx->stats.rounds) continue;  // the build was done before it
+        } else {
+            ck(ctx, cudaEventElapsedTime(&ms, r.a, r.b), "cudaEventElapsedTime");
+        }
         lcg_kernel_launch kl{};
         std::strncpy(kl.name, r.name, sizeof(kl.name) - 1);
         kl.round = r.round;
@@ -304,24 +321,28 @@ void grow_level(lcg_ctx* ctx, Level& L, u64 need_g, u64 need_G) {
         if (L.rhs_off) {
             ck(ctx, cudaMemcpyAsync(ro, L.rhs_off, (L.g + 1) * sizeof(u64), cudaMemcpyDeviceToDevice, ctx->st), "copy");
             ck(ctx, cudaMemcpyAsync(F, L.F, L.g * sizeof(u32), cudaMemcpyDeviceToDevice, ctx->st), "copy");
-            dfree(ctx, L.rhs_off);
-            dfree(ctx, L.F);
+            if (!L.shared_rules) {
+                dfree(ctx, L.rhs_off);
+                dfree(ctx, L.F);
+            }
         } else {
             ck(ctx, cudaMemsetAsync(ro, 0, sizeof(u64), ctx->st), "memset");
         }
         L.rhs_off = ro;
         L.F = F;
         L.cap_g = cap;
+        L.shared_rules = false;
     }
     if (need_G > L.cap_G || L.rhs == nullptr) {
         u64 cap = std::max<u64>(need_G, std::max<u64>(L.cap_G * 2, 1024));
         u32* r = dalloc<u32>(ctx, cap);
         if (L.rhs) {
             ck(ctx, cudaMemcpyAsync(r, L.rhs, L.G * sizeof(u32), cudaMemcpyDeviceToDevice, ctx->st), "copy");
-            dfree(ctx, L.rhs);
+            if (!L.shared_rhs) dfree(ctx, L.rhs);
         }
         L.rhs = r;
         L.cap_G = cap;
+        L.shared_rhs = false;
     }
 }
 
@@ -397,11 +418,14 @@ void free_grammar_now(lcg_grammar* G) {
     };
     release(G->F0);
     for (Level& L : G->lv) {
-        release(L.rhs_off);
-        release(L.rhs);
-        release(L.F);
+        if (!L.shared_rules) {
+            release(L.rhs_off);
+            release(L.F);
+        }
+        if (!L.shared_rhs) release(L.rhs);
         release(L.rtab);
     }
+    for (void* p : G->slabs) release(p);
     release(G->c_level);
     release(G->c_rank);
     delete G;
@@ -637,8 +661,7 @@ void set_table(RoundArgs& a, RoundBufs& b) {
     a.rank_of = b.rank_of;
 }
 
-// The round's phrases: tile strings, breaks, tile scan, strings.  A short round
-// runs them with the parse (enqueue_parse).
+// The round's phrases: tile strings, breaks, tile scan, strings.
 void enqueue_phrases(lcg_ctx* ctx, RoundArgs& a, u64 n_for_bytes) {
     // k_breaks' look-ahead words: a buffer of their own, so that no other
     // kernel's data can read as a head of this launch's epoch
@@ -646,7 +669,6 @@ void enqueue_phrases(lcg_ctx* ctx, RoundArgs& a, u64 n_for_bytes) {
     ensure_lb(ctx, &ctx->heads, &ctx->heads_steps, steps, steps * sizeof(u64));
     a.heads = reinterpret_cast<u64*>(ctx->heads);
     a.brk_epoch = ++ctx->epoch;
-    if (round_is_small(a)) return;
     const Range range("phrases, round", a.level);
     const int ht = kt_begin(ctx, "k_tile_strings", 4.0 * (double)a.tiles_bound, a.level);
     ck(ctx, launch_tile_strings(a, ctx->st), "k_tile_strings");
@@ -672,16 +694,6 @@ void enqueue_phrases(lcg_ctx* ctx, RoundArgs& a, u64 n_for_bytes) {
 // Parse: the phrases' lookups, and the next sequence.
 void enqueue_parse(lcg_ctx* ctx, RoundArgs& a, u64 n_for_bytes) {
     const Range range("parse, round", a.level);
-    if (round_is_small(a)) {
-        // a short round: tile strings, breaks, scan, strings and parse in one cooperative launch
-        const int hs = kt_begin(ctx, "k_parse_small", 5.0 * (double)n_for_bytes, a.level);
-        const u64 bar = ctx->ctr_val;  // the grid barriers' counter values
-        ctx->ctr_val += (u64)kSmallParseBarriers * small_round_grid(a);
-        ck(ctx, launch_parse_small(a, bar, ctx->st), "k_parse_small");
-        kt_end(ctx, hs);
-        ctx->launches += 1;
-        return;
-    }
     const double tab_bytes = a.tab_cap * (double)slot_bytes();
     const double tbytes = tab_bytes > kL2Bytes ? 32.0 * (double)n_for_bytes / 3.0 : 0.0;
     const int h = kt_begin(ctx, "k_parse",
@@ -700,16 +712,6 @@ void enqueue_naming(lcg_ctx* ctx, RoundArgs& a, RoundBufs& b, double g_bytes, do
     a.rrec = b.rrec;
     a.r_cap = b.r_cap;
     const u64 g_grid = std::max<u64>(1, b.r_cap);
-    if (round_is_small(a)) {
-        // a short round: marks, popcount prefix, ranks, offsets and rules in one cooperative launch
-        const int hs = kt_begin(ctx, "k_naming_small", 100.0 * g_bytes + 4.0 * G_bytes, a.level);
-        const u64 bar = ctx->ctr_val;
-        ctx->ctr_val += (u64)kSmallNamingBarriers * small_round_grid(a);
-        ck(ctx, launch_naming_small(a, bar, ctx->st), "k_naming_small");
-        kt_end(ctx, hs);
-        ctx->launches += 1;
-        return;
-    }
     int h = kt_begin(ctx, "k_mark", 8.0 * g_bytes, a.level);
     ck(ctx, launch_mark(a, g_grid, ctx->st), "k_mark");
     kt_end(ctx, h);
@@ -756,6 +758,271 @@ void next_input(lcg_ctx* ctx, RoundInput& in, RoundBufs& b) {
     in.symb = 4;
     in.soff = b.soff_next;
     in.sid = b.sid_next;
+}
+
+// ---- the short rounds ------------------------------------------------------
+//
+// A round whose tile is the smallest (see round_tile) and that has at most
+// kTailSymbols symbols, and every round after it, run in two launches.  All
+// their buffers are parts of one allocation, sized by what a round can have at
+// most (n symbols in k strings: (n + k) / 2 phrases), so nothing is planned,
+// regrown or waited for; the levels of a fresh build share one allocation too.
+
+bool is_tail(const lcg_ctx* ctx, u64 n) { return n <= kTailSymbols && round_tile(ctx, n) == 1024; }
+
+// Offsets of the parts of one allocation.
+struct Parts {
+    u64 size = 0;
+    u64 take(u64 bytes) {
+        const u64 at = size;
+        size += (bytes + 255) & ~255ull;
+        return at;
+    }
+};
+
+// Enqueue round i and those after it (at most n_bound symbols in kk strings
+// enter it); returns how many there may be.  `in` becomes what follows the
+// last (nothing); cap[r]: the table slots of round r.
+u32 tail_enqueue(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, u64 n_bound, u32 kk, bool against_resident,
+                 const DevStatus* ds_prev, u64* cap) {
+    fail_if(ctx, i >= ctx->levels || i > kMaxRounds,
+            LCG_ELEVELS, "hash family too short: needs more than " + std::to_string(ctx->levels) + " functions");
+    const u32 most = std::min<u32>({kTailRounds, ctx->levels - i, kMaxRounds - i + 1});
+    const u32 tp = parse_unit(1024);
+    struct Size {
+        u64 n, k, P, units, cap, ids, words;
+        u64 sbm, first, tab, minpos;                                          // cleared parts
+        u64 string_first, soff, sid, R_phr, R_sid, cnt, pfx, brk, T, F, crec, rank_of, rrec;
+        u64 off, rhs, lvF;                                                    // in the levels' slab
+    };
+    std::vector<Size> z;
+    Parts zero, ones, plain, slab;
+    const u64 bar = zero.take(4 * sizeof(u64));
+    u64 chunks = 0;
+    u32 chunk_ids = 32;
+    for (u64 n = n_bound, k = std::min<u64>(kk, n_bound / 2 + 1); z.size() < most && n > 0; ) {
+        Size x{};
+        x.n = n;
+        x.k = k;
+        x.P = (n + k) / 2 + 1;
+        x.units = (n + tp - 1) / tp;
+        x.cap = 3 * x.P + 64;
+        // the parse's blocks take numbers for a warp's claims at a time, at least
+        x.ids = x.P + (u64)chunk_ids * std::min<u64>((u64)ctx->sms, (x.units + kParseWarps - 1) / kParseWarps);
+        x.words = x.P / 32 + 1;
+        x.sbm = zero.take((n / 32 + 2) * 4);
+        x.first = zero.take(x.words * sizeof(uint2));
+        x.tab = ones.take(x.cap * slot_bytes());
+        x.minpos = ones.take(x.ids * 8);
+        x.string_first = plain.take(k * 8);
+        x.soff = plain.take((k + 1) * 8);
+        x.sid = plain.take(k * 4);
+        x.R_phr = plain.take(k * 8);
+        x.R_sid = plain.take(k * 4);
+        x.cnt = plain.take(x.units * 4);
+        x.pfx = plain.take(x.units * 8);
+        x.brk = plain.take((x.units * tp / 32) * 4);
+        x.T = plain.take(x.P * 4);
+        x.F = plain.take(x.P * 4);
+        x.crec = plain.take(x.ids * claim_rec_bytes());
+        x.rank_of = plain.take(x.ids * 4);
+        x.rrec = plain.take(x.P * claim_rec_bytes());
+        x.off = slab.take((x.P + 1) * 8);
+        x.rhs = slab.take(n * 4);
+        x.lvF = slab.take(x.P * 4);
+        chunks += rule_chunks(x.P);
+        z.push_back(x);
+        // the strings left have two symbols or more each
+        const u64 n1 = (n + k) / 2;
+        k = std::min<u64>(k, n1 / 2);
+        n = k ? n1 : 0;
+    }
+    const u32 rounds = (u32)z.size();
+    const u64 chunk_len = plain.take(chunks * 8);
+    unsigned char* base = dalloc<unsigned char>(ctx, zero.size + ones.size + plain.size);
+    unsigned char *b0 = base, *b1 = base + zero.size, *b2 = b1 + ones.size;
+    ck(ctx, cudaMemsetAsync(b0, 0, zero.size, ctx->st), "memset");
+    ck(ctx, cudaMemsetAsync(b1, 0xFF, ones.size, ctx->st), "memset tables");
+    unsigned char* lv = nullptr;
+    if (!against_resident) {
+        lv = dalloc<unsigned char>(ctx, slab.size);
+        R->slabs.push_back(lv);
+    }
+    const u64 steps = breaks_steps(z[0].units, tp);
+    ensure_lb(ctx, &ctx->heads, &ctx->heads_steps, steps, steps * sizeof(u64));
+    TailArgs t{};
+    t.rounds = rounds;
+    t.bar = (u64*)(b0 + bar);
+    t.chunk_len = (u64*)(b2 + chunk_len);
+    for (u32 r = 0; r < rounds; r++) {
+        const Size& x = z[r];
+        const u32 lev = i + r;
+        if (R->lv.size() < lev) R->lv.emplace_back();
+        Level& L = R->lv[lev - 1];
+        if (against_resident) {
+            if (L.g > 0) ensure_resident(ctx, R, lev, L.g + x.P);
+            grow_level(ctx, L, L.g + x.P, L.G + x.n);
+            if (L.g == 0) ensure_resident(ctx, R, lev, x.P);
+        } else {
+            L.rhs_off = (u64*)(lv + x.off);
+            L.rhs = (u32*)(lv + x.rhs);
+            L.F = (u32*)(lv + x.lvF);
+            L.cap_g = x.P;
+            L.cap_G = x.n;
+            L.shared_rules = L.shared_rhs = true;
+            L.rvalid = false;
+        }
+        RoundArgs& a = t.r[r];
+        a.sym_bytes = r == 0 ? in.symb : 4;
+        a.S = r == 0 ? in.S : b2 + z[r - 1].T;
+        a.Sf = r == 0 ? in.Sf : (u32*)(b2 + z[r - 1].F);
+        a.n = r == 0 ? in.n : 0;
+        a.d_n = r == 0 ? in.d_n : &ctx->rc_arr[lev - 2].n_next;
+        a.soff = r == 0 ? in.soff : (u64*)(b2 + z[r - 1].soff);
+        a.sid = r == 0 ? in.sid : (u32*)(b2 + z[r - 1].sid);
+        a.k = r == 0 ? in.kk : 0;
+        a.d_k = r == 0 ? in.d_k : &ctx->rc_arr[lev - 2].k_next;
+        a.Fprev = fprev_of(R, lev);
+        a.lh = level_hash(ctx, lev);
+        a.level = lev;
+        a.stripes = 1;
+        a.tp = tp;
+        a.prev_base = r == 0 ? in.prev_base : t.r[r - 1].id_base;
+        a.id_base = against_resident ? (u32)L.g : 0;
+        a.rank_prev = r == 0 ? in.rank_prev : t.r[r - 1].rank_of;
+        a.tiles_bound = x.units;
+        a.brk = (u32*)(b2 + x.brk);
+        a.sbm = (u32*)(b0 + x.sbm);
+        a.sbm_words = x.n / 32 + 2;
+        a.tile_cnt = (u32*)(b2 + x.cnt);
+        a.tile_pfx = (u64*)(b2 + x.pfx);
+        a.string_first = (u64*)(b2 + x.string_first);
+        a.heads = (u64*)ctx->heads;
+        a.brk_epoch = ++ctx->epoch;
+        a.ds = ctx->ds_arr + (lev - 1);
+        a.ds_prev = r == 0 ? ds_prev : ctx->ds_arr + (lev - 2);
+        a.rc = ctx->rc_arr + (lev - 1);
+        a.d_tiles = &a.rc->tiles;
+        a.total = ctx->tot_arr + 3 * (lev - 1);
+        a.soff_next = (u64*)(b2 + x.soff);
+        a.sid_next = (u32*)(b2 + x.sid);
+        if (r + 1 < rounds) {
+            a.sbm_next = (u32*)(b0 + z[r + 1].sbm);
+            a.sbm_next_words = z[r + 1].n / 32 + 2;
+        }
+        a.R_phr = (u64*)(b2 + x.R_phr);
+        a.R_sid = (u32*)(b2 + x.R_sid);
+        a.tab = b1 + x.tab;
+        a.tab_cap = x.cap;
+        a.id_cap = x.ids;
+        a.id_chunk = chunk_ids;
+        a.crec = b2 + x.crec;
+        a.minpos = (u64*)(b1 + x.minpos);
+        a.rank_of = (u32*)(b2 + x.rank_of);
+        a.T_cap = x.P;
+        a.Tnext = (u32*)(b2 + x.T);
+        a.Fnext = (u32*)(b2 + x.F);
+        a.c_level = R->c_level;
+        a.c_rank = R->c_rank;
+        a.d_gnew = &a.ds->claims;
+        a.d_ids = &a.ds->aux[1];
+        a.d_Gnew = &a.ds->claim_len;
+        a.cap_g = L.cap_g;
+        a.cap_G = L.cap_G;
+        a.first_words = x.words;
+        a.first = (uint2*)(b0 + x.first);
+        a.r_cap = x.P;
+        a.rrec = b2 + x.rrec;
+        a.g_base = L.g;
+        a.G_base = L.G;
+        a.rhs = L.rhs;
+        a.rhs_off = L.rhs_off;
+        a.F = L.F;
+        // keys as narrow as the symbols' ids allow (tables of resident grammars
+        // keep the full width)
+        a.sym_w = a.sym_bytes == 1 ? 8 : against_resident ? 31
+                  : rank_width(r == 0 ? in.prev_base + in.prev_cap : z[r - 1].ids);
+        if (against_resident) {
+            if (L.g > 0) {
+                a.rtab = L.rtab;
+                a.rtab_cap = L.rcap;
+                a.rrhs = L.rhs;
+                a.rrhs_off = L.rhs_off;
+            }
+            a.rtab_w = L.rtab;
+            a.rtab_w_cap = L.rcap;
+        }
+        cap[lev] = x.cap;
+    }
+    const Range range("short rounds from", i);
+    int h = kt_begin(ctx, "k_parse_small", 5.0 * (double)n_bound, i);
+    ck(ctx, launch_parse_small(t, ctx->st), "k_parse_small");
+    kt_end(ctx, h);
+    kt_parts(ctx, h, rounds - 1);
+    h = kt_begin(ctx, "k_naming_small", 12.0 * (double)n_bound, i);
+    ck(ctx, launch_naming_small(t, ctx->st), "k_naming_small");
+    kt_end(ctx, h);
+    ctx->launches += 2;
+    free_round_input(ctx, in);
+    dfree(ctx, base);
+    const u64 n = in.n;
+    in = RoundInput{};
+    in.n = n;
+    return rounds;
+}
+
+// The short rounds of a build that is run round by round: one host
+// synchronisation after all of them.
+void tail_sync(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32& i, bool against_resident) {
+    u64 cap[kMaxRounds + kTailRounds + 2] = {0};
+    u64 n = in.n;
+    u32 k = in.kk;
+    const u32 rounds = tail_enqueue(ctx, R, in, i, in.n, in.kk, against_resident, nullptr, cap);
+    std::vector<DevStatus> st(rounds);
+    std::vector<RoundCounts> rc(rounds);
+    ck(ctx, cudaMemcpyAsync(st.data(), ctx->ds_arr + (i - 1), rounds * sizeof(DevStatus), cudaMemcpyDeviceToHost,
+                            ctx->st), "read status");
+    ck(ctx, cudaMemcpyAsync(rc.data(), ctx->rc_arr + (i - 1), rounds * sizeof(RoundCounts), cudaMemcpyDeviceToHost,
+                            ctx->st), "read counts");
+    sync(ctx);
+    for (const DevStatus& x : st) {
+        check_device_status(ctx, x);
+        fail_if(ctx, x.overflow != 0, LCG_ETABLE, "phrase table full");  // not reached: it has room for every phrase
+    }
+    u32 r = 0;
+    for (; r < rounds && k > 0; r++) {
+        Level& L = R->lv[i + r - 1];
+        fail_if(ctx, L.g + st[r].claims > kMaxRank, LCG_EOVERFLOW, "level with 2^31 rules or more");
+        L.g += st[r].claims;
+        L.G += st[r].claim_len;
+        lcg_round_stats& rs = ctx->stats.round[std::min<u32>(i + r - 1, 63)];
+        rs.n = n;
+        rs.strings = k;
+        rs.phrases = rc[r].phrases;
+        rs.g = st[r].claims;
+        rs.G = st[r].claim_len;
+        rs.table_cap = cap[i + r];
+        record_hints(ctx, i + r, n, rc[r].phrases, st[r].claims, st[r].claim_len);
+        n = rc[r].n_next;
+        k = (u32)rc[r].k_next;
+        ctx->stats.rounds = i + r;
+    }
+    // levels that no round reached
+    while (R->lv.size() > (size_t)(i + r - 1) && R->lv.back().g == 0) {
+        Level& L = R->lv.back();
+        if (!L.shared_rules) {
+            dfree(ctx, L.rhs_off);
+            dfree(ctx, L.F);
+        }
+        if (!L.shared_rhs) dfree(ctx, L.rhs);
+        dfree(ctx, L.rtab);
+        R->lv.pop_back();
+    }
+    i += r;
+    in.kk = k;
+    in.n = n;
+    fail_if(ctx, k > 0, LCG_ELEVELS,
+            "hash family too short: needs more than " + std::to_string(ctx->levels) + " functions");
 }
 
 // One round with a host synchronisation after the parse: the table is
@@ -817,10 +1084,9 @@ void round_sync(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, bool agains
     ck(ctx, cudaMemsetAsync(a.ds, 0, sizeof(DevStatus), ctx->st), "reset counters");
     enqueue_phrases(ctx, a, n);
     // The next sequence: at most Pmax symbols; a large one gets exactly the
-    // round's phrases, which the host then waits for (the short rounds' parse
-    // counts them itself).
+    // round's phrases, which the host then waits for.
     u64 t_cap = b.Pmax;
-    if (!round_is_small(a) && t_cap > kExactNext) {
+    if (t_cap > kExactNext) {
         ck(ctx, cudaMemcpyAsync(&rc, a.rc, sizeof(rc), cudaMemcpyDeviceToHost, ctx->st), "read counts");
         ck(ctx, cudaMemcpyAsync(&st, a.ds, sizeof(st), cudaMemcpyDeviceToHost, ctx->st), "read status");
         sync(ctx);
@@ -895,6 +1161,7 @@ void round_sync(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, bool agains
 struct RoundPlan {
     u64 n_bound = 0, n_est = 0, n_alloc = 0, cap = 0, g_alloc = 0, G_alloc = 0, t_cap = 0;
     double P_est = 0, g_est = 0, G_est = 0;
+    bool tail = false;  // this round and all after it run as the short rounds (n_alloc symbols at most)
 };
 
 // x rounded up to a step of 2^(1/4) (about 19 %): plans from slightly
@@ -920,6 +1187,11 @@ std::vector<RoundPlan> plan_rounds(lcg_ctx* ctx, u64 n1, u32 kk, u32 planned) {
         // the round's sequence is at most the planned next sequence of the
         // round before (which flags a capacity error past it)
         p.n_alloc = (r == 1) ? n_bound : std::min<u64>(n_bound, v[r - 1].t_cap);
+        p.tail = is_tail(ctx, p.n_alloc);
+        if (p.tail) {
+            v.resize(r + 1);
+            break;
+        }
         p.P_est = ctx->p_hint[r] * (double)n_est;
         p.g_est = ctx->ratio_hint[r] * p.P_est;
         p.G_est = ctx->glen_hint[r] * p.g_est;
@@ -943,21 +1215,29 @@ std::vector<RoundPlan> plan_rounds(lcg_ctx* ctx, u64 n1, u32 kk, u32 planned) {
 // Rounds enqueued without host synchronisation, between their enqueueing and
 // the reading of their statuses.
 struct AsyncRounds {
-    u32 planned = 0, kk = 0;
+    u32 planned = 0, kk = 0;  // rounds (with those of the tail), strings
     std::vector<RoundPlan> plan;
-    std::vector<u64> g_base, G_base;
+    std::vector<u64> g_base, G_base, cap;
 };
 
 // Enqueue the planned rounds of a fresh build: every size comes from the plan;
 // kernels read the actual sizes from the device and flag a round that
 // outgrows its buffers.
 void rounds_async_enqueue(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, AsyncRounds& ar) {
-    const u32 planned = ar.planned;
     const u32 kk = ar.kk;
-    ar.g_base.assign(planned + 1, 0);
-    ar.G_base.assign(planned + 1, 0);
-    for (u32 r = 1; r <= planned; r++) {
+    ar.planned = (u32)ar.plan.size() - 1;
+    ar.g_base.assign(kMaxRounds + 1, 0);
+    ar.G_base.assign(kMaxRounds + 1, 0);
+    ar.cap.assign(kMaxRounds + 1, 0);
+    for (u32 r = 1; r < ar.plan.size(); r++) {
         const RoundPlan& p = ar.plan[r];
+        if (p.tail) {
+            const DevStatus* before = r > 1 ? ctx->ds_arr + (r - 2) : nullptr;
+            const u32 rounds = tail_enqueue(ctx, R, in, r, p.n_alloc, kk, false, before, ar.cap.data());
+            ar.planned = r - 1 + rounds;
+            return;
+        }
+        ar.cap[r] = p.cap;
         if (R->lv.size() < r) R->lv.emplace_back();
         Level& L = R->lv[r - 1];
         RoundBufs b;
@@ -1021,9 +1301,11 @@ int rounds_async_finish(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, const Asyn
     while (R->lv.size() > used && R->lv.back().g == 0 && ar.g_base.size() > R->lv.size()) {
         Level& L = R->lv.back();
         if (st[R->lv.size() - 1].claims != 0) break;
-        dfree(ctx, L.rhs_off);
-        dfree(ctx, L.rhs);
-        dfree(ctx, L.F);
+        if (!L.shared_rules) {
+            dfree(ctx, L.rhs_off);
+            dfree(ctx, L.F);
+        }
+        if (!L.shared_rhs) dfree(ctx, L.rhs);
         dfree(ctx, L.rtab);
         R->lv.pop_back();
     }
@@ -1039,7 +1321,7 @@ int rounds_async_finish(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, const Asyn
         rs.n = n;
         rs.strings = (r == 1) ? kk : rc[r - 2].k_next;
         rs.phrases = c.phrases;
-        rs.table_cap = ar.plan[r].cap;
+        rs.table_cap = ar.cap[r];
         rs.g = s.claims;
         rs.G = s.claim_len;
         record_hints(ctx, r, n, c.phrases, s.claims, s.claim_len);
@@ -1123,6 +1405,7 @@ bool plan_covers(const std::vector<RoundPlan>& have, const std::vector<RoundPlan
     for (size_t r = 1; r < have.size(); r++) {
         const RoundPlan& h = have[r];
         const RoundPlan& n = need[r];
+        if (h.tail || n.tail) return h.tail && n.tail && h.n_alloc >= n.n_alloc;
         if (h.n_bound != n.n_bound || h.n_alloc < n.n_alloc || h.cap < n.cap || h.cap > 4 * n.cap ||
             h.g_alloc < n.g_alloc || h.G_alloc < n.G_alloc || h.t_cap < n.t_cap)
             return false;
@@ -1141,6 +1424,7 @@ void destroy_graph(lcg_ctx* ctx) {
                                     [](const lcg_ctx::KRec& r) { return r.graph; }),
                      ctx->krecs.end());
     for (auto& r : gb->krecs) {
+        if (r.part) continue;
         cudaEventDestroy(r.a);
         cudaEventDestroy(r.b);
     }
@@ -1170,8 +1454,12 @@ void capture_graph(lcg_ctx* ctx, const unsigned char* d_in, const std::vector<u6
     // look-back buffers and timing events for every launch, made before the
     // capture (the graph must not reallocate them)
     u64 t1 = 1, t2 = 1, hs = 1;
-    for (u32 r = 1; r <= planned; r++) {
+    for (u32 r = 1; r < plan.size(); r++) {
         const RoundPlan& p = plan[r];
+        if (p.tail) {
+            hs = std::max(hs, breaks_steps((kTailSymbols + parse_unit(1024) - 1) / parse_unit(1024), parse_unit(1024)));
+            break;
+        }
         const u32 tp = parse_unit(round_tile(ctx, p.n_alloc));
         const u64 tiles = (p.n_alloc + tp - 1) / tp;
         t1 = std::max({t1, tiles, popscan_tiles_for((p.t_cap + k) / 32 + 1), rule_offs_tiles(std::max<u64>(1, p.g_alloc))});
@@ -1416,7 +1704,10 @@ void build_into(lcg_ctx* ctx, lcg_grammar* R, const uint8_t* data, const uint64_
         }
     }
     double prev_ratio = 0.0, p_ratio = 0.35;
-    for (; in.kk > 0; i++) round_sync(ctx, R, in, i, against_resident, prev_ratio, p_ratio);
+    while (in.kk > 0) {
+        if (is_tail(ctx, in.n)) tail_sync(ctx, R, in, i, against_resident);
+        else round_sync(ctx, R, in, i++, against_resident, prev_ratio, p_ratio);
+    }
     check_device_status(ctx, read_status(ctx));
     ctx->hint_rounds = ctx->stats.rounds;
     free_round_input(ctx, in);
@@ -1930,7 +2221,7 @@ void lcg_ctx_destroy(lcg_ctx* ctx) {
     destroy_graph(ctx);
     if (ctx->upload) cudaFree(ctx->upload);
     for (auto& r : ctx->krecs) {
-        if (r.graph) continue;  // destroyed with the graph
+        if (r.graph || r.part) continue;  // destroyed with the graph
         cudaEventDestroy(r.a);
         cudaEventDestroy(r.b);
     }

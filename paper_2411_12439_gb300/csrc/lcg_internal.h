@@ -99,7 +99,7 @@ struct RoundArgs {
     u32* brk;             // break bitmap of T^i (k_breaks), one bit per position
     u32* sbm;             // bitmap of string starts of T^i (and of n)
     u64 sbm_words;
-    u32* step_str;        // per block step of k_breaks: the string holding its first position
+    u32* step_str;        // per block step of k_breaks: the string holding its first position (or null)
     u32* tile_cnt;        // per parse unit: phrases starting in it
     u64* tile_pfx;        // exclusive prefix of tile_cnt: global index of a unit's first phrase
     u64* string_first;    // unit * tp + q of each active string's first phrase (q: its index in the unit)
@@ -114,6 +114,8 @@ struct RoundArgs {
     // strings
     u64* soff_next;
     u32* sid_next;
+    u32* sbm_next;        // the next round's bitmap of string starts, when this round's strings fill it, or null
+    u64 sbm_next_words;
     u64* R_phr;           // phrase indices (ascending) of the strings that became one phrase
     u32* R_sid;           // their string indices
     RoundCounts* rc;
@@ -157,9 +159,21 @@ bool parse_tile_valid(u32 tp);                 // 1024, 2048 or 4096 positions
 u32 parse_unit(u32 tile);                      // positions that each warp of a block takes of a tile
 constexpr u32 kParseBlocksMax = 4;             // k_parse blocks per SM at most (its launch bounds)
 constexpr u32 kParseWarps = 8;                 // warps of a block, a unit each
-bool round_is_small(const RoundArgs& a);        // the round runs as k_parse_small and k_naming_small
-u32 small_round_grid(const RoundArgs& a);       // their blocks (one launch of each per round)
-constexpr u32 kSmallParseBarriers = 3, kSmallNamingBarriers = 4;  // grid barriers of each
+// The short rounds at a build's end: one launch for their phrases and parses,
+// one for their naming.
+constexpr u64 kTailSymbols = 131072;  // of the first of them, at most
+constexpr u32 kTailRounds = 20;       // (each has at most half the symbols and a symbol per string)
+struct TailArgs {
+    u32 rounds;
+    u64* bar;        // two zeroed counters of grid barriers for each launch
+    u64* chunk_len;  // naming: symbols of each chunk of rules
+    RoundArgs r[kTailRounds];
+};
+static_assert(sizeof(TailArgs) <= 32000, "kernel parameters");
+cudaError_t launch_parse_small(const TailArgs& t, cudaStream_t st);
+cudaError_t launch_naming_small(const TailArgs& t, cudaStream_t st);
+u64 rule_chunks(u64 g);  // chunks of g rules
+
 size_t claim_rec_bytes();                       // bytes of one ClaimRec
 u64 breaks_steps(u64 units, u32 tp);           // k_breaks' block steps over a round's parse units
 u64 popscan_tiles_for(u64 nw);
@@ -170,8 +184,6 @@ size_t slot_bytes();  // bytes of one phrase-table slot
 cudaError_t launch_tile_strings(const RoundArgs& a, cudaStream_t st);
 cudaError_t launch_breaks(const RoundArgs& a, cudaStream_t st);
 cudaError_t launch_parse(const RoundArgs& a, cudaStream_t st);
-cudaError_t launch_parse_small(const RoundArgs& a, u64 bar_base, cudaStream_t st);
-cudaError_t launch_naming_small(const RoundArgs& a, u64 bar_base, cudaStream_t st);
 int parse_max_blocks(int sym_bytes);  // resident k_parse blocks per SM at most
 cudaError_t launch_strings(const RoundArgs& a, cudaStream_t st);
 cudaError_t launch_mark(const RoundArgs& a, u64 g_grid, cudaStream_t st);

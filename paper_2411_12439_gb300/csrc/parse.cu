@@ -31,12 +31,12 @@
 // a rewrite pass followed the naming and read (F^i, rank) of every phrase
 // from an array indexed by slot: one random DRAM sector per phrase in the
 // rounds whose table is beyond L2 (4 x 3.1 Gbp: 42.3 ms of 218 ms).
-// A short round (at most kSmallTiles tiles) runs the same steps as two
-// cooperative launches instead: k_parse_small (tile strings to parse) and
-// k_naming_small (marks to rules), with grid barriers between the steps.
+// The short rounds at a build's end (and the whole of a small build) run in two
+// cooperative launches: k_parse_small and k_naming_small, further down.
 // Every kernel of the round starts with pdl_wait(): it is launched with
 // programmatic dependent launch after the one before it.
 #include <algorithm>
+#include <type_traits>
 #include <utility>
 
 #include "lcg_dev.cuh"
@@ -104,11 +104,6 @@ __device__ __forceinline__ u32 string_of(const u64* soff, u32 k, u64 pos) {
 
 constexpr int kParseThreads = 32 * (int)kParseWarps;
 constexpr int kUnitMin = 128, kUnitMax = 512;
-// Rounds of at most kSmallUnits units of kUnitMin positions run as two
-// cooperative launches (parse; naming) whose steps are separated by grid
-// barriers, instead of ten launches: launch latency, not work, bounds such
-// rounds.
-constexpr u64 kSmallUnits = 1024;
 constexpr int kHalo = 64;  // symbols staged past the unit's end
 
 // Unit order of the rank rounds' parse: with `stripes` = k > 1
@@ -392,7 +387,9 @@ __device__ __forceinline__ void body_breaks(const RoundArgs& a, u64 nblocks) {
             s_pre[tid] = pre - __shfl_sync(0xffffffffu, pre, lane & ~(int)(lpu - 1));
             __syncthreads();
             const u32 kact = round_k(a);
-            for (u32 jj = a.step_str[b] + (u32)tid;; jj += kBrkThreads) {
+            // (the rounds of one launch have no table of the steps' strings)
+            const u32 j0 = a.step_str != nullptr ? a.step_str[b] : string_of(a.soff, kact, base);
+            for (u32 jj = j0 + (u32)tid;; jj += kBrkThreads) {
                 const u64 s = jj < kact ? __ldg(a.soff + jj) : ~0ull;
                 if (s >= base && s < bend) {
                     const u32 x = (u32)(s - base);
@@ -1031,8 +1028,9 @@ __device__ __forceinline__ void body_tile_strings(const RoundArgs& a, u64 tiles)
     }
     if (round_halted(a)) return;
     const u64 steps = (min(tiles * a.tp, n) + kBrkSpan - 1) / kBrkSpan;
-    for (u64 t = blockIdx.x * (u64)blockDim.x + threadIdx.x; t < steps; t += (u64)gridDim.x * blockDim.x)
-        a.step_str[t] = string_of(a.soff, k, t * kBrkSpan);
+    if (a.step_str != nullptr)
+        for (u64 t = blockIdx.x * (u64)blockDim.x + threadIdx.x; t < steps; t += (u64)gridDim.x * blockDim.x)
+            a.step_str[t] = string_of(a.soff, k, t * kBrkSpan);
     // bitmap of string starts (and of n), zeroed by the host
     for (u64 j = blockIdx.x * (u64)blockDim.x + threadIdx.x; j <= k; j += (u64)gridDim.x * blockDim.x) {
         const u64 s0 = __ldg(a.soff + j);
@@ -1067,14 +1065,20 @@ __device__ __forceinline__ void body_strings(const RoundArgs& a) {
                 a.R_phr[rb] = first;
                 a.R_sid[rb] = a.sid[j];
             } else {
-                a.soff_next[j - rb] = first - rb;
+                const u64 s0 = first - rb;
+                a.soff_next[j - rb] = s0;
                 a.sid_next[j - rb] = a.sid[j];
+                if (a.sbm_next != nullptr && (s0 >> 5) < a.sbm_next_words)
+                    atomicOr(a.sbm_next + (s0 >> 5), 1u << (s0 & 31));
             }
         }
         carry += tot;
     }
     if (threadIdx.x == 0) {
-        a.soff_next[k - carry] = P - carry;
+        const u64 s0 = P - carry;
+        a.soff_next[k - carry] = s0;
+        if (a.sbm_next != nullptr && (s0 >> 5) < a.sbm_next_words)
+            atomicOr(a.sbm_next + (s0 >> 5), 1u << (s0 & 31));
         a.rc->phrases = P;
         a.rc->retired = carry;
         a.rc->k_next = k - carry;
@@ -1237,32 +1241,21 @@ __device__ __forceinline__ u32 sym_rank(const RoundArgs& a, u32 v) {
     return v < a.prev_base ? v : __ldg(a.rank_prev + (v - a.prev_base));
 }
 
-// The new rules of level i in rank order: right-hand sides (ids translated to
-// ranks) and F^i.  When the grammar keeps a table of its rules, the new rules
-// enter it.  The roots of the retired strings get their ranks.
+// The new rules first, first + stride, ... below `end` of this thread (in rank
+// order; a warp's 32 threads take consecutive ones): right-hand sides (ids
+// translated to ranks) and F^i; their offsets are written.
 template <typename T>
-__device__ __forceinline__ void body_rules(const RoundArgs& a) {
-    pdl_wait();
+__device__ __forceinline__ void rules_range(const RoundArgs& a, u64 first, u64 stride, u64 end) {
     const T* S = (const T*)a.S;
     const ContentTable rw{(Slot*)a.rtab_w, a.rtab_w_cap};
-    if (round_halted(a)) return;
-    const u64 g_new = round_gnew(a);
-    if (!rules_fit(a)) return;
-    for (u64 x = blockIdx.x * (u64)blockDim.x + threadIdx.x; x < a.rc->retired; x += (u64)gridDim.x * blockDim.x) {
-        const u32 id = a.c_rank[a.R_sid[x]];
-        if (id < a.id_base) continue;
-        if (id - a.id_base < a.id_cap) a.c_rank[a.R_sid[x]] = a.rank_of[id - a.id_base];
-        else set_error(a.ds, kErrCapacity);
-    }
     // whole warps step through the ranks, so that a warp can take its long
     // rules (more than kLongLen symbols) together after its short ones
     const u32 lane = threadIdx.x & 31;
     const ClaimRec* rec = (const ClaimRec*)a.rrec;
-    const u64 stride = (u64)gridDim.x * blockDim.x;
-    for (u64 r0 = blockIdx.x * (u64)blockDim.x + (threadIdx.x & ~31u); r0 < g_new; r0 += stride) {
+    for (u64 r0 = first - lane; r0 < end; r0 += stride) {
         const u64 r = r0 + lane;
         bool longr = false;
-        if (r < g_new) {
+        if (r < end) {
             const Key128 k = rec[r].key;
             const u64 len = key_len(k);
             const bool hashed = key_is_hashed(k);
@@ -1312,6 +1305,24 @@ __device__ __forceinline__ void body_rules(const RoundArgs& a) {
             }
         }
     }
+}
+
+// The new rules of level i in rank order: right-hand sides (ids translated to
+// ranks) and F^i.  When the grammar keeps a table of its rules, the new rules
+// enter it.  The roots of the retired strings get their ranks.
+template <typename T>
+__device__ __forceinline__ void body_rules(const RoundArgs& a) {
+    pdl_wait();
+    if (round_halted(a)) return;
+    const u64 g_new = round_gnew(a);
+    if (!rules_fit(a)) return;
+    for (u64 x = blockIdx.x * (u64)blockDim.x + threadIdx.x; x < a.rc->retired; x += (u64)gridDim.x * blockDim.x) {
+        const u32 id = a.c_rank[a.R_sid[x]];
+        if (id < a.id_base) continue;
+        if (id - a.id_base < a.id_cap) a.c_rank[a.R_sid[x]] = a.rank_of[id - a.id_base];
+        else set_error(a.ds, kErrCapacity);
+    }
+    rules_range<T>(a, blockIdx.x * (u64)blockDim.x + threadIdx.x, (u64)gridDim.x * blockDim.x, g_new);
 }
 
 // --------------------------------------------------------------------------
@@ -1377,12 +1388,67 @@ __global__ void k_rank(const RoundArgs a) { body_rank(a); }
 template <typename T>
 __global__ void k_rules(const RoundArgs a) { body_rules<T>(a); }
 
-// Exclusive prefix of get(0 .. n) by one block of kSmallThreads threads:
-// put(i, prefix) for every i, and the sum to every thread.
-constexpr int kSmallThreads = 256;
-constexpr int kSmallItems = 16;
+// --------------------------------------------------------------------------
+// the short rounds: all that are left of a build in two launches
+// --------------------------------------------------------------------------
+//
+// Once a round has at most kTailSymbols symbols, it and every round after it
+// run in one cooperative launch for their phrases and parses (k_parse_small)
+// and one for their naming (k_naming_small): no later round reads a round's
+// ranks (the sequences hold ids), so the naming of all of them can wait.
+// What bounds such rounds is latency: before, each took two cooperative
+// launches of its own with 3 and 4 grid barriers (55-95 us a round; a string of
+// 20 kB has 10 rounds and nothing else); now a round has two barriers and all
+// namings share four.  The sizes need no plan and cannot be outgrown: a round
+// of n symbols in k strings has at most (n + k) / 2 phrases.
+
+// Barrier over the grid of a cooperative launch, the idx-th of the launch
+// (idx = 0, 1, ...); bar: two zeroed counters (arrivals, releases).  The last
+// block to arrive runs `work` before it lets the others go.  Bounded: after
+// kSpinLimit polls the round fails with kErrTimeout and the later steps do
+// nothing.
+template <typename Work>
+__device__ __forceinline__ void grid_barrier_work(u64* bar, u64 idx, DevStatus* ds, Work work) {
+    __shared__ u32 s_last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_last = atomicAdd(&bar[0], 1ull) == (idx + 1) * gridDim.x - 1 ? 1u : 0u;
+    }
+    __syncthreads();
+    if (s_last) {
+        __threadfence();
+        work();
+        __syncthreads();
+        if (threadIdx.x == 0)
+            asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(&bar[1]), "l"(idx + 1) : "memory");
+    } else if (threadIdx.x == 0) {
+        u64 it = 0;
+        while (true) {
+            u64 v;
+            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(&bar[1]) : "memory");
+            if (v > idx) break;
+            if (++it > kSpinLimit) {
+                set_error(ds, kErrTimeout);
+                break;
+            }
+            __nanosleep(32);
+        }
+    }
+    __syncthreads();
+}
+__device__ __forceinline__ void grid_barrier(u64* bar, u64 idx, DevStatus* ds) {
+    grid_barrier_work(bar, idx, ds, [] {});
+}
+
+constexpr int kSmallThreads = kParseThreads;
+static_assert(kSmallThreads == kBrkThreads, "one block shape");
+
+// Exclusive prefix of get(0 .. n) by one block: put(i, prefix) for every i;
+// returns the sum (every thread).
+constexpr int kSmallItems = 4;
 template <typename Get, typename Put>
-__device__ u64 block_scan_small(Get get, u64 n, Put put) {
+__device__ __forceinline__ u64 block_scan_small(Get get, u64 n, Put put) {
     u64 carry = 0;
     for (u64 base = 0; base < n; base += (u64)kSmallThreads * kSmallItems) {
         const u64 p0 = base + (u64)threadIdx.x * kSmallItems;
@@ -1406,80 +1472,175 @@ __device__ u64 block_scan_small(Get get, u64 n, Put put) {
     return carry;
 }
 
-// Barrier over the grid of a cooperative launch: the k-th barrier of a launch
-// waits until the round's counter has reached base + k * gridDim.x (every
-// block arrived).  Bounded: after kSpinLimit polls the round fails with
-// kErrTimeout and the kernel's later steps return at once.
-__device__ void grid_barrier(u64* ctr, u64 target, DevStatus* ds) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(ctr, 1ull);
-        u64 it = 0;
-        u32 backoff = 32;
-        while (true) {
-            u64 v;
-            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(ctr) : "memory");
-            if (v >= target) break;
-            if (++it > kSpinLimit) {
-                set_error(ds, kErrTimeout);
-                break;
-            }
-            __nanosleep(backoff);
-            if (backoff < 256) backoff <<= 1;
+// Rounds of at most this many symbols are left to block 0 alone, which needs no
+// grid barrier.
+constexpr u64 kSoloSymbols = 1024;
+
+// The phrases and the parse of the rounds t.r[0 .. t.rounds), until no string
+// is left.
+template <bool kByte>
+__global__ void __launch_bounds__(kSmallThreads) k_parse_small(const __grid_constant__ TailArgs t) {
+    pdl_wait();
+    bool solo = gridDim.x == 1;
+    u64 idx = 0;
+    for (u32 r = 0; r < t.rounds; r++) {
+        const RoundArgs& a = t.r[r];
+        const u64 n = round_n(a);
+        if (n == 0) break;
+        if (!solo && n <= kSoloSymbols) {
+            if (blockIdx.x != 0) return;
+            solo = true;
         }
-        __threadfence();
+        auto barrier = [&](auto work) {
+            if (solo) {
+                __syncthreads();
+                __threadfence();
+                work();
+                __syncthreads();
+            } else {
+                grid_barrier_work(t.bar, idx++, a.ds, work);
+            }
+        };
+        if (r == 0) {
+            body_tile_strings(a, a.tiles_bound);
+            barrier([] {});
+        }
+        const u64 steps = (n + kBrkSpan - 1) / kBrkSpan;
+        if (kByte && r == 0) body_breaks<unsigned char>(a, steps);
+        else body_breaks<u32>(a, steps);
+        // places of the units' phrases; the strings, and their starts in T^{i+1}
+        barrier([&] {
+            const u64 units = min((n + a.tp - 1) / a.tp, a.tiles_bound);
+            const u64 P = block_scan_small([&](u64 i) { return a.tile_cnt[i]; }, units,
+                                           [&](u64 i, u64 e) { a.tile_pfx[i] = e; });
+            if (threadIdx.x == 0) *a.total = P;
+            __syncthreads();
+            body_strings(a);
+        });
+        if (kByte && r == 0) body_parse<unsigned char, kUnitMin>(a, a.tiles_bound);
+        else body_parse<u32, kUnitMin>(a, a.tiles_bound);
+        barrier([] {});
+    }
+}
+
+// The naming of the same rounds: marks, popcount prefixes (a round's by one
+// block), ranks, then the rules in chunks of kRuleChunk: the chunks' lengths,
+// and each chunk's offsets and right-hand sides by one block.
+constexpr u32 kRuleChunk = 512;
+
+template <bool kByte>
+__global__ void __launch_bounds__(kSmallThreads) k_naming_small(const __grid_constant__ TailArgs t) {
+    pdl_wait();
+    __shared__ u32 s_chunk0[kTailRounds + 1];  // first chunk of each round
+    __shared__ u64 s_ids[kTailRounds], s_g[kTailRounds], s_words[kTailRounds], s_retired[kTailRounds];
+    __shared__ u32 s_halt;
+    const u64 gthreads = (u64)gridDim.x * blockDim.x, gtid = blockIdx.x * (u64)blockDim.x + threadIdx.x;
+    if (threadIdx.x == 0) s_halt = 0;
+    __syncthreads();
+    if (threadIdx.x < t.rounds) {
+        const RoundArgs& a = t.r[threadIdx.x];
+        const u64 g = *a.d_gnew;
+        if (vload(&a.ds->error) || vload(&a.ds->overflow)) s_halt = 1;
+        if (threadIdx.x == 0 && a.ds_prev && (vload(&a.ds_prev->error) || vload(&a.ds_prev->overflow))) s_halt = 1;
+        if (g > a.r_cap || a.g_base + g > a.cap_g || a.G_base + *a.d_Gnew > a.cap_G) {
+            set_error(a.ds, kErrCapacity);  // not reached: the sizes are bounds
+            s_halt = 1;
+        }
+        s_g[threadIdx.x] = g;
+        s_ids[threadIdx.x] = min(*a.d_ids, a.id_cap);
+        s_words[threadIdx.x] = g ? min(a.first_words, (*a.total + 31) / 32) : 0;
+        s_retired[threadIdx.x] = a.rc->retired;
     }
     __syncthreads();
-}
-
-// A short round's parse in one cooperative launch instead of five: tile
-// strings, breaks, block 0 scans the tiles' phrase counts and runs the
-// per-string pass, then k_parse over the tiles (grid-stride, like the
-// launches).  Grid barriers separate the steps.  Same buffers and results as
-// the launches.
-template <typename T>
-__global__ void __launch_bounds__(kSmallThreads) k_parse_small(const __grid_constant__ RoundArgs a, u64 tiles, u64 nsteps,
-                                                                u64 bar_base) {
-    static_assert(kSmallThreads == kParseThreads && kSmallThreads == kBrkThreads, "one block shape");
-    const u64 g = gridDim.x;
-    body_tile_strings(a, tiles);
-    grid_barrier(a.ctr, bar_base + g, a.ds);
-    body_breaks<T>(a, nsteps);
-    grid_barrier(a.ctr, bar_base + 2 * g, a.ds);
-    if (blockIdx.x == 0) {
-        const u64 P = block_scan_small([&](u64 i) { return a.tile_cnt[i]; }, min(tiles, *a.d_tiles),
-                                       [&](u64 i, u64 e) { a.tile_pfx[i] = e; });
-        if (threadIdx.x == 0) *a.total = P;
-        body_strings(a);
+    // (the answer is the same in every block: the rounds are over, and a
+    // capacity that a block finds exceeded is exceeded for all)
+    if (s_halt) return;
+    if (threadIdx.x == 0) {
+        u32 c = 0;
+        for (u32 r = 0; r < t.rounds; r++) {
+            s_chunk0[r] = c;
+            c += (u32)((s_g[r] + kRuleChunk - 1) / kRuleChunk);
+        }
+        s_chunk0[t.rounds] = c;
     }
-    grid_barrier(a.ctr, bar_base + 3 * g, a.ds);
-    body_parse<T, kUnitMin>(a, tiles);
-}
-
-// A short round's naming in one cooperative launch instead of five: marks,
-// (block 0) the prefix of the marks' popcounts, ranks, (block 0) the rules'
-// offsets, rules.
-template <typename T>
-__global__ void __launch_bounds__(kSmallThreads) k_naming_small(const RoundArgs a, u64 bar_base) {
-    const u64 g = gridDim.x;
-    body_mark(a);
-    grid_barrier(a.ctr, bar_base + g, a.ds);
-    if (blockIdx.x == 0)
-        block_scan_small([&](u64 w) { return (u32)__popc(a.first[w].x); }, min(a.first_words, (*a.total + 31) / 32),
+    // 1. marks
+    for (u32 r = 0; r < t.rounds; r++) {
+        const RoundArgs& a = t.r[r];
+        for (u64 c = gtid; c < s_ids[r]; c += gthreads) {
+            const u64 m = a.minpos[c];
+            if (m < a.first_words * 32) atomicOr(&a.first[m >> 5].x, 1u << (m & 31));
+        }
+    }
+    DevStatus* ds = t.r[0].ds;
+    grid_barrier(t.bar + 2, 0, ds);
+    // 2. popcount prefixes
+    for (u32 r = blockIdx.x; r < t.rounds; r += gridDim.x) {
+        const RoundArgs& a = t.r[r];
+        block_scan_small([&](u64 w) { return (u32)__popc(a.first[w].x); }, s_words[r],
                          [&](u64 w, u64 e) { a.first[w].y = (u32)e; });
-    grid_barrier(a.ctr, bar_base + 2 * g, a.ds);
-    body_rank(a);
-    grid_barrier(a.ctr, bar_base + 3 * g, a.ds);
-    if (blockIdx.x == 0 && rules_fit(a)) {
-        const u64 g_new = min(*a.d_gnew, a.r_cap);
-        const ClaimRec* rec = (const ClaimRec*)a.rrec;
-        const u64 G = block_scan_small([&](u64 r) { return (u32)key_len(rec[r].key); }, g_new,
-                                       [&](u64 r, u64 e) { a.rhs_off[a.g_base + r] = a.G_base + e; });
-        if (threadIdx.x == 0) a.rhs_off[a.g_base + g_new] = a.G_base + G;
     }
-    grid_barrier(a.ctr, bar_base + 4 * g, a.ds);
-    body_rules<T>(a);
+    grid_barrier(t.bar + 2, 1, ds);
+    // 3. ranks
+    for (u32 r = 0; r < t.rounds; r++) {
+        const RoundArgs& a = t.r[r];
+        const ClaimRec* crec = (const ClaimRec*)a.crec;
+        ClaimRec* rrec = (ClaimRec*)a.rrec;
+        for (u64 c = gtid; c < s_ids[r]; c += gthreads) {
+            const u64 m = a.minpos[c];
+            const ClaimRec rec = crec[c];
+            if (m >= a.first_words * 32) continue;  // no claim
+            const uint2 f = a.first[m >> 5];
+            const u64 rank = f.y + __popc(f.x & ((1u << (m & 31)) - 1u));
+            if (rank >= s_g[r]) continue;  // not reached
+            a.rank_of[c] = (u32)(a.g_base + rank);
+            a.F[a.g_base + rank] = rec.fp;  // (read below by the level above's rules)
+            rrec[rank] = rec;
+        }
+    }
+    grid_barrier(t.bar + 2, 2, ds);
+    // 4. symbols of each chunk of rules
+    const u32 chunks = s_chunk0[t.rounds];
+    auto round_of = [&](u32 ch) {
+        u32 r = 0;
+        while (s_chunk0[r + 1] <= ch) r++;
+        return r;
+    };
+    for (u32 ch = blockIdx.x; ch < chunks; ch += gridDim.x) {
+        const u32 r = round_of(ch);
+        const ClaimRec* rec = (const ClaimRec*)t.r[r].rrec;
+        const u64 r0 = (u64)(ch - s_chunk0[r]) * kRuleChunk, r1 = min(s_g[r], r0 + kRuleChunk);
+        u64 sum = 0, tot;
+        for (u64 x = r0 + threadIdx.x; x < r1; x += blockDim.x) sum += key_len(rec[x].key);
+        block_excl_scan(sum, tot);
+        if (threadIdx.x == 0) t.chunk_len[ch] = tot;
+    }
+    // the retired strings' roots
+    for (u32 r = blockIdx.x; r < t.rounds; r += gridDim.x) {
+        const RoundArgs& a = t.r[r];
+        for (u64 x = threadIdx.x; x < s_retired[r]; x += blockDim.x) {
+            const u32 id = a.c_rank[a.R_sid[x]];
+            if (id >= a.id_base && id - a.id_base < a.id_cap) a.c_rank[a.R_sid[x]] = a.rank_of[id - a.id_base];
+        }
+    }
+    grid_barrier(t.bar + 2, 3, ds);
+    // 5. offsets and right-hand sides
+    for (u32 ch = blockIdx.x; ch < chunks; ch += gridDim.x) {
+        const u32 r = round_of(ch);
+        const RoundArgs& a = t.r[r];
+        const ClaimRec* rec = (const ClaimRec*)a.rrec;
+        const u64 r0 = (u64)(ch - s_chunk0[r]) * kRuleChunk, r1 = min(s_g[r], r0 + kRuleChunk);
+        u64 before = 0, base;
+        for (u32 x = s_chunk0[r] + threadIdx.x; x < ch; x += blockDim.x) before += t.chunk_len[x];
+        block_excl_scan(before, base);
+        u64* off = a.rhs_off + a.g_base;
+        const u64 len = block_scan_small([&](u64 x) { return (u32)key_len(rec[r0 + x].key); }, r1 - r0,
+                                         [&](u64 x, u64 e) { off[r0 + x] = a.G_base + base + e; });
+        if (r1 == s_g[r] && threadIdx.x == 0) off[r1] = a.G_base + base + len;
+        __syncthreads();
+        if (kByte && r == 0) rules_range<unsigned char>(a, r0 + threadIdx.x, blockDim.x, r1);
+        else rules_range<u32>(a, r0 + threadIdx.x, blockDim.x, r1);
+        __syncthreads();
+    }
 }
 
 static unsigned grid_for(u64 n, u64 cap = 152ull * 32) {
@@ -1578,43 +1739,43 @@ cudaError_t launch_parse(const RoundArgs& a, cudaStream_t st) {
     return launch_parse_t<u32>(a, st);
 }
 
-bool round_is_small(const RoundArgs& a) { return a.tp == (u32)kUnitMin && a.tiles_bound <= kSmallUnits; }
-
-// Blocks of a short round's cooperative launches: a warp per unit, at most one
-// block per SM (and never more than can be resident at once).
-u32 small_round_grid(const RoundArgs& a) {
+// Blocks of the short rounds' launches: a warp per unit, at most one block per
+// SM (and never more than can be resident at once).
+template <bool kByte>
+static u32 tail_grid(u64 units) {
+    using T0 = std::conditional_t<kByte, unsigned char, u32>;
+    constexpr size_t smem = std::max(sizeof(ParseSmem<T0, kUnitMin>), sizeof(ParseSmem<u32, kUnitMin>));
     static const int cap = [] {
-        int dev = 0, sms = 0, o1 = 0, o2 = 0, o3 = 0, o4 = 0;
+        int dev = 0, sms = 0, o1 = 0, o2 = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        constexpr int s1 = (int)sizeof(ParseSmem<unsigned char, kUnitMin>), s4 = (int)sizeof(ParseSmem<u32, kUnitMin>);
-        cudaFuncSetAttribute(k_parse_small<unsigned char>, cudaFuncAttributeMaxDynamicSharedMemorySize, s1);
-        cudaFuncSetAttribute(k_parse_small<u32>, cudaFuncAttributeMaxDynamicSharedMemorySize, s4);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o1, k_parse_small<unsigned char>, kSmallThreads, s1);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o2, k_parse_small<u32>, kSmallThreads, s4);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o3, k_naming_small<unsigned char>, kSmallThreads, 0);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o4, k_naming_small<u32>, kSmallThreads, 0);
-        // one block per SM (a cooperative launch checks that they fit)
-        return (std::min({o1, o2, o3, o4}) >= 1 && sms > 0) ? sms : 1;
+        cudaFuncSetAttribute(k_parse_small<kByte>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o1, k_parse_small<kByte>, kSmallThreads, smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o2, k_naming_small<kByte>, kSmallThreads, 0);
+        return (std::min(o1, o2) >= 1 && sms > 0) ? sms : 1;  // (a cooperative launch checks that they fit)
     }();
-    return (u32)std::min<u64>((u64)cap, std::max<u64>(1, (a.tiles_bound + kParseThreads / 32 - 1) / (kParseThreads / 32)));
+    return (u32)std::min<u64>((u64)cap, std::max<u64>(1, (units + kWarps - 1) / kWarps));
 }
 
-cudaError_t launch_parse_small(const RoundArgs& a, u64 bar_base, cudaStream_t st) {
-    const u64 nsteps = (a.tiles_bound * (u64)a.tp + kBrkSpan - 1) / kBrkSpan;
-    const u32 g = small_round_grid(a);
-    if (a.sym_bytes == 1)
-        return launch_coop(k_parse_small<unsigned char>, g, kSmallThreads, sizeof(ParseSmem<unsigned char, kUnitMin>),
-                           st, a, a.tiles_bound, nsteps, bar_base);
-    return launch_coop(k_parse_small<u32>, g, kSmallThreads, sizeof(ParseSmem<u32, kUnitMin>), st, a, a.tiles_bound,
-                       nsteps, bar_base);
+template <bool kByte>
+static cudaError_t launch_parse_small_t(const TailArgs& t, cudaStream_t st) {
+    using T0 = std::conditional_t<kByte, unsigned char, u32>;
+    constexpr size_t smem = std::max(sizeof(ParseSmem<T0, kUnitMin>), sizeof(ParseSmem<u32, kUnitMin>));
+    return launch_coop(k_parse_small<kByte>, tail_grid<kByte>(t.r[0].tiles_bound), kSmallThreads, smem, st, t);
 }
 
-cudaError_t launch_naming_small(const RoundArgs& a, u64 bar_base, cudaStream_t st) {
-    const u32 g = small_round_grid(a);
-    if (a.sym_bytes == 1) return launch_coop(k_naming_small<unsigned char>, g, kSmallThreads, 0, st, a, bar_base);
-    return launch_coop(k_naming_small<u32>, g, kSmallThreads, 0, st, a, bar_base);
+cudaError_t launch_parse_small(const TailArgs& t, cudaStream_t st) {
+    return t.r[0].sym_bytes == 1 ? launch_parse_small_t<true>(t, st) : launch_parse_small_t<false>(t, st);
 }
+
+cudaError_t launch_naming_small(const TailArgs& t, cudaStream_t st) {
+    const u64 units = t.r[0].tiles_bound;
+    if (t.r[0].sym_bytes == 1)
+        return launch_coop(k_naming_small<true>, tail_grid<true>(units), kSmallThreads, 0, st, t);
+    return launch_coop(k_naming_small<false>, tail_grid<false>(units), kSmallThreads, 0, st, t);
+}
+
+u64 rule_chunks(u64 g) { return (g + kRuleChunk - 1) / kRuleChunk; }
 
 cudaError_t launch_strings(const RoundArgs& a, cudaStream_t st) {
     return launch_pdl(k_strings, 1, 1024, st, a);
