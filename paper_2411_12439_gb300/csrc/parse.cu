@@ -58,9 +58,11 @@ __device__ bool round_halted(const RoundArgs& a) {
     __shared__ int s_halt;
     __syncthreads();
     if (threadIdx.x == 0) {
-        bool h = vload(&a.ds->error) != 0 || vload(&a.ds->overflow) != 0;
-        if (a.ds_prev) h = h || vload(&a.ds_prev->error) != 0 || vload(&a.ds_prev->overflow) != 0;
-        s_halt = h ? 1 : 0;
+        // (four reads in flight together)
+        const DevStatus* before = a.ds_prev ? a.ds_prev : a.ds;
+        const u32 h0 = vload(&a.ds->error), h1 = vload(&a.ds->overflow);
+        const u32 h2 = vload(&before->error), h3 = vload(&before->overflow);
+        s_halt = (h0 | h1 | h2 | h3) != 0 ? 1 : 0;
     }
     __syncthreads();
     return s_halt != 0;
@@ -225,7 +227,9 @@ __device__ __forceinline__ u32 spread_down(u32 src, u32 pass) {
 // Kernel bodies are device functions: k_X launches body_X on a grid, and the
 // short rounds' cooperative kernels (k_parse_small, k_naming_small) run several of
 // them in one launch.
-template <typename T>
+// `own_step`: block b takes step nblocks - 1 - b and no other (a launch whose
+// blocks are all resident, at least as many as steps): no counter.
+template <typename T, bool own_step = false>
 __device__ __forceinline__ void body_breaks(const RoundArgs& a, u64 nblocks) {
     pdl_wait();
     constexpr bool kByte = sizeof(T) == 1;
@@ -253,10 +257,10 @@ __device__ __forceinline__ void body_breaks(const RoundArgs& a, u64 nblocks) {
     if (blockIdx.x >= nblocks && blockIdx.x > 0) return;  // more blocks than steps: no counter traffic
     u64* heads = a.heads;
     const int warp = tid >> 5;
-    while (true) {
+    for (bool once = true; once; once = !own_step) {
         // the next block step, in decreasing order (the counter starts at 0 every round)
         if (tid == 0) {
-            const u64 t = atomicAdd(&a.ds->aux[0], 1ull);
+            const u64 t = own_step ? (u64)blockIdx.x : atomicAdd(&a.ds->aux[0], 1ull);
             s_step = t < nblocks ? nblocks - 1 - t : ~0ull;
         }
         __syncthreads();  // also: sF0 loaded
@@ -826,39 +830,6 @@ __device__ __forceinline__ void body_parse(const RoundArgs& a, u64 nunits) {
     nunits = min(nunits, (n + U - 1) / U);
     const u64 nr = a.rc->retired;
     u32 nq = 0;  // the warp's queued phrases
-    if constexpr (kByte) {
-        for (int x = threadIdx.x; x < 256; x += kParseThreads) sm.sF[x] = a.Fprev[x];
-        for (int x = threadIdx.x; x < kCacheSlots; x += kParseThreads) {
-            sm.ckey[x] = kEmpty;
-            sm.cval[x] = ~0ull;
-        }
-    }
-    if (threadIdx.x == 0) {
-        ParseArgs& pa = sm.args;
-        pa.S = a.S;
-        pa.Sf = a.Sf;
-        pa.Tnext = a.Tnext;
-        pa.Fnext = a.Fnext;
-        pa.n = n;
-        pa.T_cap = a.T_cap;
-        pa.retired = nr;
-        pa.lh = a.lh;
-        pa.table = RoundTable{(Slot*)a.tab, a.tab_cap, a.minpos, (ClaimRec*)a.crec, a.id_cap, a.id_chunk, a.ds};
-        pa.rtab_cap = a.rtab_cap;
-        pa.all = &a;
-        pa.sym_w = (u32)a.sym_w;
-        pa.inline_most = (u32)inline_max(a.sym_w);
-        pa.find_inline = a.rtab_cap ? 0u : pa.inline_most;  // phrases looked up in the table at once
-        pa.id_base = a.id_base;
-        pa.prev_base = a.prev_base;
-    }
-    if (threadIdx.x < (u32)kLongLen) sm.cpow[threadIdx.x] = powmod61(a.lh.c, threadIdx.x);
-    if (threadIdx.x == 0) sm.ids = ClaimIds{0, 0, 0};
-    if (lane == 0) {
-        w.claims = w.claim_len = 0;
-    }
-    __syncthreads();
-
     // The warps of the grid take units in turn (rank rounds in stripes when
     // asked) and wait for no other: unit lt of the logical order.
     const u32 stripes = kByte ? 1u : a.stripes;
@@ -897,7 +868,40 @@ __device__ __forceinline__ void body_parse(const RoundArgs& a, u64 nunits) {
     };
 
     u32 lt = blockIdx.x * (kParseThreads / 32) + warp;
-    fetch(lt, 0);
+    fetch(lt, 0);  // (its reads run beside the set-up)
+    if constexpr (kByte) {
+        for (int x = threadIdx.x; x < 256; x += kParseThreads) sm.sF[x] = a.Fprev[x];
+        for (int x = threadIdx.x; x < kCacheSlots; x += kParseThreads) {
+            sm.ckey[x] = kEmpty;
+            sm.cval[x] = ~0ull;
+        }
+    }
+    if (threadIdx.x == 0) {
+        ParseArgs& pa = sm.args;
+        pa.S = a.S;
+        pa.Sf = a.Sf;
+        pa.Tnext = a.Tnext;
+        pa.Fnext = a.Fnext;
+        pa.n = n;
+        pa.T_cap = a.T_cap;
+        pa.retired = nr;
+        pa.lh = a.lh;
+        pa.table = RoundTable{(Slot*)a.tab, a.tab_cap, a.minpos, (ClaimRec*)a.crec, a.id_cap, a.id_chunk, a.ds};
+        pa.rtab_cap = a.rtab_cap;
+        pa.all = &a;
+        pa.sym_w = (u32)a.sym_w;
+        pa.inline_most = (u32)inline_max(a.sym_w);
+        pa.find_inline = a.rtab_cap ? 0u : pa.inline_most;  // phrases looked up in the table at once
+        pa.id_base = a.id_base;
+        pa.prev_base = a.prev_base;
+    }
+    if (threadIdx.x < (u32)kLongLen) sm.cpow[threadIdx.x] = powmod61(a.lh.c, threadIdx.x);
+    if (threadIdx.x == 0) sm.ids = ClaimIds{0, 0, 0};
+    if (lane == 0) {
+        w.claims = w.claim_len = 0;
+    }
+    __syncthreads();
+
     for (u32 iter = 0;; lt += step, iter++) {
         const bool have = lt < nlog;  // past the last unit: the queue is emptied
         if (!have && nq == 0) break;
@@ -905,8 +909,10 @@ __device__ __forceinline__ void body_parse(const RoundArgs& a, u64 nunits) {
         if ((iter & 15) == 0) {
             u32 h = 0;
             if (lane == 0) {
-                h = vload(&a.ds->error) | vload(&a.ds->overflow);
-                if (a.ds_prev) h |= vload(&a.ds_prev->error) | vload(&a.ds_prev->overflow);
+                const DevStatus* before = a.ds_prev ? a.ds_prev : a.ds;
+                const u32 h0 = vload(&a.ds->error), h1 = vload(&a.ds->overflow);
+                const u32 h2 = vload(&before->error), h3 = vload(&before->overflow);
+                h = h0 | h1 | h2 | h3;
             }
             if (__shfl_sync(0xffffffffu, h, 0)) break;
         }
@@ -1395,7 +1401,8 @@ __global__ void k_rules(const RoundArgs a) { body_rules<T>(a); }
 // Once a round has at most kTailSymbols symbols, it and every round after it
 // run in one cooperative launch for their phrases and parses (k_parse_small)
 // and one for their naming (k_naming_small): no later round reads a round's
-// ranks (the sequences hold ids), so the naming of all of them can wait.
+// ranks (the sequences hold ids), so the naming of all of them can wait.  The
+// last rounds, of at most kSoloSymbols symbols, are one block's (solo_rounds).
 // What bounds such rounds is latency: before, each took two cooperative
 // launches of its own with 3 and 4 grid barriers (55-95 us a round; a string of
 // 20 kB has 10 rounds and nothing else); now a round has two barriers and all
@@ -1472,42 +1479,294 @@ __device__ __forceinline__ u64 block_scan_small(Get get, u64 n, Put put) {
     return carry;
 }
 
-// Rounds of at most this many symbols are left to block 0 alone, which needs no
-// grid barrier.
-constexpr u64 kSoloSymbols = 1024;
+// The rounds of at most kSoloSymbols symbols, by block 0 alone with everything
+// in its shared memory (the last 7 or 8 rounds of a build; through global
+// memory and the round's general steps each took about 25 us of round trips).
+// Phrases are compared by content in a small table, and numbered in the order
+// of their first occurrences, so a claim's number is its rank already.
+constexpr int kSoloSymbols = 1024;
+constexpr int kSoloWords = kSoloSymbols / 32;
+constexpr int kSoloStrings = kSoloSymbols / 2;                 // two symbols each, at least
+constexpr int kSoloPhrases = (kSoloSymbols + kSoloStrings) / 2;
+constexpr int kSoloSlots = 2048;
+static_assert(kSoloWords == 32, "a warp takes a word per lane");
+
+struct SoloSmem {
+    u32 T[2][kSoloSymbols], F[2][kSoloSymbols];  // the round's sequence and the next
+    u32 sid[2][kSoloStrings];
+    unsigned short soff[2][kSoloStrings + 1];
+    unsigned short sfirst[kSoloStrings + 1];     // first phrase of each string
+    unsigned short start[kSoloPhrases + 1];      // of each phrase
+    unsigned short slot_of[kSoloPhrases];
+    u32 pF[kSoloPhrases];                        // its fingerprint
+    u32 slot[kSoloSlots];                        // a phrase with the slot's content (~0: none), later its id
+    u32 first[kSoloSlots];                       // the first such phrase
+    u32 st[kSoloWords], gt[kSoloWords], lt[kSoloWords], stop[kSoloWords], bits[kSoloWords], pre[kSoloWords];
+    u32 ret[kSoloWords], rpre[kSoloWords];       // phrases that are whole strings, and how many before each word
+    u32 phrases;
+};
+
+template <bool kByte>
+__device__ __noinline__ void solo_rounds(const TailArgs& t, u32 r) {
+    extern __shared__ __align__(16) unsigned char dyn_smem[];
+    SoloSmem& sm = *reinterpret_cast<SoloSmem*>(dyn_smem);
+    const u32 tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr u32 NT = kSmallThreads, NW = NT / 32;
+    if (round_halted(t.r[r])) return;
+    u32 n, k;
+    {
+        const RoundArgs& a = t.r[r];
+        n = (u32)round_n(a);
+        k = round_k(a);
+        if (n > a.tiles_bound * a.tp || k > (u32)kSoloStrings) {  // more than the buffers were sized for
+            if (tid == 0) set_error(a.ds, kErrCapacity);
+            return;
+        }
+        for (u32 x = tid; x < n; x += NT) {
+            if (kByte && r == 0) {
+                const u32 s = ((const unsigned char*)a.S)[x];
+                sm.T[0][x] = s;
+                sm.F[0][x] = a.Fprev[s];
+            } else {
+                sm.T[0][x] = ((const u32*)a.S)[x];
+                sm.F[0][x] = a.Sf[x];
+            }
+        }
+        for (u32 j = tid; j <= k; j += NT) sm.soff[0][j] = (unsigned short)a.soff[j];
+        for (u32 j = tid; j < k; j += NT) sm.sid[0][j] = a.sid[j];
+    }
+    for (u32 cur = 0; r < t.rounds && k > 0; r++, cur ^= 1) {
+        const RoundArgs& a = t.r[r];
+        const u32* T = sm.T[cur];
+        const u32* F = sm.F[cur];
+        const unsigned short* soff = sm.soff[cur];
+        const u32 nw = (n + 31) / 32;
+        for (u32 x = tid; x < (u32)kSoloSlots; x += NT) sm.slot[x] = sm.first[x] = ~0u;
+        if (tid < (u32)kSoloWords) sm.st[tid] = sm.ret[tid] = 0;
+        __syncthreads();
+        // string starts (and the end of the sequence, when a word holds it)
+        for (u32 j = tid; j <= k; j += NT)
+            if (soff[j] < kSoloSymbols) atomicOr(&sm.st[soff[j] >> 5], 1u << (soff[j] & 31));
+        __syncthreads();
+        // right neighbour larger, smaller, or in no string (see k_breaks)
+        for (u32 w = warp; w < nw; w += NW) {
+            const u32 x = w * 32 + lane, x1 = x + 1;
+            const bool end = x1 >= n || ((sm.st[x1 >> 5] >> (x1 & 31)) & 1u);
+            const u32 f0 = x < n ? F[x] : 0u, f1 = x1 < n ? F[x1] : 0u;
+            const u32 g = __ballot_sync(0xffffffffu, !end && f1 > f0), l = __ballot_sync(0xffffffffu, !end && f1 < f0);
+            const u32 s = __ballot_sync(0xffffffffu, end);
+            if (lane == 0) sm.gt[w] = g, sm.lt[w] = l, sm.stop[w] = s;
+        }
+        __syncthreads();
+        if (warp == 0) {
+            // one word per lane: types, breaks and the phrases before the word
+            const u32 g = lane < nw ? sm.gt[lane] : 0u, l = lane < nw ? sm.lt[lane] : 0u;
+            const u32 dec = lane < nw ? g | l | sm.stop[lane] : ~0u;
+            u32 s = spread_down(g, ~dec);
+            const unsigned decided = __ballot_sync(0xffffffffu, dec != 0);
+            const u32 later = lane < 31 ? decided >> (lane + 1) : 0u;
+            // is the first position of the next decided word of type S?
+            const u32 from = later ? lane + (u32)__ffs(later) : lane;
+            const u32 next_s = __shfl_sync(0xffffffffu, s & 1u, (int)from);
+            if (!(dec >> 31) && later && next_s) {
+                const int hi = 31 - __clz(dec | 1u);
+                s |= dec == 0 ? ~0u : ~((2u << hi) - 1u);
+            }
+            const u32 lp = __shfl_up_sync(0xffffffffu, l, 1);
+            u32 b = sm.st[lane] | (((l << 1) | (lane ? lp >> 31 : 0u)) & s);
+            if (lane * 32 >= n) b = 0;
+            else if (n - lane * 32 < 32) b &= (1u << (n - lane * 32)) - 1u;
+            u32 o = (u32)__popc(b);
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const u32 y = __shfl_up_sync(0xffffffffu, o, d);
+                if (lane >= (u32)d) o += y;
+            }
+            sm.bits[lane] = b;
+            sm.pre[lane] = o - (u32)__popc(b);
+            if (lane == 31) {
+                sm.phrases = o;
+                if (o <= (u32)kSoloPhrases) sm.start[o] = (unsigned short)n;
+            }
+        }
+        __syncthreads();
+        const u32 P = sm.phrases;
+        if (P > (u32)kSoloPhrases) {  // not reached: a phrase but a string's first has two symbols
+            if (tid == 0) set_error(a.ds, kErrCapacity);
+            return;
+        }
+        for (u32 w = warp; w < nw; w += NW) {
+            const u32 b = sm.bits[w];
+            if ((b >> lane) & 1u)
+                sm.start[sm.pre[w] + __popc(b & ((1u << lane) - 1u))] = (unsigned short)(w * 32 + lane);
+        }
+        for (u32 j = tid; j < k; j += NT) {
+            const u32 x = soff[j];
+            sm.sfirst[j] = (unsigned short)(sm.pre[x >> 5] + __popc(sm.bits[x >> 5] & ((1u << (x & 31)) - 1u)));
+        }
+        if (tid == 0) sm.sfirst[k] = (unsigned short)P;
+        __syncthreads();
+        // the strings that become one phrase, and the others' places
+        constexpr u32 kPer = kSoloStrings / NT;
+        static_assert(kPer * NT == kSoloStrings, "strings per thread");
+        u32 one = 0;
+#pragma unroll
+        for (u32 i = 0; i < kPer; i++) {
+            const u32 j = tid * kPer + i;
+            if (j < k && sm.sfirst[j + 1] - sm.sfirst[j] == 1) one |= 1u << i;
+        }
+        u64 retired;
+        u32 rb = (u32)block_excl_scan((u64)__popc(one), retired);
+#pragma unroll
+        for (u32 i = 0; i < kPer; i++) {
+            const u32 j = tid * kPer + i;
+            if (j >= k) continue;
+            const u32 q = sm.sfirst[j];
+            if ((one >> i) & 1u) {
+                a.R_phr[rb] = q;
+                a.R_sid[rb] = sm.sid[cur][j];
+                atomicOr(&sm.ret[q >> 5], 1u << (q & 31));
+                rb++;
+            } else {
+                sm.soff[cur ^ 1][j - rb] = (unsigned short)(q - rb);
+                sm.sid[cur ^ 1][j - rb] = sm.sid[cur][j];
+            }
+        }
+        const u32 k1 = k - (u32)retired, n1 = P - (u32)retired;
+        if (tid == 0) sm.soff[cur ^ 1][k1] = (unsigned short)n1;
+        // fingerprints, and equal phrases to one slot
+        auto same = [&](u32 q0, u32 q1) {
+            const u32 s0 = sm.start[q0], s1 = sm.start[q1], len = sm.start[q0 + 1] - s0;
+            if (sm.start[q1 + 1] - s1 != len) return false;
+            for (u32 j = 0; j < len; j++)
+                if (T[s0 + j] != T[s1 + j]) return false;
+            return true;
+        };
+        auto poly = [&](u32 q) -> u64 {
+            u64 H = 0;
+            for (u32 x = sm.start[q + 1]; x-- > sm.start[q];) H = addmod61(mulmod61(H, a.lh.c), (u64)F[x]);
+            return H;
+        };
+        for (u32 q = tid; q < P; q += NT) {
+            const u32 f = finish_hash(a.lh, poly(q));
+            sm.pF[q] = f;
+            u32 s = (f * 0x9E3779B1u) >> 21;
+            while (true) {
+                const u32 old = atomicCAS(&sm.slot[s], ~0u, q);
+                if (old == ~0u || same(old, q)) break;
+                s = (s + 1) & (kSoloSlots - 1);
+            }
+            sm.slot_of[q] = (unsigned short)s;
+            atomicMin(&sm.first[s], q);
+        }
+        static_assert(kSoloSlots == 1 << 11 && kSoloPhrases < kSoloSlots, "a slot for every phrase");
+        __syncthreads();
+        // ids: resident rules, and the new ones in the order of their first occurrences
+        constexpr u32 kPerQ = (kSoloPhrases + NT - 1) / NT;
+        u32 fresh = 0;
+        u64 len_sum = 0;
+        for (u32 i = 0; i < kPerQ; i++) {
+            const u32 q = tid * kPerQ + i;
+            if (q >= P || sm.first[sm.slot_of[q]] != q) continue;
+            const u32 st = sm.start[q], len = sm.start[q + 1] - st;
+            u64 rank = ~0ull;
+            if (a.rtab_cap) {
+                bool res = true;
+                if (a.sym_bytes != 1)
+                    for (u32 j = 0; j < len; j++) res = res && T[st + j] < a.prev_base;
+                if (res) {
+                    const bool hashed = len > (u32)inline_max(a.sym_w);
+                    const Key128 key = hashed ? key_hashed(poly(q), len, st) : key_inline32(T + st, len, a.sym_w);
+                    rank = table_find(ContentTable{(Slot*)a.rtab, a.rtab_cap}, key, hashed, [&](u64 rk) {
+                        const u64 o = a.rrhs_off[rk];
+                        for (u32 j = 0; j < len; j++)
+                            if (T[st + j] != a.rrhs[o + j]) return false;
+                        return true;
+                    });
+                }
+            }
+            if (rank == ~0ull) {
+                fresh |= 1u << i;
+                len_sum += len;
+            } else {
+                sm.slot[sm.slot_of[q]] = (u32)rank;
+            }
+        }
+        u64 g_new, G_new;
+        u32 c = (u32)block_excl_scan((u64)__popc(fresh), g_new);
+        block_excl_scan(len_sum, G_new);
+        for (u32 i = 0; i < kPerQ; i++) {
+            if (!((fresh >> i) & 1u)) continue;
+            const u32 q = tid * kPerQ + i, st = sm.start[q], len = sm.start[q + 1] - st;
+            const Key128 key = len > (u32)inline_max(a.sym_w) ? key_hashed(poly(q), len, st)
+                                                              : key_inline32(T + st, len, a.sym_w);
+            ((ClaimRec*)a.crec)[c] = ClaimRec{key, sm.pF[q], {0u, 0u, 0u}};
+            a.minpos[c] = q;
+            sm.slot[sm.slot_of[q]] = a.id_base + c;
+            c++;
+        }
+        if (warp == 0) {
+            u32 o = (u32)__popc(sm.ret[lane]);
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const u32 y = __shfl_up_sync(0xffffffffu, o, d);
+                if (lane >= (u32)d) o += y;
+            }
+            sm.rpre[lane] = o - (u32)__popc(sm.ret[lane]);
+        }
+        __syncthreads();
+        // the next sequence (in global memory too: long rules are read there), and the roots
+        for (u32 q = tid; q < P; q += NT) {
+            const u32 id = sm.slot[sm.slot_of[q]];
+            const u32 w = q >> 5, before = sm.rpre[w] + __popc(sm.ret[w] & ((1u << (q & 31)) - 1u));
+            if ((sm.ret[w] >> (q & 31)) & 1u) {
+                const u32 j = a.R_sid[before];
+                a.c_level[j] = a.level;
+                a.c_rank[j] = id;  // k_naming_small makes it a rank
+            } else {
+                sm.T[cur ^ 1][q - before] = id;
+                sm.F[cur ^ 1][q - before] = sm.pF[q];
+                a.Tnext[q - before] = id;
+            }
+        }
+        if (tid == 0) {
+            a.rc->phrases = P;
+            a.rc->retired = retired;
+            a.rc->k_next = k1;
+            a.rc->n_next = n1;
+            *a.total = P;
+            a.ds->claims = g_new;
+            a.ds->claim_len = G_new;
+            a.ds->aux[1] = g_new;
+        }
+        n = n1;
+        k = k1;
+        __syncthreads();
+    }
+}
 
 // The phrases and the parse of the rounds t.r[0 .. t.rounds), until no string
 // is left.
 template <bool kByte>
 __global__ void __launch_bounds__(kSmallThreads) k_parse_small(const __grid_constant__ TailArgs t) {
     pdl_wait();
-    bool solo = gridDim.x == 1;
     u64 idx = 0;
     for (u32 r = 0; r < t.rounds; r++) {
         const RoundArgs& a = t.r[r];
         const u64 n = round_n(a);
         if (n == 0) break;
-        if (!solo && n <= kSoloSymbols) {
-            if (blockIdx.x != 0) return;
-            solo = true;
+        if (n <= (u64)kSoloSymbols) {
+            if (blockIdx.x == 0) solo_rounds<kByte>(t, r);
+            return;
         }
-        auto barrier = [&](auto work) {
-            if (solo) {
-                __syncthreads();
-                __threadfence();
-                work();
-                __syncthreads();
-            } else {
-                grid_barrier_work(t.bar, idx++, a.ds, work);
-            }
-        };
+        auto barrier = [&](auto work) { grid_barrier_work(t.bar, idx++, a.ds, work); };
         if (r == 0) {
             body_tile_strings(a, a.tiles_bound);
             barrier([] {});
         }
         const u64 steps = (n + kBrkSpan - 1) / kBrkSpan;
-        if (kByte && r == 0) body_breaks<unsigned char>(a, steps);
-        else body_breaks<u32>(a, steps);
+        if (kByte && r == 0) body_breaks<unsigned char, true>(a, steps);
+        else body_breaks<u32, true>(a, steps);
         // places of the units' phrases; the strings, and their starts in T^{i+1}
         barrier([&] {
             const u64 units = min((n + a.tp - 1) / a.tp, a.tiles_bound);
@@ -1744,7 +2003,7 @@ cudaError_t launch_parse(const RoundArgs& a, cudaStream_t st) {
 template <bool kByte>
 static u32 tail_grid(u64 units) {
     using T0 = std::conditional_t<kByte, unsigned char, u32>;
-    constexpr size_t smem = std::max(sizeof(ParseSmem<T0, kUnitMin>), sizeof(ParseSmem<u32, kUnitMin>));
+    constexpr size_t smem = std::max({sizeof(ParseSmem<T0, kUnitMin>), sizeof(ParseSmem<u32, kUnitMin>), sizeof(SoloSmem)});
     static const int cap = [] {
         int dev = 0, sms = 0, o1 = 0, o2 = 0;
         cudaGetDevice(&dev);
@@ -1760,7 +2019,7 @@ static u32 tail_grid(u64 units) {
 template <bool kByte>
 static cudaError_t launch_parse_small_t(const TailArgs& t, cudaStream_t st) {
     using T0 = std::conditional_t<kByte, unsigned char, u32>;
-    constexpr size_t smem = std::max(sizeof(ParseSmem<T0, kUnitMin>), sizeof(ParseSmem<u32, kUnitMin>));
+    constexpr size_t smem = std::max({sizeof(ParseSmem<T0, kUnitMin>), sizeof(ParseSmem<u32, kUnitMin>), sizeof(SoloSmem)});
     return launch_coop(k_parse_small<kByte>, tail_grid<kByte>(t.r[0].tiles_bound), kSmallThreads, smem, st, t);
 }
 
