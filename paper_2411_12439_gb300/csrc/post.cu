@@ -14,8 +14,10 @@
 // rules.  A run-length rule is stored as [base id, run length] with kind 1.
 //
 // Kernels here take one thread per rule: right-hand sides are short, and a
-// rule's runs never cross its boundaries.  The host side (abi.cu) runs them
-// level by level with the library's scans in between.
+// rule's runs never cross its boundaries.  The run-length passes take rules of
+// more than kPPLong symbols (an N-run of DNA is one rule of up to 50 k) by whole
+// warps.  The host side (abi.cu) runs them level by level with the library's
+// scans in between.
 #include "lcg_dev.cuh"
 #include "lcg_internal.h"
 
@@ -31,23 +33,67 @@ static unsigned pp_grid(u64 n) {
     return (unsigned)(b < cap ? b : cap);
 }
 
+// Rules longer than this are taken by a whole warp, after the 32 rules of its
+// threads: one thread walks such a rule one dependent read at a time (16 x
+// 2 Mbp with N-runs: k_rl_count 2.36 ms and k_rl_write 2.08 ms, most of it the
+// longest run's walk; 0.14 ms each so).
+constexpr u64 kPPLong = 64;
+
 // Runs of rule r: out_len[r] = runs, rl_len[r] = runs of length >= 2.
 __global__ void k_rl_count(const u64* __restrict__ off, const u32* __restrict__ rhs, u64 g, u32* out_len,
                            u32* rl_len) {
-    for (u64 r = blockIdx.x * (u64)blockDim.x + threadIdx.x; r < g; r += (u64)gridDim.x * blockDim.x) {
-        const u64 a = off[r], b = off[r + 1];
-        u32 runs = 0, long_runs = 0;
-        u64 p = a;
-        while (p < b) {
-            const u32 y = rhs[p];
-            u64 e = p + 1;
-            while (e < b && rhs[e] == y) e++;
-            runs++;
-            long_runs += (e - p >= 2) ? 1u : 0u;
-            p = e;
+    const u32 lane = threadIdx.x & 31;
+    for (u64 r0 = blockIdx.x * (u64)blockDim.x + (threadIdx.x & ~31u); r0 < g; r0 += (u64)gridDim.x * blockDim.x) {
+        const u64 r = r0 + lane;
+        const u64 a = r < g ? off[r] : 0, b = r < g ? off[r + 1] : 0;
+        if (r < g && b - a <= kPPLong) {
+            u32 runs = 0, long_runs = 0;
+            u64 p = a;
+            while (p < b) {
+                const u32 y = rhs[p];
+                u64 e = p + 1;
+                while (e < b && rhs[e] == y) e++;
+                runs++;
+                long_runs += (e - p >= 2) ? 1u : 0u;
+                p = e;
+            }
+            out_len[r] = runs;
+            rl_len[r] = long_runs;
         }
-        out_len[r] = runs;
-        rl_len[r] = long_runs;
+        for (unsigned m = __ballot_sync(0xffffffffu, b - a > kPPLong); m; m &= m - 1) {
+            // a run starts where the symbol differs from the one before, and is
+            // long when the next symbol starts none
+            const int l = __ffs(m) - 1;
+            const u64 wa = __shfl_sync(0xffffffffu, a, l), wb = __shfl_sync(0xffffffffu, b, l);
+            u32 runs = 0, long_runs = 0;
+            constexpr int kPer = 16;  // words of 32 symbols whose reads are in flight together
+            u32 last = 0;             // the symbol before the word
+            unsigned before = 0;      // and whether a run starts there
+            for (u64 p0 = wa; p0 < wb; p0 += 32 * kPer) {
+                u32 v[kPer];
+#pragma unroll
+                for (int i = 0; i < kPer; i++) {
+                    const u64 p = p0 + 32 * i + lane;
+                    v[i] = p < wb ? rhs[p] : 0u;
+                }
+#pragma unroll
+                for (int i = 0; i < kPer; i++) {
+                    const u64 p = p0 + 32 * i + lane;
+                    u32 prev = __shfl_up_sync(0xffffffffu, v[i], 1);
+                    if (lane == 0) prev = last;
+                    last = __shfl_sync(0xffffffffu, v[i], 31);
+                    const unsigned in = __ballot_sync(0xffffffffu, p < wb);
+                    const unsigned st = __ballot_sync(0xffffffffu, p < wb && (p == wa || v[i] != prev));
+                    runs += (u32)__popc(st);
+                    long_runs += (u32)__popc(in & ~st & ((st << 1) | before));
+                    before = st >> 31;
+                }
+            }
+            if (lane == 0) {
+                out_len[r0 + l] = runs;
+                rl_len[r0 + l] = long_runs;
+            }
+        }
     }
 }
 
@@ -74,28 +120,80 @@ __device__ u64 pp_claim(u64* keys, u64 mask, u64 key) {
 __global__ void k_rl_write(const u64* __restrict__ off, const u32* __restrict__ rhs, u64 g,
                            const u64* __restrict__ new_off, const u64* __restrict__ rl_off, u32* new_rhs,
                            u32* run_y, u32* run_len, u64* run_pos, u64* keys, u64* vals, u64 mask, DevStatus* ds) {
-    for (u64 r = blockIdx.x * (u64)blockDim.x + threadIdx.x; r < g; r += (u64)gridDim.x * blockDim.x) {
-        const u64 a = off[r], b = off[r + 1];
-        u64 w = new_off[r], m = rl_off[r];
-        u64 p = a;
-        while (p < b) {
-            const u32 y = rhs[p];
-            u64 e = p + 1;
-            while (e < b && rhs[e] == y) e++;
-            if (e - p >= 2) {
-                run_y[m] = y;
-                run_len[m] = (u32)(e - p);
-                run_pos[m] = w;
-                const u64 s = pp_claim(keys, mask, pp_key(y, e - p));
-                if (s == ~0ull) set_error(ds, kErrTableFull);
-                else atomicMin((unsigned long long*)&vals[s], (unsigned long long)m);
-                new_rhs[w] = kRLFlag;  // named by k_rl_fix
-                m++;
-            } else {
-                new_rhs[w] = y;
+    const u32 lane = threadIdx.x & 31;
+    // the run of `len` symbols y: output entry w, and entry m of the list when len >= 2
+    auto run = [&](u32 y, u64 len, u64 w, u64 m) {
+        if (len < 2) {
+            new_rhs[w] = y;
+            return;
+        }
+        run_y[m] = y;
+        run_len[m] = (u32)len;
+        run_pos[m] = w;
+        const u64 s = pp_claim(keys, mask, pp_key(y, len));
+        if (s == ~0ull) set_error(ds, kErrTableFull);
+        else atomicMin((unsigned long long*)&vals[s], (unsigned long long)m);
+        new_rhs[w] = kRLFlag;  // named by k_rl_fix
+    };
+    for (u64 r0 = blockIdx.x * (u64)blockDim.x + (threadIdx.x & ~31u); r0 < g; r0 += (u64)gridDim.x * blockDim.x) {
+        const u64 r = r0 + lane;
+        const u64 a = r < g ? off[r] : 0, b = r < g ? off[r + 1] : 0;
+        if (r < g && b - a <= kPPLong) {
+            u64 w = new_off[r], m = rl_off[r];
+            u64 p = a;
+            while (p < b) {
+                const u32 y = rhs[p];
+                u64 e = p + 1;
+                while (e < b && rhs[e] == y) e++;
+                run(y, e - p, w, m);
+                m += e - p >= 2 ? 1 : 0;
+                w++;
+                p = e;
             }
-            w++;
-            p = e;
+        }
+        for (unsigned lm = __ballot_sync(0xffffffffu, b - a > kPPLong); lm; lm &= lm - 1) {
+            const int l = __ffs(lm) - 1;
+            const u64 wa = __shfl_sync(0xffffffffu, a, l), wb = __shfl_sync(0xffffffffu, b, l);
+            u64 w = new_off[r0 + l], m = rl_off[r0 + l];  // of the open run
+            u64 open = wa;                                // where it starts
+            u32 open_y = rhs[wa];
+            // kPer words of 32 symbols at a time: their reads are in flight together
+            constexpr int kPer = 8;
+            u32 last = open_y;  // the symbol before the word
+            for (u64 p0 = wa; p0 < wb; p0 += 32 * kPer) {
+                u32 v[kPer];
+#pragma unroll
+                for (int i = 0; i < kPer; i++) {
+                    const u64 p = p0 + 32 * i + lane;
+                    v[i] = p < wb ? rhs[p] : 0u;
+                }
+#pragma unroll
+                for (int i = 0; i < kPer; i++) {
+                    const u64 q0 = p0 + 32 * i, p = q0 + lane;
+                    u32 prev = __shfl_up_sync(0xffffffffu, v[i], 1);
+                    if (lane == 0) prev = last;
+                    last = __shfl_sync(0xffffffffu, v[i], 31);
+                    const unsigned st = __ballot_sync(0xffffffffu, p < wb && p != wa && v[i] != prev);
+                    if (st == 0) continue;
+                    // the first start closes the open run; the others close the ones
+                    // that start in this word
+                    const u64 first = q0 + (u32)__ffs(st) - 1;
+                    if (lane == 0) run(open_y, first - open, w, m);
+                    m += first - open >= 2 ? 1 : 0;
+                    w++;
+                    const unsigned above = lane < 31 ? st >> (lane + 1) : 0u;
+                    const bool mine = ((st >> lane) & 1u) && above;  // starts and ends here
+                    const u64 len = mine ? (u64)__ffs(above) : 0;
+                    const unsigned longs = __ballot_sync(0xffffffffu, len >= 2), below = (1u << lane) - 1u;
+                    if (mine) run(v[i], len, w + __popc(st & below), m + __popc(longs & below));
+                    m += __popc(longs);
+                    w += __popc(st) - 1;
+                    const int top = 31 - __clz(st);
+                    open = q0 + (u64)top;
+                    open_y = __shfl_sync(0xffffffffu, v[i], top);
+                }
+            }
+            if (lane == 0) run(open_y, wb - open, w, m);
         }
     }
 }
@@ -149,7 +247,9 @@ __global__ void k_pp_uses(const u64* __restrict__ off, const u32* __restrict__ r
     for (u64 r = blockIdx.x * (u64)blockDim.x + threadIdx.x; r < g; r += (u64)gridDim.x * blockDim.x) {
         for (u64 p = off[r]; p < off[r + 1]; p++) {
             const u32 v = rhs[p];
-            if (!(v & kRLFlag)) atomicAdd(&uses_below[v], 1u);
+            // (only 0, 1 and more are told apart, so a symbol used all over is
+            // not counted on)
+            if (!(v & kRLFlag) && vload(&uses_below[v]) < 2) atomicAdd(&uses_below[v], 1u);
         }
     }
 }
