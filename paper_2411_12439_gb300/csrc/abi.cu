@@ -1802,54 +1802,101 @@ void merge(lcg_ctx* ctx, lcg_grammar* A, const lcg_grammar* B) {
 
 void decompress(lcg_ctx* ctx, const lcg_grammar* G, u32 j, uint8_t* out, u64 cap, uint64_t* out_len, int on_dev) {
     fail_if(ctx, j >= G->k, LCG_EINVAL, "string index out of range");
-    u32 lev = 0, r = 0;
-    ck(ctx, cudaMemcpyAsync(&lev, G->c_level + j, 4, cudaMemcpyDeviceToHost, ctx->st), "read C");
-    ck(ctx, cudaMemcpyAsync(&r, G->c_rank + j, 4, cudaMemcpyDeviceToHost, ctx->st), "read C");
-    sync(ctx);
-    u32* cur = dalloc<u32>(ctx, 1);
-    ck(ctx, cudaMemcpyAsync(cur, &r, 4, cudaMemcpyHostToDevice, ctx->st), "copy");
-    u64 cnt = 1;
-    for (u32 l = lev; l >= 1; l--) {
+    // the upper levels, and the whole of a short string, in one launch
+    ExpandState st{1, 0, 0};
+    u32* cur = nullptr;
+    u8* tmp = nullptr;  // bytes for a host buffer
+    if (G->lv.size() <= 64) {
+        ExpandLevels lv{};
+        for (size_t l = 0; l < G->lv.size(); l++) {
+            lv.off[l] = G->lv[l].rhs_off;
+            lv.rhs[l] = G->lv[l].rhs;
+        }
+        cur = dalloc<u32>(ctx, kExpandSmall);
+        if (!on_dev) tmp = dalloc<u8>(ctx, kExpandSmallBytes);
+        ExpandState* d = (ExpandState*)(ctx->scratch + 4);
+        ck(ctx, launch_expand_small(lv, G->c_level, G->c_rank, j, on_dev ? out : tmp,
+                                    on_dev ? cap : std::min<u64>(cap, kExpandSmallBytes), cur, d, ctx->st),
+           "k_expand_small");
+        ctx->launches++;
+        ck(ctx, cudaMemcpyAsync(&st, d, sizeof(st), cudaMemcpyDeviceToHost, ctx->st), "read state");
+        sync(ctx);
+    } else {
+        u32 r = 0;
+        ck(ctx, cudaMemcpyAsync(&st.level, G->c_level + j, 4, cudaMemcpyDeviceToHost, ctx->st), "read C");
+        ck(ctx, cudaMemcpyAsync(&r, G->c_rank + j, 4, cudaMemcpyDeviceToHost, ctx->st), "read C");
+        cur = dalloc<u32>(ctx, 1);
+        ck(ctx, cudaMemcpyAsync(cur, G->c_rank + j, 4, cudaMemcpyDeviceToDevice, ctx->st), "copy");
+        sync(ctx);
+        if (st.level == 0 && cap >= 1) {
+            const u8 b = (u8)r;
+            if (!on_dev) tmp = dalloc<u8>(ctx, 1);
+            ck(ctx, cudaMemcpyAsync(on_dev ? out : tmp, &b, 1, cudaMemcpyHostToDevice, ctx->st), "copy");
+        }
+    }
+    u64 cnt = st.count;
+    auto too_small = [&] {
+        *out_len = cnt;
+        dfree(ctx, cur);
+        dfree(ctx, tmp);
+        sync(ctx);
+        fail_if(ctx, true, LCG_EINVAL, "output buffer too small");
+    };
+    if (st.level == 0 && cap < cnt) too_small();
+    for (u32 l = st.level; l >= 1; l--) {
         const Level& L = G->lv[l - 1];
-        u32* lens = dalloc<u32>(ctx, cnt);
-        u64* offs = dalloc<u64>(ctx, cnt);
-        ck(ctx, launch_rule_lens(cur, cnt, L.rhs_off, lens, ctx->st), "rule lens");
-        u64 grid = 0;
-        const u64 stiles = std::max<u64>(1, scan2_tiles_for(cnt));
+        const u64 tiles = expand_tiles_for(cnt);
+        u32* sums = dalloc<u32>(ctx, 2 * tiles);
+        u64* places = dalloc<u64>(ctx, 2 * tiles);
+        ck(ctx, launch_expand_count(cur, cnt, L.rhs_off, sums, sums + tiles, ctx->st), "k_expand_count");
+        const u64 stiles = std::max<u64>(1, scan2_tiles_for(tiles));
         ensure_lb(ctx, &ctx->lb2, &ctx->lb2_tiles, stiles, scan2_lb_bytes(stiles));
-        ck(ctx, launch_scan2(lens, nullptr, cnt, offs, nullptr, ctx->scratch + 1, ctx->lb2, ++ctx->epoch, ctx->ctr,
-                             ctx->ctr_val, ctx->ds, ctx->st, &grid),
+        u64 grid = 0, tot[2] = {0, 0};
+        ck(ctx, launch_scan2(sums, sums + tiles, tiles, places, places + tiles, ctx->scratch + 1, ctx->lb2,
+                             ++ctx->epoch, ctx->ctr, ctx->ctr_val, ctx->ds, ctx->st, &grid),
            "scan");
         ctx->ctr_val += grid;
-        u64 total = 0;
-        ck(ctx, cudaMemcpyAsync(&total, ctx->scratch + 1, 8, cudaMemcpyDeviceToHost, ctx->st), "read total");
+        ck(ctx, cudaMemcpyAsync(tot, ctx->scratch + 1, 16, cudaMemcpyDeviceToHost, ctx->st), "read total");
         check_device_status(ctx, read_status(ctx));
-        u32* next = dalloc<u32>(ctx, total);
-        ck(ctx, launch_expand(cur, cnt, offs, L.rhs_off, L.rhs, next, ctx->st), "expand");
+        const u64 total = tot[0] + (tot[1] << 32);
+        u32* next = nullptr;
+        u8 *bytes = nullptr, *packed = nullptr;
+        if (l == 1) {
+            if (cap < total) {
+                cnt = total;
+                dfree(ctx, sums);
+                dfree(ctx, places);
+                too_small();
+            }
+            if (!on_dev) {
+                dfree(ctx, tmp);
+                tmp = dalloc<u8>(ctx, total);
+            }
+            bytes = on_dev ? out : tmp;
+            // the level's right-hand sides as bytes, when they are read several times
+            if (total >= 4 * L.G) {
+                packed = dalloc<u8>(ctx, L.G + 16);
+                ck(ctx, launch_expand_pack(L.rhs, L.G, packed, ctx->st), "k_expand_pack");
+                ctx->launches++;
+            }
+        } else {
+            next = dalloc<u32>(ctx, total);
+        }
+        ck(ctx, launch_expand_tiles(cur, cnt, L.rhs_off, L.rhs, packed, places, places + tiles, next, bytes, ctx->st),
+           "k_expand_tiles");
+        dfree(ctx, packed);
         ctx->launches += 3;
-        dfree(ctx, lens);
-        dfree(ctx, offs);
+        dfree(ctx, sums);
+        dfree(ctx, places);
         dfree(ctx, cur);
         cur = next;
         cnt = total;
     }
     *out_len = cnt;
-    if (cap < cnt) {
-        dfree(ctx, cur);
-        sync(ctx);
-        fail_if(ctx, true, LCG_EINVAL, "output buffer too small");
-    }
-    if (on_dev) {
-        ck(ctx, launch_to_bytes(cur, cnt, out, ctx->st), "to bytes");
-    } else {
-        unsigned char* tmp = dalloc<unsigned char>(ctx, cnt);
-        ck(ctx, launch_to_bytes(cur, cnt, tmp, ctx->st), "to bytes");
-        ck(ctx, cudaMemcpyAsync(out, tmp, cnt, cudaMemcpyDeviceToHost, ctx->st), "copy out");
-        dfree(ctx, tmp);
-    }
-    ctx->launches++;
+    if (!on_dev) ck(ctx, cudaMemcpyAsync(out, tmp, cnt, cudaMemcpyDeviceToHost, ctx->st), "copy out");
+    dfree(ctx, tmp);
     dfree(ctx, cur);
-    sync(ctx);
+    if (st.level != 0 || !on_dev) sync(ctx);
 }
 
 // --------------------------------------------------------------------------

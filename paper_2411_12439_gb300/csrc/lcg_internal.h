@@ -219,6 +219,25 @@ struct FTable {
 cudaError_t launch_roots(const u32* c_level, const u32* c_rank, u32 j0, u32 cnt, const FTable& ft, u32* out,
                          cudaStream_t st);
 cudaError_t launch_remap_c(const u32* c_level, u32* c_rank, u32 k, u32 level, const u32* M, cudaStream_t st);
+// Expansion of one string.
+constexpr u32 kExpandSmall = 8192;         // symbols of a level, at most, while one block expands
+constexpr u64 kExpandSmallBytes = 65536;   // and bytes
+struct ExpandLevels {
+    const u64* off[64];  // right-hand-side offsets of level i + 1
+    const u32* rhs[64];
+};
+struct ExpandState {
+    u64 count;  // symbols of level `level` (the string's bytes when it is 0)
+    u32 level;
+    u32 pad;
+};
+cudaError_t launch_expand_small(const ExpandLevels& lv, const u32* c_level, const u32* c_rank, u32 j,
+                                unsigned char* out, u64 cap, u32* rest, ExpandState* state, cudaStream_t st);
+u64 expand_tiles_for(u64 cnt);
+cudaError_t launch_expand_count(const u32* cur, u64 cnt, const u64* off, u32* lo, u32* hi, cudaStream_t st);
+cudaError_t launch_expand_tiles(const u32* cur, u64 cnt, const u64* off, const u32* rhs, const u8* packed,
+                                const u64* lo, const u64* hi, u32* next, u8* bytes, cudaStream_t st);
+cudaError_t launch_expand_pack(const u32* rhs, u64 n, u8* out, cudaStream_t st);  // out: n bytes and 3 more
 cudaError_t launch_rule_lens(const u32* cur, u64 cnt, const u64* rhs_off, u32* lens, cudaStream_t st);
 cudaError_t launch_expand(const u32* cur, u64 cnt, const u64* offs, const u64* rhs_off, const u32* rhs, u32* next,
                           cudaStream_t st);
