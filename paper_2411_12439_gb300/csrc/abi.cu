@@ -355,6 +355,8 @@ void ensure_resident(lcg_ctx* ctx, lcg_grammar* G, u32 i, u64 need_g) {
     if (L.rvalid && L.rcap >= 2 * need_g) return;
     const u64 cap = std::max<u64>(1024, 3 * need_g);
     dfree(ctx, L.rtab);
+    L.rtab = nullptr;
+    L.rvalid = false;
     L.rtab = dalloc<unsigned char>(ctx, cap * slot_bytes());
     L.rcap = cap;
     ck(ctx, cudaMemsetAsync(L.rtab, 0xFF, cap * slot_bytes(), ctx->st), "memset table");
@@ -363,6 +365,25 @@ void ensure_resident(lcg_ctx* ctx, lcg_grammar* G, u32 i, u64 need_g) {
        "resident build");
     ctx->launches++;
     L.rvalid = true;
+}
+
+// The rules of an imported grammar against their fingerprints (the host reads the
+// status afterwards); `temps` gets what is to be freed then.
+void check_fingerprints(lcg_ctx* ctx, const lcg_grammar* G, std::vector<void*>& temps) {
+    std::vector<FpLevel> lv;
+    u64 blocks = 0;
+    for (u32 i = 1; i <= G->lv.size(); i++) {
+        const Level& L = G->lv[i - 1];
+        if (L.g == 0) continue;
+        lv.push_back(FpLevel{L.rhs, L.rhs_off, fprev_of(G, i), L.F, L.g, blocks, level_hash(ctx, i)});
+        blocks += (L.g + 255) / 256;
+    }
+    if (lv.empty()) return;
+    FpLevel* d = dalloc<FpLevel>(ctx, lv.size());
+    temps.push_back(d);
+    ck(ctx, cudaMemcpyAsync(d, lv.data(), lv.size() * sizeof(FpLevel), cudaMemcpyHostToDevice, ctx->st), "levels");
+    ck(ctx, launch_check_fp(d, (u32)lv.size(), blocks, ctx->ds, ctx->st), "k_check_fp");
+    ctx->launches++;
 }
 
 void grow_c(lcg_ctx* ctx, lcg_grammar* G, u32 need) {
@@ -1719,81 +1740,123 @@ void build_into(lcg_ctx* ctx, lcg_grammar* R, const uint8_t* data, const uint64_
 // MergeGrams
 // --------------------------------------------------------------------------
 
+// A level grows to what it may need at most, without waiting for what it does
+// need, up to this many rules and symbols (16 + 8 MB; a doubling of the arrays adds
+// as much).
+constexpr u64 kMergeAheadRules = 1ull << 20, kMergeAheadSymbols = 1ull << 21;
+
+// All levels are enqueued before the host waits once, but for a level that is large
+// and does not fit its arrays whatever G_b adds: there the host reads what it adds.
+// G_a's sizes are set at the end, so that a failure leaves G_a as it was.
 void merge(lcg_ctx* ctx, lcg_grammar* A, const lcg_grammar* B) {
     fail_if(ctx, A == B, LCG_EINVAL, "cannot merge a grammar into itself");
     fail_if(ctx, A->tag != B->tag || A->tag != ctx->tag, LCG_EMISMATCH, "grammars of different hash families");
     fail_if(ctx, (u64)A->k + B->k > 0xffffffffull, LCG_EOVERFLOW, "too many strings");
     const u32 kb = B->k;
-    u32* cb_rank = dalloc<u32>(ctx, kb);
-    if (kb)
-        ck(ctx, cudaMemcpyAsync(cb_rank, B->c_rank, kb * 4, cudaMemcpyDeviceToDevice, ctx->st), "copy");
-    u32* Mprev = nullptr;
-    for (u32 i = 1; i <= B->lv.size(); i++) {
-        if (A->lv.size() < i) A->lv.emplace_back();
-        Level& LA = A->lv[i - 1];
-        const Level& LB = B->lv[i - 1];
-        const u64 gb = LB.g;
-        const u32* brhs = LB.rhs;
-        u32* brhs_tmp = nullptr;
-        if (i > 1 && LB.G > 0) {
-            brhs_tmp = dalloc<u32>(ctx, LB.G);
-            ck(ctx, launch_remap(LB.rhs, LB.G, Mprev, brhs_tmp, ctx->st), "remap");
+    const u32 nb = (u32)B->lv.size();
+    std::vector<u64> tot(2 * (size_t)nb, 0);
+    std::vector<void*> temps;
+    auto temp = [&](auto* p) {
+        temps.push_back(p);
+        return p;
+    };
+    try {
+        u32* cb_rank = temp(dalloc<u32>(ctx, kb));
+        u64* d_tot = temp(dalloc<u64>(ctx, 2 * (size_t)nb));
+        if (nb) ck(ctx, cudaMemsetAsync(d_tot, 0, tot.size() * 8, ctx->st), "memset totals");
+        if (kb) ck(ctx, cudaMemcpyAsync(cb_rank, B->c_rank, kb * 4, cudaMemcpyDeviceToDevice, ctx->st), "copy");
+        const u32* Mprev = nullptr;
+        for (u32 i = 1; i <= nb; i++) {
+            if (A->lv.size() < i) A->lv.emplace_back();
+            Level& LA = A->lv[i - 1];
+            const Level& LB = B->lv[i - 1];
+            const u64 gb = LB.g;
+            if (LA.rhs_off == nullptr) grow_level(ctx, LA, 0, 0);
+            if (gb == 0) {
+                Mprev = nullptr;
+                continue;
+            }
+            ensure_resident(ctx, A, i, LA.g + gb);
+            LA.rvalid = false;  // until the rules it will hold are the level's
+            MergeLevel m{};
+            m.brhs = LB.rhs;
+            m.boff = LB.rhs_off;
+            m.bF = LB.F;
+            m.gb = gb;
+            m.Mprev = Mprev;
+            m.aFprev = fprev_of(A, i);
+            m.lh = level_hash(ctx, i);
+            m.slots = LA.rtab;
+            m.cap = LA.rcap;
+            m.ga = LA.g;
+            m.Ga = LA.G;
+            // one allocation per level for the ranks (kept for the next level) and one
+            // for what this level alone needs
+            m.M = temp(dalloc<u32>(ctx, gb));
+            u64* x = dalloc<u64>(ctx, 3 * gb);
+            temps.push_back(x);
+            m.xrank = x;
+            m.xlen = x + gb;
+            m.miss = (u32*)(x + 2 * gb);
+            m.mlen = m.miss + gb;
+            m.totals = d_tot + 2 * (size_t)(i - 1);
+            m.c_level = B->c_level;
+            m.c_rank = B->c_rank;
+            m.c_out = cb_rank;
+            m.kb = kb;
+            m.level = i;
+            m.ds = ctx->ds;
+            const u64 stiles = std::max<u64>(1, scan2_tiles_for(gb));
+            ensure_lb(ctx, &ctx->lb2, &ctx->lb2_tiles, stiles, scan2_lb_bytes(stiles));
+            // (the lookup reads G_a's arrays as they are before they grow)
+            m.arhs = LA.rhs;
+            m.aoff = LA.rhs_off;
+            m.aF = LA.F;
+            ck(ctx, launch_merge_lookup(m, i == 1, ctx->st), "merge lookup");
+            u64 grid = 0;
+            ck(ctx, launch_scan2(m.miss, m.mlen, gb, x, x + gb, d_tot + 2 * (size_t)(i - 1), ctx->lb2, ++ctx->epoch,
+                                 ctx->ctr, ctx->ctr_val, ctx->ds, ctx->st, &grid),
+               "scan");
+            ctx->ctr_val += grid;
+            ctx->launches += 2;
+            u64 more[2] = {gb, LB.G};
+            const bool fits = m.ga + gb <= LA.cap_g && m.Ga + LB.G <= LA.cap_G;
+            if (m.ga + gb > kMaxRank || (!fits && (m.ga + gb > kMergeAheadRules || m.Ga + LB.G > kMergeAheadSymbols))) {
+                ck(ctx, cudaMemcpyAsync(more, m.totals, 16, cudaMemcpyDeviceToHost, ctx->st), "read totals");
+                check_device_status(ctx, read_status(ctx));
+                fail_if(ctx, m.ga + more[0] > kMaxRank, LCG_EOVERFLOW, "level with 2^31 rules or more");
+            }
+            grow_level(ctx, LA, m.ga + more[0], m.Ga + more[1]);
+            m.arhs = LA.rhs;
+            m.aoff = LA.rhs_off;
+            m.aF = LA.F;
+            ck(ctx, launch_merge_append(m, i == 1, ctx->st), "merge append");
             ctx->launches++;
-            brhs = brhs_tmp;
+            dfree(ctx, temps.back());
+            temps.pop_back();
+            Mprev = m.M;
         }
-        if (LA.rhs_off == nullptr) grow_level(ctx, LA, 0, 0);
-        ensure_resident(ctx, A, i, LA.g + gb);
-        u32* M = dalloc<u32>(ctx, gb);
-        u32* miss = dalloc<u32>(ctx, gb);
-        u32* mlen = dalloc<u32>(ctx, gb);
-        u64* xrank = dalloc<u64>(ctx, gb);
-        u64* xlen = dalloc<u64>(ctx, gb);
-        ck(ctx, launch_merge_lookup(brhs, LB.rhs_off, LB.F, gb, i == 1, fprev_of(A, i), level_hash(ctx, i), LA.rtab,
-                                    LA.rcap, LA.rhs, LA.rhs_off, LA.F, M, miss, mlen, ctx->ds, ctx->st),
-           "merge lookup");
-        u64 grid = 0;
-        const u64 stiles = std::max<u64>(1, scan2_tiles_for(gb));
-        ensure_lb(ctx, &ctx->lb2, &ctx->lb2_tiles, stiles, scan2_lb_bytes(stiles));
-        ck(ctx, launch_scan2(miss, mlen, gb, xrank, xlen, ctx->scratch + 1, ctx->lb2, ++ctx->epoch, ctx->ctr,
-                             ctx->ctr_val, ctx->ds, ctx->st, &grid),
-           "scan");
-        ctx->ctr_val += grid;
-        ctx->launches += 2;
-        u64 tot[2] = {0, 0};
-        if (gb) ck(ctx, cudaMemcpyAsync(tot, ctx->scratch + 1, 16, cudaMemcpyDeviceToHost, ctx->st), "read totals");
+        grow_c(ctx, A, A->k + kb);
+        if (kb) {
+            ck(ctx, cudaMemcpyAsync(A->c_level + A->k, B->c_level, kb * 4, cudaMemcpyDeviceToDevice, ctx->st), "copy");
+            ck(ctx, cudaMemcpyAsync(A->c_rank + A->k, cb_rank, kb * 4, cudaMemcpyDeviceToDevice, ctx->st), "copy");
+        }
+        if (nb)
+            ck(ctx, cudaMemcpyAsync(tot.data(), d_tot, tot.size() * 8, cudaMemcpyDeviceToHost, ctx->st), "read totals");
         check_device_status(ctx, read_status(ctx));
-        const u64 ga = LA.g, Ga = LA.G;
-        fail_if(ctx, ga + tot[0] > kMaxRank, LCG_EOVERFLOW, "level with 2^31 rules or more");
-        grow_level(ctx, LA, ga + tot[0], Ga + tot[1]);
-        ck(ctx, launch_merge_append(brhs, LB.rhs_off, LB.F, gb, miss, xrank, xlen, ga, Ga, LA.rhs, LA.rhs_off, LA.F,
-                                    M, ga + tot[0], Ga + tot[1], ctx->st),
-           "merge append");
-        ctx->launches += 2;
-        LA.g = ga + tot[0];
-        LA.G = Ga + tot[1];
-        // the appended rules join the table of the level
-        ck(ctx, launch_resident_build(LA.rhs, LA.rhs_off, ga, tot[0], i == 1, fprev_of(A, i), level_hash(ctx, i),
-                                      LA.rtab, LA.rcap, ctx->ds, ctx->st),
-           "table insert");
-        ck(ctx, launch_remap_c(B->c_level, cb_rank, kb, i, M, ctx->st), "remap C");
-        ctx->launches += 2;
-        dfree(ctx, brhs_tmp);
-        dfree(ctx, miss);
-        dfree(ctx, mlen);
-        dfree(ctx, xrank);
-        dfree(ctx, xlen);
-        dfree(ctx, Mprev);
-        Mprev = M;
+    } catch (...) {
+        for (void* p : temps) dfree(ctx, p);
+        throw;
     }
-    dfree(ctx, Mprev);
-    grow_c(ctx, A, A->k + kb);
-    if (kb) {
-        ck(ctx, cudaMemcpyAsync(A->c_level + A->k, B->c_level, kb * 4, cudaMemcpyDeviceToDevice, ctx->st), "copy");
-        ck(ctx, cudaMemcpyAsync(A->c_rank + A->k, cb_rank, kb * 4, cudaMemcpyDeviceToDevice, ctx->st), "copy");
+    for (void* p : temps) dfree(ctx, p);
+    for (u32 i = 0; i < nb; i++) {
+        Level& L = A->lv[i];
+        if (B->lv[i].g == 0) continue;
+        L.g += tot[2 * (size_t)i];
+        L.G += tot[2 * (size_t)i + 1];
+        L.rvalid = true;
     }
     A->k += kb;
-    dfree(ctx, cb_rank);
-    check_device_status(ctx, read_status(ctx));
 }
 
 // --------------------------------------------------------------------------
@@ -2624,10 +2687,10 @@ int lcg_import(lcg_ctx* ctx, uint32_t k, uint32_t nlevels, const uint64_t* g, co
             L.g = gi;
             L.G = Gi;
             L.rvalid = false;
-            ck(ctx, launch_check_fp(L.rhs, L.rhs_off, gi, fprev_of(G, i), level_hash(ctx, i), L.F, ctx->ds, ctx->st),
-               "k_check_fp");
-            ctx->launches++;
         }
+        std::vector<void*> temps;
+        check_fingerprints(ctx, G, temps);
+        for (void* p : temps) dfree(ctx, p);
         const DevStatus st = read_status(ctx);
         fail_if(ctx, st.error == kErrMismatch, LCG_EMISMATCH,
                 "imported fingerprints differ from those of this context's hash family");
@@ -3216,13 +3279,7 @@ int lcg_import_vbyte(lcg_ctx* ctx, const void* buf, uint64_t size, int buf_on_de
         DevStatus st = read_status(ctx);
         fail_if(ctx, st.error == kErrFormat, LCG_EINVAL, "malformed VByte form");
         check_device_status(ctx, st);
-        for (u64 i = 0; i < nl; i++) {
-            const Level& L = G->lv[i];
-            ck(ctx, launch_check_fp(L.rhs, L.rhs_off, L.g, fprev_of(G, (u32)i + 1), level_hash(ctx, (u32)i + 1), L.F,
-                                    ctx->ds, ctx->st),
-               "k_check_fp");
-            ctx->launches++;
-        }
+        check_fingerprints(ctx, G, temps);
         uint32_t mine[256], theirs[256];
         ck(ctx, cudaMemcpyAsync(mine, G->F0, sizeof(mine), cudaMemcpyDeviceToHost, ctx->st), "read F0");
         ck(ctx, cudaMemcpyAsync(theirs, src + off_F0, sizeof(theirs), cudaMemcpyDeviceToHost, ctx->st), "read F0");

@@ -87,68 +87,175 @@ cudaError_t launch_scan2(const u32* in0, const u32* in1, u64 n, u64* out0, u64* 
 // MergeGrams
 // --------------------------------------------------------------------------
 
-// out[x] = M[in[x]]: rewrite right-hand sides of G_b into G_a's ranks.
-__global__ void k_remap(const u32* __restrict__ in, u64 n, const u32* __restrict__ M, u32* __restrict__ out) {
-    for (u64 x = blockIdx.x * (u64)blockDim.x + threadIdx.x; x < n; x += (u64)gridDim.x * blockDim.x)
-        out[x] = M[in[x]];
+// Three launches per level and no wait of the host between levels: the lookup reads
+// G_b's symbols through Mprev (no rewritten copy of G_b), the append takes the
+// totals of the scan from device memory, enters the new rules in G_a's table and
+// renames G_b's roots.  Two grammars of 3.5 M rules in 15 levels: 2.0 ms with
+// eight launches and two waits per level, 1.5 ms with these.
+//
+// A rule of more than kRuleLong symbols (an N-run of DNA) is read, hashed and
+// compared by a whole warp, after the 32 rules of its threads: a thread alone
+// takes a round trip per symbol.
+constexpr u64 kRuleLong = 32;
+
+// Calls `one(r, s, len)` for the rules r of [r_first, r_end) that are this thread's
+// (s: where their symbols start; block `block` of `blocks` takes 256 at a time) and
+// `whole(r, s, len)` with the whole warp for the long ones.
+template <typename One, typename Whole>
+__device__ __forceinline__ void for_rules(const u64* off, u64 r_first, u64 r_end, u64 block, u64 blocks, One one,
+                                          Whole whole) {
+    const u32 lane = threadIdx.x & 31;
+    for (u64 r0 = r_first + block * blockDim.x + (threadIdx.x & ~31u); r0 < r_end; r0 += blocks * blockDim.x) {
+        const u64 r = r0 + lane;
+        const u64 s = r < r_end ? off[r] : 0, e = r < r_end ? off[r + 1] : 0;
+        if (r < r_end && e - s <= kRuleLong) one(r, s, e - s);
+        __syncwarp();
+        for (unsigned m = __ballot_sync(0xffffffffu, e - s > kRuleLong); m; m &= m - 1) {
+            const int l = __ffs(m) - 1;
+            const u64 ws = __shfl_sync(0xffffffffu, s, l), we = __shfl_sync(0xffffffffu, e, l);
+            whole(r0 + l, ws, we - ws);
+            __syncwarp();
+        }
+    }
 }
 
-// For every rule of G_b (right-hand side already over G_a's ranks): its rank
-// in G_a when G_a has the same right-hand side (looked up in G_a's table of
-// the level, hashed keys confirmed by comparing contents), else a miss.
+// H of a rule whose symbol j is get(j), by one thread, four fingerprints in
+// flight at a time.
+template <typename Get>
+__device__ __forceinline__ u64 rule_poly(Get get, u64 len, const u32* __restrict__ F, u64 c) {
+    u64 H = 0;
+    for (u64 j = len; j > 0;) {
+        u32 f[4];
+        const u64 m = j < 4 ? j : 4;
+#pragma unroll
+        for (int u = 0; u < 4; u++) f[u] = (u64)u < m ? __ldg(F + get(j - 1 - u)) : 0u;
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+            if ((u64)u < m) H = addmod61(mulmod61(H, c), (u64)f[u]);
+        j -= m;
+    }
+    return H;
+}
+
+// Key of a rule of at most kRuleLong symbols for a table whose values are ranks
+// (see rule_key); H is only computed when the key needs it.
+template <bool kByte, typename Get>
+__device__ __forceinline__ Key128 rank_key(Get get, u64 len, const u32* __restrict__ Fprev, u64 c, u64 rank) {
+    constexpr int w = kByte ? 8 : kRankBits;
+    if (len <= inline_max(w)) return key_inline(get, len, w);
+    return key_hashed(rule_poly(get, len, Fprev, c), len, rank);
+}
+
+// Rules r0 .. r0+cnt-1 of a level enter its table (values: ranks).
 template <bool kByte>
-__global__ void k_merge_lookup(const u32* __restrict__ brhs, const u64* __restrict__ brhs_off,
-                               const u32* __restrict__ bF, u64 gb, const u32* __restrict__ aFprev, LevelHash lh,
-                               ContentTable at, const u32* __restrict__ arhs, const u64* __restrict__ arhs_off,
-                               const u32* __restrict__ aF, u32* __restrict__ M, u32* __restrict__ miss,
-                               u32* __restrict__ mlen, DevStatus* ds) {
-    for (u64 r = blockIdx.x * (u64)blockDim.x + threadIdx.x; r < gb; r += (u64)gridDim.x * blockDim.x) {
-        const u64 s = brhs_off[r], e = brhs_off[r + 1], len = e - s;
-        u64 H = 0;
-        for (u64 x = e; x-- > s;) H = addmod61(mulmod61(H, lh.c), (u64)__ldg(aFprev + brhs[x]));
-        const int w = kByte ? 8 : kRankBits;
-        const bool hashed = len > inline_max(w);
-        const Key128 key = hashed ? key_hashed(H, len, 0) : key_inline([&](u64 j) { return brhs[s + j]; }, len, w);
-        u64 found = ~0ull;
-        if (at.cap) {
-            found = table_find(at, key, hashed, [&](u64 ra) {
-                const u64 o = arhs_off[ra];
-                if (arhs_off[ra + 1] - o != len) return false;
-                for (u64 x = 0; x < len; x++)
-                    if (arhs[o + x] != brhs[s + x]) return false;
-                return true;
-            });
-        }
+__global__ void __launch_bounds__(256) k_resident_build(const u32* __restrict__ rhs, const u64* __restrict__ rhs_off,
+                                                        u64 r0, u64 cnt, const u32* __restrict__ Fprev, LevelHash lh,
+                                                        ContentTable t, DevStatus* ds) {
+    pdl_wait();
+    for_rules(rhs_off, r0, r0 + cnt, blockIdx.x, gridDim.x,
+              [&](u64 r, u64 s, u64 len) {
+                  table_put(t, rank_key<kByte>([&](u64 j) { return __ldg(rhs + s + j); }, len, Fprev, lh.c, r), r, ds);
+              },
+              [&](u64 r, u64 s, u64 len) {
+                  const u64 H = warp_poly61([&](u64 j) -> u64 { return __ldg(Fprev + __ldg(rhs + s + j)); }, len, lh.c);
+                  if ((threadIdx.x & 31) == 0) table_put(t, key_hashed(H, len, r), r, ds);
+              });
+}
+
+// Symbol x of G_b's right-hand sides in G_a's ranks.
+template <bool kByte>
+__device__ __forceinline__ u32 merge_sym(const MergeLevel& m, u64 x) {
+    const u32 v = __ldg(m.brhs + x);
+    if constexpr (kByte) return v;
+    else return __ldg(m.Mprev + v);
+}
+
+// An earlier level's failure: what this one would read may not have been written.
+__device__ __forceinline__ bool merge_failed(const MergeLevel& m) {
+    return vload(&m.ds->error) != 0 || vload(&m.ds->overflow) != 0;
+}
+
+// For every rule of G_b: its rank in G_a when G_a has the same right-hand side
+// (G_b's symbols through Mprev are G_a's ranks; looked up in G_a's table of the
+// level, hashed keys confirmed by comparing contents), else a miss.  Bound by the
+// round trips of a thread's rule: its bounds, its symbols, their ranks, the slot.
+template <bool kByte>
+__global__ void __launch_bounds__(256) k_merge_lookup(const __grid_constant__ MergeLevel m) {
+    pdl_wait();
+    if (merge_failed(m)) return;
+    const ContentTable at{(Slot*)m.slots, m.cap};
+    auto put = [&](u64 r, u64 len, u64 found) {
         if (found != ~0ull) {
-            if (aF[found] != bF[r]) set_error(ds, kErrMismatch);
-            M[r] = (u32)found;
-            miss[r] = 0;
-            mlen[r] = 0;
-        } else {
-            miss[r] = 1;
-            mlen[r] = (u32)len;
+            if (m.aF[found] != m.bF[r]) set_error(m.ds, kErrMismatch);
+            m.M[r] = (u32)found;
         }
-    }
+        m.miss[r] = found == ~0ull ? 1u : 0u;
+        m.mlen[r] = found == ~0ull ? (u32)len : 0u;
+    };
+    for_rules(m.boff, 0, m.gb, blockIdx.x, gridDim.x,
+              [&](u64 r, u64 s, u64 len) {
+                  const Key128 key = rank_key<kByte>([&](u64 j) { return merge_sym<kByte>(m, s + j); }, len, m.aFprev,
+                                                     m.lh.c, 0);
+                  put(r, len, table_find(at, key, key_is_hashed(key), [&](u64 ra) {
+                          const u64 o = m.aoff[ra];
+                          for (u64 x = 0; x < len; x++)
+                              if (m.arhs[o + x] != merge_sym<kByte>(m, s + x)) return false;
+                          return true;
+                      }));
+              },
+              [&](u64 r, u64 s, u64 len) {
+                  const u64 H = warp_poly61([&](u64 j) -> u64 { return __ldg(m.aFprev + merge_sym<kByte>(m, s + j)); },
+                                            len, m.lh.c);
+                  const u64 found = table_find_warp(at, key_hashed(H, len, 0), [&](u64 ra) {
+                      const u64 o = m.aoff[ra];
+                      return warp_equal([&](u64 x) { return m.arhs[o + x]; },
+                                        [&](u64 x) { return merge_sym<kByte>(m, s + x); }, len);
+                  });
+                  if ((threadIdx.x & 31) == 0) put(r, len, found);
+              });
 }
 
-// Append the missed rules of G_b to G_a in G_b's rank order.
-__global__ void k_merge_append(const u32* __restrict__ brhs, const u64* __restrict__ brhs_off,
-                               const u32* __restrict__ bF, u64 gb, const u32* __restrict__ miss,
-                               const u64* __restrict__ xrank, const u64* __restrict__ xlen, u64 ga, u64 Ga,
-                               u32* __restrict__ arhs, u64* __restrict__ arhs_off, u32* __restrict__ aF,
-                               u32* __restrict__ M) {
-    for (u64 r = blockIdx.x * (u64)blockDim.x + threadIdx.x; r < gb; r += (u64)gridDim.x * blockDim.x) {
-        if (!miss[r]) continue;
-        const u64 nr = ga + xrank[r], o = Ga + xlen[r];
-        const u64 s = brhs_off[r], e = brhs_off[r + 1];
-        arhs_off[nr] = o;
-        for (u64 x = s; x < e; x++) arhs[o + (x - s)] = brhs[x];
-        aF[nr] = bF[r];
-        M[r] = (u32)nr;
-    }
+// Append the missed rules of G_b to G_a in G_b's rank order (totals: their number
+// and symbols, read here so that the host need not wait for them) and to G_a's
+// table, and give G_b's roots of this level their ranks in G_a.
+template <bool kByte>
+__global__ void __launch_bounds__(256) k_merge_append(const __grid_constant__ MergeLevel m) {
+    pdl_wait();
+    if (merge_failed(m)) return;
+    const ContentTable at{(Slot*)m.slots, m.cap};
+    if (blockIdx.x == 0 && threadIdx.x == 0) m.aoff[m.ga + m.totals[0]] = m.Ga + m.totals[1];
+    for (u32 j = blockIdx.x * blockDim.x + threadIdx.x; j < m.kb; j += gridDim.x * blockDim.x)
+        if (m.c_level[j] == m.level) {
+            const u32 r = m.c_rank[j];
+            m.c_out[j] = m.miss[r] ? (u32)(m.ga + m.xrank[r]) : m.M[r];
+        }
+    for_rules(m.boff, 0, m.gb, blockIdx.x, gridDim.x,
+              [&](u64 r, u64 s, u64 len) {
+                  if (!m.miss[r]) return;
+                  const u64 nr = m.ga + m.xrank[r], o = m.Ga + m.xlen[r];
+                  m.aoff[nr] = o;
+                  m.aF[nr] = m.bF[r];
+                  m.M[r] = (u32)nr;
+                  for (u64 x = 0; x < len; x++) m.arhs[o + x] = merge_sym<kByte>(m, s + x);
+                  table_put(at, rank_key<kByte>([&](u64 j) { return merge_sym<kByte>(m, s + j); }, len, m.aFprev,
+                                                m.lh.c, nr),
+                            nr, m.ds);
+              },
+              [&](u64 r, u64 s, u64 len) {
+                  if (!m.miss[r]) return;  // (the same for the whole warp)
+                  const u32 lane = threadIdx.x & 31;
+                  const u64 nr = m.ga + m.xrank[r], o = m.Ga + m.xlen[r];
+                  for (u64 x = lane; x < len; x += 32) m.arhs[o + x] = merge_sym<kByte>(m, s + x);
+                  const u64 H = warp_poly61([&](u64 j) -> u64 { return __ldg(m.aFprev + merge_sym<kByte>(m, s + j)); },
+                                            len, m.lh.c);
+                  if (lane == 0) {
+                      m.aoff[nr] = o;
+                      m.aF[nr] = m.bF[r];
+                      m.M[r] = (u32)nr;
+                      table_put(at, key_hashed(H, len, nr), nr, m.ds);
+                  }
+              });
 }
-
-__global__ void k_set_u64(u64* p, u64 v) { *p = v; }
 
 // F^0[s] = h^0(s) = ((a_0 s + b_0) mod p) mod m for every byte s (Sec. 3.2).
 __global__ void k_h0(LevelHash h0, u32* __restrict__ F0) {
@@ -161,26 +268,34 @@ cudaError_t launch_h0(LevelHash h0, u32* F0, cudaStream_t st) {
     return launch_pdl(k_h0, 1, 256, st, h0, F0);
 }
 
-// C_b entries of level `level` move to G_a's ranks.
 // Imported rules: F^i[r] must be h^i of the rule's right-hand side
 // (Eq. fast_hash over F^{i-1}); a difference means the grammar was built with
-// another hash family (or was altered).
-__global__ void k_check_fp(const u32* __restrict__ rhs, const u64* __restrict__ rhs_off, u64 g,
-                           const u32* __restrict__ Fprev, LevelHash lh, const u32* __restrict__ F, DevStatus* ds) {
-    for (u64 r = blockIdx.x * (u64)blockDim.x + threadIdx.x; r < g; r += (u64)gridDim.x * blockDim.x) {
-        const u64 s = rhs_off[r], e = rhs_off[r + 1];
-        u64 H = 0;
-        for (u64 y = e; y-- > s;) H = addmod61(mulmod61(H, lh.c), (u64)__ldg(Fprev + rhs[y]));
-        if (finish_hash(lh, H) != F[r]) set_error(ds, kErrMismatch);
+// another hash family (or was altered).  All levels in one launch: block b has
+// 256 rules of the level whose blocks start at blk0 <= b.
+__global__ void __launch_bounds__(256) k_check_fp(const FpLevel* __restrict__ lv, u32 nl, DevStatus* ds) {
+    pdl_wait();
+    u32 lo = 0, hi = nl - 1;
+    while (lo < hi) {
+        const u32 mid = (lo + hi + 1) / 2;
+        if (lv[mid].blk0 <= blockIdx.x) lo = mid;
+        else hi = mid - 1;
     }
+    const FpLevel L = lv[lo];
+    for_rules(L.off, 0, L.g, blockIdx.x - L.blk0, 1ull << 32,
+              [&](u64 r, u64 s, u64 len) {
+                  const u64 H = rule_poly([&](u64 j) { return __ldg(L.rhs + s + j); }, len, L.Fprev, L.lh.c);
+                  if (finish_hash(L.lh, H) != L.F[r]) set_error(ds, kErrMismatch);
+              },
+              [&](u64 r, u64 s, u64 len) {
+                  const u64 H =
+                      warp_poly61([&](u64 j) -> u64 { return __ldg(L.Fprev + __ldg(L.rhs + s + j)); }, len, L.lh.c);
+                  if ((threadIdx.x & 31) == 0 && finish_hash(L.lh, H) != L.F[r]) set_error(ds, kErrMismatch);
+              });
 }
 
-cudaError_t launch_check_fp(const u32* rhs, const u64* rhs_off, u64 g, const u32* Fprev, LevelHash lh, const u32* F,
-                            DevStatus* ds, cudaStream_t st) {
-    if (g == 0) return cudaSuccess;
-    const u64 b = (g + 255) / 256;
-    k_check_fp<<<(unsigned)(b < 152 * 16 ? b : 152 * 16), 256, 0, st>>>(rhs, rhs_off, g, Fprev, lh, F, ds);
-    return cudaGetLastError();
+cudaError_t launch_check_fp(const FpLevel* lv, u32 nl, u64 blocks, DevStatus* ds, cudaStream_t st) {
+    if (blocks == 0) return cudaSuccess;
+    return launch_pdl(k_check_fp, (unsigned)blocks, 256, st, lv, nl, ds);
 }
 
 // Root of strings j0 .. j0+cnt-1: C[j] = (level, rank) and the fingerprint
@@ -202,53 +317,28 @@ cudaError_t launch_roots(const u32* c_level, const u32* c_rank, u32 j0, u32 cnt,
     return cudaGetLastError();
 }
 
-__global__ void k_remap_c(const u32* __restrict__ c_level, u32* __restrict__ c_rank, u32 k, u32 level,
-                          const u32* __restrict__ M) {
-    for (u32 j = blockIdx.x * blockDim.x + threadIdx.x; j < k; j += gridDim.x * blockDim.x)
-        if (c_level[j] == level) c_rank[j] = M[c_rank[j]];
-}
-
 static unsigned grid_for(u64 n, unsigned cap = 152 * 32) {
     u64 b = (n + 255) / 256;
     if (b == 0) b = 1;
     return (unsigned)(b < cap ? b : cap);
 }
 
-cudaError_t launch_remap(const u32* in, u64 n, const u32* M, u32* out, cudaStream_t st) {
-    if (n == 0) return cudaSuccess;
-    k_remap<<<grid_for(n), 256, 0, st>>>(in, n, M, out);
-    return cudaGetLastError();
+cudaError_t launch_resident_build(const u32* rhs, const u64* rhs_off, u64 r0, u64 cnt, bool bytes, const u32* Fprev,
+                                  LevelHash lh, void* slots, u64 cap, DevStatus* ds, cudaStream_t st) {
+    if (cnt == 0) return cudaSuccess;
+    const ContentTable t{(Slot*)slots, cap};
+    return launch_pdl(bytes ? k_resident_build<true> : k_resident_build<false>, grid_for(cnt), 256, st, rhs, rhs_off,
+                      r0, cnt, Fprev, lh, t, ds);
 }
 
-cudaError_t launch_merge_lookup(const u32* brhs, const u64* brhs_off, const u32* bF, u64 gb, bool bytes,
-                                const u32* aFprev, LevelHash lh, void* aslots, u64 acap, const u32* arhs,
-                                const u64* arhs_off, const u32* aF, u32* M, u32* miss, u32* mlen, DevStatus* ds,
-                                cudaStream_t st) {
-    if (gb == 0) return cudaSuccess;
-    const ContentTable at{(Slot*)aslots, acap};
-    if (bytes)
-        k_merge_lookup<true><<<grid_for(gb), 256, 0, st>>>(brhs, brhs_off, bF, gb, aFprev, lh, at, arhs, arhs_off, aF,
-                                                           M, miss, mlen, ds);
-    else
-        k_merge_lookup<false><<<grid_for(gb), 256, 0, st>>>(brhs, brhs_off, bF, gb, aFprev, lh, at, arhs, arhs_off,
-                                                            aF, M, miss, mlen, ds);
-    return cudaGetLastError();
+cudaError_t launch_merge_lookup(const MergeLevel& m, bool bytes, cudaStream_t st) {
+    if (m.gb == 0) return cudaSuccess;
+    return launch_pdl(bytes ? k_merge_lookup<true> : k_merge_lookup<false>, grid_for(m.gb), 256, st, m);
 }
 
-cudaError_t launch_merge_append(const u32* brhs, const u64* brhs_off, const u32* bF, u64 gb, const u32* miss,
-                                const u64* xrank, const u64* xlen, u64 ga, u64 Ga, u32* arhs, u64* arhs_off,
-                                u32* aF, u32* M, u64 ga_new, u64 Ga_new, cudaStream_t st) {
-    if (gb > 0)
-        k_merge_append<<<grid_for(gb), 256, 0, st>>>(brhs, brhs_off, bF, gb, miss, xrank, xlen, ga, Ga, arhs,
-                                                     arhs_off, aF, M);
-    k_set_u64<<<1, 1, 0, st>>>(arhs_off + ga_new, Ga_new);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_remap_c(const u32* c_level, u32* c_rank, u32 k, u32 level, const u32* M, cudaStream_t st) {
-    if (k == 0) return cudaSuccess;
-    k_remap_c<<<grid_for(k, 152), 256, 0, st>>>(c_level, c_rank, k, level, M);
-    return cudaGetLastError();
+cudaError_t launch_merge_append(const MergeLevel& m, bool bytes, cudaStream_t st) {
+    if (m.gb == 0) return cudaSuccess;
+    return launch_pdl(bytes ? k_merge_append<true> : k_merge_append<false>, grid_for(m.gb), 256, st, m);
 }
 
 // --------------------------------------------------------------------------

@@ -194,23 +194,47 @@ u64 rule_offs_tiles(u64 g);
 cudaError_t launch_rules(const RoundArgs& a, u64 g_grid, cudaStream_t st);
 cudaError_t launch_level0(const unsigned char* data, const u64* pos, const u32* ids, u32 cnt, u32* c_level,
                           u32* c_rank, cudaStream_t st);
-cudaError_t launch_resident_build(const u32* rhs, const u64* rhs_off, u64 r0, u64 cnt, bool bytes, const u32* Fprev,
-                                  LevelHash lh, void* slots, u64 cap, DevStatus* ds, cudaStream_t st);
 cudaError_t launch_h0(LevelHash h0, u32* F0, cudaStream_t st);
 cudaError_t launch_gather_strings(const unsigned char* data, const u64* src_off, const u64* dst_off, u32 k,
                                   unsigned char* out, cudaStream_t st);
 
 // grammar.cu
-cudaError_t launch_remap(const u32* in, u64 n, const u32* M, u32* out, cudaStream_t st);
-cudaError_t launch_merge_lookup(const u32* brhs, const u64* brhs_off, const u32* bF, u64 gb, bool bytes,
-                                const u32* aFprev, LevelHash lh, void* aslots, u64 acap, const u32* arhs,
-                                const u64* arhs_off, const u32* aF, u32* M, u32* miss, u32* mlen, DevStatus* ds,
-                                cudaStream_t st);
-cudaError_t launch_merge_append(const u32* brhs, const u64* brhs_off, const u32* bF, u64 gb, const u32* miss,
-                                const u64* xrank, const u64* xlen, u64 ga, u64 Ga, u32* arhs, u64* arhs_off,
-                                u32* aF, u32* M, u64 ga_new, u64 Ga_new, cudaStream_t st);
-cudaError_t launch_check_fp(const u32* rhs, const u64* rhs_off, u64 g, const u32* Fprev, LevelHash lh, const u32* F,
-                            DevStatus* ds, cudaStream_t st);
+cudaError_t launch_resident_build(const u32* rhs, const u64* rhs_off, u64 r0, u64 cnt, bool bytes, const u32* Fprev,
+                                  LevelHash lh, void* slots, u64 cap, DevStatus* ds, cudaStream_t st);
+// One level of a merge of G_b into G_a.
+struct MergeLevel {
+    const u32* brhs;  // G_b's rules: right-hand sides (over G_b's ranks), offsets, fingerprints
+    const u64* boff;
+    const u32* bF;
+    u64 gb;
+    const u32* Mprev;   // G_a's ranks of G_b's rules of the level below
+    const u32* aFprev;  // G_a's fingerprints of the level below, the appended ones included
+    LevelHash lh;
+    void* slots;  // G_a's table of the level
+    u64 cap;
+    u32* arhs;  // G_a's rules, with room for the appended ones
+    u64* aoff;
+    u32* aF;
+    u64 ga, Ga;            // G_a's rules and symbols before the merge
+    u32 *M, *miss, *mlen;  // gb each: rank in G_a; 1 for a rule G_a does not have; its length then
+    const u64 *xrank, *xlen, *totals;  // scans of miss and mlen, and their sums
+    const u32 *c_level, *c_rank;       // G_b's roots
+    u32* c_out;                        // their ranks in G_a
+    u32 kb, level;
+    DevStatus* ds;
+};
+cudaError_t launch_merge_lookup(const MergeLevel& m, bool bytes, cudaStream_t st);
+cudaError_t launch_merge_append(const MergeLevel& m, bool bytes, cudaStream_t st);
+// A level of an imported grammar, blocks of 256 rules from block blk0 on.
+struct FpLevel {
+    const u32* rhs;
+    const u64* off;
+    const u32* Fprev;
+    const u32* F;
+    u64 g, blk0;
+    LevelHash lh;
+};
+cudaError_t launch_check_fp(const FpLevel* lv, u32 nl, u64 blocks, DevStatus* ds, cudaStream_t st);
 // F arrays of a grammar by level (F[0] = F^0).
 struct FTable {
     const u32* F[65];
@@ -218,7 +242,6 @@ struct FTable {
 };
 cudaError_t launch_roots(const u32* c_level, const u32* c_rank, u32 j0, u32 cnt, const FTable& ft, u32* out,
                          cudaStream_t st);
-cudaError_t launch_remap_c(const u32* c_level, u32* c_rank, u32 k, u32 level, const u32* M, cudaStream_t st);
 // Expansion of one string.
 constexpr u32 kExpandSmall = 8192;         // symbols of a level, at most, while one block expands
 constexpr u64 kExpandSmallBytes = 65536;   // and bytes

@@ -1332,25 +1332,6 @@ __device__ __forceinline__ void body_rules(const RoundArgs& a) {
 }
 
 // --------------------------------------------------------------------------
-// k_resident_build: table over existing rules of a level
-// --------------------------------------------------------------------------
-
-// Rules r0 .. r0+cnt-1 of a level enter its table (values: ranks).
-template <bool kByte>
-__global__ void k_resident_build(const u32* __restrict__ rhs, const u64* __restrict__ rhs_off, u64 r0, u64 cnt,
-                                 const u32* __restrict__ Fprev, LevelHash lh, ContentTable t, DevStatus* ds) {
-    pdl_wait();
-    for (u64 x = blockIdx.x * (u64)blockDim.x + threadIdx.x; x < cnt; x += (u64)gridDim.x * blockDim.x) {
-        const u64 r = r0 + x;
-        const u64 s = rhs_off[r], e = rhs_off[r + 1];
-        u64 H = 0;
-        for (u64 y = e; y-- > s;) H = addmod61(mulmod61(H, lh.c), (u64)__ldg(Fprev + rhs[y]));
-        const Key128 k = rule_key([&](u64 j) { return rhs[s + j]; }, e - s, kByte ? 8 : kRankBits, H, r);
-        table_put(t, k, r, ds);
-    }
-}
-
-// --------------------------------------------------------------------------
 // round 0 helpers: strings of length one, and gathering the active strings
 // --------------------------------------------------------------------------
 
@@ -2077,15 +2058,6 @@ cudaError_t launch_gather_strings(const unsigned char* data, const u64* src_off,
     if (k == 0) return cudaSuccess;
     const unsigned blocks = k < 152 * 8 ? k : 152 * 8;
     k_gather_strings<<<blocks, 256, 0, st>>>(data, src_off, dst_off, k, out);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_resident_build(const u32* rhs, const u64* rhs_off, u64 r0, u64 cnt, bool bytes, const u32* Fprev,
-                                  LevelHash lh, void* slots, u64 cap, DevStatus* ds, cudaStream_t st) {
-    if (cnt == 0) return cudaSuccess;
-    const ContentTable t{(Slot*)slots, cap};
-    if (bytes) k_resident_build<true><<<grid_for(cnt), 256, 0, st>>>(rhs, rhs_off, r0, cnt, Fprev, lh, t, ds);
-    else k_resident_build<false><<<grid_for(cnt), 256, 0, st>>>(rhs, rhs_off, r0, cnt, Fprev, lh, t, ds);
     return cudaGetLastError();
 }
 
