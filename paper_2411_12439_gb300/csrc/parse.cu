@@ -1389,6 +1389,10 @@ __global__ void k_rules(const RoundArgs a) { body_rules<T>(a); }
 // 20 kB has 10 rounds and nothing else); now a round has two barriers and all
 // namings share four.  The sizes need no plan and cannot be outgrown: a round
 // of n symbols in k strings has at most (n + k) / 2 phrases.
+// Why 524288: six builds of 12 MB into a growing grammar take 8.66 ms when the
+// short rounds begin at 131072 symbols, 8.27 at 262144, 7.94 at 524288 and 7.82 at
+// 1048576; a build of 8 x 1 MB 947, 948, 917 and 916 us; the larger builds do not
+// tell them apart.  The buffers, some 200 bytes a symbol, grow with it.
 
 // Barrier over the grid of a cooperative launch, the idx-th of the launch
 // (idx = 0, 1, ...); bar: two zeroed counters (arrivals, releases).  The last
