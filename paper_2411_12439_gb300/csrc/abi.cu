@@ -1745,6 +1745,120 @@ void build_into(lcg_ctx* ctx, lcg_grammar* R, const uint8_t* data, const uint64_
 // as much).
 constexpr u64 kMergeAheadRules = 1ull << 20, kMergeAheadSymbols = 1ull << 21;
 
+// The levels i0 + 1 .. of G_b, all of them small, in one launch.  `temps` gets what is
+// to be freed afterwards.
+void merge_small(lcg_ctx* ctx, lcg_grammar* A, const lcg_grammar* B, u32 i0, const u32* Mprev, u64* bar, u64* d_tot,
+                 u32* cb_rank, std::vector<void*>& temps) {
+    const u32 nb = (u32)B->lv.size();
+    const u32 blocks = merge_small_blocks();
+    MergeSmall a{};
+    a.bar = bar;
+    Parts tmp, grown;
+    struct At {
+        u64 M, off, F, rhs, cap_g, cap_G;
+        bool rules, syms, table;
+    };
+    std::vector<At> at;
+    const u64 counts = tmp.take(2 * (u64)blocks * sizeof(u64));
+    while (A->lv.size() < nb) A->lv.emplace_back();
+    for (u32 i = i0 + 1; i <= nb; i++) {
+        const Level &LA = A->lv[i - 1], &LB = B->lv[i - 1];
+        At x{};
+        x.M = tmp.take(LB.g * sizeof(u32));
+        x.rules = LA.rhs_off == nullptr || LA.g + LB.g > LA.cap_g;
+        x.syms = LA.rhs == nullptr || LA.G + LB.G > LA.cap_G;
+        x.table = !(LA.rvalid && LA.rcap >= 2 * (LA.g + LB.g));
+        if (x.rules) {
+            x.cap_g = std::max<u64>({LA.g + LB.g, 2 * LA.cap_g, 256});
+            x.off = grown.take((x.cap_g + 1) * sizeof(u64));
+            x.F = grown.take(x.cap_g * sizeof(u32));
+        }
+        if (x.syms) {
+            x.cap_G = std::max<u64>({LA.G + LB.G, 2 * LA.cap_G, 1024});
+            x.rhs = grown.take(x.cap_G * sizeof(u32));
+        }
+        at.push_back(x);
+    }
+    unsigned char* t = dalloc<unsigned char>(ctx, tmp.size);
+    temps.push_back(t);
+    a.counts = (u64*)(t + counts);
+    unsigned char* g = nullptr;
+    if (grown.size) {
+        g = dalloc<unsigned char>(ctx, grown.size);
+        A->slabs.push_back(g);
+    }
+    std::vector<void*> tables;
+    try {
+        for (u32 i = i0 + 1; i <= nb; i++)
+            tables.push_back(at[i - i0 - 1].table ? dalloc<unsigned char>(ctx, std::max<u64>(1024, 3 * (A->lv[i - 1].g + B->lv[i - 1].g)) * slot_bytes()) : nullptr);
+    } catch (...) {
+        for (void* p : tables) dfree(ctx, p);
+        throw;
+    }
+    // nothing below fails but the launch itself
+    const u32* F_below = i0 == 0 ? A->F0 : A->lv[i0 - 1].F;
+    for (u32 i = i0 + 1; i <= nb; i++) {
+        Level& LA = A->lv[i - 1];
+        const Level& LB = B->lv[i - 1];
+        const At& x = at[i - i0 - 1];
+        MergeLevel& m = a.lv[a.levels];
+        MergeOld& o = a.old[a.levels];
+        if (x.rules) {
+            o.off = LA.rhs_off;
+            o.F = LA.F;
+            o.first = LA.rhs_off == nullptr;
+            if (LA.rhs_off && !LA.shared_rules) {
+                temps.push_back(LA.rhs_off);
+                temps.push_back(LA.F);
+            }
+            LA.rhs_off = (u64*)(g + x.off);
+            LA.F = (u32*)(g + x.F);
+            LA.cap_g = x.cap_g;
+            LA.shared_rules = true;
+        }
+        if (x.syms) {
+            o.rhs = LA.rhs;
+            if (LA.rhs && !LA.shared_rhs) temps.push_back(LA.rhs);
+            LA.rhs = (u32*)(g + x.rhs);
+            LA.cap_G = x.cap_G;
+            LA.shared_rhs = true;
+        }
+        if (x.table) {
+            dfree(ctx, LA.rtab);
+            LA.rtab = tables[i - i0 - 1];
+            LA.rcap = std::max<u64>(1024, 3 * (LA.g + LB.g));
+            o.fresh = true;
+        }
+        LA.rvalid = false;
+        m.brhs = LB.rhs;
+        m.boff = LB.rhs_off;
+        m.bF = LB.F;
+        m.gb = LB.g;
+        m.M = (u32*)(t + x.M);
+        m.Mprev = Mprev;
+        m.aFprev = F_below;
+        m.lh = level_hash(ctx, i);
+        m.slots = LA.rtab;
+        m.cap = LA.rcap;
+        m.arhs = LA.rhs;
+        m.aoff = LA.rhs_off;
+        m.aF = LA.F;
+        m.ga = LA.g;
+        m.Ga = LA.G;
+        m.c_level = B->c_level;
+        m.c_rank = B->c_rank;
+        m.c_out = cb_rank;
+        m.kb = B->k;
+        m.level = i;
+        m.ds = ctx->ds;
+        a.totals[a.levels++] = d_tot + 2 * (size_t)(i - 1);
+        Mprev = m.M;
+        F_below = LA.F;
+    }
+    ck(ctx, launch_merge_small(a, blocks, ctx->st), "merge levels");
+    ctx->launches++;
+}
+
 // All levels are enqueued before the host waits once, but for a level that is large
 // and does not fit its arrays whatever G_b adds: there the host reads what it adds.
 // G_a's sizes are set at the end, so that a failure leaves G_a as it was.
@@ -1762,11 +1876,19 @@ void merge(lcg_ctx* ctx, lcg_grammar* A, const lcg_grammar* B) {
     };
     try {
         u32* cb_rank = temp(dalloc<u32>(ctx, kb));
-        u64* d_tot = temp(dalloc<u64>(ctx, 2 * (size_t)nb));
-        if (nb) ck(ctx, cudaMemsetAsync(d_tot, 0, tot.size() * 8, ctx->st), "memset totals");
+        u64* d_tot = temp(dalloc<u64>(ctx, 2 * (size_t)nb + 2));  // and the small levels' barrier
+        ck(ctx, cudaMemsetAsync(d_tot, 0, (tot.size() + 2) * 8, ctx->st), "memset totals");
         if (kb) ck(ctx, cudaMemcpyAsync(cb_rank, B->c_rank, kb * 4, cudaMemcpyDeviceToDevice, ctx->st), "copy");
         const u32* Mprev = nullptr;
-        for (u32 i = 1; i <= nb; i++) {
+        u32 large = nb;  // levels before the small ones
+        while (large > 0 && nb - large < kMergeSmallLevels) {
+            const Level& LB = B->lv[large - 1];
+            const u64 g = LB.g + (large <= A->lv.size() ? A->lv[large - 1].g : 0);
+            const u64 G = LB.G + (large <= A->lv.size() ? A->lv[large - 1].G : 0);
+            if (LB.g == 0 || g > kMergeSmallRules || G > kMergeSmallSymbols) break;
+            large--;
+        }
+        for (u32 i = 1; i <= large; i++) {
             if (A->lv.size() < i) A->lv.emplace_back();
             Level& LA = A->lv[i - 1];
             const Level& LB = B->lv[i - 1];
@@ -1836,6 +1958,7 @@ void merge(lcg_ctx* ctx, lcg_grammar* A, const lcg_grammar* B) {
             temps.pop_back();
             Mprev = m.M;
         }
+        if (large < nb) merge_small(ctx, A, B, large, Mprev, d_tot + tot.size(), d_tot, cb_rank, temps);
         grow_c(ctx, A, A->k + kb);
         if (kb) {
             ck(ctx, cudaMemcpyAsync(A->c_level + A->k, B->c_level, kb * 4, cudaMemcpyDeviceToDevice, ctx->st), "copy");

@@ -99,11 +99,12 @@ cudaError_t launch_scan2(const u32* in0, const u32* in1, u64 n, u64* out0, u64* 
 // MergeGrams
 // --------------------------------------------------------------------------
 
-// Three launches per level and no wait of the host between levels: the lookup reads
-// G_b's symbols through Mprev (no rewritten copy of G_b), the append takes the
-// totals of the scan from device memory, enters the new rules in G_a's table and
-// renames G_b's roots.  Two grammars of 3.5 M rules in 15 levels: 2.0 ms with
-// eight launches and two waits per level, 1.5 ms with these.
+// Three launches per large level: the lookup reads G_b's symbols through Mprev (no
+// rewritten copy of G_b), the append takes the totals of the scan from device memory,
+// enters the new rules in G_a's table and renames G_b's roots.  Bound by random
+// sectors: the table's slots in DRAM, ranks and fingerprints in L2.  (Tiles of 1024
+// rules with their symbols in shared memory and four rules a thread, and claiming the
+// slots in the lookup, were slower: 543 + 223 us against 267 + 342.)
 //
 // A rule of more than kRuleLong symbols (an N-run of DNA) is read, hashed and
 // compared by a whole warp, after the 32 rules of its threads: a thread alone
@@ -140,7 +141,7 @@ __device__ __forceinline__ u64 rule_poly(Get get, u64 len, const u32* __restrict
         u32 f[4];
         const u64 m = j < 4 ? j : 4;
 #pragma unroll
-        for (int u = 0; u < 4; u++) f[u] = (u64)u < m ? __ldg(F + get(j - 1 - u)) : 0u;
+        for (int u = 0; u < 4; u++) f[u] = (u64)u < m ? F[get(j - 1 - u)] : 0u;
 #pragma unroll
         for (int u = 0; u < 4; u++)
             if ((u64)u < m) H = addmod61(mulmod61(H, c), (u64)f[u]);
@@ -174,12 +175,14 @@ __global__ void __launch_bounds__(256) k_resident_build(const u32* __restrict__ 
               });
 }
 
-// Symbol x of G_b's right-hand sides in G_a's ranks.
+// Symbol x of G_b's right-hand sides in G_a's ranks.  (What a merge itself writes --
+// ranks, rules, fingerprints -- is read by plain loads: k_merge_small reads it in the
+// launch that wrote it.)
 template <bool kByte>
 __device__ __forceinline__ u32 merge_sym(const MergeLevel& m, u64 x) {
     const u32 v = __ldg(m.brhs + x);
     if constexpr (kByte) return v;
-    else return __ldg(m.Mprev + v);
+    else return m.Mprev[v];
 }
 
 // An earlier level's failure: what this one would read may not have been written.
@@ -191,20 +194,10 @@ __device__ __forceinline__ bool merge_failed(const MergeLevel& m) {
 // (G_b's symbols through Mprev are G_a's ranks; looked up in G_a's table of the
 // level, hashed keys confirmed by comparing contents), else a miss.  Bound by the
 // round trips of a thread's rule: its bounds, its symbols, their ranks, the slot.
-template <bool kByte>
-__global__ void __launch_bounds__(256) k_merge_lookup(const __grid_constant__ MergeLevel m) {
-    pdl_wait();
-    if (merge_failed(m)) return;
+template <bool kByte, typename Put>
+__device__ __forceinline__ void merge_lookup(const MergeLevel& m, u64 r_first, u64 r_end, u64 block, u64 blocks, Put put) {
     const ContentTable at{(Slot*)m.slots, m.cap};
-    auto put = [&](u64 r, u64 len, u64 found) {
-        if (found != ~0ull) {
-            if (m.aF[found] != m.bF[r]) set_error(m.ds, kErrMismatch);
-            m.M[r] = (u32)found;
-        }
-        m.miss[r] = found == ~0ull ? 1u : 0u;
-        m.mlen[r] = found == ~0ull ? (u32)len : 0u;
-    };
-    for_rules(m.boff, 0, m.gb, blockIdx.x, gridDim.x,
+    for_rules(m.boff, r_first, r_end, block, blocks,
               [&](u64 r, u64 s, u64 len) {
                   const Key128 key = rank_key<kByte>([&](u64 j) { return merge_sym<kByte>(m, s + j); }, len, m.aFprev,
                                                      m.lh.c, 0);
@@ -216,8 +209,8 @@ __global__ void __launch_bounds__(256) k_merge_lookup(const __grid_constant__ Me
                       }));
               },
               [&](u64 r, u64 s, u64 len) {
-                  const u64 H = warp_poly61([&](u64 j) -> u64 { return __ldg(m.aFprev + merge_sym<kByte>(m, s + j)); },
-                                            len, m.lh.c);
+                  const u64 H = warp_poly61([&](u64 j) -> u64 { return m.aFprev[merge_sym<kByte>(m, s + j)]; }, len,
+                                            m.lh.c);
                   const u64 found = table_find_warp(at, key_hashed(H, len, 0), [&](u64 ra) {
                       const u64 o = m.aoff[ra];
                       return warp_equal([&](u64 x) { return m.arhs[o + x]; },
@@ -225,6 +218,20 @@ __global__ void __launch_bounds__(256) k_merge_lookup(const __grid_constant__ Me
                   });
                   if ((threadIdx.x & 31) == 0) put(r, len, found);
               });
+}
+
+template <bool kByte>
+__global__ void __launch_bounds__(256) k_merge_lookup(const __grid_constant__ MergeLevel m) {
+    pdl_wait();
+    if (merge_failed(m)) return;
+    merge_lookup<kByte>(m, 0, m.gb, blockIdx.x, gridDim.x, [&](u64 r, u64 len, u64 found) {
+        if (found != ~0ull) {
+            if (m.aF[found] != m.bF[r]) set_error(m.ds, kErrMismatch);
+            m.M[r] = (u32)found;
+        }
+        m.miss[r] = found == ~0ull ? 1u : 0u;
+        m.mlen[r] = found == ~0ull ? (u32)len : 0u;
+    });
 }
 
 // Append the missed rules of G_b to G_a in G_b's rank order (totals: their number
@@ -258,7 +265,7 @@ __global__ void __launch_bounds__(256) k_merge_append(const __grid_constant__ Me
                   const u32 lane = threadIdx.x & 31;
                   const u64 nr = m.ga + m.xrank[r], o = m.Ga + m.xlen[r];
                   for (u64 x = lane; x < len; x += 32) m.arhs[o + x] = merge_sym<kByte>(m, s + x);
-                  const u64 H = warp_poly61([&](u64 j) -> u64 { return __ldg(m.aFprev + merge_sym<kByte>(m, s + j)); },
+                  const u64 H = warp_poly61([&](u64 j) -> u64 { return m.aFprev[merge_sym<kByte>(m, s + j)]; },
                                             len, m.lh.c);
                   if (lane == 0) {
                       m.aoff[nr] = o;
@@ -267,6 +274,163 @@ __global__ void __launch_bounds__(256) k_merge_append(const __grid_constant__ Me
                       table_put(at, key_hashed(H, len, nr), nr, m.ds);
                   }
               });
+}
+
+// --------------------------------------------------------------------------
+// the small levels of a merge: all of them in one cooperative launch
+// --------------------------------------------------------------------------
+//
+// Launch by launch a level of a few thousand rules takes eight launches and copies in
+// a row, 45 us, whatever its size; two grammars of 3.5 M rules have eleven such levels
+// of 15.  Here G_a's tables and grown arrays of all of them are filled at once, and a
+// level then takes two barriers: each block looks its part of G_b's rules up and
+// counts what is new, then appends it after what the blocks before it counted.
+// All eleven in 231 us (32768 rules a level at most, both grammars together: 2.48 ms
+// for importing, merging and exporting the two, 131072: 2.42, 262144: 2.40, 655360:
+// 2.40, none: 2.64).
+
+constexpr u32 kNoRank = 0xffffffffu;
+
+template <bool kByte>
+__device__ __forceinline__ void merge_build(const MergeLevel& m) {
+    const ContentTable t{(Slot*)m.slots, m.cap};
+    for_rules(m.aoff, 0, m.ga, blockIdx.x, gridDim.x,
+              [&](u64 r, u64 s, u64 len) {
+                  table_put(t, rank_key<kByte>([&](u64 j) { return m.arhs[s + j]; }, len, m.aFprev, m.lh.c, r), r, m.ds);
+              },
+              [&](u64 r, u64 s, u64 len) {
+                  const u64 H = warp_poly61([&](u64 j) -> u64 { return m.aFprev[m.arhs[s + j]]; }, len, m.lh.c);
+                  if ((threadIdx.x & 31) == 0) table_put(t, key_hashed(H, len, r), r, m.ds);
+              });
+}
+
+// Part `block` of G_b's rules: M[r] their ranks, kNoRank for new ones, whose number and
+// symbols go to counts[2 block], counts[2 block + 1].
+template <bool kByte>
+__device__ __forceinline__ void merge_part_lookup(const MergeLevel& m, u64 lo, u64 hi, u64* counts) {
+    u64 n = 0, G = 0;
+    merge_lookup<kByte>(m, lo, hi, 0, 1, [&](u64 r, u64 len, u64 found) {
+        if (found != ~0ull) {
+            if (m.aF[found] != m.bF[r]) set_error(m.ds, kErrMismatch);
+        } else {
+            n++;
+            G += len;
+        }
+        m.M[r] = found == ~0ull ? kNoRank : (u32)found;
+    });
+    u64 tn, tG;
+    block_excl_scan(n, tn);
+    block_excl_scan(G, tG);
+    if (threadIdx.x == 0) {
+        counts[2 * blockIdx.x] = tn;
+        counts[2 * blockIdx.x + 1] = tG;
+    }
+}
+
+template <bool kByte>
+__device__ __forceinline__ void merge_part_append(const MergeLevel& m, u64 lo, u64 hi, const u64* counts, u64* totals) {
+    const u32 lane = threadIdx.x & 31;
+    const ContentTable at{(Slot*)m.slots, m.cap};
+    u64 bn = 0, bG = 0, an = 0, aG = 0;  // new rules and symbols before this part, and in all
+    for (u32 b = threadIdx.x; b < gridDim.x; b += blockDim.x) {
+        const u64 x = counts[2 * b], y = counts[2 * b + 1];
+        an += x;
+        aG += y;
+        if (b < blockIdx.x) bn += x, bG += y;
+    }
+    u64 t;
+    block_excl_scan(bn, t);
+    u64 nr0 = m.ga + t;
+    block_excl_scan(bG, t);
+    u64 o0 = m.Ga + t;
+    block_excl_scan(an, t);
+    an = t;
+    block_excl_scan(aG, t);
+    aG = t;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        totals[0] = an;
+        totals[1] = aG;
+        m.aoff[m.ga + an] = m.Ga + aG;
+    }
+    for (u64 base = lo; base < hi; base += blockDim.x) {
+        const u64 r = base + threadIdx.x;
+        const bool miss = r < hi && m.M[r] == kNoRank;
+        const u64 s = miss ? m.boff[r] : 0, len = miss ? m.boff[r + 1] - s : 0;
+        u64 tot;  // lengths are below 2^28, new rules of a turn at most 1024
+        const u64 e = block_excl_scan(len << 16 | (miss ? 1u : 0u), tot);
+        const u64 nr = nr0 + (e & 0xffffu), o = o0 + (e >> 16);
+        if (miss) {
+            m.aoff[nr] = o;
+            m.aF[nr] = m.bF[r];
+            m.M[r] = (u32)nr;
+            if (len <= kRuleLong) {
+                for (u64 x = 0; x < len; x++) m.arhs[o + x] = merge_sym<kByte>(m, s + x);
+                table_put(at, rank_key<kByte>([&](u64 j) { return merge_sym<kByte>(m, s + j); }, len, m.aFprev, m.lh.c,
+                                              nr),
+                          nr, m.ds);
+            }
+        }
+        __syncwarp();
+        for (unsigned q = __ballot_sync(0xffffffffu, len > kRuleLong); q; q &= q - 1) {
+            const int l = __ffs(q) - 1;
+            const u64 ws = __shfl_sync(0xffffffffu, s, l), wl = __shfl_sync(0xffffffffu, len, l),
+                      wo = __shfl_sync(0xffffffffu, o, l), wr = __shfl_sync(0xffffffffu, nr, l);
+            for (u64 x = lane; x < wl; x += 32) m.arhs[wo + x] = merge_sym<kByte>(m, ws + x);
+            const u64 H = warp_poly61([&](u64 j) -> u64 { return m.aFprev[merge_sym<kByte>(m, ws + j)]; }, wl, m.lh.c);
+            if (lane == 0) table_put(at, key_hashed(H, wl, wr), wr, m.ds);
+            __syncwarp();
+        }
+        nr0 += tot & 0xffffu;
+        o0 += tot >> 16;
+    }
+}
+
+__global__ void __launch_bounds__(kMergeSmallThreads) k_merge_small(const __grid_constant__ MergeSmall a) {
+    pdl_wait();
+    u64 barriers = 0;
+    const u64 t0 = (u64)blockIdx.x * blockDim.x + threadIdx.x, stride = (u64)gridDim.x * blockDim.x;
+    for (u32 i = 0; i < a.levels; i++) {
+        const MergeLevel& m = a.lv[i];
+        const MergeOld& o = a.old[i];
+        if (o.off != nullptr) {
+            for (u64 x = t0; x <= m.ga; x += stride) m.aoff[x] = o.off[x];
+            for (u64 x = t0; x < m.ga; x += stride) m.aF[x] = o.F[x];
+        }
+        if (o.first && t0 == 0) m.aoff[0] = 0;
+        if (o.rhs != nullptr)
+            for (u64 x = t0; x < m.Ga; x += stride) m.arhs[x] = o.rhs[x];
+        if (o.fresh)
+            for (u64 x = t0; x < 2 * m.cap; x += stride)
+                reinterpret_cast<uint4*>(m.slots)[x] = make_uint4(~0u, ~0u, ~0u, ~0u);
+    }
+    DevStatus* const ds = a.lv[0].ds;
+    if (merge_failed(a.lv[0])) return;  // (by an earlier launch: the same for every block)
+    grid_barrier(a.bar, barriers++, ds);
+    for (u32 i = 0; i < a.levels; i++) {
+        const MergeLevel& m = a.lv[i];
+        if (!a.old[i].fresh) continue;
+        if (m.level == 1) merge_build<true>(m);
+        else merge_build<false>(m);
+    }
+    grid_barrier(a.bar, barriers++, ds);
+    for (u32 i = 0; i < a.levels; i++) {
+        const MergeLevel& m = a.lv[i];
+        const u64 part = (m.gb + gridDim.x - 1) / gridDim.x;
+        const u64 lo = min(m.gb, blockIdx.x * part), hi = min(m.gb, lo + part);
+        if (m.level == 1) merge_part_lookup<true>(m, lo, hi, a.counts);
+        else merge_part_lookup<false>(m, lo, hi, a.counts);
+        grid_barrier(a.bar, barriers++, ds);
+        if (m.level == 1) merge_part_append<true>(m, lo, hi, a.counts, a.totals[i]);
+        else merge_part_append<false>(m, lo, hi, a.counts, a.totals[i]);
+        grid_barrier(a.bar, barriers++, ds);
+    }
+    const u32 kb = a.lv[0].kb;
+    for (u64 j = t0; j < kb; j += stride) {
+        const u32 lvl = a.lv[0].c_level[j];
+        if (lvl >= a.lv[0].level)
+            for (u32 i = 0; i < a.levels; i++)
+                if (a.lv[i].level == lvl) a.lv[0].c_out[j] = a.lv[i].M[a.lv[0].c_rank[j]];
+    }
 }
 
 // F^0[s] = h^0(s) = ((a_0 s + b_0) mod p) mod m for every byte s (Sec. 3.2).
@@ -346,6 +510,17 @@ cudaError_t launch_resident_build(const u32* rhs, const u64* rhs_off, u64 r0, u6
 cudaError_t launch_merge_lookup(const MergeLevel& m, bool bytes, cudaStream_t st) {
     if (m.gb == 0) return cudaSuccess;
     return launch_pdl(bytes ? k_merge_lookup<true> : k_merge_lookup<false>, grid_for(m.gb), 256, st, m);
+}
+
+u32 merge_small_blocks() {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms > 0 ? (u32)sms : 1u;
+}
+
+cudaError_t launch_merge_small(const MergeSmall& a, u32 blocks, cudaStream_t st) {
+    return launch_coop(k_merge_small, blocks, kMergeSmallThreads, 0, st, a);
 }
 
 cudaError_t launch_merge_append(const MergeLevel& m, bool bytes, cudaStream_t st) {

@@ -290,6 +290,45 @@ __device__ void block_lookback(LBSlot<NV>* st, u64 tile, u64 epoch, const u64 (&
     lookback_finish<NV>(st, tile, epoch, agg, excl, ds);
 }
 
+// Barrier over the grid of a cooperative launch, the idx-th of the launch
+// (idx = 0, 1, ...); bar: two zeroed counters (arrivals, releases).  The last
+// block to arrive runs `work` before it lets the others go.  Bounded: after
+// kSpinLimit polls the round fails with kErrTimeout and the later steps do
+// nothing.
+template <typename Work>
+__device__ __forceinline__ void grid_barrier_work(u64* bar, u64 idx, DevStatus* ds, Work work) {
+    __shared__ u32 s_last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_last = atomicAdd(&bar[0], 1ull) == (idx + 1) * gridDim.x - 1 ? 1u : 0u;
+    }
+    __syncthreads();
+    if (s_last) {
+        __threadfence();
+        work();
+        __syncthreads();
+        if (threadIdx.x == 0)
+            asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(&bar[1]), "l"(idx + 1) : "memory");
+    } else if (threadIdx.x == 0) {
+        u64 it = 0;
+        while (true) {
+            u64 v;
+            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(&bar[1]) : "memory");
+            if (v > idx) break;
+            if (++it > kSpinLimit) {
+                set_error(ds, kErrTimeout);
+                break;
+            }
+            __nanosleep(32);
+        }
+    }
+    __syncthreads();
+}
+__device__ __forceinline__ void grid_barrier(u64* bar, u64 idx, DevStatus* ds) {
+    grid_barrier_work(bar, idx, ds, [] {});
+}
+
 // Tile index in launch order from a counter that is never reset: the host
 // passes the counter's value at launch (`ctr_base`).
 __device__ __forceinline__ u64 dynamic_tile(u64* ctr, u64 ctr_base) {

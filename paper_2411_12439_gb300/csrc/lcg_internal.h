@@ -225,6 +225,28 @@ struct MergeLevel {
 };
 cudaError_t launch_merge_lookup(const MergeLevel& m, bool bytes, cudaStream_t st);
 cudaError_t launch_merge_append(const MergeLevel& m, bool bytes, cudaStream_t st);
+// The small levels of a merge, in one launch.
+constexpr u32 kMergeSmallLevels = 40;         // of one launch
+constexpr u64 kMergeSmallRules = 262144;      // of a level, both grammars' together
+constexpr u64 kMergeSmallSymbols = 4 * kMergeSmallRules;
+constexpr int kMergeSmallThreads = 512;
+struct MergeOld {
+    const u64* off;  // G_a's arrays before they grew (null: they did not)
+    const u32* F;
+    const u32* rhs;
+    bool first;  // G_a had no such level
+    bool fresh;  // its table is to be filled
+};
+struct MergeSmall {
+    u32 levels;  // consecutive ones, the lowest first
+    u64* bar;    // two zeroed counters
+    u64* counts;  // two per block
+    u64* totals[kMergeSmallLevels];
+    MergeLevel lv[kMergeSmallLevels];  // (no miss, mlen, xrank, xlen)
+    MergeOld old[kMergeSmallLevels];
+};
+u32 merge_small_blocks();
+cudaError_t launch_merge_small(const MergeSmall& a, u32 blocks, cudaStream_t st);
 // A level of an imported grammar, blocks of 256 rules from block blk0 on.
 struct FpLevel {
     const u32* rhs;
