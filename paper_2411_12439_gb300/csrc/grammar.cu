@@ -444,19 +444,52 @@ cudaError_t launch_h0(LevelHash h0, u32* F0, cudaStream_t st) {
     return launch_pdl(k_h0, 1, 256, st, h0, F0);
 }
 
+// The entry of a list whose blocks (from blk0 on, ascending) contain block b.
+template <typename T>
+__device__ __forceinline__ u32 owner_of(const T* list, u32 n, u64 b) {
+    u32 lo = 0, hi = n - 1;
+    while (lo < hi) {
+        const u32 mid = (lo + hi + 1) / 2;
+        if (list[mid].blk0 <= b) lo = mid;
+        else hi = mid - 1;
+    }
+    return lo;
+}
+
+// A grammar's columns copied in one launch: as copies of their own, 2 us each
+// however short, the 17 of a grammar of 15 levels took 50 us.
+constexpr u32 kCopyEach = 16;  // words per thread
+__global__ void __launch_bounds__(256) k_copy_cols(const CopyCol* __restrict__ cols, u32 ncols) {
+    pdl_wait();
+    const CopyCol c = cols[owner_of(cols, ncols, blockIdx.x)];
+    const u64 x0 = (blockIdx.x - c.blk0) * (256ull * kCopyEach);
+    const u32 m = (u32)min((u64)256 * kCopyEach, c.n - x0);
+    if (c.pad && x0 == 0 && threadIdx.x == 0) c.dst[c.n] = 0;
+    if (((reinterpret_cast<uintptr_t>(c.dst) | reinterpret_cast<uintptr_t>(c.src)) & 7) == 0) {
+        // (x0 is even: pairs stay aligned)
+        for (u32 x = threadIdx.x; x < m / 2; x += 256)
+            reinterpret_cast<uint2*>(c.dst + x0)[x] = __ldg(reinterpret_cast<const uint2*>(c.src + x0) + x);
+        if (threadIdx.x == 0 && (m & 1)) c.dst[x0 + m - 1] = c.src[x0 + m - 1];
+    } else {
+        for (u32 x = threadIdx.x; x < m; x += 256) c.dst[x0 + x] = __ldg(c.src + x0 + x);
+    }
+}
+
+u64 copy_blocks(u64 n) { return (n + 256 * kCopyEach - 1) / (256 * kCopyEach); }
+
+cudaError_t launch_copy_cols(const CopyCol* cols, u32 ncols, u64 blocks, cudaStream_t st) {
+    if (blocks == 0) return cudaSuccess;
+    return launch_pdl(k_copy_cols, (unsigned)blocks, 256, st, cols, ncols);
+}
+
 // Imported rules: F^i[r] must be h^i of the rule's right-hand side
 // (Eq. fast_hash over F^{i-1}); a difference means the grammar was built with
 // another hash family (or was altered).  All levels in one launch: block b has
 // 256 rules of the level whose blocks start at blk0 <= b.
 __global__ void __launch_bounds__(256) k_check_fp(const FpLevel* __restrict__ lv, u32 nl, DevStatus* ds) {
     pdl_wait();
-    u32 lo = 0, hi = nl - 1;
-    while (lo < hi) {
-        const u32 mid = (lo + hi + 1) / 2;
-        if (lv[mid].blk0 <= blockIdx.x) lo = mid;
-        else hi = mid - 1;
-    }
-    const FpLevel L = lv[lo];
+    if (vload(&ds->error) != 0) return;  // (a malformed stream: an earlier launch's)
+    const FpLevel L = lv[owner_of(lv, nl, blockIdx.x)];
     for_rules(L.off, 0, L.g, blockIdx.x - L.blk0, 1ull << 32,
               [&](u64 r, u64 s, u64 len) {
                   const u64 H = rule_poly([&](u64 j) { return __ldg(L.rhs + s + j); }, len, L.Fprev, L.lh.c);

@@ -257,6 +257,15 @@ struct FpLevel {
     LevelHash lh;
 };
 cudaError_t launch_check_fp(const FpLevel* lv, u32 nl, u64 blocks, DevStatus* ds, cudaStream_t st);
+// Columns to copy, blocks from blk0 on.
+struct CopyCol {
+    u32* dst;
+    const u32* src;
+    u64 n, blk0;
+    bool pad;  // a zero after them
+};
+u64 copy_blocks(u64 n);
+cudaError_t launch_copy_cols(const CopyCol* cols, u32 ncols, u64 blocks, cudaStream_t st);
 // F arrays of a grammar by level (F[0] = F^0).
 struct FTable {
     const u32* F[65];
