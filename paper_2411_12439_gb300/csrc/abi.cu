@@ -2202,23 +2202,27 @@ void free_pp(lcg_pp* pp) {
 }
 
 // Exclusive scan of up to two u32 columns (the library's single-pass scan);
-// returns the column totals.
-void pp_scan(lcg_ctx* ctx, const u32* in0, const u32* in1, u64 n, u64* out0, u64* out1, u64 tot[2]) {
-    tot[0] = tot[1] = 0;
-    if (n == 0) return;
+// their totals go to totals[0] and [1] (on the device), the first also to *end0.
+void pp_scan(lcg_ctx* ctx, const u32* in0, const u32* in1, u64 n, u64* out0, u64* out1, u64* totals,
+             u64* end0 = nullptr) {
     u64 grid = 0;
     const u64 stiles = std::max<u64>(1, scan2_tiles_for(n));
     ensure_lb(ctx, &ctx->lb2, &ctx->lb2_tiles, stiles, scan2_lb_bytes(stiles));
-    ck(ctx, launch_scan2(in0, in1, n, out0, out1, ctx->scratch + 1, ctx->lb2, ++ctx->epoch, ctx->ctr, ctx->ctr_val,
-                         ctx->ds, ctx->st, &grid),
+    ck(ctx, launch_scan2(in0, in1, n, out0, out1, totals, ctx->lb2, ++ctx->epoch, ctx->ctr, ctx->ctr_val,
+                         ctx->ds, ctx->st, &grid, nullptr, end0),
        "scan");
     ctx->ctr_val += grid;
     ctx->launches++;
-    ck(ctx, cudaMemcpyAsync(tot, ctx->scratch + 1, 16, cudaMemcpyDeviceToHost, ctx->st), "read totals");
-    check_device_status(ctx, read_status(ctx));
 }
 
-// Temporary device arrays of one post-processing call, freed in stream order.
+// The totals of the scans since the last wait.
+std::vector<u64> pp_totals(lcg_ctx* ctx, const u64* d, u64 n) {
+    std::vector<u64> t(n, 0);
+    if (n) ck(ctx, cudaMemcpyAsync(t.data(), d, n * 8, cudaMemcpyDeviceToHost, ctx->st), "read totals");
+    check_device_status(ctx, read_status(ctx));
+    return t;
+}
+
 struct PPTemps {
     lcg_ctx* ctx;
     std::vector<void*> ptrs;
@@ -2233,11 +2237,8 @@ struct PPTemps {
     }
 };
 
-void set_u64(lcg_ctx* ctx, u64* dst, u64 v) {
-    ck(ctx, cudaMemcpyAsync(dst, &v, 8, cudaMemcpyHostToDevice, ctx->st), "set value");
-    sync(ctx);  // v lives on the host stack
-}
-
+// Each step runs over all levels before the host waits for what it needs of them:
+// five waits in all.  (Level by level it was three to five waits a level.)
 lcg_pp* postprocess(lcg_ctx* ctx, const lcg_grammar* G) {
     const u32 nl = (u32)G->lv.size();
     fail_if(ctx, nl > (u32)kPPMaxLevels, LCG_EINVAL, "grammar with too many levels");
@@ -2249,53 +2250,83 @@ lcg_pp* postprocess(lcg_ctx* ctx, const lcg_grammar* G) {
     lv.n = nl;
     std::vector<u32*> uses(nl);
     u64 rl_total = 0, size_before = 0, size_rl = 0;
-    // RL, level by level
+    // RL: the lengths of the rewritten rules and the runs of every level
+    u64* d_tot = tmp.get<u64>(2 * (u64)nl + 2);
+    std::vector<u64*> new_off(nl), rl_off(nl);
     for (u32 i = 0; i < nl; i++) {
         const Level& L = G->lv[i];
-        const u64 g = L.g;
         size_before += L.G;
-        u32* out_len = tmp.get<u32>(g);
-        u32* rl_len = tmp.get<u32>(g);
-        u64* new_off = tmp.get<u64>(g + 1);
-        u64* rl_off = tmp.get<u64>(g);
-        ck(ctx, launch_rl_count(L.rhs_off, L.rhs, g, out_len, rl_len, ctx->st), "k_rl_count");
-        u64 tot[2];
-        pp_scan(ctx, out_len, rl_len, g, new_off, rl_off, tot);
-        const u64 Gn = tot[0], R = tot[1];
-        set_u64(ctx, new_off + g, Gn);
-        u32* new_rhs = tmp.get<u32>(Gn);
-        u32* run_y = tmp.get<u32>(R);
-        u32* run_len = tmp.get<u32>(R);
-        u64* run_pos = tmp.get<u64>(R);
+        u32* out_len = tmp.get<u32>(L.g);
+        u32* rl_len = tmp.get<u32>(L.g);
+        new_off[i] = tmp.get<u64>(L.g + 1);
+        rl_off[i] = tmp.get<u64>(L.g);
+        ck(ctx, launch_rl_count(L.rhs_off, L.rhs, L.g, out_len, rl_len, ctx->st), "k_rl_count");
+        pp_scan(ctx, out_len, rl_len, L.g, new_off[i], rl_off[i], d_tot + 2 * i, new_off[i] + L.g);
+        ctx->launches++;
+    }
+    std::vector<u64> tot = pp_totals(ctx, d_tot, 2 * (u64)nl);
+    std::vector<u64> Gn(nl);
+    // the rules without runs, and the distinct runs of the levels that have any
+    struct Runs {
+        u64 R = 0;
+        u32 *y = nullptr, *len = nullptr;
+        u64 *pos = nullptr, *first = nullptr, *rank_of = nullptr;
+        u32* rhs = nullptr;
+    };
+    std::vector<Runs> runs(nl);
+    bool any = false;
+    for (u32 i = 0; i < nl; i++) {
+        const Level& L = G->lv[i];
+        const u64 R = tot[2 * i + 1];
+        Gn[i] = tot[2 * i];
+        Runs& x = runs[i];
+        x.R = R;
+        x.rhs = tmp.get<u32>(Gn[i]);
+        size_rl += Gn[i];
         u64 cap = 64;
         while (cap < 2 * R + 16) cap <<= 1;
-        u64* keys = tmp.get<u64>(cap);
-        u64* vals = tmp.get<u64>(cap);
-        ck(ctx, cudaMemsetAsync(keys, 0xFF, cap * 8, ctx->st), "memset");
-        ck(ctx, cudaMemsetAsync(vals, 0xFF, cap * 8, ctx->st), "memset");
-        ck(ctx, launch_rl_write(L.rhs_off, L.rhs, g, new_off, rl_off, new_rhs, run_y, run_len, run_pos, keys, vals,
+        u64 *keys = nullptr, *vals = nullptr;
+        if (R) {
+            x.y = tmp.get<u32>(R);
+            x.len = tmp.get<u32>(R);
+            x.pos = tmp.get<u64>(R);
+            x.first = tmp.get<u64>(R);
+            x.rank_of = tmp.get<u64>(R);
+            keys = tmp.get<u64>(cap);
+            vals = tmp.get<u64>(cap);
+            ck(ctx, cudaMemsetAsync(keys, 0xFF, cap * 8, ctx->st), "memset");
+            ck(ctx, cudaMemsetAsync(vals, 0xFF, cap * 8, ctx->st), "memset");
+        }
+        ck(ctx, launch_rl_write(L.rhs_off, L.rhs, L.g, new_off[i], rl_off[i], x.rhs, x.y, x.len, x.pos, keys, vals,
                                 cap - 1, ctx->ds, ctx->st),
            "k_rl_write");
-        u32* first = tmp.get<u32>(R);
-        u64* run_first = tmp.get<u64>(R);
-        u64* rank_of = tmp.get<u64>(R);
-        ck(ctx, launch_rl_first(run_y, run_len, R, keys, vals, cap - 1, first, run_first, ctx->ds, ctx->st),
-           "k_rl_first");
-        pp_scan(ctx, first, nullptr, R, rank_of, nullptr, tot);
-        const u64 Rd = tot[0];
+        ctx->launches++;
+        if (R) {
+            any = true;
+            u32* first = tmp.get<u32>(R);
+            ck(ctx, launch_rl_first(x.y, x.len, R, keys, vals, cap - 1, first, x.first, ctx->ds, ctx->st), "k_rl_first");
+            pp_scan(ctx, first, nullptr, R, x.rank_of, nullptr, d_tot + 2 * i);
+            ctx->launches++;
+        }
+    }
+    if (any) tot = pp_totals(ctx, d_tot, 2 * (u64)nl);
+    for (u32 i = 0; i < nl; i++) {
+        const Runs& x = runs[i];
+        const u64 Rd = x.R ? tot[2 * i] : 0;
+        const u64 g = G->lv[i].g;
         u32* rl_y = tmp.get<u32>(Rd);
         u32* rl_l = tmp.get<u32>(Rd);
-        ck(ctx, launch_rl_fix(run_y, run_len, run_pos, run_first, rank_of, R, new_rhs, rl_y, rl_l, ctx->ds, ctx->st),
+        ck(ctx, launch_rl_fix(x.y, x.len, x.pos, x.first, x.rank_of, x.R, x.rhs, rl_y, rl_l, ctx->ds, ctx->st),
            "k_rl_fix");
-        ctx->launches += 4;
-        lv.off[i] = new_off;
-        lv.rhs[i] = new_rhs;
+        ctx->launches++;
+        lv.off[i] = new_off[i];
+        lv.rhs[i] = x.rhs;
         lv.g[i] = g;
         lv.nrl[i] = Rd;
         lv.rl_y[i] = rl_y;
         lv.rl_l[i] = rl_l;
         rl_total += Rd;
-        size_rl += Gn + 2 * Rd;
+        size_rl += 2 * Rd;
         uses[i] = tmp.get<u32>(g);
         lv.pinned[i] = tmp.get<u8>(g);
         ck(ctx, cudaMemsetAsync(uses[i], 0, g * 4, ctx->st), "memset");
@@ -2303,7 +2334,7 @@ lcg_pp* postprocess(lcg_ctx* ctx, const lcg_grammar* G) {
     }
     // Simp: uses, kept rules, surviving rules and their ids
     for (u32 i = 1; i < nl; i++) {
-        ck(ctx, launch_pp_uses(lv.off[i], lv.rhs[i], lv.g[i], uses[i - 1], ctx->st), "k_pp_uses");
+        ck(ctx, launch_pp_uses(lv.rhs[i], Gn[i], uses[i - 1], ctx->st), "k_pp_uses");
         ck(ctx, launch_pp_pin_bases(lv.rl_y[i], lv.nrl[i], lv.pinned[i - 1], ctx->st), "k_pp_pin_bases");
         ctx->launches += 2;
     }
@@ -2313,18 +2344,20 @@ lcg_pp* postprocess(lcg_ctx* ctx, const lcg_grammar* G) {
         u32* surv = tmp.get<u32>(lv.g[i]);
         u64* spre = tmp.get<u64>(lv.g[i]);
         ck(ctx, launch_pp_survive(uses[i], lv.pinned[i], lv.g[i], surv, ctx->st), "k_pp_survive");
-        u64 tot[2];
-        pp_scan(ctx, surv, nullptr, lv.g[i], spre, nullptr, tot);
+        pp_scan(ctx, surv, nullptr, lv.g[i], spre, nullptr, d_tot + 2 * i);
         lv.surv[i] = surv;
         lv.spre[i] = spre;
-        lv.S[i] = tot[0];
-        lv.base[i] = next;
         lv.explen[i] = tmp.get<u32>(lv.g[i]);
         lv.dst[i] = tmp.get<u64>(lv.g[i]);
         ck(ctx, cudaMemsetAsync(lv.dst[i], 0xFF, lv.g[i] * 8, ctx->st), "memset");
+        ctx->launches += 1;
+    }
+    tot = pp_totals(ctx, d_tot, 2 * (u64)nl);
+    for (u32 i = 0; i < nl; i++) {
+        lv.S[i] = tot[2 * i];
+        lv.base[i] = next;
         next += lv.S[i] + lv.nrl[i];
         removed += lv.g[i] - lv.S[i];
-        ctx->launches += 2;
     }
     const u64 rules = next - 256;
     fail_if(ctx, next > 0xffffffffull, LCG_EOVERFLOW, "post-processed grammar with 2^32 symbols or more");
@@ -2339,10 +2372,8 @@ lcg_pp* postprocess(lcg_ctx* ctx, const lcg_grammar* G) {
     pp->k = G->k;
     try {
         pp->rhs_off = dalloc<u64>(ctx, rules + 1);
-        u64 tot[2];
-        pp_scan(ctx, fin_len, nullptr, rules, pp->rhs_off, nullptr, tot);
-        pp->size = tot[0];
-        set_u64(ctx, pp->rhs_off + rules, pp->size);
+        pp_scan(ctx, fin_len, nullptr, rules, pp->rhs_off, nullptr, d_tot, pp->rhs_off + rules);
+        pp->size = pp_totals(ctx, d_tot, 1)[0];
         pp->rhs = dalloc<u32>(ctx, pp->size);
         pp->kind = dalloc<u8>(ctx, rules);
         pp->c = dalloc<u32>(ctx, G->k);

@@ -52,7 +52,7 @@ __device__ __forceinline__ void scan_store(u64* out, u64 p0, u64 n, const u32 (&
 __global__ void __launch_bounds__(kScanThreads) k_scan2(const u32* __restrict__ in0, const u32* __restrict__ in1,
                                                         u64 n, u64* __restrict__ out0, u64* __restrict__ out1,
                                                         u64* __restrict__ totals, LBSlot<2>* lb, u64 epoch, u64* ctr,
-                                                        u64 ctr_base, DevStatus* ds, const u64* n_dev) {
+                                                        u64 ctr_base, DevStatus* ds, const u64* n_dev, u64* end0) {
     pdl_wait();
     const u64 tile = dynamic_tile(ctr, ctr_base);
     if (n_dev != nullptr) n = min(*n_dev, n);
@@ -78,6 +78,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan2(const u32* __restrict__ 
     if (out1 != nullptr) scan_store(out1, p0, n, b, eb);
     if ((tile + 1) * (u64)kScanTile >= n && threadIdx.x == 0) {
         totals[0] = excl[0] + ta;
+        if (end0 != nullptr) *end0 = excl[0] + ta;
         totals[1] = excl[1] + tb;
     }
 }
@@ -87,12 +88,12 @@ size_t scan2_lb_bytes(u64 tiles) { return scan2_lb_bytes_static(tiles); }
 
 cudaError_t launch_scan2(const u32* in0, const u32* in1, u64 n, u64* out0, u64* out1, u64* totals, void* lb,
                          u64 epoch, u64* ctr, u64 ctr_base, DevStatus* ds, cudaStream_t st, u64* grid_out,
-                         const u64* n_dev) {
+                         const u64* n_dev, u64* end0) {
     u64 tiles = scan2_tiles_for(n);
     if (tiles == 0) tiles = 1;
     *grid_out = tiles;
     return launch_pdl(k_scan2, (unsigned)tiles, kScanThreads, st, in0, in1, n, out0, out1, totals, (LBSlot<2>*)lb,
-                      epoch, ctr, ctr_base, ds, n_dev);
+                      epoch, ctr, ctr_base, ds, n_dev, end0);
 }
 
 // --------------------------------------------------------------------------

@@ -300,7 +300,7 @@ cudaError_t launch_to_bytes(const u32* cur, u64 cnt, unsigned char* out, cudaStr
 // read on the device (n then only bounds the grid).
 cudaError_t launch_scan2(const u32* in0, const u32* in1, u64 n, u64* out0, u64* out1, u64* totals, void* lb,
                          u64 epoch, u64* ctr, u64 ctr_base, DevStatus* ds, cudaStream_t st, u64* grid_out,
-                         const u64* n_dev = nullptr);
+                         const u64* n_dev = nullptr, u64* end0 = nullptr);
 u64 scan2_tiles_for(u64 n);
 size_t scan2_lb_bytes(u64 tiles);
 constexpr size_t scan2_lb_bytes_static(u64 tiles) { return tiles * sizeof(LBSlot<2>); }
@@ -334,7 +334,7 @@ cudaError_t launch_rl_first(const u32* run_y, const u32* run_len, u64 R, const u
 cudaError_t launch_rl_fix(const u32* run_y, const u32* run_len, const u64* run_pos, const u64* run_first,
                           const u64* rank_of, u64 R, u32* new_rhs, u32* rl_y, u32* rl_l, DevStatus* ds,
                           cudaStream_t st);
-cudaError_t launch_pp_uses(const u64* off, const u32* rhs, u64 g, u32* uses_below, cudaStream_t st);
+cudaError_t launch_pp_uses(const u32* rhs, u64 G, u32* uses_below, cudaStream_t st);
 cudaError_t launch_pp_pin_bases(const u32* rl_y, u64 nrl, u8* pinned_below, cudaStream_t st);
 cudaError_t launch_pp_pin_roots(const u32* c_level, const u32* c_rank, u32 k, const PPLevels& lv, cudaStream_t st);
 cudaError_t launch_pp_survive(const u32* uses, const u8* pinned, u64 g, u32* surv, cudaStream_t st);
