@@ -789,7 +789,12 @@ void next_input(lcg_ctx* ctx, RoundInput& in, RoundBufs& b) {
 // most (n symbols in k strings: (n + k) / 2 phrases), so nothing is planned,
 // regrown or waited for; the levels of a fresh build share one allocation too.
 
-bool is_tail(const lcg_ctx* ctx, u64 n) { return n <= kTailSymbols && round_tile(ctx, n) == 1024; }
+// (Where the slots of a table are limited the rounds that could need more run one by
+// one: theirs start within the limit.)
+bool is_tail(const lcg_ctx* ctx, u64 n) {
+    const u64 most = ctx->tuning.table_slots_max;
+    return n <= kTailSymbols && round_tile(ctx, n) == 1024 && (most == 0 || 3 * n <= most);
+}
 
 // Offsets of the parts of one allocation.
 struct Parts {

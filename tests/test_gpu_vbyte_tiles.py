@@ -2,6 +2,8 @@
 four of either to a counting block) and of the 16-byte lines of the output, for
 streams of shortest, longest and mixed values; values that reach over the edge of a
 tile, whole and malformed."""
+import gc
+
 import numpy as np
 import pytest
 
@@ -16,7 +18,8 @@ from paper_2411_12439_gb300 import Context, LCGError  # noqa: E402
 
 @pytest.fixture(scope="module")
 def ctx():
-    return Context(li.hash_family(), device=0)
+    yield Context(li.hash_family(), device=0)
+    gc.collect()  # tensors held by the tracebacks of refused calls go now, not in a later test
 
 
 def _values(kind, n):
@@ -33,6 +36,14 @@ def _bytes(b, shift=0):
     t = torch.zeros(len(b) + shift + 16, dtype=torch.uint8, device="cuda")
     t[shift:shift + len(b)] = torch.from_numpy(np.frombuffer(b, dtype=np.uint8).copy()).cuda()
     return t[shift:shift + len(b)]
+
+
+def _code(ctx, b, n):
+    try:
+        ctx.vbyte_decode(_bytes(b), n)
+    except LCGError as e:
+        return e.code
+    return 0
 
 
 @pytest.mark.parametrize("kind", ["short", "long", "mixed"])
@@ -68,8 +79,5 @@ def test_values_over_a_tile_edge(ctx, before):
         want[before] = sum((x & 0x7F) << (7 * j) for j, x in enumerate(bytes.fromhex(tail)))
         assert np.array_equal(ctx.vbyte_decode(_bytes(b), before + 4).cpu().numpy().view(np.uint32), want)
     for tail in ("808080808000", "ffffffff10", "ffffffffffffffffffff00", "80" * 20 + "00"):
-        with pytest.raises(LCGError) as e:
-            ctx.vbyte_decode(_bytes(lead + bytes.fromhex(tail)), before + 1)
-        assert e.value.code == -1
-    with pytest.raises(LCGError):
-        ctx.vbyte_decode(_bytes(lead + b"\x80"), before + 1)
+        assert _code(ctx, lead + bytes.fromhex(tail), before + 1) == -1
+    assert _code(ctx, lead + b"\x80", before + 1) == -1
