@@ -7,6 +7,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <initializer_list>
 #include <mutex>
 #include <new>
 #include <string>
@@ -97,6 +98,7 @@ struct lcg_ctx {
     // per-kernel CUDA-event timing (optional)
     int ktime = 0;  // 0 off, 1 every launch, 2 parse launches only
     bool capturing = false;              // the stream is being captured into a graph
+    unsigned char* mail = nullptr;       // page-locked: what the host reads of a step (see fetch)
     unsigned char* upload = nullptr;     // host input of graph builds, at a fixed address
     u64 upload_cap = 0;
     struct KRec {
@@ -260,10 +262,45 @@ void reset_status(lcg_ctx* ctx) {
     ck(ctx, cudaMemsetAsync(ctx->ds, 0, sizeof(DevStatus), ctx->st), "reset status");
 }
 
+// Waits for the stream and reads small values from the device, all of them through the
+// context's page-locked buffer: a copy to pageable memory is a wait of its own, and a
+// step mostly reads two or three (some 10 us each on the host, the device idle).
+constexpr u64 kMailBytes = 16384;
+struct Read {
+    void* dst;
+    const void* src;
+    u64 bytes;
+};
+void fetch(lcg_ctx* ctx, std::initializer_list<Read> reads) {
+    u64 total = 0;
+    for (const Read& r : reads) total += (r.bytes + 15) & ~15ull;
+    const bool mail = total <= kMailBytes;
+    u64 at = 0;
+    for (const Read& r : reads) {
+        if (r.bytes)
+            ck(ctx, cudaMemcpyAsync(mail ? (void*)(ctx->mail + at) : r.dst, r.src, r.bytes, cudaMemcpyDeviceToHost,
+                                    ctx->st),
+               "read");
+        at += (r.bytes + 15) & ~15ull;
+    }
+    sync(ctx);
+    at = 0;
+    for (const Read& r : reads) {
+        if (mail && r.bytes) std::memcpy(r.dst, ctx->mail + at, r.bytes);
+        at += (r.bytes + 15) & ~15ull;
+    }
+}
+
 DevStatus read_status(lcg_ctx* ctx) {
     DevStatus h;
-    ck(ctx, cudaMemcpyAsync(&h, ctx->ds, sizeof(h), cudaMemcpyDeviceToHost, ctx->st), "read status");
-    sync(ctx);
+    fetch(ctx, {{&h, ctx->ds, sizeof(h)}});
+    return h;
+}
+
+// The status, and another value of the same step.
+DevStatus read_status(lcg_ctx* ctx, void* dst, const void* src, u64 bytes) {
+    DevStatus h;
+    fetch(ctx, {{&h, ctx->ds, sizeof(h)}, {dst, src, bytes}});
     return h;
 }
 
@@ -1006,11 +1043,8 @@ void tail_sync(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32& i, bool agains
     const u32 rounds = tail_enqueue(ctx, R, in, i, in.n, in.kk, against_resident, nullptr, cap);
     std::vector<DevStatus> st(rounds);
     std::vector<RoundCounts> rc(rounds);
-    ck(ctx, cudaMemcpyAsync(st.data(), ctx->ds_arr + (i - 1), rounds * sizeof(DevStatus), cudaMemcpyDeviceToHost,
-                            ctx->st), "read status");
-    ck(ctx, cudaMemcpyAsync(rc.data(), ctx->rc_arr + (i - 1), rounds * sizeof(RoundCounts), cudaMemcpyDeviceToHost,
-                            ctx->st), "read counts");
-    sync(ctx);
+    fetch(ctx, {{st.data(), ctx->ds_arr + (i - 1), rounds * sizeof(DevStatus)},
+                {rc.data(), ctx->rc_arr + (i - 1), rounds * sizeof(RoundCounts)}});
     for (const DevStatus& x : st) {
         check_device_status(ctx, x);
         fail_if(ctx, x.overflow != 0, LCG_ETABLE, "phrase table full");  // not reached: it has room for every phrase
@@ -1113,9 +1147,7 @@ void round_sync(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, bool agains
     // round's phrases, which the host then waits for.
     u64 t_cap = b.Pmax;
     if (t_cap > kExactNext) {
-        ck(ctx, cudaMemcpyAsync(&rc, a.rc, sizeof(rc), cudaMemcpyDeviceToHost, ctx->st), "read counts");
-        ck(ctx, cudaMemcpyAsync(&st, a.ds, sizeof(st), cudaMemcpyDeviceToHost, ctx->st), "read status");
-        sync(ctx);
+        fetch(ctx, {{&rc, a.rc, sizeof(rc)}, {&st, a.ds, sizeof(st)}});
         check_device_status(ctx, st);
         t_cap = rc.phrases + 1;
     }
@@ -1131,9 +1163,7 @@ void round_sync(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, bool agains
         alloc_table(ctx, b, cap, std::min<u64>(max_ids, most));
         set_table(a, b);
         enqueue_parse(ctx, a, n);
-        ck(ctx, cudaMemcpyAsync(&rc, a.rc, sizeof(rc), cudaMemcpyDeviceToHost, ctx->st), "read counts");
-        ck(ctx, cudaMemcpyAsync(&st, a.ds, sizeof(st), cudaMemcpyDeviceToHost, ctx->st), "read status");
-        sync(ctx);
+        fetch(ctx, {{&rc, a.rc, sizeof(rc)}, {&st, a.ds, sizeof(st)}});
         check_device_status(ctx, st);
         if (!st.overflow) break;
         free_table(ctx, b);
@@ -1308,11 +1338,8 @@ int rounds_async_finish(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, const Asyn
     const u32 kk = ar.kk;
     std::vector<DevStatus> st(planned);
     std::vector<RoundCounts> rc(planned);
-    ck(ctx, cudaMemcpyAsync(st.data(), ctx->ds_arr, planned * sizeof(DevStatus), cudaMemcpyDeviceToHost, ctx->st),
-       "read status");
-    ck(ctx, cudaMemcpyAsync(rc.data(), ctx->rc_arr, planned * sizeof(RoundCounts), cudaMemcpyDeviceToHost, ctx->st),
-       "read counts");
-    sync(ctx);
+    fetch(ctx, {{st.data(), ctx->ds_arr, planned * sizeof(DevStatus)},
+                {rc.data(), ctx->rc_arr, planned * sizeof(RoundCounts)}});
     for (u32 r = 0; r < planned; r++) {
         if (st[r].overflow || st[r].error == kErrCapacity || st[r].error == kErrHalted) return -1;
         check_device_status(ctx, st[r]);
@@ -1949,8 +1976,7 @@ void merge(lcg_ctx* ctx, lcg_grammar* A, const lcg_grammar* B) {
             u64 more[2] = {gb, LB.G};
             const bool fits = m.ga + gb <= LA.cap_g && m.Ga + LB.G <= LA.cap_G;
             if (m.ga + gb > kMaxRank || (!fits && (m.ga + gb > kMergeAheadRules || m.Ga + LB.G > kMergeAheadSymbols))) {
-                ck(ctx, cudaMemcpyAsync(more, m.totals, 16, cudaMemcpyDeviceToHost, ctx->st), "read totals");
-                check_device_status(ctx, read_status(ctx));
+                check_device_status(ctx, read_status(ctx, more, m.totals, 16));
                 fail_if(ctx, m.ga + more[0] > kMaxRank, LCG_EOVERFLOW, "level with 2^31 rules or more");
             }
             grow_level(ctx, LA, m.ga + more[0], m.Ga + more[1]);
@@ -1969,9 +1995,7 @@ void merge(lcg_ctx* ctx, lcg_grammar* A, const lcg_grammar* B) {
             ck(ctx, cudaMemcpyAsync(A->c_level + A->k, B->c_level, kb * 4, cudaMemcpyDeviceToDevice, ctx->st), "copy");
             ck(ctx, cudaMemcpyAsync(A->c_rank + A->k, cb_rank, kb * 4, cudaMemcpyDeviceToDevice, ctx->st), "copy");
         }
-        if (nb)
-            ck(ctx, cudaMemcpyAsync(tot.data(), d_tot, tot.size() * 8, cudaMemcpyDeviceToHost, ctx->st), "read totals");
-        check_device_status(ctx, read_status(ctx));
+        check_device_status(ctx, read_status(ctx, tot.data(), d_tot, tot.size() * 8));
     } catch (...) {
         for (void* p : temps) dfree(ctx, p);
         throw;
@@ -2010,8 +2034,7 @@ void decompress(lcg_ctx* ctx, const lcg_grammar* G, u32 j, uint8_t* out, u64 cap
                                     on_dev ? cap : std::min<u64>(cap, kExpandSmallBytes), cur, d, ctx->st),
            "k_expand_small");
         ctx->launches++;
-        ck(ctx, cudaMemcpyAsync(&st, d, sizeof(st), cudaMemcpyDeviceToHost, ctx->st), "read state");
-        sync(ctx);
+        fetch(ctx, {{&st, d, sizeof(st)}});
     } else {
         u32 r = 0;
         ck(ctx, cudaMemcpyAsync(&st.level, G->c_level + j, 4, cudaMemcpyDeviceToHost, ctx->st), "read C");
@@ -2047,8 +2070,7 @@ void decompress(lcg_ctx* ctx, const lcg_grammar* G, u32 j, uint8_t* out, u64 cap
                              ++ctx->epoch, ctx->ctr, ctx->ctr_val, ctx->ds, ctx->st, &grid),
            "scan");
         ctx->ctr_val += grid;
-        ck(ctx, cudaMemcpyAsync(tot, ctx->scratch + 1, 16, cudaMemcpyDeviceToHost, ctx->st), "read total");
-        check_device_status(ctx, read_status(ctx));
+        check_device_status(ctx, read_status(ctx, tot, ctx->scratch + 1, 16));
         const u64 total = tot[0] + (tot[1] << 32);
         u32* next = nullptr;
         u8 *bytes = nullptr, *packed = nullptr;
@@ -2137,9 +2159,7 @@ void decompress_static(lcg_ctx* ctx, const lcg_grammar* G, u32 j, uint8_t* out, 
     fail_if(ctx, j >= G->k, LCG_EINVAL, "string index out of range");
     StaticScratch* sc = static_scratch_of_device(ctx);
     u32 lev = 0, r = 0;
-    ck(ctx, cudaMemcpyAsync(&lev, G->c_level + j, 4, cudaMemcpyDeviceToHost, ctx->st), "read C");
-    ck(ctx, cudaMemcpyAsync(&r, G->c_rank + j, 4, cudaMemcpyDeviceToHost, ctx->st), "read C");
-    sync(ctx);
+    fetch(ctx, {{&lev, G->c_level + j, 4}, {&r, G->c_rank + j, 4}});
     u32* cur = sc->cur;
     u32* nxt = sc->next;
     ck(ctx, cudaMemcpyAsync(cur, &r, 4, cudaMemcpyHostToDevice, ctx->st), "copy");
@@ -2156,8 +2176,7 @@ void decompress_static(lcg_ctx* ctx, const lcg_grammar* G, u32 j, uint8_t* out, 
            "scan");
         ctx->ctr_val += grid;
         u64 total = 0;
-        ck(ctx, cudaMemcpyAsync(&total, sc->totals, 8, cudaMemcpyDeviceToHost, ctx->st), "read total");
-        check_device_status(ctx, read_status(ctx));
+        check_device_status(ctx, read_status(ctx, &total, sc->totals, 8));
         if (total > kStaticMaxSymbols) {
             *out_len = total;  // a lower bound of the string's length
             fail_if(ctx, true, LCG_EOVERFLOW,
@@ -2223,8 +2242,7 @@ void pp_scan(lcg_ctx* ctx, const u32* in0, const u32* in1, u64 n, u64* out0, u64
 // The totals of the scans since the last wait.
 std::vector<u64> pp_totals(lcg_ctx* ctx, const u64* d, u64 n) {
     std::vector<u64> t(n, 0);
-    if (n) ck(ctx, cudaMemcpyAsync(t.data(), d, n * 8, cudaMemcpyDeviceToHost, ctx->st), "read totals");
-    check_device_status(ctx, read_status(ctx));
+    check_device_status(ctx, read_status(ctx, t.data(), d, n * 8));
     return t;
 }
 
@@ -2462,6 +2480,7 @@ int lcg_ctx_create(int device, const lcg_hash_family* H, void* stream, lcg_ctx**
             u64 thr = ~0ull;
             cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
         }
+        ck(ctx, cudaHostAlloc((void**)&ctx->mail, kMailBytes, cudaHostAllocDefault), "cudaHostAlloc");
         ck(ctx, cudaMalloc(&ctx->ds, sizeof(DevStatus)), "cudaMalloc");
         ck(ctx, cudaMalloc(&ctx->rc, sizeof(RoundCounts)), "cudaMalloc");
         ck(ctx, cudaMalloc(&ctx->ctr, sizeof(u64)), "cudaMalloc");
@@ -2489,6 +2508,7 @@ void lcg_ctx_destroy(lcg_ctx* ctx) {
     ctx->live.clear();
     destroy_graph(ctx);
     if (ctx->upload) cudaFree(ctx->upload);
+    if (ctx->mail) cudaFreeHost(ctx->mail);
     for (auto& r : ctx->krecs) {
         if (r.graph || r.part) continue;  // destroyed with the graph
         cudaEventDestroy(r.a);
@@ -2886,9 +2906,8 @@ int lcg_string_roots(lcg_ctx* ctx, const lcg_grammar* G, uint32_t j0, uint32_t c
     u32* d = dalloc<u32>(ctx, 3ull * count);
     ck(ctx, launch_roots(G->c_level, G->c_rank, j0, count, ft, d, ctx->st), "k_roots");
     std::vector<u32> h(3ull * count);
-    ck(ctx, cudaMemcpyAsync(h.data(), d, h.size() * 4, cudaMemcpyDeviceToHost, ctx->st), "roots");
+    fetch(ctx, {{h.data(), d, h.size() * 4}});
     dfree(ctx, d);
-    sync(ctx);
     for (u32 x = 0; x < count; x++) {
         level[x] = h[3 * x];
         rank[x] = h[3 * x + 1];
@@ -3158,9 +3177,8 @@ static std::vector<u64> vb_section_bytes(lcg_ctx* ctx, const lcg_grammar* G) {
         ck(ctx, launch_vb_count(L.rhs, nullptr, L.G, d + 2 * i + 1, sms, ctx->st), "k_vb_count");
         ctx->launches += (L.g != 0) + (L.G != 0);
     }
-    ck(ctx, cudaMemcpyAsync(nb.data(), d, 16 * nl, cudaMemcpyDeviceToHost, ctx->st), "read sizes");
+    fetch(ctx, {{nb.data(), d, 16 * nl}});
     dfree(ctx, d);
-    sync(ctx);
     return nb;
 }
 
@@ -3187,8 +3205,7 @@ int lcg_vbyte_encode(lcg_ctx* ctx, const uint32_t* in, uint64_t n, uint8_t* out,
         off = dalloc<u64>(ctx, tiles);
         vb_count_col(ctx, in, nullptr, n, cnt, off, ctx->scratch + 1);
         u64 nb = 0;
-        ck(ctx, cudaMemcpyAsync(&nb, ctx->scratch + 1, 8, cudaMemcpyDeviceToHost, ctx->st), "read size");
-        sync(ctx);
+        fetch(ctx, {{&nb, ctx->scratch + 1, 8}});
         *out_bytes = nb;
         fail_if(ctx, cap < nb, LCG_EINVAL, "output buffer too small");
         vb_write_col(ctx, in, nullptr, n, off, out, false, nb);
@@ -3292,8 +3309,7 @@ int lcg_export_vbyte(lcg_ctx* ctx, const lcg_grammar* G, void* out, uint64_t cap
             vb_scan(ctx, cnt, T, off, ctx->scratch + 1);
         }
         std::vector<u64> nb(ncols + 1);
-        ck(ctx, cudaMemcpyAsync(nb.data(), colb, 8 * (ncols + 1), cudaMemcpyDeviceToHost, ctx->st), "read sizes");
-        sync(ctx);
+        fetch(ctx, {{nb.data(), colb, 8 * (ncols + 1)}});
         for (u32 c = 0; c < ncols; c++) out_bytes += (double)nb[c];
         const u64 total = vb_total_bytes(G, nb);
         if (bytes) *bytes = total;
@@ -3386,8 +3402,7 @@ int lcg_import_vbyte(lcg_ctx* ctx, const void* buf, uint64_t size, int buf_on_de
         auto read_host = [&](void* dst, u64 off, u64 n) {
             if (n == 0) return;
             if (buf_on_device) {
-                ck(ctx, cudaMemcpyAsync(dst, b + off, n, cudaMemcpyDeviceToHost, ctx->st), "read");
-                sync(ctx);
+                fetch(ctx, {{dst, b + off, n}});
             } else {
                 std::memcpy(dst, b + off, n);
             }
