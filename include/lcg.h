@@ -145,7 +145,8 @@ int lcg_set_kernel_timing(lcg_ctx* ctx, int enable);
  * paper_2411_12439_gb300/autotune.py; the results do not depend on them):
  *   table_load          phrase-table slots per expected new rule is 1 / table_load
  *                       (0.3 .. 0.78; a table past 0.8 is regrown and the round rerun);
- *   parse_blocks_per_sm resident k_parse blocks per SM, 0 = as many as fit;
+ *   parse_blocks_per_sm resident k_parse blocks per SM in the rounds over ranks, 0 =
+ *                       as many as fit (a block of the byte round fills its SM);
  *   miss_flush          accepted (32 .. 256) and kept; it has no effect: every warp of
  *                       the parse looks its queued phrases up as soon as there are 32;
  *   table_slots_max     0, or at most this many slots (>= 1024) in the first phrase

@@ -106,6 +106,14 @@ __device__ __forceinline__ u32 string_of(const u64* soff, u32 k, u64 pos) {
 
 constexpr int kParseThreads = 32 * (int)kParseWarps;
 constexpr int kUnitMin = 128, kUnitMax = 512;
+// Warps of a k_parse block.  A byte round's blocks fill their SM, so that its warps
+// share one phrase cache of 8192 places instead of four of 2048 (round 1 of 4 x 3.1
+// Gbp, 22 k phrases: 39.6 ms, now 37.2; 64 x 5 Mbp 1.06 ms, 0.97).  Three probes in
+// it: text, whose phrases fill any cache, takes 0.72 ms so and 0.76 with eight.
+template <typename T>
+constexpr int parse_warps = sizeof(T) == 1 ? 32 : (int)kParseWarps;
+template <int W>
+constexpr int parse_blocks = W >= 32 ? 1 : W >= 16 ? 2 : (int)kParseBlocksMax;
 constexpr int kHalo = 64;  // symbols staged past the unit's end
 
 // Unit order of the rank rounds' parse: with `stripes` = k > 1
@@ -127,9 +135,7 @@ __device__ __forceinline__ u64 stripe_tile(u64 l, u64 ntiles, u32 stripes) {
     const u64 per = (ntiles + stripes - 1) / stripes;
     return (l % stripes) * per + l / stripes;
 }
-constexpr int kCacheBits = 11;
-constexpr int kCacheSlots = 1 << kCacheBits;  // per-block phrase cache (byte rounds)
-constexpr int kCacheProbes = 8;
+constexpr int kCacheProbes = 3;
 // Byte rounds: so many misses among a warp's 32 phrases are looked up in the table
 // at once (text, whose phrases are too many for the cache); fewer go to the
 // queue, where a full warp takes the long path.  Round 1 of 32 x 2 MB of text:
@@ -424,9 +430,11 @@ struct ParseArgs {
 
 // Shared memory of a k_parse block (dynamic).  A warp's part holds its unit's
 // symbols (and those of the unit it takes next), phrase starts and queue.
-template <typename T, int U>
+template <typename T, int U, int W>
 struct ParseSmem {
     static constexpr bool kByte = sizeof(T) == 1;
+    static constexpr int kCacheBits = W >= 32 ? 13 : W >= 16 ? 12 : 11;
+    static constexpr int kCacheSlots = 1 << kCacheBits;
     static constexpr int kSP = U + kHalo;            // staged symbols
     // phrase starts: a phrase has two symbols or more unless it is a string's
     // first, and a string in a round two or more, so at most two phrases start
@@ -438,7 +446,7 @@ struct ParseSmem {
         u64 claims, claim_len;  // what the warp claimed
         unsigned short start[kStarts];
     };
-    Warp w[kParseThreads / 32];
+    Warp w[W];
     ClaimIds ids;
     ParseArgs args;
     // byte rounds: the block's phrase cache, packed bytes -> CacheVal
@@ -451,10 +459,10 @@ struct ParseSmem {
 // A queued phrase: where it starts in S, its length, what is known of its home
 // slot, and the cache slot it may take (0: none); with its index p.
 constexpr int kPosBits = 44;  // positions and phrase indices are below 2^44
-__device__ __forceinline__ u64 queue_word(u64 pos, u32 len, u32 home, u32 cache) {
-    return pos | ((u64)len << kPosBits) | ((u64)home << (kPosBits + 6)) | ((u64)cache << (kPosBits + 8));
+__device__ __forceinline__ ulonglong2 queue_entry(u64 pos, u32 len, u32 home, u32 cache, u64 p) {
+    return make_ulonglong2(pos | ((u64)len << kPosBits) | ((u64)home << (kPosBits + 6)), p | ((u64)cache << kPosBits));
 }
-static_assert(kLongLen < 64 && kCacheBits + 1 <= 64 - kPosBits - 8, "queue word");
+static_assert(kLongLen < 64, "queue entry");
 
 // First index with R_phr >= p (the phrases of the strings that retire, ascending).
 __device__ __noinline__ u64 retired_before(const RoundArgs& a, u64 p) {
@@ -483,11 +491,11 @@ __device__ __noinline__ void emit_slow(const RoundArgs& a, u64 p, u32 id, u32 F)
     __stcs(a.Fnext + (p - lo), F);
 }
 
-template <typename T, int U>
-__device__ __forceinline__ ParseSmem<T, U>& parse_smem() {
-    static_assert((sizeof(ParseSmem<T, U>) + 1024) * kParseBlocksMax <= 228 * 1024, "shared memory of an SM");
+template <typename T, int U, int W>
+__device__ __forceinline__ ParseSmem<T, U, W>& parse_smem() {
+    static_assert((sizeof(ParseSmem<T, U, W>) + 1024) * parse_blocks<W> <= 228 * 1024, "shared memory of an SM");
     extern __shared__ __align__(16) unsigned char dyn_smem[];
-    return *reinterpret_cast<ParseSmem<T, U>*>(dyn_smem);
+    return *reinterpret_cast<ParseSmem<T, U, W>*>(dyn_smem);
 }
 
 // The resident rank of a phrase given its key (a hashed key names the
@@ -546,9 +554,9 @@ __device__ __forceinline__ Key128 byte_key(const u64* s64, u32 st, u32 len) {
 // Byte rounds: a phrase found or claimed enters the cache at its free place
 // `cache` - 1 (0: none; then it is not short either), valid from a place
 // after its first occurrence (at or before `first`) on.
-template <int U>
+template <int U, int W>
 __device__ __forceinline__ void cache_put(u32 cache, const Key128& key, u32 len, u32 id, u32 F, u64 first) {
-    ParseSmem<unsigned char, U>& sm = parse_smem<unsigned char, U>();
+    ParseSmem<unsigned char, U, W>& sm = parse_smem<unsigned char, U, W>();
     if (cache == 0 || id >= (1u << 26)) return;
     const u64 ck = ((u64)len << 56) | (key.hi & ((1ull << (8 * len)) - 1));
     if (atomicCAS((unsigned long long*)&sm.ckey[cache - 1], (unsigned long long)kEmpty, (unsigned long long)ck) == kEmpty)
@@ -558,9 +566,9 @@ __device__ __forceinline__ void cache_put(u32 cache, const Key128& key, u32 len,
 // A phrase of more than kLongLen symbols at `pos`, by the whole warp: the
 // fingerprint polynomial H (Eq. fast_hash) and the content comparisons of its
 // hashed key are spread over the lanes.
-template <typename T, int U>
+template <typename T, int U, int W>
 __device__ __noinline__ void parse_long(u64 pos, u64 len, u64 p) {
-    ParseSmem<T, U>& sm = parse_smem<T, U>();
+    ParseSmem<T, U, W>& sm = parse_smem<T, U, W>();
     const RoundArgs& a = *sm.args.all;
     const T* S = (const T*)a.S;
     const u32 lane = threadIdx.x & 31;
@@ -604,9 +612,9 @@ __device__ __noinline__ void parse_long(u64 pos, u64 len, u64 p) {
 // The long path on the warp's queued phrases first .. first + take - 1 (at
 // most 32): fingerprint, resident lookup, find or claim, and the symbol of
 // T^{i+1}.  Not inlined, so that the loop over the units keeps its registers.
-template <typename T, int U>
+template <typename T, int U, int W>
 __device__ __noinline__ void parse_queued(u32 first, u32 take) {
-    ParseSmem<T, U>& sm = parse_smem<T, U>();
+    ParseSmem<T, U, W>& sm = parse_smem<T, U, W>();
     const ParseArgs& a = sm.args;
     constexpr bool kByte = sizeof(T) == 1;
     const T* S = (const T*)a.S;
@@ -615,7 +623,8 @@ __device__ __noinline__ void parse_queued(u32 first, u32 take) {
     const bool act = lane < take;
     ulonglong2 e = make_ulonglong2(0ull, 0ull);
     if (act) e = w.queue[first + lane];
-    const u64 pos = e.x & ((1ull << kPosBits) - 1), p = e.y;
+    constexpr u64 kPosMask = (1ull << kPosBits) - 1;
+    const u64 pos = e.x & kPosMask, p = e.y & kPosMask;
     const u32 plen = (u32)(e.x >> kPosBits) & 63u, home = (u32)(e.x >> (kPosBits + 6)) & 3u;
     Key128 k;
     u64 H = 0;
@@ -693,7 +702,7 @@ __device__ __noinline__ void parse_queued(u32 first, u32 take) {
     if (act && (r != ~0ull || pub != kNoPub)) {
         const u32 id = r != ~0ull ? (u32)r : a.id_base + (u32)pub;
         if constexpr (kByte) {
-            cache_put<U>((u32)(e.x >> (kPosBits + 8)), k, plen, id, F, first_occ);
+            cache_put<U, W>((u32)(e.y >> kPosBits), k, plen, id, F, first_occ);
         }
         if (a.retired == 0 && p < a.T_cap) {
             __stcs(a.Tnext + p, id);
@@ -714,10 +723,10 @@ __device__ __noinline__ void parse_queued(u32 first, u32 take) {
 // 4 x 3.1 Gbp took 52.7 ms, now 37.1).  One phrase per thread at a time: with
 // two in flight round 2 of the same took 45.2 ms (44.4), with four 52.2: the
 // rounds with large tables are bound by random sectors, not by their latency.
-template <typename T, int U>
+template <typename T, int U, int W>
 __device__ __noinline__ u32 parse_unit_find(u32 buf, u64 t0, u64 p0, u64 out, u32 span, u32 nq, bool direct) {
-    using Smem = ParseSmem<T, U>;
-    Smem& sm = parse_smem<T, U>();
+    using Smem = ParseSmem<T, U, W>;
+    Smem& sm = parse_smem<T, U, W>();
     const ParseArgs& a = sm.args;
     constexpr bool kByte = Smem::kByte;
     const u32 lane = threadIdx.x & 31;
@@ -753,7 +762,7 @@ __device__ __noinline__ u32 parse_unit_find(u32 buf, u64 t0, u64 p0, u64 out, u3
                     const u64 lo = s64[0], hi = s64[1];
                     const u64 v = sh ? (lo >> sh) | (hi << (64 - sh)) : lo;
                     const u64 k = ((u64)len << 56) | (v & ((1ull << (8 * len)) - 1));
-                    u32 h = (u32)((k * 0x9E3779B97F4A7C15ull) >> (64 - kCacheBits));
+                    u32 h = (u32)((k * 0x9E3779B97F4A7C15ull) >> (64 - Smem::kCacheBits));
                     for (int probe = 0; probe < kCacheProbes; probe++) {
                         const u64 ck = ckey[h];
                         if (ck == k) {
@@ -769,7 +778,7 @@ __device__ __noinline__ u32 parse_unit_find(u32 buf, u64 t0, u64 p0, u64 out, u3
                             cache = h + 1;
                             break;
                         }
-                        h = (h + 1) & (kCacheSlots - 1);
+                        h = (h + 1) & (Smem::kCacheSlots - 1);
                     }
                 }
             }
@@ -784,7 +793,7 @@ __device__ __noinline__ u32 parse_unit_find(u32 buf, u64 t0, u64 p0, u64 out, u3
                 const u32 id = id_base + (u32)c.pub, F = (u32)(c.pub >> 32);
                 state = kDone;
                 emit(q, id, F);
-                if constexpr (kByte) cache_put<U>(cache, key, len, id, F, c.val);
+                if constexpr (kByte) cache_put<U, W>(cache, key, len, id, F, c.val);
             } else if (c.key.hi == kEmptyHi) {
                 state = kHomeEmpty;
             } else if (c.key.hi != key.hi) {
@@ -802,7 +811,7 @@ __device__ __noinline__ u32 parse_unit_find(u32 buf, u64 t0, u64 p0, u64 out, u3
         }
         if (state < kDone)
             w.queue[nq + __popc(m & ((1u << lane) - 1u))] =
-                make_ulonglong2(queue_word(t0 + st, len, state, cache), p0 + q);
+                queue_entry(t0 + st, len, state, cache, p0 + q);
         nq += (u32)__popc(m);
         longs |= __ballot_sync(0xffffffffu, state == kLong);
         __syncwarp();
@@ -810,17 +819,17 @@ __device__ __noinline__ u32 parse_unit_find(u32 buf, u64 t0, u64 p0, u64 out, u3
     return min(q0, cnt) | (nq << 10) | ((longs ? 1u : 0u) << 18);
 }
 
-template <typename T, int U>
+template <typename T, int U, int W>
 __device__ __forceinline__ void body_parse(const RoundArgs& a, u64 nunits) {
     pdl_wait();
-    using Smem = ParseSmem<T, U>;
+    using Smem = ParseSmem<T, U, W>;
     constexpr bool kByte = Smem::kByte;
     constexpr int kSP = Smem::kSP;
     constexpr int kWords = U / 32;  // break words of a unit
     constexpr int kBits = U / 32;   // positions per lane in the phrase list
     static_assert(kWords + kHalo / 32 <= 32 && kHalo % 32 == 0 && kBits <= 32, "a unit's break words fit one per lane");
     static_assert(kHalo > kLongLen, "a phrase that is not long lies in the staged symbols");
-    Smem& sm = parse_smem<T, U>();
+    Smem& sm = parse_smem<T, U, W>();
     const u32 lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     typename Smem::Warp& w = sm.w[warp];
 
@@ -833,7 +842,7 @@ __device__ __forceinline__ void body_parse(const RoundArgs& a, u64 nunits) {
     // The warps of the grid take units in turn (rank rounds in stripes when
     // asked) and wait for no other: unit lt of the logical order.
     const u32 stripes = kByte ? 1u : a.stripes;
-    const u32 nlog = (u32)stripe_tiles(nunits, stripes), step = gridDim.x * (kParseThreads / 32);
+    const u32 nlog = (u32)stripe_tiles(nunits, stripes), step = gridDim.x * W;
     // A unit's symbols go to buffer b; its break words (one per lane) and first
     // phrase index to registers.
     u32 nx_bits = 0;
@@ -867,11 +876,11 @@ __device__ __forceinline__ void body_parse(const RoundArgs& a, u64 nunits) {
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
 
-    u32 lt = blockIdx.x * (kParseThreads / 32) + warp;
+    u32 lt = blockIdx.x * W + warp;
     fetch(lt, 0);  // (its reads run beside the set-up)
     if constexpr (kByte) {
-        for (int x = threadIdx.x; x < 256; x += kParseThreads) sm.sF[x] = a.Fprev[x];
-        for (int x = threadIdx.x; x < kCacheSlots; x += kParseThreads) {
+        for (int x = threadIdx.x; x < 256; x += 32 * W) sm.sF[x] = a.Fprev[x];
+        for (int x = threadIdx.x; x < Smem::kCacheSlots; x += 32 * W) {
             sm.ckey[x] = kEmpty;
             sm.cval[x] = ~0ull;
         }
@@ -987,7 +996,7 @@ __device__ __forceinline__ void body_parse(const RoundArgs& a, u64 nunits) {
         bool longs = false;
         for (u32 q0 = 0;;) {
             if (q0 < cnt) {
-                const u32 r = parse_unit_find<T, U>(iter & 1, t0, p0, out, q0 | (cnt << 16), nq, direct);
+                const u32 r = parse_unit_find<T, U, W>(iter & 1, t0, p0, out, q0 | (cnt << 16), nq, direct);
                 q0 = r & 0x3FFu;
                 nq = (r >> 10) & 0xFFu;
                 longs = longs || (r >> 18) != 0;
@@ -995,7 +1004,7 @@ __device__ __forceinline__ void body_parse(const RoundArgs& a, u64 nunits) {
             if (nq < 32 && (have || nq == 0)) break;  // (the whole unit has been looked at)
             const u32 take = min(nq, 32u);
             nq -= take;
-            parse_queued<T, U>(nq, take);
+            parse_queued<T, U, W>(nq, take);
         }
 
         // 3. long phrases, one at a time by the whole warp
@@ -1006,7 +1015,7 @@ __device__ __forceinline__ void body_parse(const RoundArgs& a, u64 nunits) {
                 for (; m; m &= m - 1) {
                     const u32 x = q0 + (u32)__ffs(m) - 1;
                     const u64 st = w.start[x], en = x + 1 < cnt ? (u64)w.start[x + 1] : tail;
-                    parse_long<T, U>(t0 + st, en - st, p0 + x);
+                    parse_long<T, U, W>(t0 + st, en - st, p0 + x);
                 }
             }
         }
@@ -1365,8 +1374,9 @@ __global__ void k_gather_strings(const unsigned char* __restrict__ data, const u
 template <typename T>
 __global__ void __launch_bounds__(kBrkThreads) k_breaks(const RoundArgs a, u64 nblocks) { body_breaks<T>(a, nblocks); }
 template <typename T, int U>
-__global__ void __launch_bounds__(kParseThreads, kParseBlocksMax) k_parse(const __grid_constant__ RoundArgs a, u64 nunits) {
-    body_parse<T, U>(a, nunits);
+__global__ void __launch_bounds__(32 * parse_warps<T>, parse_blocks<parse_warps<T>>)
+    k_parse(const __grid_constant__ RoundArgs a, u64 nunits) {
+    body_parse<T, U, parse_warps<T>>(a, nunits);
 }
 __global__ void k_tile_strings(const RoundArgs a, u64 tiles) { body_tile_strings(a, tiles); }
 __global__ void __launch_bounds__(1024) k_strings(const RoundArgs a) { body_strings(a); }
@@ -1722,8 +1732,8 @@ __global__ void __launch_bounds__(kSmallThreads) k_parse_small(const __grid_cons
             __syncthreads();
             body_strings(a);
         });
-        if (kByte && r == 0) body_parse<unsigned char, kUnitMin>(a, a.tiles_bound);
-        else body_parse<u32, kUnitMin>(a, a.tiles_bound);
+        if (kByte && r == 0) body_parse<unsigned char, kUnitMin, kParseWarps>(a, a.tiles_bound);
+        else body_parse<u32, kUnitMin, kParseWarps>(a, a.tiles_bound);
         barrier([] {});
     }
 }
@@ -1875,9 +1885,9 @@ static int parse_occupancy(int* sms_out) {
         int dev = 0, sms = 0, occ = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        constexpr int smem = (int)sizeof(ParseSmem<T, U>);
+        constexpr int smem = (int)sizeof(ParseSmem<T, U, parse_warps<T>>);
         cudaFuncSetAttribute(k_parse<T, U>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_parse<T, U>, kParseThreads, smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_parse<T, U>, 32 * parse_warps<T>, smem);
         return std::make_pair(occ > 0 ? occ : 1, sms);
     }();
     if (sms_out) *sms_out = occ_sms.second;
@@ -1890,7 +1900,7 @@ static unsigned persistent_grid(u64 units, u32 per_sm) {
     int sms = 0;
     const int occ = parse_occupancy<T, U>(&sms);
     const u64 b = (per_sm == 0 || per_sm > (u32)occ) ? (u64)occ : (u64)per_sm;
-    const u64 g = b * (u64)sms, most = (units + kWarps - 1) / kWarps;
+    const u64 g = b * (u64)sms, most = (units + parse_warps<T> - 1) / parse_warps<T>;
     return (unsigned)(most < g ? (most ? most : 1) : g);
 }
 
@@ -1925,8 +1935,8 @@ cudaError_t launch_breaks(const RoundArgs& a, cudaStream_t st) {
 template <typename T, int U>
 static cudaError_t launch_parse_tp(const RoundArgs& a, cudaStream_t st) {
     const u64 tiles = a.tiles_bound;
-    return launch_pdl_smem(k_parse<T, U>, persistent_grid<T, U>(tiles, a.parse_blocks), kParseThreads,
-                           sizeof(ParseSmem<T, U>), st, a, tiles);
+    return launch_pdl_smem(k_parse<T, U>, persistent_grid<T, U>(tiles, a.parse_blocks), 32 * parse_warps<T>,
+                           sizeof(ParseSmem<T, U, parse_warps<T>>), st, a, tiles);
 }
 
 template <typename T>
@@ -1949,7 +1959,7 @@ cudaError_t launch_parse(const RoundArgs& a, cudaStream_t st) {
 template <bool kByte>
 static u32 tail_grid(u64 units) {
     using T0 = std::conditional_t<kByte, unsigned char, u32>;
-    constexpr size_t smem = std::max({sizeof(ParseSmem<T0, kUnitMin>), sizeof(ParseSmem<u32, kUnitMin>), sizeof(SoloSmem)});
+    constexpr size_t smem = std::max({sizeof(ParseSmem<T0, kUnitMin, kParseWarps>), sizeof(ParseSmem<u32, kUnitMin, kParseWarps>), sizeof(SoloSmem)});
     static const int cap = [] {
         int dev = 0, sms = 0, o1 = 0, o2 = 0;
         cudaGetDevice(&dev);
@@ -1965,7 +1975,7 @@ static u32 tail_grid(u64 units) {
 template <bool kByte>
 static cudaError_t launch_parse_small_t(const TailArgs& t, cudaStream_t st) {
     using T0 = std::conditional_t<kByte, unsigned char, u32>;
-    constexpr size_t smem = std::max({sizeof(ParseSmem<T0, kUnitMin>), sizeof(ParseSmem<u32, kUnitMin>), sizeof(SoloSmem)});
+    constexpr size_t smem = std::max({sizeof(ParseSmem<T0, kUnitMin, kParseWarps>), sizeof(ParseSmem<u32, kUnitMin, kParseWarps>), sizeof(SoloSmem)});
     return launch_coop(k_parse_small<kByte>, tail_grid<kByte>(t.r[0].tiles_bound), kSmallThreads, smem, st, t);
 }
 
