@@ -187,9 +187,11 @@ constexpr u64 kBrkSpan = (u64)kBrkThreads * 32;  // positions per block step
 static_assert(kUnitMax <= 32 * 32, "a warp of k_breaks covers whole parse units");
 
 // Head of block step b in the look-ahead words: (epoch << 8) | (state << 2) |
-// type, state 1 = open, 2 = decided.
+// type, state 1 = open, 2 = decided.  The word is all that passes between steps, so
+// it needs no order with other accesses (as a release the store held the block's warps
+// at the barrier after it).
 __device__ __forceinline__ void brk_publish(u64* heads, u64 b, u64 epoch, u32 state, u32 type) {
-    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(heads + b), "l"((epoch << 8) | (state << 2) | type)
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(heads + b), "l"((epoch << 8) | (state << 2) | type)
                  : "memory");
 }
 
@@ -201,7 +203,7 @@ __device__ u32 brk_lookahead(const u64* heads, u64 j, u64 nsteps, u64 epoch, u32
         u32 backoff = 32;
         while (true) {
             u64 w;
-            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(heads + j) : "memory");
+            asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(heads + j) : "memory");
             if ((w >> 8) == epoch) {
                 if (((w >> 2) & 3u) == 2u) return (u32)(w & 3u);
                 break;  // open: one run throughout, look at the next step
@@ -245,7 +247,7 @@ __device__ __forceinline__ void body_breaks(const RoundArgs& a, u64 nblocks) {
     __shared__ u32 sst[SW + 1];      // string starts at base .. base + kBrkSpan
     __shared__ u32 sfirst[kBrkThreads];  // type of each thread's first position
     __shared__ u32 s_bits[kBrkThreads], s_pre[kBrkThreads];
-    __shared__ u64 s_step;
+    __shared__ u64 s_step[2];
     __shared__ u32 s_open, s_carry;
     if (round_halted(a)) return;
     const T* S = (const T*)a.S;
@@ -263,22 +265,38 @@ __device__ __forceinline__ void body_breaks(const RoundArgs& a, u64 nblocks) {
     if (blockIdx.x >= nblocks && blockIdx.x > 0) return;  // more blocks than steps: no counter traffic
     u64* heads = a.heads;
     const int warp = tid >> 5;
-    for (bool once = true; once; once = !own_step) {
-        // the next block step, in decreasing order (the counter starts at 0 every round)
-        if (tid == 0) {
-            const u64 t = own_step ? (u64)blockIdx.x : atomicAdd(&a.ds->aux[0], 1ull);
-            s_step = t < nblocks ? nblocks - 1 - t : ~0ull;
-        }
-        __syncthreads();  // also: sF0 loaded
-        const u64 b = s_step;
-        if (b == ~0ull) break;
+    // Block steps in decreasing order (the counter starts at 0 every round).  In the
+    // rounds over ranks, with many steps a block, the step after the next is asked for
+    // and the next one's string starts are read while a step is worked on (rounds 2 and
+    // 3 of 4 x 3.1 Gbp: 4.29 and 1.39 ms, now 3.68 and 1.22); with few, a step that a
+    // block holds back would be one that another could have begun.  Not so the byte
+    // round, whose steps more often end in a run and wait for the next one's head (10.2
+    // ms, 10.0 without).
+    const bool ahead = !kByte && !own_step && nblocks > 4 * (u64)gridDim.x;
+    auto step_of = [&](u64 t) { return t < nblocks ? nblocks - 1 - t : ~0ull; };
+    auto ticket = [&]() { return step_of(own_step ? (u64)blockIdx.x : atomicAdd(&a.ds->aux[0], 1ull)); };
+    // string starts of a step (bitmap of k_tile_strings; n counts as one): this
+    // thread's word, and the one past the step
+    auto starts = [&](u64 b, u32 w) {
+        const u64 gw = b * (kBrkSpan / 32) + (u64)w;
+        return b != ~0ull && gw < a.sbm_words ? __ldg(a.sbm + gw) : 0u;
+    };
+    if (tid == 0) {
+        s_step[0] = ticket();
+        s_step[1] = ahead ? ticket() : ~0ull;
+    }
+    __syncthreads();  // also: sF0 loaded
+    u64 b = s_step[0], b_next = s_step[1];
+    u32 my_starts = starts(b, (u32)tid), end_starts = tid == 0 ? starts(b, SW) : 0u;
+    for (u32 it = 0; b != ~0ull; it++) {
+        u64 asked = ~0ull;
+        if (ahead && tid == 0) asked = ticket();
+        const u32 next_starts = ahead ? starts(b_next, (u32)tid) : 0u,
+                  next_end = ahead && tid == 0 ? starts(b_next, SW) : 0u;
         const u64 base = b * kBrkSpan;
         const u64 bend = min(base + kBrkSpan, n);
-        // string starts (bitmap of k_tile_strings; n counts as one)
-        for (int w = tid; w <= SW; w += kBrkThreads) {
-            const u64 gw = base / 32 + (u64)w;
-            sst[w] = gw < a.sbm_words ? __ldg(a.sbm + gw) : 0u;
-        }
+        sst[tid] = my_starts;
+        if (tid == 0) sst[SW] = end_starts;
         const u64 x0 = base + 32ull * (u64)tid;
         u32 f[32];
         if (aligned && x0 + 32 <= n) {
@@ -385,6 +403,7 @@ __device__ __forceinline__ void body_breaks(const RoundArgs& a, u64 nblocks) {
         if ((lane & (int)(lpu - 1)) == 0 && x0 < bend) a.tile_cnt[x0 / a.tp] = ucnt;
         // the first phrase of every string that starts in the step: its index
         // among its unit's phrases
+        if (!own_step && tid == 0) s_step[it & 1] = ahead ? asked : ticket();
         if (__syncthreads_or((int)(st & bits))) {
             u32 pre = (u32)__popc(bits);
 #pragma unroll
@@ -408,6 +427,18 @@ __device__ __forceinline__ void body_breaks(const RoundArgs& a, u64 nblocks) {
                 }
                 if (__shfl_sync(0xffffffffu, s < bend ? 1u : 0u, 31) == 0) break;
             }
+        }
+        if (own_step) break;
+        const u64 fresh = s_step[it & 1];
+        if (ahead) {
+            b = b_next;
+            b_next = fresh;
+            my_starts = next_starts;
+            end_starts = next_end;
+        } else {
+            b = fresh;
+            my_starts = starts(b, (u32)tid);
+            end_starts = tid == 0 ? starts(b, SW) : 0u;
         }
     }
 }
@@ -1372,7 +1403,10 @@ __global__ void k_gather_strings(const unsigned char* __restrict__ data, const u
 // --------------------------------------------------------------------------
 
 template <typename T>
-__global__ void __launch_bounds__(kBrkThreads) k_breaks(const RoundArgs a, u64 nblocks) { body_breaks<T>(a, nblocks); }
+// Blocks per SM: six in the byte round (10.0 ms for 12.4 GB; 10.2 with five, 10.5 with
+// four), four over ranks, whose steps read four times as much (3.7 ms for 3.6 G
+// symbols; 4.4 with three, 4.3 with five).
+__global__ void __launch_bounds__(kBrkThreads, sizeof(T) == 1 ? 6 : 4) k_breaks(const RoundArgs a, u64 nblocks) { body_breaks<T>(a, nblocks); }
 template <typename T, int U>
 __global__ void __launch_bounds__(32 * parse_warps<T>, parse_blocks<parse_warps<T>>)
     k_parse(const __grid_constant__ RoundArgs a, u64 nunits) {
