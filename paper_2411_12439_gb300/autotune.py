@@ -2,9 +2,9 @@
 with a cache of the best setting per class of collection.
 
 The parse tile size, the rank rounds' tile order (tiles taken in interleaved
-stripes), the parse kernel's resident blocks per SM, the phrase tables' load
-factor and the byte rounds' miss-queue threshold change the build's speed,
-never its result.
+stripes), the parse kernel's resident blocks per SM in those rounds and the
+phrase tables' load factor change the build's speed, never its result
+(``miss_flush`` is a field of the tuning that has no effect).
 ``autotune`` times builds of a sample collection on a context and keeps, one
 parameter at a time (coordinate descent, two sweeps), the value with the
 shortest median build time; the context keeps the best setting.

@@ -494,7 +494,7 @@ void free_grammar_now(lcg_grammar* G) {
 // --------------------------------------------------------------------------
 
 // Per-round ratios that size the next build's buffers: the largest seen,
-// decaying by 10 % per build, so that a context that sees collections of
+// decaying by 2 % per build, so that a context that sees collections of
 // changing make-up (a serving loop) keeps plans that fit.
 void record_hints(lcg_ctx* ctx, u32 i, u64 n, u64 P, u64 g, u64 G) {
     if (i >= 64) return;
@@ -1119,7 +1119,7 @@ void round_sync(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, bool agains
         a.rrhs_off = L.rhs_off;
     }
     // Phrase table: sized from the distinct/phrase ratio of this level in the
-    // context's previous build when there is one (at the tuning's load, 0.5 by
+    // context's previous build when there is one (at the tuning's load, 0.35 by
     // default: short probe sequences), else from a generous guess; an
     // overflowing table is regrown and the parse rerun.
     const double hint = ctx->ratio_hint[std::min<u32>(i, 63)];
@@ -1633,7 +1633,17 @@ lcg_grammar* build_with_graph(lcg_ctx* ctx, const unsigned char* d_in, const std
     ck(ctx, cudaMemcpyAsync(gb->soff, soff_h.data(), (k + 1) * sizeof(u64), cudaMemcpyHostToDevice, ctx->st),
        "upload offsets");
     ck(ctx, cudaMemcpyAsync(gb->sid, sid_h.data(), k * sizeof(u32), cudaMemcpyHostToDevice, ctx->st), "upload ids");
-    ck(ctx, cudaGraphLaunch(gb->exec, ctx->st), "graph launch");
+    cudaError_t el = cudaGraphLaunch(gb->exec, ctx->st);
+    if (el == cudaErrorMemoryAllocation) {
+        // the graph has memory of its own beside the pool's: what earlier builds left in
+        // the pool goes back to the device
+        cudaGetLastError();
+        sync(ctx);
+        cudaMemPool_t pool;
+        if (cudaDeviceGetDefaultMemPool(&pool, ctx->device) == cudaSuccess) cudaMemPoolTrimTo(pool, 0);
+        el = cudaGraphLaunch(gb->exec, ctx->st);
+    }
+    ck(ctx, el, "graph launch");
     ctx->ctr_val = gb->ctr_end;
     ctx->launches += gb->launches;
     for (const auto& r : gb->krecs) ctx->krecs.push_back(r);
@@ -2997,36 +3007,30 @@ int lcg_export_packed(lcg_ctx* ctx, const lcg_grammar* G, void* out, uint64_t ca
     add(G->c_level, 4ull * G->k);
     add(G->c_rank, 4ull * G->k);
     add(G->F0, 4 * 256);
-    struct Run {
-        u64 pos, bytes, at;
+    auto copy = [&](const Col& x) {
+        if (x.bytes) ck(ctx, cudaMemcpyAsync(o + x.pos, x.src, x.bytes, cudaMemcpyDeviceToHost, ctx->st), "export");
+        if (x.span > x.bytes) std::memset(o + x.pos + x.bytes, 0, x.span - x.bytes);
     };
-    std::vector<Run> runs;
-    Copies gather;
-    u64 staged = 0;
     for (size_t c = 0; c < cols.size();) {
         size_t e = c;
         while (e < cols.size() && cols[e].bytes <= kPackGather) e++;
         if (e < c + 2) {
-            const Col& x = cols[c++];
-            if (x.bytes) ck(ctx, cudaMemcpyAsync(o + x.pos, x.src, x.bytes, cudaMemcpyDeviceToHost, ctx->st), "export");
-            if (x.span > x.bytes) std::memset(o + x.pos + x.bytes, 0, x.span - x.bytes);
+            copy(cols[c++]);
             continue;
         }
-        const u64 bytes = cols[e - 1].pos + cols[e - 1].span - cols[c].pos;
-        runs.push_back(Run{cols[c].pos, bytes, staged});
-        for (; c < e; c++)
-            gather.add((void*)(staged + (cols[c].pos - runs.back().pos)), cols[c].src, cols[c].bytes / 4, true);
-        staged += bytes;
-    }
-    if (!runs.empty()) {
-        std::vector<void*> temps;
+        const u64 from = cols[c].pos, bytes = cols[e - 1].pos + cols[e - 1].span - from;
+        void* stage = nullptr;
+        if (cudaMallocAsync(&stage, bytes, ctx->st) != cudaSuccess) {  // (the form needs no device memory)
+            cudaGetLastError();
+            for (; c < e; c++) copy(cols[c]);
+            continue;
+        }
+        std::vector<void*> temps{stage};
         try {
-            u8* stage = dalloc<u8>(ctx, staged);
-            temps.push_back(stage);
-            for (CopyCol& x : gather.cols) x.dst = (u32*)(stage + (u64)(uintptr_t)x.dst);
+            Copies gather;
+            for (; c < e; c++) gather.add((u8*)stage + (cols[c].pos - from), cols[c].src, cols[c].bytes / 4, true);
             gather.run(ctx, temps);
-            for (const Run& r : runs)
-                ck(ctx, cudaMemcpyAsync(o + r.pos, stage + r.at, r.bytes, cudaMemcpyDeviceToHost, ctx->st), "export");
+            ck(ctx, cudaMemcpyAsync(o + from, stage, bytes, cudaMemcpyDeviceToHost, ctx->st), "export");
         } catch (...) {
             for (void* p : temps) dfree(ctx, p);
             throw;
