@@ -1792,7 +1792,7 @@ constexpr u64 kMergeAheadRules = 1ull << 20, kMergeAheadSymbols = 1ull << 21;
 void merge_small(lcg_ctx* ctx, lcg_grammar* A, const lcg_grammar* B, u32 i0, const u32* Mprev, u64* bar, u64* d_tot,
                  u32* cb_rank, std::vector<void*>& temps) {
     const u32 nb = (u32)B->lv.size();
-    const u32 blocks = merge_small_blocks();
+    const u32 blocks = coop_blocks();
     MergeSmall a{};
     a.bar = bar;
     Parts tmp, grown;
@@ -2029,7 +2029,7 @@ void decompress(lcg_ctx* ctx, const lcg_grammar* G, u32 j, uint8_t* out, u64 cap
     fail_if(ctx, j >= G->k, LCG_EINVAL, "string index out of range");
     // the upper levels, and the whole of a short string, in one launch
     ExpandState st{1, 0, 0};
-    u32* cur = nullptr;
+    u32 *cur = nullptr, *own = nullptr;  // the sequence, and the allocation that holds it
     u8* tmp = nullptr;  // bytes for a host buffer
     if (G->lv.size() <= 64) {
         ExpandLevels lv{};
@@ -2045,11 +2045,29 @@ void decompress(lcg_ctx* ctx, const lcg_grammar* G, u32 j, uint8_t* out, u64 cap
            "k_expand_small");
         ctx->launches++;
         fetch(ctx, {{&st, d, sizeof(st)}});
+        own = cur;
+        if (st.level >= 2) {
+            const u32 blocks = coop_blocks();
+            u64* words = dalloc<u64>(ctx, 2 + blocks);
+            u32* mid = dalloc<u32>(ctx, 2 * kExpandMid);
+            ck(ctx, cudaMemsetAsync(words, 0, 2 * sizeof(u64), ctx->st), "memset barrier");
+            ck(ctx, launch_expand_mid(lv, cur, mid, words + 2, words, d, ctx->ds, blocks, ctx->st), "k_expand_mid");
+            ctx->launches++;
+            dfree(ctx, words);
+            check_device_status(ctx, read_status(ctx, &st, d, sizeof(st)));
+            if (st.which < 2) {
+                dfree(ctx, own);
+                own = mid;
+                cur = mid + st.which * kExpandMid;
+            } else {
+                dfree(ctx, mid);
+            }
+        }
     } else {
         u32 r = 0;
         ck(ctx, cudaMemcpyAsync(&st.level, G->c_level + j, 4, cudaMemcpyDeviceToHost, ctx->st), "read C");
         ck(ctx, cudaMemcpyAsync(&r, G->c_rank + j, 4, cudaMemcpyDeviceToHost, ctx->st), "read C");
-        cur = dalloc<u32>(ctx, 1);
+        own = cur = dalloc<u32>(ctx, 1);
         ck(ctx, cudaMemcpyAsync(cur, G->c_rank + j, 4, cudaMemcpyDeviceToDevice, ctx->st), "copy");
         sync(ctx);
         if (st.level == 0 && cap >= 1) {
@@ -2061,7 +2079,7 @@ void decompress(lcg_ctx* ctx, const lcg_grammar* G, u32 j, uint8_t* out, u64 cap
     u64 cnt = st.count;
     auto too_small = [&] {
         *out_len = cnt;
-        dfree(ctx, cur);
+        dfree(ctx, own);
         dfree(ctx, tmp);
         sync(ctx);
         fail_if(ctx, true, LCG_EINVAL, "output buffer too small");
@@ -2111,14 +2129,14 @@ void decompress(lcg_ctx* ctx, const lcg_grammar* G, u32 j, uint8_t* out, u64 cap
         ctx->launches += 3;
         dfree(ctx, sums);
         dfree(ctx, places);
-        dfree(ctx, cur);
-        cur = next;
+        dfree(ctx, own);
+        own = cur = next;
         cnt = total;
     }
     *out_len = cnt;
     if (!on_dev) ck(ctx, cudaMemcpyAsync(out, tmp, cnt, cudaMemcpyDeviceToHost, ctx->st), "copy out");
     dfree(ctx, tmp);
-    dfree(ctx, cur);
+    dfree(ctx, own);
     if (st.level != 0 || !on_dev) sync(ctx);
 }
 

@@ -245,7 +245,7 @@ struct MergeSmall {
     MergeLevel lv[kMergeSmallLevels];  // (no miss, mlen, xrank, xlen)
     MergeOld old[kMergeSmallLevels];
 };
-u32 merge_small_blocks();
+u32 coop_blocks();  // of a cooperative launch: one per SM
 cudaError_t launch_merge_small(const MergeSmall& a, u32 blocks, cudaStream_t st);
 // A level of an imported grammar, blocks of 256 rules from block blk0 on.
 struct FpLevel {
@@ -283,10 +283,15 @@ struct ExpandLevels {
 struct ExpandState {
     u64 count;  // symbols of level `level` (the string's bytes when it is 0)
     u32 level;
-    u32 pad;
+    u32 which;  // k_expand_mid: the half of its buffer that holds them (2: none)
 };
 cudaError_t launch_expand_small(const ExpandLevels& lv, const u32* c_level, const u32* c_rank, u32 j,
                                 unsigned char* out, u64 cap, u32* rest, ExpandState* state, cudaStream_t st);
+constexpr u64 kExpandMid = 1u << 20;  // symbols of a level, at most, while one launch expands
+// Needs 2 kExpandMid symbols at `mid`, `blocks` (coop_blocks()) words at `counts` and
+// two zeroed words at `bar`.
+cudaError_t launch_expand_mid(const ExpandLevels& lv, const u32* first, u32* mid, u64* counts, u64* bar,
+                              ExpandState* state, DevStatus* ds, u32 blocks, cudaStream_t st);
 u64 expand_tiles_for(u64 cnt);
 cudaError_t launch_expand_count(const u32* cur, u64 cnt, const u64* off, u32* lo, u32* hi, cudaStream_t st);
 cudaError_t launch_expand_tiles(const u32* cur, u64 cnt, const u64* off, const u32* rhs, const u8* packed,

@@ -51,3 +51,6 @@ def test_forms(hf, n, k, kind):
         ctx.build_into(h, coll.data, coll.offsets)
         assert h.export()["c_rank"].size == 3 * k
         assert all(np.array_equal(x["rhs"], y["rhs"]) for x, y in zip(h.export()["levels"], want["levels"]))
+        h.free()
+    g.free()
+    ctx.close()
