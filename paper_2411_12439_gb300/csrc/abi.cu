@@ -514,6 +514,7 @@ struct RoundInput {
     const u32* Sf;
     int symb;
     u64 n;          // |T^i| (host value when known)
+    u64 n_cap;      // symbols that the buffers S and Sf hold
     u32 kk;         // active strings (host value when known)
     u64* soff;
     u32* sid;
@@ -669,6 +670,7 @@ RoundArgs round_args(lcg_ctx* ctx, lcg_grammar* R, const RoundInput& in, RoundBu
     a.Sf = in.Sf;
     a.n = in.n;
     a.d_n = in.d_n;
+    a.n_cap = in.n_cap;
     a.soff = in.soff;
     a.sid = in.sid;
     a.k = in.kk;
@@ -813,6 +815,7 @@ void next_input(lcg_ctx* ctx, RoundInput& in, RoundBufs& b) {
     in.S = b.Tnext;
     in.S_owned = b.Tnext;
     in.Sf = b.Fnext;
+    in.n_cap = b.Tcap;
     in.symb = 4;
     in.soff = b.soff_next;
     in.sid = b.sid_next;
@@ -941,6 +944,7 @@ u32 tail_enqueue(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, u64 n_boun
         a.Sf = r == 0 ? in.Sf : (u32*)(b2 + z[r - 1].F);
         a.n = r == 0 ? in.n : 0;
         a.d_n = r == 0 ? in.d_n : &ctx->rc_arr[lev - 2].n_next;
+        a.n_cap = r == 0 ? in.n_cap : z[r - 1].P;
         a.soff = r == 0 ? in.soff : (u64*)(b2 + z[r - 1].soff);
         a.sid = r == 0 ? in.sid : (u32*)(b2 + z[r - 1].sid);
         a.k = r == 0 ? in.kk : 0;
@@ -1567,7 +1571,7 @@ void capture_graph(lcg_ctx* ctx, const unsigned char* d_in, const std::vector<u6
         RoundInput in{};
         in.S = d_in;
         in.symb = 1;
-        in.n = gb->n1;
+        in.n = in.n_cap = gb->n1;
         in.kk = k;
         in.soff = gb->soff;
         in.sid = gb->sid;
@@ -1755,7 +1759,7 @@ void build_into(lcg_ctx* ctx, lcg_grammar* R, const uint8_t* data, const uint64_
     in.S_owned = S_owned;
     in.Sf = nullptr;
     in.symb = 1;
-    in.n = n1;
+    in.n = in.n_cap = n1;
     in.kk = kk;
     in.soff = d_soff;
     in.sid = d_sid;

@@ -80,6 +80,7 @@ struct RoundArgs {
     const u32* Sf;        // fingerprints of T^i (rounds >= 2)
     u64 n;                // |T^i| (when d_n is null)
     const u64* d_n;       // |T^i| on the device (rounds enqueued without a host sync), or null
+    u64 n_cap;            // symbols that S (and Sf) hold: past a plan that was outgrown *d_n is more
     const u64* soff;      // k+1 string offsets into T^i
     const u32* sid;       // original string index of each active string
     u32 k;                // active strings (when d_k is null)

@@ -865,7 +865,11 @@ __device__ __forceinline__ void body_parse(const RoundArgs& a, u64 nunits) {
     typename Smem::Warp& w = sm.w[warp];
 
     const T* S = (const T*)a.S;
-    const u64 n = round_n(a);
+    // After a planned round that outgrew its next sequence *d_n is the number of
+    // symbols that there should have been.  Such a round is halted, but the first unit
+    // is fetched before its status is known, so all that is read lies within the
+    // buffers whatever the status.
+    const u64 n = min(round_n(a), min(a.n_cap, nunits * (u64)U));
     const u64 nwords = (n + 31) / 32;  // words of the break bitmap
     nunits = min(nunits, (n + U - 1) / U);
     const u64 nr = a.rc->retired;
@@ -1568,7 +1572,7 @@ __device__ __noinline__ void solo_rounds(const TailArgs& t, u32 r) {
         const RoundArgs& a = t.r[r];
         n = (u32)round_n(a);
         k = round_k(a);
-        if (n > a.tiles_bound * a.tp || k > (u32)kSoloStrings) {  // more than the buffers were sized for
+        if (n > min(a.n_cap, a.tiles_bound * a.tp) || k > (u32)kSoloStrings) {  // more than the buffers were sized for
             if (tid == 0) set_error(a.ds, kErrCapacity);
             return;
         }

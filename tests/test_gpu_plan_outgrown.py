@@ -1,0 +1,55 @@
+"""Builds whose planned rounds get fewer places for the next sequence than the strings
+need: a context that has seen runs only is given as many bytes of a periodic string,
+which has many phrases but few different ones, so no table overflows and it is the
+sequence that outgrows its plan.  The build is redone round by round and equals the
+oracle's, with the round after it an ordinary or a short one, as launches and as a
+graph."""
+import numpy as np
+import pytest
+
+import lcg_inputs as li
+from oracle import oracle as O
+
+pytestmark = pytest.mark.gpu
+
+
+def _runs(n, phrases, k):
+    """k strings of n bytes in all with about `phrases` phrases."""
+    x = np.full(n, ord("N"), dtype=np.uint8)
+    x[:4 * phrases] = np.resize(np.frombuffer(b"ACGT", dtype=np.uint8), 4 * phrases)
+    return li.from_strings(np.array_split(x, k))
+
+
+def _periodic(n, k):
+    return li.from_strings(np.array_split(np.resize(np.frombuffer(b"ACGT", dtype=np.uint8), n), k))
+
+
+# (bytes, phrases of the strings that the plan is made from): the next round is planned
+# as a short one of some 4 k, 70 k or 150 k symbols, or as an ordinary one of some 700 k
+SIZES = [(530_001, 100), (900_001, 60_000), (1_500_007, 130_000), (6_000_011, 600_000)]
+
+
+@pytest.mark.parametrize("n,phrases", SIZES)
+@pytest.mark.parametrize("k", [1, 7])
+@pytest.mark.parametrize("graph", [False, True])
+def test_next_sequence_outgrows_its_plan(hf, n, phrases, k, graph):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2411_12439_gb300 import Context
+    few, many = _runs(n, phrases, k), _periodic(n, k)
+    want = O.build(many, hf).export()
+    ctx = Context(hf, device=0)
+    ctx.set_graph(graph)
+    buf = torch.from_numpy(few.data.copy()).cuda()
+    plan = ctx.build(buf, few.offsets)
+    assert not ctx.last_build_stats()["redone"]
+    plan.free()
+    buf.copy_(torch.from_numpy(many.data))
+    torch.cuda.synchronize()
+    g = ctx.build(buf, many.offsets)
+    st = ctx.last_build_stats()
+    assert st["redone"], st
+    assert all(r["retries"] == 0 for r in st["per_round"]), st  # no table was too small
+    assert O.grammars_equal(g.export(), want)
+    g.free()
