@@ -2589,6 +2589,7 @@ int lcg_set_graph(lcg_ctx* ctx, int enable) {
 
 int lcg_set_tuning(lcg_ctx* ctx, const lcg_tuning* t) {
     if (!ctx || !t) return LCG_EINVAL;
+    if (cudaSetDevice(ctx->device) != cudaSuccess) return LCG_EDEVICE;  // whose blocks per SM are asked for
     const int maxb = std::max(parse_max_blocks(1), parse_max_blocks(4));
     if (!(t->table_load >= 0.3 && t->table_load <= 0.78) || t->parse_blocks_per_sm > (uint32_t)maxb ||
         t->miss_flush < 32 || t->miss_flush > 256 || (t->table_slots_max != 0 && t->table_slots_max < 1024) ||

@@ -2,6 +2,7 @@
 // expansion exp(C[j]) (Sec. 2.2), and a generic two-column exclusive scan.
 #include "lcg_dev.cuh"
 #include "lcg_internal.h"
+#include "per_device.h"
 #include "table.cuh"
 
 namespace lcg {
@@ -907,9 +908,17 @@ __global__ void __launch_bounds__(kEtThreads, 4) k_expand_tiles(const u32* __res
 
 cudaError_t launch_expand_small(const ExpandLevels& lv, const u32* c_level, const u32* c_rank, u32 j,
                                 unsigned char* out, u64 cap, u32* rest, ExpandState* state, cudaStream_t st) {
-    static const cudaError_t attr = cudaFuncSetAttribute(k_expand_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                         (int)sizeof(ExpandSmem));
-    if (attr != cudaSuccess) return attr;
+    static PerDevice<bool> raised;  // (the limit of dynamic shared memory is each device's own)
+    int dev = 0;
+    bool set = false;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess)
+        e = raised.get(dev, set, [](bool& b) {
+            b = true;
+            return cudaFuncSetAttribute(k_expand_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)sizeof(ExpandSmem));
+        });
+    if (e != cudaSuccess) return e;
     k_expand_small<<<1, kExpThreads, sizeof(ExpandSmem), st>>>(lv, c_level, c_rank, j, out, cap, rest, state);
     return cudaGetLastError();
 }

@@ -41,6 +41,7 @@
 
 #include "lcg_dev.cuh"
 #include "lcg_internal.h"
+#include "per_device.h"
 #include "table.cuh"
 
 namespace lcg {
@@ -1975,65 +1976,79 @@ cudaError_t launch_tile_strings(const RoundArgs& a, cudaStream_t st) {
     return launch_pdl(k_tile_strings, grid_for(a.tiles_bound), 256, st, a, a.tiles_bound);
 }
 
+// What the current device can hold of a kernel with `smem` bytes of dynamic shared
+// memory, whose limit is raised there (CUDA keeps it per device).
+struct Fit {
+    int per_sm = 0;  // resident blocks of an SM
+    int sms = 0;
+};
+template <typename Kernel>
+static cudaError_t fit_of(PerDevice<Fit>& known, Kernel* kernel, int threads, size_t smem, Fit& out) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    return known.get(dev, out, [&](Fit& f) {
+        cudaError_t err = cudaDeviceGetAttribute(&f.sms, cudaDevAttrMultiProcessorCount, dev);
+        if (err == cudaSuccess && smem > 0)
+            err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (err == cudaSuccess)
+            err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&f.per_sm, kernel, threads, smem);
+        if (err == cudaSuccess && (f.per_sm < 1 || f.sms < 1)) err = cudaErrorInvalidConfiguration;
+        return err;
+    });
+}
+
 template <typename T, int U>
-static int parse_occupancy(int* sms_out) {
-    // queried once per instantiation (thread-safe static initialisation:
-    // contexts on several host threads launch at once)
-    static const std::pair<int, int> occ_sms = [] {
-        int dev = 0, sms = 0, occ = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        constexpr int smem = (int)sizeof(ParseSmem<T, U, parse_warps<T>>);
-        cudaFuncSetAttribute(k_parse<T, U>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_parse<T, U>, 32 * parse_warps<T>, smem);
-        return std::make_pair(occ > 0 ? occ : 1, sms);
-    }();
-    if (sms_out) *sms_out = occ_sms.second;
-    return occ_sms.first;
+static cudaError_t parse_fit(Fit& out) {
+    static PerDevice<Fit> known;
+    return fit_of(known, k_parse<T, U>, 32 * parse_warps<T>, sizeof(ParseSmem<T, U, parse_warps<T>>), out);
 }
 
 // Persistent grid: `per_sm` blocks per SM (0 or more than fit: as many as fit).
-template <typename T, int U>
-static unsigned persistent_grid(u64 units, u32 per_sm) {
-    int sms = 0;
-    const int occ = parse_occupancy<T, U>(&sms);
-    const u64 b = (per_sm == 0 || per_sm > (u32)occ) ? (u64)occ : (u64)per_sm;
-    const u64 g = b * (u64)sms, most = (units + parse_warps<T> - 1) / parse_warps<T>;
+template <typename T>
+static unsigned persistent_grid(const Fit& fit, u64 units, u32 per_sm) {
+    const u64 b = (per_sm == 0 || per_sm > (u32)fit.per_sm) ? (u64)fit.per_sm : (u64)per_sm;
+    const u64 g = b * (u64)fit.sms, most = (units + parse_warps<T> - 1) / parse_warps<T>;
     return (unsigned)(most < g ? (most ? most : 1) : g);
 }
 
-// Most k_parse blocks that fit on an SM, over every unit size.
+// Most k_parse blocks that fit on an SM of the current device, over every unit size
+// (at least 1).
+template <typename T>
+static int parse_max_blocks_t() {
+    int most = 1;
+    for (auto fit : {parse_fit<T, 128>, parse_fit<T, 256>, parse_fit<T, 512>}) {
+        Fit f;
+        if (fit(f) == cudaSuccess) most = std::max(most, f.per_sm);
+    }
+    return most;
+}
 int parse_max_blocks(int sym_bytes) {
-    if (sym_bytes == 1)
-        return std::max({parse_occupancy<unsigned char, 128>(nullptr), parse_occupancy<unsigned char, 256>(nullptr),
-                         parse_occupancy<unsigned char, 512>(nullptr)});
-    return std::max({parse_occupancy<u32, 128>(nullptr), parse_occupancy<u32, 256>(nullptr),
-                     parse_occupancy<u32, 512>(nullptr)});
+    return sym_bytes == 1 ? parse_max_blocks_t<unsigned char>() : parse_max_blocks_t<u32>();
 }
 
 template <typename T>
-static unsigned breaks_grid(u64 blocks) {
-    static const u64 cap = [] {
-        int dev = 0, sms = 0, occ = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_breaks<T>, kBrkThreads, 0);
-        return (u64)(occ > 0 ? occ : 1) * (u64)sms;
-    }();
-    return (unsigned)(blocks < cap ? (blocks ? blocks : 1) : cap);
+static cudaError_t launch_breaks_t(const RoundArgs& a, cudaStream_t st) {
+    static PerDevice<Fit> known;
+    Fit fit;
+    const cudaError_t e = fit_of(known, k_breaks<T>, kBrkThreads, 0, fit);
+    if (e != cudaSuccess) return e;
+    const u64 steps = (a.tiles_bound * (u64)a.tp + kBrkSpan - 1) / kBrkSpan;
+    const u64 blocks = std::max<u64>(1, std::min<u64>(steps, (u64)fit.per_sm * (u64)fit.sms));
+    return launch_pdl(k_breaks<T>, (unsigned)blocks, kBrkThreads, st, a, steps);
 }
 
 cudaError_t launch_breaks(const RoundArgs& a, cudaStream_t st) {
-    const u64 blocks = (a.tiles_bound * (u64)a.tp + kBrkSpan - 1) / kBrkSpan;
-    if (a.sym_bytes == 1)
-        return launch_pdl(k_breaks<unsigned char>, breaks_grid<unsigned char>(blocks), kBrkThreads, st, a, blocks);
-    return launch_pdl(k_breaks<u32>, breaks_grid<u32>(blocks), kBrkThreads, st, a, blocks);
+    return a.sym_bytes == 1 ? launch_breaks_t<unsigned char>(a, st) : launch_breaks_t<u32>(a, st);
 }
 
 template <typename T, int U>
 static cudaError_t launch_parse_tp(const RoundArgs& a, cudaStream_t st) {
     const u64 tiles = a.tiles_bound;
-    return launch_pdl_smem(k_parse<T, U>, persistent_grid<T, U>(tiles, a.parse_blocks), 32 * parse_warps<T>,
+    Fit fit;
+    const cudaError_t e = parse_fit<T, U>(fit);
+    if (e != cudaSuccess) return e;
+    return launch_pdl_smem(k_parse<T, U>, persistent_grid<T>(fit, tiles, a.parse_blocks), 32 * parse_warps<T>,
                            sizeof(ParseSmem<T, U, parse_warps<T>>), st, a, tiles);
 }
 
@@ -2052,29 +2067,30 @@ cudaError_t launch_parse(const RoundArgs& a, cudaStream_t st) {
     return launch_parse_t<u32>(a, st);
 }
 
-// Blocks of the short rounds' launches: a warp per unit, at most one block per
-// SM (and never more than can be resident at once).
-template <bool kByte>
-static u32 tail_grid(u64 units) {
-    using T0 = std::conditional_t<kByte, unsigned char, u32>;
-    constexpr size_t smem = std::max({sizeof(ParseSmem<T0, kUnitMin, kParseWarps>), sizeof(ParseSmem<u32, kUnitMin, kParseWarps>), sizeof(SoloSmem)});
-    static const int cap = [] {
-        int dev = 0, sms = 0, o1 = 0, o2 = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaFuncSetAttribute(k_parse_small<kByte>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o1, k_parse_small<kByte>, kSmallThreads, smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o2, k_naming_small<kByte>, kSmallThreads, 0);
-        return (std::min(o1, o2) >= 1 && sms > 0) ? sms : 1;  // (a cooperative launch checks that they fit)
-    }();
-    return (u32)std::min<u64>((u64)cap, std::max<u64>(1, (units + kWarps - 1) / kWarps));
+// Blocks of the short rounds' launches: a warp per unit, at most one block per SM (all
+// of them resident at once: one fits an SM).
+static u32 tail_grid(const Fit& fit, u64 units) {
+    return (u32)std::min<u64>((u64)fit.sms, std::max<u64>(1, (units + kWarps - 1) / kWarps));
 }
 
 template <bool kByte>
 static cudaError_t launch_parse_small_t(const TailArgs& t, cudaStream_t st) {
     using T0 = std::conditional_t<kByte, unsigned char, u32>;
     constexpr size_t smem = std::max({sizeof(ParseSmem<T0, kUnitMin, kParseWarps>), sizeof(ParseSmem<u32, kUnitMin, kParseWarps>), sizeof(SoloSmem)});
-    return launch_coop(k_parse_small<kByte>, tail_grid<kByte>(t.r[0].tiles_bound), kSmallThreads, smem, st, t);
+    static PerDevice<Fit> known;
+    Fit fit;
+    const cudaError_t e = fit_of(known, k_parse_small<kByte>, kSmallThreads, smem, fit);
+    if (e != cudaSuccess) return e;
+    return launch_coop(k_parse_small<kByte>, tail_grid(fit, t.r[0].tiles_bound), kSmallThreads, smem, st, t);
+}
+
+template <bool kByte>
+static cudaError_t launch_naming_small_t(const TailArgs& t, cudaStream_t st) {
+    static PerDevice<Fit> known;
+    Fit fit;
+    const cudaError_t e = fit_of(known, k_naming_small<kByte>, kSmallThreads, 0, fit);
+    if (e != cudaSuccess) return e;
+    return launch_coop(k_naming_small<kByte>, tail_grid(fit, t.r[0].tiles_bound), kSmallThreads, 0, st, t);
 }
 
 cudaError_t launch_parse_small(const TailArgs& t, cudaStream_t st) {
@@ -2082,10 +2098,7 @@ cudaError_t launch_parse_small(const TailArgs& t, cudaStream_t st) {
 }
 
 cudaError_t launch_naming_small(const TailArgs& t, cudaStream_t st) {
-    const u64 units = t.r[0].tiles_bound;
-    if (t.r[0].sym_bytes == 1)
-        return launch_coop(k_naming_small<true>, tail_grid<true>(units), kSmallThreads, 0, st, t);
-    return launch_coop(k_naming_small<false>, tail_grid<false>(units), kSmallThreads, 0, st, t);
+    return t.r[0].sym_bytes == 1 ? launch_naming_small_t<true>(t, st) : launch_naming_small_t<false>(t, st);
 }
 
 u64 rule_chunks(u64 g) { return (g + kRuleChunk - 1) / kRuleChunk; }
