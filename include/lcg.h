@@ -215,6 +215,11 @@ int lcg_last_kernel_launches(const lcg_ctx* ctx, lcg_kernel_launch* out, uint32_
  * before (look-back slots carry a launch epoch).  Any other return value means
  * the bounded wait is broken. */
 int lcg_selftest_wait_timeout(lcg_ctx* ctx);
+/* Self-test of the launches whose blocks wait for one another (short rounds,
+ * small levels of a merge, middle levels of an expansion): later calls of the
+ * context give them at most `most` blocks (0, the default: one per SM), as a
+ * device of as many SMs would.  Results do not depend on it. */
+int lcg_selftest_blocks(lcg_ctx* ctx, uint32_t most);
 
 /* BuildGram(T, H) (Sec. 3.3).
  * data: the k strings concatenated (uint8), `data_on_device` = 1 when it is a

@@ -67,6 +67,7 @@ struct lcg_ctx {
     // table load, k_parse blocks per SM, miss flush, slots cap, stripes, parse tile
     lcg_tuning tuning{0.35, 0, 64, 0, 1, 4096, 16};
     bool own_stream = false;
+    u32 blocks_max = 0;  // of cooperative launches (lcg_selftest_blocks), 0: one per SM
     std::vector<u64> a, b, c;
     u32 levels = 0, m_bits = 32;
     u64 mmask = 0xffffffffull;
@@ -148,6 +149,11 @@ T* dalloc(lcg_ctx* ctx, u64 count) {
 
 void dfree(lcg_ctx* ctx, void* p) {
     if (p) cudaFreeAsync(p, ctx->st);
+}
+
+// Blocks of a cooperative launch: one per SM.
+u32 coop_blocks(const lcg_ctx* ctx) {
+    return ctx->blocks_max ? std::min(ctx->blocks_max, (u32)ctx->sms) : (u32)ctx->sms;
 }
 
 void sync(lcg_ctx* ctx) { ck(ctx, cudaStreamSynchronize(ctx->st), "stream synchronize"); }
@@ -1023,11 +1029,11 @@ u32 tail_enqueue(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, u64 n_boun
     }
     const Range range("short rounds from", i);
     int h = kt_begin(ctx, "k_parse_small", 5.0 * (double)n_bound, i);
-    ck(ctx, launch_parse_small(t, ctx->st), "k_parse_small");
+    ck(ctx, launch_parse_small(t, ctx->blocks_max, ctx->st), "k_parse_small");
     kt_end(ctx, h);
     kt_parts(ctx, h, rounds - 1);
     h = kt_begin(ctx, "k_naming_small", 12.0 * (double)n_bound, i);
-    ck(ctx, launch_naming_small(t, ctx->st), "k_naming_small");
+    ck(ctx, launch_naming_small(t, ctx->blocks_max, ctx->st), "k_naming_small");
     kt_end(ctx, h);
     ctx->launches += 2;
     free_round_input(ctx, in);
@@ -1801,7 +1807,7 @@ constexpr u64 kMergeAheadRules = 1ull << 20, kMergeAheadSymbols = 1ull << 21;
 void merge_small(lcg_ctx* ctx, lcg_grammar* A, const lcg_grammar* B, u32 i0, const u32* Mprev, u64* bar, u64* d_tot,
                  u32* cb_rank, std::vector<void*>& temps) {
     const u32 nb = (u32)B->lv.size();
-    const u32 blocks = coop_blocks();
+    const u32 blocks = coop_blocks(ctx);
     MergeSmall a{};
     a.bar = bar;
     Parts tmp, grown;
@@ -2056,7 +2062,7 @@ void decompress(lcg_ctx* ctx, const lcg_grammar* G, u32 j, uint8_t* out, u64 cap
         fetch(ctx, {{&st, d, sizeof(st)}});
         own = cur;
         if (st.level >= 2) {
-            const u32 blocks = coop_blocks();
+            const u32 blocks = coop_blocks(ctx);
             u64* words = dalloc<u64>(ctx, 2 + blocks);
             u32* mid = dalloc<u32>(ctx, 2 * kExpandMid);
             ck(ctx, cudaMemsetAsync(words, 0, 2 * sizeof(u64), ctx->st), "memset barrier");
@@ -2775,6 +2781,13 @@ int lcg_decompress_static(lcg_ctx* ctx, const lcg_grammar* G, uint32_t j, uint8_
     decompress_static(ctx, G, j, out_dev, cap, out_len);
     return LCG_OK;
     LCG_GUARD_END
+}
+
+int lcg_selftest_blocks(lcg_ctx* ctx, uint32_t most) {
+    if (!ctx) return LCG_EINVAL;
+    ctx->blocks_max = most;
+    destroy_graph(ctx);  // (captured with another number)
+    return LCG_OK;
 }
 
 int lcg_selftest_wait_timeout(lcg_ctx* ctx) {

@@ -547,13 +547,6 @@ cudaError_t launch_merge_lookup(const MergeLevel& m, bool bytes, cudaStream_t st
     return launch_pdl(bytes ? k_merge_lookup<true> : k_merge_lookup<false>, grid_for(m.gb), 256, st, m);
 }
 
-u32 coop_blocks() {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return sms > 0 ? (u32)sms : 1u;
-}
-
 cudaError_t launch_merge_small(const MergeSmall& a, u32 blocks, cudaStream_t st) {
     return launch_coop(k_merge_small, blocks, kMergeSmallThreads, 0, st, a);
 }

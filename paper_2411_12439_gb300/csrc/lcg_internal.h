@@ -171,8 +171,9 @@ struct TailArgs {
     RoundArgs r[kTailRounds];
 };
 static_assert(sizeof(TailArgs) <= 32000, "kernel parameters");
-cudaError_t launch_parse_small(const TailArgs& t, cudaStream_t st);
-cudaError_t launch_naming_small(const TailArgs& t, cudaStream_t st);
+// (`most`: blocks at most, 0 for one per SM)
+cudaError_t launch_parse_small(const TailArgs& t, u32 most, cudaStream_t st);
+cudaError_t launch_naming_small(const TailArgs& t, u32 most, cudaStream_t st);
 u64 rule_chunks(u64 g);  // chunks of g rules
 
 size_t claim_rec_bytes();                       // bytes of one ClaimRec
@@ -246,7 +247,6 @@ struct MergeSmall {
     MergeLevel lv[kMergeSmallLevels];  // (no miss, mlen, xrank, xlen)
     MergeOld old[kMergeSmallLevels];
 };
-u32 coop_blocks();  // of a cooperative launch: one per SM
 cudaError_t launch_merge_small(const MergeSmall& a, u32 blocks, cudaStream_t st);
 // A level of an imported grammar, blocks of 256 rules from block blk0 on.
 struct FpLevel {
@@ -289,7 +289,7 @@ struct ExpandState {
 cudaError_t launch_expand_small(const ExpandLevels& lv, const u32* c_level, const u32* c_rank, u32 j,
                                 unsigned char* out, u64 cap, u32* rest, ExpandState* state, cudaStream_t st);
 constexpr u64 kExpandMid = 1u << 20;  // symbols of a level, at most, while one launch expands
-// Needs 2 kExpandMid symbols at `mid`, `blocks` (coop_blocks()) words at `counts` and
+// Needs 2 kExpandMid symbols at `mid`, `blocks` words at `counts` and
 // two zeroed words at `bar`.
 cudaError_t launch_expand_mid(const ExpandLevels& lv, const u32* first, u32* mid, u64* counts, u64* bar,
                               ExpandState* state, DevStatus* ds, u32 blocks, cudaStream_t st);

@@ -236,8 +236,9 @@ __device__ __forceinline__ u32 spread_down(u32 src, u32 pass) {
 // Kernel bodies are device functions: k_X launches body_X on a grid, and the
 // short rounds' cooperative kernels (k_parse_small, k_naming_small) run several of
 // them in one launch.
-// `own_step`: block b takes step nblocks - 1 - b and no other (a launch whose
-// blocks are all resident, at least as many as steps): no counter.
+// `own_step`: block b takes the steps nblocks - 1 - b, nblocks - 1 - b - gridDim.x, ...
+// (a launch whose blocks are all resident, mostly more than steps): no counter, and the
+// steps after the one that a block waits for are done or another block's, so it ends.
 template <typename T, bool own_step = false>
 __device__ __forceinline__ void body_breaks(const RoundArgs& a, u64 nblocks) {
     pdl_wait();
@@ -275,7 +276,16 @@ __device__ __forceinline__ void body_breaks(const RoundArgs& a, u64 nblocks) {
     // ms, 10.0 without).
     const bool ahead = !kByte && !own_step && nblocks > 4 * (u64)gridDim.x;
     auto step_of = [&](u64 t) { return t < nblocks ? nblocks - 1 - t : ~0ull; };
-    auto ticket = [&]() { return step_of(own_step ? (u64)blockIdx.x : atomicAdd(&a.ds->aux[0], 1ull)); };
+    u64 own = blockIdx.x;
+    auto ticket = [&]() {
+        if constexpr (own_step) {
+            const u64 t = own;
+            own += gridDim.x;
+            return step_of(t);
+        } else {
+            return step_of(atomicAdd(&a.ds->aux[0], 1ull));
+        }
+    };
     // string starts of a step (bitmap of k_tile_strings; n counts as one): this
     // thread's word, and the one past the step
     auto starts = [&](u64 b, u32 w) {
@@ -404,7 +414,7 @@ __device__ __forceinline__ void body_breaks(const RoundArgs& a, u64 nblocks) {
         if ((lane & (int)(lpu - 1)) == 0 && x0 < bend) a.tile_cnt[x0 / a.tp] = ucnt;
         // the first phrase of every string that starts in the step: its index
         // among its unit's phrases
-        if (!own_step && tid == 0) s_step[it & 1] = ahead ? asked : ticket();
+        if (tid == 0) s_step[it & 1] = ahead ? asked : ticket();
         if (__syncthreads_or((int)(st & bits))) {
             u32 pre = (u32)__popc(bits);
 #pragma unroll
@@ -429,7 +439,6 @@ __device__ __forceinline__ void body_breaks(const RoundArgs& a, u64 nblocks) {
                 if (__shfl_sync(0xffffffffu, s < bend ? 1u : 0u, 31) == 0) break;
             }
         }
-        if (own_step) break;
         const u64 fresh = s_step[it & 1];
         if (ahead) {
             b = b_next;
@@ -2069,36 +2078,37 @@ cudaError_t launch_parse(const RoundArgs& a, cudaStream_t st) {
 
 // Blocks of the short rounds' launches: a warp per unit, at most one block per SM (all
 // of them resident at once: one fits an SM).
-static u32 tail_grid(const Fit& fit, u64 units) {
-    return (u32)std::min<u64>((u64)fit.sms, std::max<u64>(1, (units + kWarps - 1) / kWarps));
+static u32 tail_grid(const Fit& fit, u64 units, u32 most) {
+    const u64 blocks = std::min<u64>((u64)fit.sms, std::max<u64>(1, (units + kWarps - 1) / kWarps));
+    return (u32)(most ? std::min<u64>(blocks, most) : blocks);
 }
 
 template <bool kByte>
-static cudaError_t launch_parse_small_t(const TailArgs& t, cudaStream_t st) {
+static cudaError_t launch_parse_small_t(const TailArgs& t, u32 most, cudaStream_t st) {
     using T0 = std::conditional_t<kByte, unsigned char, u32>;
     constexpr size_t smem = std::max({sizeof(ParseSmem<T0, kUnitMin, kParseWarps>), sizeof(ParseSmem<u32, kUnitMin, kParseWarps>), sizeof(SoloSmem)});
     static PerDevice<Fit> known;
     Fit fit;
     const cudaError_t e = fit_of(known, k_parse_small<kByte>, kSmallThreads, smem, fit);
     if (e != cudaSuccess) return e;
-    return launch_coop(k_parse_small<kByte>, tail_grid(fit, t.r[0].tiles_bound), kSmallThreads, smem, st, t);
+    return launch_coop(k_parse_small<kByte>, tail_grid(fit, t.r[0].tiles_bound, most), kSmallThreads, smem, st, t);
 }
 
 template <bool kByte>
-static cudaError_t launch_naming_small_t(const TailArgs& t, cudaStream_t st) {
+static cudaError_t launch_naming_small_t(const TailArgs& t, u32 most, cudaStream_t st) {
     static PerDevice<Fit> known;
     Fit fit;
     const cudaError_t e = fit_of(known, k_naming_small<kByte>, kSmallThreads, 0, fit);
     if (e != cudaSuccess) return e;
-    return launch_coop(k_naming_small<kByte>, tail_grid(fit, t.r[0].tiles_bound), kSmallThreads, 0, st, t);
+    return launch_coop(k_naming_small<kByte>, tail_grid(fit, t.r[0].tiles_bound, most), kSmallThreads, 0, st, t);
 }
 
-cudaError_t launch_parse_small(const TailArgs& t, cudaStream_t st) {
-    return t.r[0].sym_bytes == 1 ? launch_parse_small_t<true>(t, st) : launch_parse_small_t<false>(t, st);
+cudaError_t launch_parse_small(const TailArgs& t, u32 most, cudaStream_t st) {
+    return t.r[0].sym_bytes == 1 ? launch_parse_small_t<true>(t, most, st) : launch_parse_small_t<false>(t, most, st);
 }
 
-cudaError_t launch_naming_small(const TailArgs& t, cudaStream_t st) {
-    return t.r[0].sym_bytes == 1 ? launch_naming_small_t<true>(t, st) : launch_naming_small_t<false>(t, st);
+cudaError_t launch_naming_small(const TailArgs& t, u32 most, cudaStream_t st) {
+    return t.r[0].sym_bytes == 1 ? launch_naming_small_t<true>(t, most, st) : launch_naming_small_t<false>(t, most, st);
 }
 
 u64 rule_chunks(u64 g) { return (g + kRuleChunk - 1) / kRuleChunk; }

@@ -29,7 +29,7 @@ SYMBOLS = [
     "lcg_export_start", "lcg_string_roots", "lcg_import", "lcg_packed_size", "lcg_export_packed", "lcg_import_packed",
     "lcg_grammar_free", "lcg_postprocess", "lcg_pp_stats_of", "lcg_pp_export", "lcg_pp_free",
     "lcg_vbyte_encode", "lcg_vbyte_decode", "lcg_vbyte_size", "lcg_export_vbyte", "lcg_import_vbyte",
-    "lcg_last_kernel_launches", "lcg_selftest_wait_timeout",
+    "lcg_last_kernel_launches", "lcg_selftest_wait_timeout", "lcg_selftest_blocks",
 ]
 
 
@@ -110,6 +110,7 @@ def load(build_if_missing: bool = True):
     lib.lcg_last_kernel_times.argtypes = [P, P, U32, ctypes.POINTER(U32)]
     lib.lcg_last_kernel_launches.argtypes = [P, P, U32, ctypes.POINTER(U32)]
     lib.lcg_selftest_wait_timeout.argtypes = [P]
+    lib.lcg_selftest_blocks.argtypes = [P, U32]
     lib.lcg_build.argtypes = [P, P, P, U32, I, PP]
     lib.lcg_build_into.argtypes = [P, P, P, P, U32, I]
     lib.lcg_merge.argtypes = [P, P, P]
@@ -362,6 +363,11 @@ class Context:
         """lcg_selftest_wait_timeout: the return code (LCG_ETIMEOUT, -6, when
         the bounded wait works)."""
         return int(load().lcg_selftest_wait_timeout(self._h))
+
+    def selftest_blocks(self, most: int) -> None:
+        """lcg_selftest_blocks: at most ``most`` blocks (0: one per SM) in the
+        launches of later calls whose blocks wait for one another."""
+        self._check(load().lcg_selftest_blocks(self._h, int(most)))
 
     def last_build_stats(self) -> dict:
         st = BuildStatsC()
