@@ -137,7 +137,7 @@ __device__ __forceinline__ void for_rules(const u64* off, u64 r_first, u64 r_end
 // H of a rule whose symbol j is get(j), by one thread, four fingerprints in
 // flight at a time.
 template <typename Get>
-__device__ __forceinline__ u64 rule_poly(Get get, u64 len, const u32* __restrict__ F, u64 c) {
+__device__ __forceinline__ u64 rule_poly(Get get, u64 len, const u32* F, u64 c) {
     u64 H = 0;
     for (u64 j = len; j > 0;) {
         u32 f[4];
@@ -155,7 +155,7 @@ __device__ __forceinline__ u64 rule_poly(Get get, u64 len, const u32* __restrict
 // Key of a rule of at most kRuleLong symbols for a table whose values are ranks
 // (see rule_key); H is only computed when the key needs it.
 template <bool kByte, typename Get>
-__device__ __forceinline__ Key128 rank_key(Get get, u64 len, const u32* __restrict__ Fprev, u64 c, u64 rank) {
+__device__ __forceinline__ Key128 rank_key(Get get, u64 len, const u32* Fprev, u64 c, u64 rank) {
     constexpr int w = kByte ? 8 : kRankBits;
     if (len <= inline_max(w)) return key_inline(get, len, w);
     return key_hashed(rule_poly(get, len, Fprev, c), len, rank);

@@ -69,12 +69,22 @@ __device__ bool round_halted(const RoundArgs& a) {
     return s_halt != 0;
 }
 
+// A read of the round's input.  The short rounds' launches (kLive) read what their own
+// earlier steps wrote, for which the non-coherent path is not defined: it is for data
+// that nothing writes while the kernel runs.
+template <bool kLive, typename T>
+__device__ __forceinline__ T ld_in(const T* p) {
+    if constexpr (kLive) return *p;
+    else return __ldg(p);
+}
+
 // index of the string holding position `pos`: largest j with soff[j] <= pos
+template <bool kLive>
 __device__ __forceinline__ u32 string_of(const u64* soff, u32 k, u64 pos) {
     u32 lo = 0, hi = k;  // answer in [lo, hi)
     while (hi - lo > 1) {
         const u32 mid = (lo + hi) >> 1;
-        if (__ldg(soff + mid) <= pos) lo = mid; else hi = mid;
+        if (ld_in<kLive>(soff + mid) <= pos) lo = mid; else hi = mid;
     }
     return lo;
 }
@@ -259,7 +269,7 @@ __device__ __forceinline__ void body_breaks(const RoundArgs& a, u64 nblocks) {
     if constexpr (kByte)
         for (int x = tid; x < 256; x += kBrkThreads) sF0[x] = a.Fprev[x];
     auto fpos = [&](u64 x) -> u32 {  // fingerprint of position x < n
-        if constexpr (kByte) return sF0[S[x]]; else return __ldg(Sf + x);
+        if constexpr (kByte) return sF0[S[x]]; else return ld_in<own_step>(Sf + x);
     };
     const bool aligned = kByte ? (reinterpret_cast<unsigned long long>(S) & 15) == 0
                                : (reinterpret_cast<unsigned long long>(Sf) & 15) == 0;
@@ -290,7 +300,7 @@ __device__ __forceinline__ void body_breaks(const RoundArgs& a, u64 nblocks) {
     // thread's word, and the one past the step
     auto starts = [&](u64 b, u32 w) {
         const u64 gw = b * (kBrkSpan / 32) + (u64)w;
-        return b != ~0ull && gw < a.sbm_words ? __ldg(a.sbm + gw) : 0u;
+        return b != ~0ull && gw < a.sbm_words ? ld_in<own_step>(a.sbm + gw) : 0u;
     };
     if (tid == 0) {
         s_step[0] = ticket();
@@ -428,9 +438,9 @@ __device__ __forceinline__ void body_breaks(const RoundArgs& a, u64 nblocks) {
             __syncthreads();
             const u32 kact = round_k(a);
             // (the rounds of one launch have no table of the steps' strings)
-            const u32 j0 = a.step_str != nullptr ? a.step_str[b] : string_of(a.soff, kact, base);
+            const u32 j0 = a.step_str != nullptr ? a.step_str[b] : string_of<own_step>(a.soff, kact, base);
             for (u32 jj = j0 + (u32)tid;; jj += kBrkThreads) {
-                const u64 s = jj < kact ? __ldg(a.soff + jj) : ~0ull;
+                const u64 s = jj < kact ? ld_in<own_step>(a.soff + jj) : ~0ull;
                 if (s >= base && s < bend) {
                     const u32 x = (u32)(s - base);
                     a.string_first[jj] = s / a.tp * a.tp + s_pre[x >> 5] +
@@ -607,7 +617,7 @@ __device__ __forceinline__ void cache_put(u32 cache, const Key128& key, u32 len,
 // A phrase of more than kLongLen symbols at `pos`, by the whole warp: the
 // fingerprint polynomial H (Eq. fast_hash) and the content comparisons of its
 // hashed key are spread over the lanes.
-template <typename T, int U, int W>
+template <typename T, int U, int W, bool kLive>
 __device__ __noinline__ void parse_long(u64 pos, u64 len, u64 p) {
     ParseSmem<T, U, W>& sm = parse_smem<T, U, W>();
     const RoundArgs& a = *sm.args.all;
@@ -620,7 +630,7 @@ __device__ __noinline__ void parse_long(u64 pos, u64 len, u64 p) {
     }
     const u64 H = warp_poly61([&](u64 j) -> u64 {
         if constexpr (sizeof(T) == 1) return sm.sF[S[pos + j]];
-        else return __ldg(a.Sf + pos + j);
+        else return ld_in<kLive>(a.Sf + pos + j);
     }, len, a.lh.c);
     const u32 F = finish_hash(a.lh, H);
     const Key128 key = key_hashed(H, len, pos);
@@ -653,7 +663,7 @@ __device__ __noinline__ void parse_long(u64 pos, u64 len, u64 p) {
 // The long path on the warp's queued phrases first .. first + take - 1 (at
 // most 32): fingerprint, resident lookup, find or claim, and the symbol of
 // T^{i+1}.  Not inlined, so that the loop over the units keeps its registers.
-template <typename T, int U, int W>
+template <typename T, int U, int W, bool kLive>
 __device__ __noinline__ void parse_queued(u32 first, u32 take) {
     ParseSmem<T, U, W>& sm = parse_smem<T, U, W>();
     const ParseArgs& a = sm.args;
@@ -710,8 +720,8 @@ __device__ __noinline__ void parse_queued(u32 first, u32 take) {
             for (int u = 0; u < 4; u++) {
                 v[u] = f[u] = 0;
                 if ((u32)u < m) {
-                    v[u] = (u32)__ldg(S + pos + j - 1 - u);
-                    f[u] = __ldg(a.Sf + pos + j - 1 - u);
+                    v[u] = (u32)ld_in<kLive>(S + pos + j - 1 - u);
+                    f[u] = ld_in<kLive>(a.Sf + pos + j - 1 - u);
                 }
             }
 #pragma unroll
@@ -860,7 +870,7 @@ __device__ __noinline__ u32 parse_unit_find(u32 buf, u64 t0, u64 p0, u64 out, u3
     return min(q0, cnt) | (nq << 10) | ((longs ? 1u : 0u) << 18);
 }
 
-template <typename T, int U, int W>
+template <typename T, int U, int W, bool kLive = false>
 __device__ __forceinline__ void body_parse(const RoundArgs& a, u64 nunits) {
     pdl_wait();
     using Smem = ParseSmem<T, U, W>;
@@ -915,7 +925,7 @@ __device__ __forceinline__ void body_parse(const RoundArgs& a, u64 nunits) {
                 }
             }
             const u64 gw = f0 / 32 + lane;
-            nx_bits = (lane < kWords + kHalo / 32 && gw < nwords) ? __ldg(a.brk + gw) : 0u;
+            nx_bits = (lane < kWords + kHalo / 32 && gw < nwords) ? ld_in<kLive>(a.brk + gw) : 0u;
             nx_p0 = a.tile_pfx[unit];
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
@@ -1010,7 +1020,7 @@ __device__ __forceinline__ void body_parse(const RoundArgs& a, u64 nunits) {
             else {
                 tail = n - t0;
                 for (u64 gw = t0 / 32 + kWords + 2; gw < nwords; gw += 32) {
-                    const u32 x = gw + lane < nwords ? __ldg(a.brk + gw + lane) : 0u;
+                    const u32 x = gw + lane < nwords ? ld_in<kLive>(a.brk + gw + lane) : 0u;
                     const unsigned m = __ballot_sync(0xffffffffu, x != 0);
                     if (m) {
                         const int l = __ffs(m) - 1;
@@ -1049,7 +1059,7 @@ __device__ __forceinline__ void body_parse(const RoundArgs& a, u64 nunits) {
             if (nq < 32 && (have || nq == 0)) break;  // (the whole unit has been looked at)
             const u32 take = min(nq, 32u);
             nq -= take;
-            parse_queued<T, U, W>(nq, take);
+            parse_queued<T, U, W, kLive>(nq, take);
         }
 
         // 3. long phrases, one at a time by the whole warp
@@ -1060,7 +1070,7 @@ __device__ __forceinline__ void body_parse(const RoundArgs& a, u64 nunits) {
                 for (; m; m &= m - 1) {
                     const u32 x = q0 + (u32)__ffs(m) - 1;
                     const u64 st = w.start[x], en = x + 1 < cnt ? (u64)w.start[x + 1] : tail;
-                    parse_long<T, U, W>(t0 + st, en - st, p0 + x);
+                    parse_long<T, U, W, kLive>(t0 + st, en - st, p0 + x);
                 }
             }
         }
@@ -1090,7 +1100,7 @@ __device__ __forceinline__ void body_tile_strings(const RoundArgs& a, u64 tiles)
     const u64 steps = (min(tiles * a.tp, n) + kBrkSpan - 1) / kBrkSpan;
     if (a.step_str != nullptr)
         for (u64 t = blockIdx.x * (u64)blockDim.x + threadIdx.x; t < steps; t += (u64)gridDim.x * blockDim.x)
-            a.step_str[t] = string_of(a.soff, k, t * kBrkSpan);
+            a.step_str[t] = string_of<false>(a.soff, k, t * kBrkSpan);
     // bitmap of string starts (and of n), zeroed by the host
     for (u64 j = blockIdx.x * (u64)blockDim.x + threadIdx.x; j <= k; j += (u64)gridDim.x * blockDim.x) {
         const u64 s0 = __ldg(a.soff + j);
@@ -1344,16 +1354,16 @@ __global__ void __launch_bounds__(kRoThreads) k_rule_offs(const RoundArgs a) {
 }
 
 // The rank of a symbol of T^i (ids; bytes name themselves).
-template <typename T>
+template <typename T, bool kLive>
 __device__ __forceinline__ u32 sym_rank(const RoundArgs& a, u32 v) {
     if constexpr (sizeof(T) == 1) return v;
-    return v < a.prev_base ? v : __ldg(a.rank_prev + (v - a.prev_base));
+    return v < a.prev_base ? v : ld_in<kLive>(a.rank_prev + (v - a.prev_base));
 }
 
 // The new rules first, first + stride, ... below `end` of this thread (in rank
 // order; a warp's 32 threads take consecutive ones): right-hand sides (ids
 // translated to ranks) and F^i; their offsets are written.
-template <typename T>
+template <typename T, bool kLive = false>
 __device__ __forceinline__ void rules_range(const RoundArgs& a, u64 first, u64 stride, u64 end) {
     const T* S = (const T*)a.S;
     const ContentTable rw{(Slot*)a.rtab_w, a.rtab_w_cap};
@@ -1382,7 +1392,7 @@ __device__ __forceinline__ void rules_range(const RoundArgs& a, u64 first, u64 s
                         v[u] = j + u < len ? (hashed ? (u32)S[k.lo + j + u] : key_sym(k, j + u, a.sym_w)) : 0u;
 #pragma unroll
                     for (int u = 0; u < 4; u++)
-                        if (j + u < len) v[u] = sym_rank<T>(a, v[u]);
+                        if (j + u < len) v[u] = sym_rank<T, kLive>(a, v[u]);
 #pragma unroll
                     for (int u = 0; u < 4; u++)
                         if (j + u < len) a.rhs[off + j + u] = v[u];
@@ -1392,7 +1402,7 @@ __device__ __forceinline__ void rules_range(const RoundArgs& a, u64 first, u64 s
                     const int w = sizeof(T) == 1 ? 8 : kRankBits;
                     u64 H = 0;
                     if (len > inline_max(w))
-                        for (u64 j = len; j-- > 0;) H = addmod61(mulmod61(H, a.lh.c), (u64)__ldg(a.Fprev + get(j)));
+                        for (u64 j = len; j-- > 0;) H = addmod61(mulmod61(H, a.lh.c), (u64)ld_in<kLive>(a.Fprev + get(j)));
                     table_put(rw, rule_key(get, len, w, H, rank), rank, a.ds);
                 }
             }
@@ -1413,14 +1423,14 @@ __device__ __forceinline__ void rules_range(const RoundArgs& a, u64 first, u64 s
                 for (int u = 0; u < 8; u++) v[u] = j0 + 32 * u < len ? (u32)S[k.lo + j0 + 32 * u] : 0u;
 #pragma unroll
                 for (int u = 0; u < 8; u++)
-                    if (j0 + 32 * u < len) v[u] = sym_rank<T>(a, v[u]);
+                    if (j0 + 32 * u < len) v[u] = sym_rank<T, kLive>(a, v[u]);
 #pragma unroll
                 for (int u = 0; u < 8; u++)
                     if (j0 + 32 * u < len) a.rhs[off + j0 + 32 * u] = v[u];
             }
             if (rw.cap) {
                 __syncwarp();
-                const u64 H = warp_poly61([&](u64 j) -> u64 { return __ldg(a.Fprev + a.rhs[off + j]); }, len, a.lh.c);
+                const u64 H = warp_poly61([&](u64 j) -> u64 { return ld_in<kLive>(a.Fprev + a.rhs[off + j]); }, len, a.lh.c);
                 if (lane == 0) table_put(rw, key_hashed(H, len, a.g_base + rr), a.g_base + rr, a.ds);
             }
         }
@@ -1811,8 +1821,9 @@ __device__ __noinline__ void solo_rounds(const TailArgs& t, u32 r) {
 
 // The phrases and the parse of the rounds t.r[0 .. t.rounds), until no string
 // is left.
+// (one block per SM: without the bound the compiler may settle on 80 registers and spill)
 template <bool kByte>
-__global__ void __launch_bounds__(kSmallThreads) k_parse_small(const __grid_constant__ TailArgs t) {
+__global__ void __launch_bounds__(kSmallThreads, 1) k_parse_small(const __grid_constant__ TailArgs t) {
     pdl_wait();
     u64 idx = 0;
     for (u32 r = 0; r < t.rounds; r++) {
@@ -1840,8 +1851,8 @@ __global__ void __launch_bounds__(kSmallThreads) k_parse_small(const __grid_cons
             __syncthreads();
             body_strings(a);
         });
-        if (kByte && r == 0) body_parse<unsigned char, kUnitMin, kParseWarps>(a, a.tiles_bound);
-        else body_parse<u32, kUnitMin, kParseWarps>(a, a.tiles_bound);
+        if (kByte && r == 0) body_parse<unsigned char, kUnitMin, kParseWarps, true>(a, a.tiles_bound);
+        else body_parse<u32, kUnitMin, kParseWarps, true>(a, a.tiles_bound);
         barrier([] {});
     }
 }
@@ -1960,8 +1971,8 @@ __global__ void __launch_bounds__(kSmallThreads) k_naming_small(const __grid_con
                                          [&](u64 x, u64 e) { off[r0 + x] = a.G_base + base + e; });
         if (r1 == s_g[r] && threadIdx.x == 0) off[r1] = a.G_base + base + len;
         __syncthreads();
-        if (kByte && r == 0) rules_range<unsigned char>(a, r0 + threadIdx.x, blockDim.x, r1);
-        else rules_range<u32>(a, r0 + threadIdx.x, blockDim.x, r1);
+        if (kByte && r == 0) rules_range<unsigned char, true>(a, r0 + threadIdx.x, blockDim.x, r1);
+        else rules_range<u32, true>(a, r0 + threadIdx.x, blockDim.x, r1);
         __syncthreads();
     }
 }
