@@ -156,6 +156,32 @@ u32 coop_blocks(const lcg_ctx* ctx) {
     return ctx->blocks_max ? std::min(ctx->blocks_max, (u32)ctx->sms) : (u32)ctx->sms;
 }
 
+// A call's device scratch: freed when the call is done with it (drop), and at its end,
+// also when it fails.
+struct Temps {
+    explicit Temps(lcg_ctx* c) : ctx(c) {}
+    Temps(const Temps&) = delete;
+    Temps& operator=(const Temps&) = delete;
+    ~Temps() {
+        for (void* p : ptrs) dfree(ctx, p);
+    }
+    template <typename T>
+    T* get(u64 n) {
+        ptrs.reserve(ptrs.size() + 1);
+        T* p = dalloc<T>(ctx, n);
+        ptrs.push_back(p);
+        return p;
+    }
+    void drop(void* p) {
+        const auto at = std::find(ptrs.begin(), ptrs.end(), p);
+        if (at == ptrs.end()) return;
+        ptrs.erase(at);
+        dfree(ctx, p);
+    }
+    lcg_ctx* const ctx;
+    std::vector<void*> ptrs;
+};
+
 void sync(lcg_ctx* ctx) { ck(ctx, cudaStreamSynchronize(ctx->st), "stream synchronize"); }
 
 // ---- per-kernel timing: events around each launch when enabled -----------
@@ -2044,6 +2070,7 @@ void decompress(lcg_ctx* ctx, const lcg_grammar* G, u32 j, uint8_t* out, u64 cap
     fail_if(ctx, j >= G->k, LCG_EINVAL, "string index out of range");
     // the upper levels, and the whole of a short string, in one launch
     ExpandState st{1, 0, 0};
+    Temps temps(ctx);
     u32 *cur = nullptr, *own = nullptr;  // the sequence, and the allocation that holds it
     u8* tmp = nullptr;  // bytes for a host buffer
     if (G->lv.size() <= 64) {
@@ -2052,8 +2079,8 @@ void decompress(lcg_ctx* ctx, const lcg_grammar* G, u32 j, uint8_t* out, u64 cap
             lv.off[l] = G->lv[l].rhs_off;
             lv.rhs[l] = G->lv[l].rhs;
         }
-        cur = dalloc<u32>(ctx, kExpandSmall);
-        if (!on_dev) tmp = dalloc<u8>(ctx, kExpandSmallBytes);
+        cur = temps.get<u32>(kExpandSmall);
+        if (!on_dev) tmp = temps.get<u8>(kExpandSmallBytes);
         ExpandState* d = (ExpandState*)(ctx->scratch + 4);
         ck(ctx, launch_expand_small(lv, G->c_level, G->c_rank, j, on_dev ? out : tmp,
                                     on_dev ? cap : std::min<u64>(cap, kExpandSmallBytes), cur, d, ctx->st),
@@ -2061,50 +2088,51 @@ void decompress(lcg_ctx* ctx, const lcg_grammar* G, u32 j, uint8_t* out, u64 cap
         ctx->launches++;
         fetch(ctx, {{&st, d, sizeof(st)}});
         own = cur;
+        // (the launches after it are judged by the status; what an earlier call left there
+        // is not theirs)
+        if (st.level >= 1) reset_status(ctx);
         if (st.level >= 2) {
             const u32 blocks = coop_blocks(ctx);
-            u64* words = dalloc<u64>(ctx, 2 + blocks);
-            u32* mid = dalloc<u32>(ctx, 2 * kExpandMid);
+            u64* words = temps.get<u64>(2 + blocks);
+            u32* mid = temps.get<u32>(2 * kExpandMid);
             ck(ctx, cudaMemsetAsync(words, 0, 2 * sizeof(u64), ctx->st), "memset barrier");
             ck(ctx, launch_expand_mid(lv, cur, mid, words + 2, words, d, ctx->ds, blocks, ctx->st), "k_expand_mid");
             ctx->launches++;
-            dfree(ctx, words);
+            temps.drop(words);
             check_device_status(ctx, read_status(ctx, &st, d, sizeof(st)));
             if (st.which < 2) {
-                dfree(ctx, own);
+                temps.drop(own);
                 own = mid;
                 cur = mid + st.which * kExpandMid;
             } else {
-                dfree(ctx, mid);
+                temps.drop(mid);
             }
         }
     } else {
         u32 r = 0;
         ck(ctx, cudaMemcpyAsync(&st.level, G->c_level + j, 4, cudaMemcpyDeviceToHost, ctx->st), "read C");
         ck(ctx, cudaMemcpyAsync(&r, G->c_rank + j, 4, cudaMemcpyDeviceToHost, ctx->st), "read C");
-        own = cur = dalloc<u32>(ctx, 1);
+        reset_status(ctx);
+        own = cur = temps.get<u32>(1);
         ck(ctx, cudaMemcpyAsync(cur, G->c_rank + j, 4, cudaMemcpyDeviceToDevice, ctx->st), "copy");
         sync(ctx);
         if (st.level == 0 && cap >= 1) {
             const u8 b = (u8)r;
-            if (!on_dev) tmp = dalloc<u8>(ctx, 1);
+            if (!on_dev) tmp = temps.get<u8>(1);
             ck(ctx, cudaMemcpyAsync(on_dev ? out : tmp, &b, 1, cudaMemcpyHostToDevice, ctx->st), "copy");
         }
     }
     u64 cnt = st.count;
     auto too_small = [&] {
         *out_len = cnt;
-        dfree(ctx, own);
-        dfree(ctx, tmp);
-        sync(ctx);
         fail_if(ctx, true, LCG_EINVAL, "output buffer too small");
     };
     if (st.level == 0 && cap < cnt) too_small();
     for (u32 l = st.level; l >= 1; l--) {
         const Level& L = G->lv[l - 1];
         const u64 tiles = expand_tiles_for(cnt);
-        u32* sums = dalloc<u32>(ctx, 2 * tiles);
-        u64* places = dalloc<u64>(ctx, 2 * tiles);
+        u32* sums = temps.get<u32>(2 * tiles);
+        u64* places = temps.get<u64>(2 * tiles);
         ck(ctx, launch_expand_count(cur, cnt, L.rhs_off, sums, sums + tiles, ctx->st), "k_expand_count");
         const u64 stiles = std::max<u64>(1, scan2_tiles_for(tiles));
         ensure_lb(ctx, &ctx->lb2, &ctx->lb2_tiles, stiles, scan2_lb_bytes(stiles));
@@ -2120,38 +2148,31 @@ void decompress(lcg_ctx* ctx, const lcg_grammar* G, u32 j, uint8_t* out, u64 cap
         if (l == 1) {
             if (cap < total) {
                 cnt = total;
-                dfree(ctx, sums);
-                dfree(ctx, places);
                 too_small();
             }
             if (!on_dev) {
-                dfree(ctx, tmp);
-                tmp = dalloc<u8>(ctx, total);
+                temps.drop(tmp);
+                tmp = temps.get<u8>(total);
             }
             bytes = on_dev ? out : tmp;
             // the level's right-hand sides as bytes, when they are read several times
             if (total >= 4 * L.G) {
-                packed = dalloc<u8>(ctx, L.G + 16);
+                packed = temps.get<u8>(L.G + 16);
                 ck(ctx, launch_expand_pack(L.rhs, L.G, packed, ctx->st), "k_expand_pack");
                 ctx->launches++;
             }
         } else {
-            next = dalloc<u32>(ctx, total);
+            next = temps.get<u32>(total);
         }
         ck(ctx, launch_expand_tiles(cur, cnt, L.rhs_off, L.rhs, packed, places, places + tiles, next, bytes, ctx->st),
            "k_expand_tiles");
-        dfree(ctx, packed);
         ctx->launches += 3;
-        dfree(ctx, sums);
-        dfree(ctx, places);
-        dfree(ctx, own);
+        for (void* p : {(void*)packed, (void*)sums, (void*)places, (void*)own}) temps.drop(p);
         own = cur = next;
         cnt = total;
     }
     *out_len = cnt;
     if (!on_dev) ck(ctx, cudaMemcpyAsync(out, tmp, cnt, cudaMemcpyDeviceToHost, ctx->st), "copy out");
-    dfree(ctx, tmp);
-    dfree(ctx, own);
     if (st.level != 0 || !on_dev) sync(ctx);
 }
 
@@ -2201,6 +2222,7 @@ void decompress_static(lcg_ctx* ctx, const lcg_grammar* G, u32 j, uint8_t* out, 
     static_assert(scan2_lb_bytes_static(kStaticLbTiles) <= kStaticLbTiles * 48, "look-back slots");
     fail_if(ctx, j >= G->k, LCG_EINVAL, "string index out of range");
     StaticScratch* sc = static_scratch_of_device(ctx);
+    reset_status(ctx);
     u32 lev = 0, r = 0;
     fetch(ctx, {{&lev, G->c_level + j, 4}, {&r, G->c_rank + j, 4}});
     u32* cur = sc->cur;
@@ -2289,20 +2311,6 @@ std::vector<u64> pp_totals(lcg_ctx* ctx, const u64* d, u64 n) {
     return t;
 }
 
-struct PPTemps {
-    lcg_ctx* ctx;
-    std::vector<void*> ptrs;
-    template <typename T>
-    T* get(u64 n) {
-        T* p = dalloc<T>(ctx, n);
-        ptrs.push_back(p);
-        return p;
-    }
-    ~PPTemps() {
-        for (void* p : ptrs) dfree(ctx, p);
-    }
-};
-
 // Each step runs over all levels before the host waits for what it needs of them:
 // five waits in all.  (Level by level it was three to five waits a level.)
 lcg_pp* postprocess(lcg_ctx* ctx, const lcg_grammar* G) {
@@ -2311,7 +2319,7 @@ lcg_pp* postprocess(lcg_ctx* ctx, const lcg_grammar* G) {
     if (G->owner && G->owner != ctx) ck(ctx, cudaStreamSynchronize(G->owner->st), "grammar's stream");
     sync(ctx);
     reset_status(ctx);
-    PPTemps tmp{ctx, {}};
+    Temps tmp(ctx);
     PPLevels lv{};
     lv.n = nl;
     std::vector<u32*> uses(nl);
