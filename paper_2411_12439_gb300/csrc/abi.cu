@@ -2071,6 +2071,7 @@ void decompress(lcg_ctx* ctx, const lcg_grammar* G, u32 j, uint8_t* out, u64 cap
     // the upper levels, and the whole of a short string, in one launch
     ExpandState st{1, 0, 0};
     Temps temps(ctx);
+    bool waited = false;  // for all that was enqueued
     u32 *cur = nullptr, *own = nullptr;  // the sequence, and the allocation that holds it
     u8* tmp = nullptr;  // bytes for a host buffer
     if (G->lv.size() <= 64) {
@@ -2087,6 +2088,7 @@ void decompress(lcg_ctx* ctx, const lcg_grammar* G, u32 j, uint8_t* out, u64 cap
            "k_expand_small");
         ctx->launches++;
         fetch(ctx, {{&st, d, sizeof(st)}});
+        waited = st.level == 0 && on_dev;  // the whole string, in its place
         own = cur;
         // (the launches after it are judged by the status; what an earlier call left there
         // is not theirs)
@@ -2173,7 +2175,7 @@ void decompress(lcg_ctx* ctx, const lcg_grammar* G, u32 j, uint8_t* out, u64 cap
     }
     *out_len = cnt;
     if (!on_dev) ck(ctx, cudaMemcpyAsync(out, tmp, cnt, cudaMemcpyDeviceToHost, ctx->st), "copy out");
-    if (st.level != 0 || !on_dev) sync(ctx);
+    if (!waited) sync(ctx);
 }
 
 // --------------------------------------------------------------------------

@@ -65,3 +65,40 @@ def test_refused_expansion_returns_its_scratch(built, j):
         with pytest.raises(LCGError):
             g.decompress(j, small)
     assert _pool_used(rt) == used
+
+
+def test_string_of_one_byte_in_a_deep_grammar(hf):
+    """More than 64 levels, and a string that is a byte: in its place when the call is
+    back, for a reader on another stream."""
+    import torch
+    from paper_2411_12439_gb300 import Context
+    family = li.hash_family(levels=80)
+    ctx = Context(family, device=0)
+
+    # level i's only rule is level i - 1's; level 1's is the byte 65
+    levels, below = [], None
+    for i in range(1, 71):
+        below = _fingerprint(family, i, 65 if i == 1 else 0, below)
+        levels.append({"g": 1, "rhs_off": np.array([0, 1], dtype=np.uint64),
+                       "rhs": np.array([65 if i == 1 else 0], dtype=np.uint32),
+                       "F": np.array([below], dtype=np.uint32)})
+    g = ctx.import_grammar({"levels": levels, "c_level": np.array([0, 70], dtype=np.uint32),
+                            "c_rank": np.array([66, 0], dtype=np.uint32)})
+    other = torch.cuda.Stream()
+    for j, byte in ((0, 66), (1, 65)):
+        assert g.decompress(j) == bytes([byte])
+        for _ in range(50):
+            out = torch.zeros(1, dtype=torch.uint8, device="cuda")
+            torch.cuda.synchronize()
+            assert g.decompress(j, out) == 1
+            with torch.cuda.stream(other):
+                assert int(out.item()) == byte
+
+
+def _fingerprint(family, i, symbol, below):
+    """h^i of a rule of one symbol (Eq. fast_hash over the level below)."""
+    p = (1 << 61) - 1
+    a, b = int(family.a[i]), int(family.b[i])
+    if i == 1:
+        below = (int(family.a[0]) * symbol + int(family.b[0])) % p % (1 << int(family.m_bits))
+    return (a * int(below) + b) % p % (1 << int(family.m_bits))
