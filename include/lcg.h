@@ -220,6 +220,10 @@ int lcg_selftest_wait_timeout(lcg_ctx* ctx);
  * context give them at most `most` blocks (0, the default: one per SM), as a
  * device of as many SMs would.  Results do not depend on it. */
 int lcg_selftest_blocks(lcg_ctx* ctx, uint32_t most);
+/* Self-test of what a call leaves behind when device memory runs out: the
+ * nth device allocation of the context from now on (1 = the next) is refused
+ * (0: none), on the host, without asking for memory. */
+int lcg_selftest_alloc_failure(lcg_ctx* ctx, uint64_t nth);
 
 /* BuildGram(T, H) (Sec. 3.3).
  * data: the k strings concatenated (uint8), `data_on_device` = 1 when it is a

@@ -68,6 +68,7 @@ struct lcg_ctx {
     lcg_tuning tuning{0.35, 0, 64, 0, 1, 4096, 16};
     bool own_stream = false;
     u32 blocks_max = 0;  // of cooperative launches (lcg_selftest_blocks), 0: one per SM
+    u64 fail_alloc = 0;  // the allocation from now that fails (lcg_selftest_alloc_failure), 0: none
     std::vector<u64> a, b, c;
     u32 levels = 0, m_bits = 32;
     u64 mmask = 0xffffffffull;
@@ -139,11 +140,16 @@ void ck(lcg_ctx* ctx, cudaError_t e, const char* what) {
     }
 }
 
+cudaError_t alloc_async(lcg_ctx* ctx, void** p, u64 bytes) {
+    if (ctx->fail_alloc && --ctx->fail_alloc == 0) return cudaErrorMemoryAllocation;  // lcg_selftest_alloc_failure
+    return cudaMallocAsync(p, bytes, ctx->st);
+}
+
 template <typename T>
 T* dalloc(lcg_ctx* ctx, u64 count) {
     void* p = nullptr;
     if (count == 0) count = 1;
-    ck(ctx, cudaMallocAsync(&p, count * sizeof(T), ctx->st), "cudaMallocAsync");
+    ck(ctx, alloc_async(ctx, &p, count * sizeof(T)), "cudaMallocAsync");
     return (T*)p;
 }
 
@@ -375,7 +381,9 @@ void ensure_lb(lcg_ctx* ctx, void** lb, u64* have, u64 tiles, size_t bytes) {
     if (*lb && ctx->graph) destroy_graph(ctx);
     if (*lb) dfree(ctx, *lb);
     void* p = nullptr;
-    ck(ctx, cudaMallocAsync(&p, nb, ctx->st), "cudaMallocAsync lb");
+    *have = 0;
+    *lb = nullptr;
+    ck(ctx, alloc_async(ctx, &p, nb), "cudaMallocAsync lb");
     ck(ctx, cudaMemsetAsync(p, 0, nb, ctx->st), "memset lb");
     *lb = p;
     *have = want;
@@ -385,8 +393,9 @@ void ensure_lb(lcg_ctx* ctx, void** lb, u64* have, u64 tiles, size_t bytes) {
 void grow_level(lcg_ctx* ctx, Level& L, u64 need_g, u64 need_G) {
     if (need_g > L.cap_g || L.rhs_off == nullptr) {
         u64 cap = std::max<u64>(need_g, std::max<u64>(L.cap_g * 2, 256));
-        u64* ro = dalloc<u64>(ctx, cap + 1);
-        u32* F = dalloc<u32>(ctx, cap);
+        Temps fresh(ctx);  // (the level has all of its new arrays or none)
+        u64* ro = fresh.get<u64>(cap + 1);
+        u32* F = fresh.get<u32>(cap);
         if (L.rhs_off) {
             ck(ctx, cudaMemcpyAsync(ro, L.rhs_off, (L.g + 1) * sizeof(u64), cudaMemcpyDeviceToDevice, ctx->st), "copy");
             ck(ctx, cudaMemcpyAsync(F, L.F, L.g * sizeof(u32), cudaMemcpyDeviceToDevice, ctx->st), "copy");
@@ -397,6 +406,7 @@ void grow_level(lcg_ctx* ctx, Level& L, u64 need_g, u64 need_G) {
         } else {
             ck(ctx, cudaMemsetAsync(ro, 0, sizeof(u64), ctx->st), "memset");
         }
+        fresh.ptrs.clear();
         L.rhs_off = ro;
         L.F = F;
         L.cap_g = cap;
@@ -413,6 +423,18 @@ void grow_level(lcg_ctx* ctx, Level& L, u64 need_g, u64 need_G) {
         L.cap_G = cap;
         L.shared_rhs = false;
     }
+}
+
+// Drop the grammar's highest level.
+void pop_level(lcg_ctx* ctx, lcg_grammar* G) {
+    Level& L = G->lv.back();
+    if (!L.shared_rules) {
+        dfree(ctx, L.rhs_off);
+        dfree(ctx, L.F);
+    }
+    if (!L.shared_rhs) dfree(ctx, L.rhs);
+    dfree(ctx, L.rtab);
+    G->lv.pop_back();
 }
 
 const u32* fprev_of(const lcg_grammar* G, u32 i) { return i == 1 ? G->F0 : G->lv[i - 2].F; }
@@ -458,14 +480,16 @@ void check_fingerprints(lcg_ctx* ctx, const lcg_grammar* G, std::vector<void*>& 
 void grow_c(lcg_ctx* ctx, lcg_grammar* G, u32 need) {
     if (need <= G->cap_k && G->c_level) return;
     u32 cap = std::max<u32>(need, std::max<u32>(G->cap_k * 2, 16));
-    u32* cl = dalloc<u32>(ctx, cap);
-    u32* cr = dalloc<u32>(ctx, cap);
+    Temps fresh(ctx);
+    u32* cl = fresh.get<u32>(cap);
+    u32* cr = fresh.get<u32>(cap);
     if (G->c_level) {
         ck(ctx, cudaMemcpyAsync(cl, G->c_level, G->k * sizeof(u32), cudaMemcpyDeviceToDevice, ctx->st), "copy");
         ck(ctx, cudaMemcpyAsync(cr, G->c_rank, G->k * sizeof(u32), cudaMemcpyDeviceToDevice, ctx->st), "copy");
         dfree(ctx, G->c_level);
         dfree(ctx, G->c_rank);
     }
+    fresh.ptrs.clear();
     G->c_level = cl;
     G->c_rank = cr;
     G->cap_k = cap;
@@ -1104,16 +1128,7 @@ void tail_sync(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32& i, bool agains
         ctx->stats.rounds = i + r;
     }
     // levels that no round reached
-    while (R->lv.size() > (size_t)(i + r - 1) && R->lv.back().g == 0) {
-        Level& L = R->lv.back();
-        if (!L.shared_rules) {
-            dfree(ctx, L.rhs_off);
-            dfree(ctx, L.F);
-        }
-        if (!L.shared_rhs) dfree(ctx, L.rhs);
-        dfree(ctx, L.rtab);
-        R->lv.pop_back();
-    }
+    while (R->lv.size() > (size_t)(i + r - 1) && R->lv.back().g == 0) pop_level(ctx, R);
     i += r;
     in.kk = k;
     in.n = n;
@@ -1393,15 +1408,8 @@ int rounds_async_finish(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, const Asyn
         if (k_in == 0) { used = r - 1; break; }
     }
     while (R->lv.size() > used && R->lv.back().g == 0 && ar.g_base.size() > R->lv.size()) {
-        Level& L = R->lv.back();
         if (st[R->lv.size() - 1].claims != 0) break;
-        if (!L.shared_rules) {
-            dfree(ctx, L.rhs_off);
-            dfree(ctx, L.F);
-        }
-        if (!L.shared_rhs) dfree(ctx, L.rhs);
-        dfree(ctx, L.rtab);
-        R->lv.pop_back();
+        pop_level(ctx, R);
     }
     u64 n = in.n;
     for (u32 r = 1; r <= used; r++) {
@@ -1843,9 +1851,11 @@ void merge_small(lcg_ctx* ctx, lcg_grammar* A, const lcg_grammar* B, u32 i0, con
     };
     std::vector<At> at;
     const u64 counts = tmp.take(2 * (u64)blocks * sizeof(u64));
-    while (A->lv.size() < nb) A->lv.emplace_back();
+    // all that can fail but the launch itself comes before G_a changes
+    std::vector<Level> lv = A->lv;  // G_a's levels as they will be
+    if (lv.size() < nb) lv.resize(nb);
     for (u32 i = i0 + 1; i <= nb; i++) {
-        const Level &LA = A->lv[i - 1], &LB = B->lv[i - 1];
+        const Level &LA = lv[i - 1], &LB = B->lv[i - 1];
         At x{};
         x.M = tmp.take(LB.g * sizeof(u32));
         x.rules = LA.rhs_off == nullptr || LA.g + LB.g > LA.cap_g;
@@ -1862,26 +1872,14 @@ void merge_small(lcg_ctx* ctx, lcg_grammar* A, const lcg_grammar* B, u32 i0, con
         }
         at.push_back(x);
     }
-    unsigned char* t = dalloc<unsigned char>(ctx, tmp.size);
-    temps.push_back(t);
+    Temps fresh(ctx);  // what the levels get
+    unsigned char* t = fresh.get<unsigned char>(tmp.size);
     a.counts = (u64*)(t + counts);
-    unsigned char* g = nullptr;
-    if (grown.size) {
-        g = dalloc<unsigned char>(ctx, grown.size);
-        A->slabs.push_back(g);
-    }
-    std::vector<void*> tables;
-    try {
-        for (u32 i = i0 + 1; i <= nb; i++)
-            tables.push_back(at[i - i0 - 1].table ? dalloc<unsigned char>(ctx, std::max<u64>(1024, 3 * (A->lv[i - 1].g + B->lv[i - 1].g)) * slot_bytes()) : nullptr);
-    } catch (...) {
-        for (void* p : tables) dfree(ctx, p);
-        throw;
-    }
-    // nothing below fails but the launch itself
-    const u32* F_below = i0 == 0 ? A->F0 : A->lv[i0 - 1].F;
+    unsigned char* g = grown.size ? fresh.get<unsigned char>(grown.size) : nullptr;
+    std::vector<void*> old;  // and what they had
+    const u32* F_below = i0 == 0 ? A->F0 : lv[i0 - 1].F;
     for (u32 i = i0 + 1; i <= nb; i++) {
-        Level& LA = A->lv[i - 1];
+        Level& LA = lv[i - 1];
         const Level& LB = B->lv[i - 1];
         const At& x = at[i - i0 - 1];
         MergeLevel& m = a.lv[a.levels];
@@ -1891,8 +1889,8 @@ void merge_small(lcg_ctx* ctx, lcg_grammar* A, const lcg_grammar* B, u32 i0, con
             o.F = LA.F;
             o.first = LA.rhs_off == nullptr;
             if (LA.rhs_off && !LA.shared_rules) {
-                temps.push_back(LA.rhs_off);
-                temps.push_back(LA.F);
+                old.push_back(LA.rhs_off);
+                old.push_back(LA.F);
             }
             LA.rhs_off = (u64*)(g + x.off);
             LA.F = (u32*)(g + x.F);
@@ -1901,15 +1899,15 @@ void merge_small(lcg_ctx* ctx, lcg_grammar* A, const lcg_grammar* B, u32 i0, con
         }
         if (x.syms) {
             o.rhs = LA.rhs;
-            if (LA.rhs && !LA.shared_rhs) temps.push_back(LA.rhs);
+            if (LA.rhs && !LA.shared_rhs) old.push_back(LA.rhs);
             LA.rhs = (u32*)(g + x.rhs);
             LA.cap_G = x.cap_G;
             LA.shared_rhs = true;
         }
         if (x.table) {
-            dfree(ctx, LA.rtab);
-            LA.rtab = tables[i - i0 - 1];
+            if (LA.rtab) old.push_back(LA.rtab);
             LA.rcap = std::max<u64>(1024, 3 * (LA.g + LB.g));
+            LA.rtab = fresh.get<unsigned char>(LA.rcap * slot_bytes());
             o.fresh = true;
         }
         LA.rvalid = false;
@@ -1938,8 +1936,15 @@ void merge_small(lcg_ctx* ctx, lcg_grammar* A, const lcg_grammar* B, u32 i0, con
         Mprev = m.M;
         F_below = LA.F;
     }
+    temps.reserve(temps.size() + old.size() + 1);
+    A->slabs.reserve(A->slabs.size() + 1);
     ck(ctx, launch_merge_small(a, blocks, ctx->st), "merge levels");
     ctx->launches++;
+    fresh.ptrs.clear();
+    A->lv.swap(lv);
+    if (g) A->slabs.push_back(g);
+    temps.push_back(t);
+    temps.insert(temps.end(), old.begin(), old.end());
 }
 
 // All levels are enqueued before the host waits once, but for a level that is large
@@ -1951,6 +1956,7 @@ void merge(lcg_ctx* ctx, lcg_grammar* A, const lcg_grammar* B) {
     fail_if(ctx, (u64)A->k + B->k > 0xffffffffull, LCG_EOVERFLOW, "too many strings");
     const u32 kb = B->k;
     const u32 nb = (u32)B->lv.size();
+    const size_t na = A->lv.size();
     std::vector<u64> tot(2 * (size_t)nb, 0);
     std::vector<void*> temps;
     auto temp = [&](auto* p) {
@@ -2049,6 +2055,7 @@ void merge(lcg_ctx* ctx, lcg_grammar* A, const lcg_grammar* B) {
         check_device_status(ctx, read_status(ctx, tot.data(), d_tot, tot.size() * 8));
     } catch (...) {
         for (void* p : temps) dfree(ctx, p);
+        while (A->lv.size() > na) pop_level(ctx, A);  // the levels that only G_b has
         throw;
     }
     for (void* p : temps) dfree(ctx, p);
@@ -2800,6 +2807,12 @@ int lcg_selftest_blocks(lcg_ctx* ctx, uint32_t most) {
     return LCG_OK;
 }
 
+int lcg_selftest_alloc_failure(lcg_ctx* ctx, uint64_t nth) {
+    if (!ctx) return LCG_EINVAL;
+    ctx->fail_alloc = nth;
+    return LCG_OK;
+}
+
 int lcg_selftest_wait_timeout(lcg_ctx* ctx) {
     if (!ctx) return LCG_EINVAL;
     LCG_GUARD_BEGIN
@@ -3071,7 +3084,7 @@ int lcg_export_packed(lcg_ctx* ctx, const lcg_grammar* G, void* out, uint64_t ca
         }
         const u64 from = cols[c].pos, bytes = cols[e - 1].pos + cols[e - 1].span - from;
         void* stage = nullptr;
-        if (cudaMallocAsync(&stage, bytes, ctx->st) != cudaSuccess) {  // (the form needs no device memory)
+        if (alloc_async(ctx, &stage, bytes) != cudaSuccess) {  // (the form needs no device memory)
             cudaGetLastError();
             for (; c < e; c++) copy(cols[c]);
             continue;

@@ -30,6 +30,7 @@ SYMBOLS = [
     "lcg_grammar_free", "lcg_postprocess", "lcg_pp_stats_of", "lcg_pp_export", "lcg_pp_free",
     "lcg_vbyte_encode", "lcg_vbyte_decode", "lcg_vbyte_size", "lcg_export_vbyte", "lcg_import_vbyte",
     "lcg_last_kernel_launches", "lcg_selftest_wait_timeout", "lcg_selftest_blocks",
+    "lcg_selftest_alloc_failure",
 ]
 
 
@@ -111,6 +112,7 @@ def load(build_if_missing: bool = True):
     lib.lcg_last_kernel_launches.argtypes = [P, P, U32, ctypes.POINTER(U32)]
     lib.lcg_selftest_wait_timeout.argtypes = [P]
     lib.lcg_selftest_blocks.argtypes = [P, U32]
+    lib.lcg_selftest_alloc_failure.argtypes = [P, U64]
     lib.lcg_build.argtypes = [P, P, P, U32, I, PP]
     lib.lcg_build_into.argtypes = [P, P, P, P, U32, I]
     lib.lcg_merge.argtypes = [P, P, P]
@@ -368,6 +370,11 @@ class Context:
         """lcg_selftest_blocks: at most ``most`` blocks (0: one per SM) in the
         launches of later calls whose blocks wait for one another."""
         self._check(load().lcg_selftest_blocks(self._h, int(most)))
+
+    def selftest_alloc_failure(self, nth: int) -> None:
+        """lcg_selftest_alloc_failure: the ``nth`` device allocation of the
+        context from now on is refused (0: none)."""
+        self._check(load().lcg_selftest_alloc_failure(self._h, int(nth)))
 
     def last_build_stats(self) -> dict:
         st = BuildStatsC()
