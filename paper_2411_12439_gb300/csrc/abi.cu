@@ -2759,7 +2759,24 @@ int lcg_build_into(lcg_ctx* ctx, lcg_grammar* resident, const uint8_t* data, con
     ck(ctx, cudaSetDevice(ctx->device), "cudaSetDevice");
     kt_reset(ctx);
     reset_status(ctx);
-    build_into(ctx, resident, data, offsets, k, data_on_device, true, false);
+    // what the grammar goes back to when the build fails: the rounds that were done have
+    // appended rules, whose places are then free again
+    const u32 k0 = resident->k;
+    std::vector<std::pair<u64, u64>> sizes;
+    for (const Level& L : resident->lv) sizes.emplace_back(L.g, L.G);
+    try {
+        build_into(ctx, resident, data, offsets, k, data_on_device, true, false);
+    } catch (...) {
+        resident->k = k0;
+        while (resident->lv.size() > sizes.size()) pop_level(ctx, resident);
+        for (size_t i = 0; i < sizes.size(); i++) {
+            Level& L = resident->lv[i];
+            L.g = sizes[i].first;
+            L.G = sizes[i].second;
+            L.rvalid = false;  // (the table may hold rules past them)
+        }
+        throw;
+    }
     sync(ctx);
     kt_collect(ctx);
     return LCG_OK;
