@@ -671,13 +671,18 @@ void alloc_round(lcg_ctx* ctx, RoundBufs& b, u64 n_bound, u32 kk, u64 t_cap) {
 // A phrase table of `cap` slots, and numbers for `claims` claims (at most 0.8
 // of the slots: past it the table is too full).  The blocks of the parse take
 // the numbers in ranges (a quarter of the claims that a block makes on
-// average, at least a warp's worth), of which each may leave one unused.
-void alloc_table(lcg_ctx* ctx, RoundBufs& b, u64 cap, u64 claims) {
+// average, at least a warp's worth), of which each may leave all but one
+// unused.  All that may stay unused is a tenth of the slots at most (one number at a
+// time in the smallest tables), so a pass never fills more than 0.9 of them before it
+// runs out of numbers; whether more than 0.8 are full the host sees afterwards
+// (overfull).
+void alloc_table(lcg_ctx* ctx, RoundBufs& b, int sym_bytes, u64 cap, u64 claims) {
     b.cap = cap;
     claims = std::min(claims, cap - cap / 5);
-    const u64 blocks = std::min<u64>((u64)kParseBlocksMax * (u64)ctx->sms, (b.tiles + kParseWarps - 1) / kParseWarps);
-    b.id_chunk = (u32)std::min<u64>(2048, std::max<u64>(32, claims / (4 * std::max<u64>(1, blocks))));
-    b.id_cap = claims + blocks * b.id_chunk;
+    const u64 blocks = parse_blocks_most(sym_bytes, b.tiles, (u64)ctx->sms);
+    const u64 chunk = std::min<u64>(2048, std::max<u64>(32, claims / (4 * blocks)));
+    b.id_chunk = (u32)std::min<u64>(chunk, 1 + cap / 10 / blocks);
+    b.id_cap = claims + blocks * (b.id_chunk - 1);
     b.tab = dalloc<unsigned char>(ctx, cap * slot_bytes());
     b.crec = dalloc<unsigned char>(ctx, b.id_cap * claim_rec_bytes());
     b.minpos = dalloc<u64>(ctx, b.id_cap);
@@ -685,6 +690,10 @@ void alloc_table(lcg_ctx* ctx, RoundBufs& b, u64 cap, u64 claims) {
     ck(ctx, cudaMemsetAsync(b.tab, 0xFF, cap * slot_bytes(), ctx->st), "memset table");
     ck(ctx, cudaMemsetAsync(b.minpos, 0xFF, b.id_cap * sizeof(u64), ctx->st), "memset positions");
 }
+
+// Whether the pass has to be rerun with a larger table: it ran out of numbers or of
+// probes, or left the table past its load limit.
+bool overfull(const DevStatus& st, u64 cap) { return st.overflow != 0 || st.claims > cap - cap / 5; }
 
 void free_table(lcg_ctx* ctx, RoundBufs& b) {
     for (void* p : {(void*)b.tab, (void*)b.crec, (void*)b.minpos, (void*)b.rank_of}) dfree(ctx, p);
@@ -1214,12 +1223,12 @@ void round_sync(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, bool agains
         // (a large table without a hint gets numbers for half its slots: they take
         // more memory than the slots)
         const u64 most = cap <= (1ull << 26) ? cap : std::max<u64>(cap / 2, (u64)g_hint);
-        alloc_table(ctx, b, cap, std::min<u64>(max_ids, most));
+        alloc_table(ctx, b, in.symb, cap, std::min<u64>(max_ids, most));
         set_table(a, b);
         enqueue_parse(ctx, a, n);
         fetch(ctx, {{&rc, a.rc, sizeof(rc)}, {&st, a.ds, sizeof(st)}});
         check_device_status(ctx, st);
-        if (!st.overflow) break;
+        if (!overfull(st, cap)) break;
         free_table(ctx, b);
         fail_if(ctx, b.id_cap >= max_ids, LCG_EOVERFLOW, "level with 2^31 rules or more");
         cap *= 4;
@@ -1361,7 +1370,7 @@ void rounds_async_enqueue(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, AsyncRou
         // (the phrases first: the pool may take a while over the table, the largest
         // allocation, 0.4 ms for 0.5 GB in blocks that it has to piece together)
         enqueue_phrases(ctx, a, p.n_est);
-        alloc_table(ctx, b, p.cap, p.g_alloc);
+        alloc_table(ctx, b, in.symb, p.cap, p.g_alloc);
         set_table(a, b);
         enqueue_parse(ctx, a, p.n_est);
         grow_level(ctx, L, L.g + p.g_alloc, L.G + p.G_alloc);
@@ -1397,7 +1406,7 @@ int rounds_async_finish(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, const Asyn
     fetch(ctx, {{st.data(), ctx->ds_arr, planned * sizeof(DevStatus)},
                 {rc.data(), ctx->rc_arr, planned * sizeof(RoundCounts)}});
     for (u32 r = 0; r < planned; r++) {
-        if (st[r].overflow || st[r].error == kErrCapacity || st[r].error == kErrHalted) return -1;
+        if (overfull(st[r], ar.cap[r + 1]) || st[r].error == kErrCapacity || st[r].error == kErrHalted) return -1;
         check_device_status(ctx, st[r]);
     }
     // rounds past the last active string (the data needed fewer rounds than

@@ -158,6 +158,7 @@ struct RoundArgs {
 constexpr double kL2Bytes = 126.5 * 1024 * 1024;  // GB300 L2 (byte accounting, launch choices)
 bool parse_tile_valid(u32 tp);                 // 1024, 2048 or 4096 positions
 u32 parse_unit(u32 tile);                      // positions that each warp of a block takes of a tile
+u64 parse_blocks_most(int sym_bytes, u64 units, u64 sms);  // blocks of k_parse, at most
 constexpr u32 kParseBlocksMax = 4;             // k_parse blocks per SM at most (its launch bounds)
 constexpr u32 kParseWarps = 8;                 // warps of a block, a unit each
 // The short rounds at a build's end: one launch for their phrases and parses,

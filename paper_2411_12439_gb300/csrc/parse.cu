@@ -2027,9 +2027,16 @@ static cudaError_t parse_fit(Fit& out) {
 // Persistent grid: `per_sm` blocks per SM (0 or more than fit: as many as fit).
 template <typename T>
 static unsigned persistent_grid(const Fit& fit, u64 units, u32 per_sm) {
-    const u64 b = (per_sm == 0 || per_sm > (u32)fit.per_sm) ? (u64)fit.per_sm : (u64)per_sm;
+    const u64 fits = std::min<u64>((u64)fit.per_sm, parse_blocks<parse_warps<T>>);
+    const u64 b = (per_sm == 0 || per_sm > fits) ? fits : (u64)per_sm;
     const u64 g = b * (u64)fit.sms, most = (units + parse_warps<T> - 1) / parse_warps<T>;
     return (unsigned)(most < g ? (most ? most : 1) : g);
+}
+
+u64 parse_blocks_most(int sym_bytes, u64 units, u64 sms) {
+    const u64 warps = sym_bytes == 1 ? parse_warps<unsigned char> : parse_warps<u32>;
+    const u64 per_sm = sym_bytes == 1 ? parse_blocks<parse_warps<unsigned char>> : parse_blocks<parse_warps<u32>>;
+    return std::max<u64>(1, std::min(per_sm * sms, (units + warps - 1) / warps));
 }
 
 // Most k_parse blocks that fit on an SM of the current device, over every unit size

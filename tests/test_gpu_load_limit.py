@@ -1,0 +1,49 @@
+"""A phrase table that a round fills past 0.8 of its slots is regrown, however the claims
+fall on the blocks: rounds with a first table of 1.05 to 1.3 times their new rules, over
+bytes and over ranks, in tables of a few thousand slots and of millions."""
+import numpy as np
+import pytest
+
+import lcg_inputs as li
+from oracle import oracle as O
+
+pytestmark = pytest.mark.gpu
+
+LAST_SHORT = 524_288  # symbols of the largest round among the short ones
+
+
+def _collection(kind):
+    rng = np.random.default_rng(7)
+    if kind == "few":  # a few thousand different phrases
+        return li.from_strings([rng.choice(np.frombuffer(b"ACGTN", dtype=np.uint8), size=1_500_000)])
+    if kind == "text":
+        return li.from_strings([li.zipf_text(rng, 2_000_000), li.zipf_text(rng, 900_000)])
+    return li.from_strings([rng.integers(0, 256, size=6_000_000, dtype=np.uint8)])
+
+
+@pytest.mark.parametrize("kind", ["few", "text", "bytes"])
+@pytest.mark.parametrize("room", [1.05, 1.15, 1.23])
+def test_tables_past_the_limit_are_regrown(hf, kind, room):
+    from paper_2411_12439_gb300 import Context
+    coll = _collection(kind)
+    want = O.build(coll, hf).export()
+    ctx = Context(hf, device=0)
+    ctx.build(coll.data, coll.offsets).free()
+    first = [r["g"] for r in ctx.last_build_stats()["per_round"] if r["n"] > LAST_SHORT]
+    assert first
+    for i, g_i in enumerate(first):
+        slots = int(g_i * room) + 1
+        if slots < 1024:
+            continue
+        for planned in (False, True):
+            ctx = Context(hf, device=0)
+            if planned:
+                ctx.build(coll.data, coll.offsets).free()
+            ctx.set_tuning(table_slots_max=slots)
+            g = ctx.build(coll.data, coll.offsets)
+            rounds = ctx.last_build_stats()["per_round"]
+            assert O.grammars_equal(g.export(), want)
+            assert rounds[i]["retries"] >= 1, (i, slots, rounds[i])
+            for r in rounds:
+                assert r["g"] <= r["table_cap"] - r["table_cap"] // 5, r
+            g.free()
