@@ -675,14 +675,18 @@ void alloc_round(lcg_ctx* ctx, RoundBufs& b, u64 n_bound, u32 kk, u64 t_cap) {
 // unused.  All that may stay unused is a tenth of the slots at most (one number at a
 // time in the smallest tables), so a pass never fills more than 0.9 of them before it
 // runs out of numbers; whether more than 0.8 are full the host sees afterwards
-// (overfull).
-void alloc_table(lcg_ctx* ctx, RoundBufs& b, int sym_bytes, u64 cap, u64 claims) {
+// (overfull).  `most`: ids that follow the resident ones and are below 2^31.
+void alloc_table(lcg_ctx* ctx, RoundBufs& b, int sym_bytes, u64 cap, u64 claims, u64 most) {
     b.cap = cap;
     claims = std::min(claims, cap - cap / 5);
     const u64 blocks = parse_blocks_most(sym_bytes, b.tiles, (u64)ctx->sms);
     const u64 chunk = std::min<u64>(2048, std::max<u64>(32, claims / (4 * blocks)));
     b.id_chunk = (u32)std::min<u64>(chunk, 1 + cap / 10 / blocks);
     b.id_cap = claims + blocks * (b.id_chunk - 1);
+    if (b.id_cap > most) {  // a level near its last rule: no number stays unused
+        b.id_chunk = 1;
+        b.id_cap = std::min(claims, most);
+    }
     b.tab = dalloc<unsigned char>(ctx, cap * slot_bytes());
     b.crec = dalloc<unsigned char>(ctx, b.id_cap * claim_rec_bytes());
     b.minpos = dalloc<u64>(ctx, b.id_cap);
@@ -896,7 +900,11 @@ void next_input(lcg_ctx* ctx, RoundInput& in, RoundBufs& b) {
 
 // (Where the slots of a table are limited the rounds that could need more run one by
 // one: theirs start within the limit.)
-bool is_tail(const lcg_ctx* ctx, u64 n) {
+bool is_tail(const lcg_ctx* ctx, u64 n, const lcg_grammar* resident = nullptr) {
+    // (nor where a level is so full that the numbers a short round takes might not fit)
+    if (resident)
+        for (const Level& L : resident->lv)
+            if (L.g > kMaxRank - 2 * kTailSymbols) return false;
     const u64 most = ctx->tuning.table_slots_max;
     return n <= kTailSymbols && round_tile(ctx, n) == 1024 && (most == 0 || 3 * n <= most);
 }
@@ -1197,11 +1205,11 @@ void round_sync(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, bool agains
     }
     if (ctx->tuning.table_slots_max) cap = std::min<u64>(cap, ctx->tuning.table_slots_max);
     // the claims' ids follow the resident ranks and are below 2^31; the claims
-    // that the table is expected to see, with slack (a round past them is rerun
-    // with a larger table)
-    const u64 max_ids = (kMaxRank + 1 - id_base) / 5 * 4;
+    // that the table is expected to see, with slack
+    const u64 max_ids = kMaxRank + 1 - id_base;
     const double g_hint = hint * ctx->p_hint[std::min<u32>(i, 63)] * (double)n * 1.5 + 1024;
     u32 retries = 0;
+    bool all = false;  // numbers for all the claims that the table may hold
     DevStatus st;
     RoundCounts rc;
     ck(ctx, cudaMemsetAsync(a.ds, 0, sizeof(DevStatus), ctx->st), "reset counters");
@@ -1222,16 +1230,20 @@ void round_sync(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, bool agains
         fail_if(ctx, cap > kMaxRank + 1, LCG_ETABLE, "phrase table would exceed 2^31 slots");
         // (a large table without a hint gets numbers for half its slots: they take
         // more memory than the slots)
-        const u64 most = cap <= (1ull << 26) ? cap : std::max<u64>(cap / 2, (u64)g_hint);
-        alloc_table(ctx, b, in.symb, cap, std::min<u64>(max_ids, most));
+        const u64 most = all || cap <= (1ull << 26) ? cap : std::max<u64>(cap / 2, (u64)g_hint);
+        alloc_table(ctx, b, in.symb, cap, most, max_ids);
         set_table(a, b);
         enqueue_parse(ctx, a, n);
         fetch(ctx, {{&rc, a.rc, sizeof(rc)}, {&st, a.ds, sizeof(st)}});
         check_device_status(ctx, st);
         if (!overfull(st, cap)) break;
         free_table(ctx, b);
-        fail_if(ctx, b.id_cap >= max_ids, LCG_EOVERFLOW, "level with 2^31 rules or more");
-        cap *= 4;
+        const bool ran_out = st.aux[1] >= b.id_cap;  // of numbers
+        fail_if(ctx, ran_out && b.id_cap >= max_ids, LCG_EOVERFLOW, "level with 2^31 rules or more");
+        // a table with more room than numbers is tried with all of them first: the next
+        // larger one may be one too large (2^31 slots)
+        all = ran_out && b.id_cap < cap - cap / 5 && !all;
+        if (!all) cap *= 4;
         retries++;
         ck(ctx, cudaMemsetAsync(a.ds, 0, sizeof(DevStatus), ctx->st), "reset counters");
     }
@@ -1370,7 +1382,7 @@ void rounds_async_enqueue(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, AsyncRou
         // (the phrases first: the pool may take a while over the table, the largest
         // allocation, 0.4 ms for 0.5 GB in blocks that it has to piece together)
         enqueue_phrases(ctx, a, p.n_est);
-        alloc_table(ctx, b, in.symb, p.cap, p.g_alloc);
+        alloc_table(ctx, b, in.symb, p.cap, p.g_alloc, kMaxRank + 1);
         set_table(a, b);
         enqueue_parse(ctx, a, p.n_est);
         grow_level(ctx, L, L.g + p.g_alloc, L.G + p.G_alloc);
@@ -1826,7 +1838,7 @@ void build_into(lcg_ctx* ctx, lcg_grammar* R, const uint8_t* data, const uint64_
     }
     double prev_ratio = 0.0, p_ratio = 0.35;
     while (in.kk > 0) {
-        if (is_tail(ctx, in.n)) tail_sync(ctx, R, in, i, against_resident);
+        if (is_tail(ctx, in.n, against_resident ? R : nullptr)) tail_sync(ctx, R, in, i, against_resident);
         else round_sync(ctx, R, in, i++, against_resident, prev_ratio, p_ratio);
     }
     check_device_status(ctx, read_status(ctx));

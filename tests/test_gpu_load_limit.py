@@ -47,3 +47,32 @@ def test_tables_past_the_limit_are_regrown(hf, kind, room):
             for r in rounds:
                 assert r["g"] <= r["table_cap"] - r["table_cap"] // 5, r
             g.free()
+
+
+def test_large_table_with_few_numbers(hf):
+    """A table of more than 2^26 slots gets numbers for half of them at first.  A round
+    that claims more than those, and no more than the table may hold, is rerun with the
+    same table: a build whose next larger table would pass 2^31 slots is not refused."""
+    import torch
+    from paper_2411_12439_gb300 import Context
+    n = 400_000_000
+    g = torch.Generator(device="cuda").manual_seed(1)
+    data = torch.randint(0, 256, (n,), dtype=torch.uint8, device="cuda", generator=g)
+    off = np.array([0, n], dtype=np.uint64)
+    torch.cuda.synchronize()
+    ctx = Context(hf, device=0)
+    first = ctx.build(data, off)
+    rounds = ctx.last_build_stats()["per_round"]
+    i = int(np.argmax([r["g"] for r in rounds]))
+    slots = int(rounds[i]["g"] / 0.65) // 16 + 1  # reached by two steps of four
+    assert 16 * slots > 1 << 26
+    first.free()
+    ctx = Context(hf, device=0)
+    ctx.set_tuning(table_slots_max=slots)
+    grammar = ctx.build(data, off)
+    again = ctx.last_build_stats()["per_round"]
+    assert [(r["g"], r["G"]) for r in again] == [(r["g"], r["G"]) for r in rounds]
+    assert again[i]["table_cap"] == 16 * slots and again[i]["retries"] >= 3, again[i]
+    out = torch.zeros(n, dtype=torch.uint8, device="cuda")
+    assert grammar.decompress(0, out) == n
+    assert torch.equal(out, data)
