@@ -978,6 +978,7 @@ u32 tail_enqueue(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, u64 n_boun
     }
     const u32 rounds = (u32)z.size();
     const u64 chunk_len = plain.take(chunks * 8);
+    const u64 retired = plain.take((u64)ctx->sms * 8);
     unsigned char* base = dalloc<unsigned char>(ctx, zero.size + ones.size + plain.size);
     unsigned char *b0 = base, *b1 = base + zero.size, *b2 = b1 + ones.size;
     ck(ctx, cudaMemsetAsync(b0, 0, zero.size, ctx->st), "memset");
@@ -993,6 +994,7 @@ u32 tail_enqueue(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, u64 n_boun
     t.rounds = rounds;
     t.bar = (u64*)(b0 + bar);
     t.chunk_len = (u64*)(b2 + chunk_len);
+    t.retired = (u64*)(b2 + retired);
     for (u32 r = 0; r < rounds; r++) {
         const Size& x = z[r];
         const u32 lev = i + r;

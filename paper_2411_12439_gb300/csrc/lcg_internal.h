@@ -169,6 +169,7 @@ struct TailArgs {
     u32 rounds;
     u64* bar;        // two zeroed counters of grid barriers for each launch
     u64* chunk_len;  // naming: symbols of each chunk of rules
+    u64* retired;    // parse: strings that retire of each block's share (a word per SM)
     RoundArgs r[kTailRounds];
 };
 static_assert(sizeof(TailArgs) <= 32000, "kernel parameters");

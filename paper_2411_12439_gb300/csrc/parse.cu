@@ -1112,25 +1112,23 @@ __device__ __forceinline__ void body_tile_strings(const RoundArgs& a, u64 tiles)
 // k_strings: per-string phrase ranges, retirement, next offsets (one block)
 // --------------------------------------------------------------------------
 
-__device__ __forceinline__ void body_strings(const RoundArgs& a) {
-    pdl_wait();
-    if (round_halted(a)) return;
-    const u64 P = *a.total;
-    const u32 k = round_k(a);
-    u64 carry = 0;
-    for (u32 j0 = 0; j0 < k; j0 += blockDim.x) {
+// The first phrase of string j of k, and whether the string has no other.
+__device__ __forceinline__ bool string_retires(const RoundArgs& a, u32 j, u32 k, u64 P, u64& first) {
+    auto index_of = [&](u64 ok) { return a.tile_pfx[ok / a.tp] + ok % a.tp; };
+    first = index_of(a.string_first[j]);
+    return ((j + 1 < k) ? index_of(a.string_first[j + 1]) : P) - first == 1;
+}
+
+// Strings lo .. hi - 1 of the round's k, by one block; `carry`: the strings before them
+// that retire.  Returns those and its own.
+__device__ __forceinline__ u64 strings_range(const RoundArgs& a, u64 P, u32 k, u32 lo, u32 hi, u64 carry) {
+    for (u32 j0 = lo; j0 < hi; j0 += blockDim.x) {
         const u32 j = j0 + threadIdx.x;
-        u64 first = 0, nextf = 0;
-        bool retire = false;
-        if (j < k) {
-            auto index_of = [&](u64 ok) { return a.tile_pfx[ok / a.tp] + ok % a.tp; };
-            first = index_of(a.string_first[j]);
-            nextf = (j + 1 < k) ? index_of(a.string_first[j + 1]) : P;
-            retire = (nextf - first == 1);
-        }
+        u64 first = 0;
+        const bool retire = j < hi && string_retires(a, j, k, P, first);
         u64 tot;
         const u64 rb = block_excl_scan(retire ? 1ull : 0ull, tot) + carry;
-        if (j < k) {
+        if (j < hi) {
             if (retire) {
                 a.R_phr[rb] = first;
                 a.R_sid[rb] = a.sid[j];
@@ -1144,16 +1142,28 @@ __device__ __forceinline__ void body_strings(const RoundArgs& a) {
         }
         carry += tot;
     }
-    if (threadIdx.x == 0) {
-        const u64 s0 = P - carry;
-        a.soff_next[k - carry] = s0;
-        if (a.sbm_next != nullptr && (s0 >> 5) < a.sbm_next_words)
-            atomicOr(a.sbm_next + (s0 >> 5), 1u << (s0 & 31));
-        a.rc->phrases = P;
-        a.rc->retired = carry;
-        a.rc->k_next = k - carry;
-        a.rc->n_next = P - carry;
-    }
+    return carry;
+}
+
+// After all strings (one thread): the end of the next sequence and the round's counts;
+// `carry`: the strings that retire.
+__device__ __forceinline__ void strings_end(const RoundArgs& a, u64 P, u32 k, u64 carry) {
+    const u64 s0 = P - carry;
+    a.soff_next[k - carry] = s0;
+    if (a.sbm_next != nullptr && (s0 >> 5) < a.sbm_next_words) atomicOr(a.sbm_next + (s0 >> 5), 1u << (s0 & 31));
+    a.rc->phrases = P;
+    a.rc->retired = carry;
+    a.rc->k_next = k - carry;
+    a.rc->n_next = P - carry;
+}
+
+__device__ __forceinline__ void body_strings(const RoundArgs& a) {
+    pdl_wait();
+    if (round_halted(a)) return;
+    const u64 P = *a.total;
+    const u32 k = round_k(a);
+    const u64 retired = strings_range(a, P, k, 0, k, 0);
+    if (threadIdx.x == 0) strings_end(a, P, k, retired);
 }
 
 // --------------------------------------------------------------------------
@@ -1821,6 +1831,12 @@ __device__ __noinline__ void solo_rounds(const TailArgs& t, u32 r) {
 
 // The phrases and the parse of the rounds t.r[0 .. t.rounds), until no string
 // is left.
+// Strings of a round, at most, that one block takes (in the barrier); more are shared
+// out, for two barriers more (some 6 us, what one block takes for 800 strings).  100,000
+// strings of 5 bytes: 1443 us in this kernel with one block for all strings, 200 so; the
+// build 5.90 ms, 4.47 so.
+constexpr u32 kStringsAlone = 2048;
+
 // (one block per SM: without the bound the compiler may settle on 80 registers and spill)
 template <bool kByte>
 __global__ void __launch_bounds__(kSmallThreads, 1) k_parse_small(const __grid_constant__ TailArgs t) {
@@ -1834,6 +1850,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_parse_small(const __grid_c
             if (blockIdx.x == 0) solo_rounds<kByte>(t, r);
             return;
         }
+        const u32 k = round_k(a);
         auto barrier = [&](auto work) { grid_barrier_work(t.bar, idx++, a.ds, work); };
         if (r == 0) {
             body_tile_strings(a, a.tiles_bound);
@@ -1849,8 +1866,29 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_parse_small(const __grid_c
                                            [&](u64 i, u64 e) { a.tile_pfx[i] = e; });
             if (threadIdx.x == 0) *a.total = P;
             __syncthreads();
-            body_strings(a);
+            if (k <= kStringsAlone) body_strings(a);
         });
+        if (k > kStringsAlone) {
+            // each block its share of the strings: how many retire, then their places
+            const u64 P = *a.total;
+            const u32 share = (k + gridDim.x - 1) / gridDim.x;
+            const u32 lo = min(k, blockIdx.x * share), hi = min(k, lo + share);
+            const bool ok = !round_halted(a);
+            u64 mine = 0, sum;
+            for (u32 j = lo + threadIdx.x; ok && j < hi; j += blockDim.x) {
+                u64 first;
+                mine += string_retires(a, j, k, P, first) ? 1 : 0;
+            }
+            block_excl_scan(mine, sum);
+            if (threadIdx.x == 0) t.retired[blockIdx.x] = sum;
+            barrier([] {});
+            u64 before = 0;
+            for (u32 b = threadIdx.x; b < blockIdx.x; b += blockDim.x) before += t.retired[b];
+            block_excl_scan(before, sum);
+            const u64 upto = ok ? strings_range(a, P, k, lo, hi, sum) : 0;
+            if (ok && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) strings_end(a, P, k, upto);
+            barrier([] {});
+        }
         if (kByte && r == 0) body_parse<unsigned char, kUnitMin, kParseWarps, true>(a, a.tiles_bound);
         else body_parse<u32, kUnitMin, kParseWarps, true>(a, a.tiles_bound);
         barrier([] {});
@@ -1949,9 +1987,9 @@ __global__ void __launch_bounds__(kSmallThreads) k_naming_small(const __grid_con
         if (threadIdx.x == 0) t.chunk_len[ch] = tot;
     }
     // the retired strings' roots
-    for (u32 r = blockIdx.x; r < t.rounds; r += gridDim.x) {
+    for (u32 r = 0; r < t.rounds; r++) {
         const RoundArgs& a = t.r[r];
-        for (u64 x = threadIdx.x; x < s_retired[r]; x += blockDim.x) {
+        for (u64 x = gtid; x < s_retired[r]; x += gthreads) {
             const u32 id = a.c_rank[a.R_sid[x]];
             if (id >= a.id_base && id - a.id_base < a.id_cap) a.c_rank[a.R_sid[x]] = a.rank_of[id - a.id_base];
         }
