@@ -3326,7 +3326,7 @@ int lcg_vbyte_encode(lcg_ctx* ctx, const uint32_t* in, uint64_t n, uint8_t* out,
         dfree(ctx, off);
         cnt = nullptr;
         off = nullptr;
-        const DevStatus st = read_status(ctx, &nb, ctx->scratch + 1, 8);
+        const DevStatus st = fits ? read_status(ctx, &nb, ctx->scratch + 1, 8) : read_status(ctx);
         *out_bytes = nb;
         kt_collect(ctx);
         check_device_status(ctx, st);
