@@ -1334,8 +1334,11 @@ std::vector<RoundPlan> plan_rounds(lcg_ctx* ctx, u64 n1, u32 kk, u32 planned) {
         p.cap = std::min<u64>(bucket(std::max<u64>(8192, (u64)(p.g_est * 1.1 * sl / ctx->tuning.table_load) + 1024)),
                               kMaxRank + 1);
         if (ctx->tuning.table_slots_max) p.cap = std::min<u64>(p.cap, ctx->tuning.table_slots_max);
-        p.g_alloc = bucket((u64)(p.g_est * 1.25 * sl) + 1024);
-        p.G_alloc = bucket((u64)(p.G_est * 1.25 * sl) + 4096);
+        // (never more than a round can have: a context that has seen runs, then many short
+        // rules, estimates their product)
+        p.g_alloc = std::min<u64>(bucket((u64)(p.g_est * 1.25 * sl) + 1024), p.n_alloc / 2 + 2ull * kk + 1);
+        p.G_alloc = (u64)std::min((double)p.n_alloc, p.G_est * 1.25 * sl + 4096.0);
+        p.G_alloc = std::min<u64>(bucket(p.G_alloc), p.n_alloc);
         // the next sequence: the estimated phrases with the same slack (a
         // round past it flags a capacity error and the build is redone)
         p.t_cap = std::min<u64>(bucket((u64)(p.P_est * 1.1 * sl) + 4096), n_bound / 2 + 2ull * kk + 1);

@@ -53,3 +53,19 @@ def test_next_sequence_outgrows_its_plan(hf, n, phrases, k, graph):
     assert all(r["retries"] == 0 for r in st["per_round"]), st  # no table was too small
     assert O.grammars_equal(g.export(), want)
     g.free()
+
+
+def test_plan_of_unlike_collections(hf):
+    """Rules as long as a string in one collection and hundreds of thousands of short ones
+    in the next: a plan made from both asks for no more than a round can have."""
+    pytest.importorskip("torch")
+    from paper_2411_12439_gb300 import Context
+    rng = np.random.default_rng(4)
+    runs = _runs(8_000_000, 10, 1)
+    noise = li.from_strings([rng.integers(0, 256, size=2_000_000, dtype=np.uint8)])
+    last = li.from_strings([li.random_dna(rng, 1_500_000)])
+    ctx = Context(hf, device=0)
+    for coll in (runs, noise, last, runs, noise):
+        g = ctx.build(coll.data, coll.offsets)
+        assert O.grammars_equal(g.export(), O.build(coll, hf).export())
+        g.free()
