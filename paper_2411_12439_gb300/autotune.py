@@ -4,7 +4,8 @@ with a cache of the best setting per class of collection.
 The parse tile size, the rank rounds' tile order (tiles taken in interleaved
 stripes), the parse kernel's resident blocks per SM in those rounds and the
 phrase tables' load factor change the build's speed, never its result
-(``miss_flush`` is a field of the tuning that has no effect).
+(``miss_flush`` is a field of the tuning that has no effect; a context names such
+fields in ``INERT_TUNING``, and they are not searched).
 ``autotune`` times builds of a sample collection on a context and keeps, one
 parameter at a time (coordinate descent, two sweeps), the value with the
 shortest median build time; the context keeps the best setting.
@@ -63,6 +64,8 @@ def autotune(ctx, data, offsets, reps: int = 3, sweeps: int = 2, candidates=None
         for name, values in cands.items():
             if name not in best:
                 continue  # a parameter this context does not have
+            if name in getattr(ctx, "INERT_TUNING", ()):
+                continue  # or that changes nothing in it
             for v in values:
                 if v == best[name]:
                     continue

@@ -1516,9 +1516,8 @@ struct GraphBuild {
 // What a graph's launches depend on besides the input and the planned buffer
 // sizes: the number of planned rounds and the launch parameters.
 std::vector<double> graph_params(lcg_ctx* ctx, u32 planned) {
-    return {(double)planned,    (double)ctx->tuning.parse_blocks_per_sm, (double)ctx->tuning.miss_flush,
-            (double)ctx->ktime, (double)ctx->tuning.tile_stripes,        (double)ctx->tuning.parse_tile,
-            (double)ctx->tuning.parse_tile_min};
+    return {(double)planned,    (double)ctx->tuning.parse_blocks_per_sm, (double)ctx->ktime,
+            (double)ctx->tuning.tile_stripes, (double)ctx->tuning.parse_tile, (double)ctx->tuning.parse_tile_min};
 }
 
 // A captured graph serves a new plan when each of its rounds' buffers holds

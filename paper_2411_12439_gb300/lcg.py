@@ -169,6 +169,9 @@ def _data_arg(data):
 class Context:
     """A device, a stream and a hash family (``lcg_ctx``)."""
 
+    # fields of lcg_tuning that are accepted and kept and change nothing
+    INERT_TUNING = frozenset({"miss_flush"})
+
     def __init__(self, hash_family, device: int = 0, stream=None):
         lib = load()
         self._keep = [np.ascontiguousarray(x, dtype=np.uint64) for x in (hash_family.a, hash_family.b, hash_family.c)]
