@@ -364,7 +364,9 @@ def timed_builds(ctx, d, offsets, steps: int, stream, graph: bool):
 
 def round_breakdown(ctx, d, offsets, builds: int = 3):
     """Builds as launches with every launch timed: per round its sizes and
-    device time, per kernel kind its time per build."""
+    device time, per kernel kind its launches and time per build.  The short
+    rounds share their launches: the first of them has the time of all
+    (``ms_rounds``: how many), the others none."""
     ctx.set_kernel_timing(1)
     per_round, kernels = None, {}
     for _ in range(builds):
@@ -373,8 +375,11 @@ def round_breakdown(ctx, d, offsets, builds: int = 3):
         if per_round is None or len(per_round) != len(rs):
             per_round = [{k: r[k] for k in ("n", "phrases", "g", "G", "table_cap", "strings")} | {"ms": []}
                          for r in rs]
-        byround = {}
+        byround, shared = {}, set()
         for rec in ctx.last_kernel_launches():
+            if rec["shared"]:
+                shared.add(rec["round"])
+                continue
             byround[rec["round"]] = byround.get(rec["round"], 0.0) + rec["ms"]
             k = kernels.setdefault(rec["name"], {"launches": 0, "ms": 0.0})
             k["launches"] += 1
@@ -382,8 +387,9 @@ def round_breakdown(ctx, d, offsets, builds: int = 3):
         for i, pr in enumerate(per_round):
             pr["ms"].append(byround.get(i + 1, 0.0))
     ctx.set_kernel_timing(0)
-    for pr in per_round:
-        pr["ms"] = float(np.median(pr["ms"]))
+    for i, pr in enumerate(per_round):
+        pr["ms"] = None if i + 1 in shared else float(np.median(pr["ms"]))
+        pr["ms_rounds"] = 1 + len(shared) if i + 2 in shared and i + 1 not in shared else 1
     kernels = {k: {"launches": v["launches"] // builds, "ms_per_step": v["ms"] / builds}
                for k, v in sorted(kernels.items(), key=lambda kv: -kv[1]["ms"])}
     return per_round, kernels
@@ -711,8 +717,9 @@ def run_ours(args):
                 "one 32-byte sector per phrase of every round whose table exceeds L2"}
     rounds_line = [{"round": i + 1, "symbols": int(r["n"]), "phrases": int(r["phrases"]), "g": int(r["g"]),
                     "G": int(r["G"]), "table_mb": r["table_cap"] * 32 / 1e6, "ms": r["ms"],
-                    "parse_ms": parse_ms.get(i + 1),
-                    "gbs": r["n"] * (1 if i == 0 else 4) / (r["ms"] / 1e3) / 1e9 if r["ms"] > 0 else None}
+                    "ms_rounds": r["ms_rounds"], "parse_ms": parse_ms.get(i + 1),
+                    "gbs": r["n"] * (1 if i == 0 else 4) / (r["ms"] / 1e3) / 1e9
+                    if r["ms"] and r["ms_rounds"] == 1 else None}
                    for i, r in enumerate(rounds)]
 
     # ---- plain form: each string built alone, back to back (and the merge of

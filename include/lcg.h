@@ -119,7 +119,8 @@ typedef struct lcg_build_stats {
  * only while kernel timing is enabled with lcg_set_kernel_timing). */
 typedef struct lcg_kernel_time {
     char name[24];       /* kernel kind, e.g. "k_parse" */
-    uint32_t launches;
+    uint32_t launches;   /* its records: a launch that parses several short rounds
+                            (k_parse_small) counts once for each of them */
     uint32_t pad;
     double ms;           /* summed CUDA-event time of its launches */
     double bytes;        /* algorithmic bytes of its launches (see the kernel's comment) */
@@ -193,13 +194,14 @@ int lcg_get_tuning(const lcg_ctx* ctx, lcg_tuning* t);
  * `out` (host) and their number into *count. */
 int lcg_last_kernel_times(const lcg_ctx* ctx, lcg_kernel_time* out, uint32_t cap, uint32_t* count);
 
-/* One timed kernel launch of the last call (kernel timing on). */
+/* One timed kernel launch of the last call (kernel timing on), or one round of it. */
 typedef struct lcg_kernel_launch {
     char name[24];       /* kernel kind, e.g. "k_parse" */
     uint32_t round;      /* BuildGram round of a build's launch (1 = bytes), 0 for others */
-    uint32_t pad;
-    double ms;           /* CUDA-event time of the launch */
-    double bytes;        /* algorithmic bytes of the launch */
+    uint32_t shared;     /* 1: no launch of its own, but a further round of the launch
+                            recorded before it, which has the time and the bytes */
+    double ms;           /* CUDA-event time of the launch (0 when shared) */
+    double bytes;        /* algorithmic bytes of the launch (0 when shared) */
 } lcg_kernel_launch;
 /* Copy up to `cap` of the last call's timed launches, in launch order, into
  * `out` (host) and their number into *count. */

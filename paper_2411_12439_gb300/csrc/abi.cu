@@ -259,6 +259,7 @@ void kt_collect(lcg_ctx* ctx) {
         lcg_kernel_launch kl{};
         std::strncpy(kl.name, r.name, sizeof(kl.name) - 1);
         kl.round = r.round;
+        kl.shared = r.part ? 1 : 0;
         kl.ms = ms;
         kl.bytes = r.bytes;
         ctx->klaunches.push_back(kl);

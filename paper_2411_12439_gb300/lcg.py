@@ -58,7 +58,7 @@ class KernelTimeC(ctypes.Structure):
 
 
 class KernelLaunchC(ctypes.Structure):
-    _fields_ = [("name", ctypes.c_char * 24), ("round", ctypes.c_uint32), ("pad", ctypes.c_uint32),
+    _fields_ = [("name", ctypes.c_char * 24), ("round", ctypes.c_uint32), ("shared", ctypes.c_uint32),
                 ("ms", ctypes.c_double), ("bytes", ctypes.c_double)]
 
 
@@ -353,8 +353,9 @@ class Context:
                                        "bytes": float(buf[i].bytes)} for i in range(min(cnt.value, 32))}
 
     def last_kernel_launches(self) -> list:
-        """lcg_last_kernel_launches: [{"name", "round", "ms", "bytes"}] of the
-        last call's timed launches, in launch order."""
+        """lcg_last_kernel_launches: [{"name", "round", "ms", "bytes", "shared"}]
+        of the last call's timed launches, in launch order; ``shared`` records
+        are further rounds of the launch before them, without a time."""
         lib = load()
         cnt = ctypes.c_uint32(0)
         self._check(lib.lcg_last_kernel_launches(self._h, None, 0, ctypes.byref(cnt)))
@@ -362,7 +363,7 @@ class Context:
         buf = (KernelLaunchC * max(n, 1))()
         self._check(lib.lcg_last_kernel_launches(self._h, ctypes.cast(buf, ctypes.c_void_p), n, ctypes.byref(cnt)))
         return [{"name": buf[i].name.decode(), "round": int(buf[i].round), "ms": float(buf[i].ms),
-                 "bytes": float(buf[i].bytes)} for i in range(min(n, cnt.value))]
+                 "bytes": float(buf[i].bytes), "shared": bool(buf[i].shared)} for i in range(min(n, cnt.value))]
 
     def selftest_wait_timeout(self) -> int:
         """lcg_selftest_wait_timeout: the return code (LCG_ETIMEOUT, -6, when
