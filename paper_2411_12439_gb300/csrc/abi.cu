@@ -1174,8 +1174,6 @@ void round_sync(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, bool agains
     rs.strings = in.kk;
     RoundBufs b;
     alloc_round(ctx, b, n, in.kk, 0);
-    const u64 tiles = b.tiles;
-    ensure_lb(ctx, &ctx->lb1, &ctx->lb1_tiles, tiles, lb1_bytes(tiles));
     Level& L = R->lv[i - 1];
     RoundArgs a = round_args(ctx, R, in, b, i);
     a.d_n = nullptr;
@@ -1379,7 +1377,6 @@ void rounds_async_enqueue(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, AsyncRou
         Level& L = R->lv[r - 1];
         RoundBufs b;
         alloc_round(ctx, b, p.n_alloc, kk, p.t_cap);
-        ensure_lb(ctx, &ctx->lb1, &ctx->lb1_tiles, b.tiles, lb1_bytes(b.tiles));
         RoundArgs a = round_args(ctx, R, in, b, r);
         // a round stops early when the one before it failed
         if (r > 1) a.ds_prev = ctx->ds_arr + (r - 2);
@@ -1590,7 +1587,7 @@ void capture_graph(lcg_ctx* ctx, const unsigned char* d_in, const std::vector<u6
         }
         const u32 tp = parse_unit(round_tile(ctx, p.n_alloc));
         const u64 tiles = (p.n_alloc + tp - 1) / tp;
-        t1 = std::max({t1, tiles, popscan_tiles_for((p.t_cap + k) / 32 + 1), rule_offs_tiles(std::max<u64>(1, p.g_alloc))});
+        t1 = std::max({t1, popscan_tiles_for((p.t_cap + k) / 32 + 1), rule_offs_tiles(std::max<u64>(1, p.g_alloc))});
         t2 = std::max(t2, scan2_tiles_for(tiles));
         hs = std::max(hs, breaks_steps(tiles, tp));
     }
