@@ -76,7 +76,6 @@ struct lcg_ctx {
     std::string err;
     // persistent device scratch
     DevStatus* ds = nullptr;
-    RoundCounts* rc = nullptr;
     u64* ctr = nullptr;     // tile counter of single-pass kernels (never reset)
     u64 ctr_val = 0;        // its value after all launched tiles ran
     u64 epoch = 0;          // look-back epoch, one per launch
@@ -2565,7 +2564,6 @@ int lcg_ctx_create(int device, const lcg_hash_family* H, void* stream, lcg_ctx**
         }
         ck(ctx, cudaHostAlloc((void**)&ctx->mail, kMailBytes, cudaHostAllocDefault), "cudaHostAlloc");
         ck(ctx, cudaMalloc(&ctx->ds, sizeof(DevStatus)), "cudaMalloc");
-        ck(ctx, cudaMalloc(&ctx->rc, sizeof(RoundCounts)), "cudaMalloc");
         ck(ctx, cudaMalloc(&ctx->ctr, sizeof(u64)), "cudaMalloc");
         ck(ctx, cudaMalloc(&ctx->scratch, 8 * sizeof(u64)), "cudaMalloc");
         ck(ctx, cudaMalloc(&ctx->ds_arr, kMaxRounds * sizeof(DevStatus)), "cudaMalloc");
@@ -2602,7 +2600,6 @@ void lcg_ctx_destroy(lcg_ctx* ctx) {
     if (ctx->heads) cudaFree(ctx->heads);
     if (ctx->lb2) cudaFree(ctx->lb2);
     cudaFree(ctx->ds);
-    cudaFree(ctx->rc);
     cudaFree(ctx->ctr);
     cudaFree(ctx->scratch);
     cudaFree(ctx->ds_arr);

@@ -182,7 +182,6 @@ size_t claim_rec_bytes();                       // bytes of one ClaimRec
 u64 breaks_steps(u64 units, u32 tp);           // k_breaks' block steps over a round's parse units
 u64 popscan_tiles_for(u64 nw);
 size_t lb1_bytes(u64 tiles);
-size_t lb2_bytes(u64 tiles);
 size_t slot_bytes();  // bytes of one phrase-table slot
 
 cudaError_t launch_tile_strings(const RoundArgs& a, cudaStream_t st);

@@ -2214,7 +2214,6 @@ cudaError_t launch_gather_strings(const unsigned char* data, const u64* src_off,
 }
 
 size_t lb1_bytes(u64 tiles) { return tiles * sizeof(LBSlot<1>); }
-size_t lb2_bytes(u64 tiles) { return tiles * sizeof(LBSlot<2>); }
 size_t slot_bytes() { return sizeof(Slot); }
 
 }  // namespace lcg

@@ -59,17 +59,6 @@ __device__ __forceinline__ u64 inline_max(int w) {
     return m < kInlineMax ? (u64)m : (u64)kInlineMax;
 }
 
-__device__ __forceinline__ void put_bits(u64& hi, u64& lo, int pos, u64 v, int b) {
-    if (pos + b <= kHiBits) {
-        hi |= v << pos;
-    } else if (pos >= kHiBits) {
-        lo |= v << (pos - kHiBits);
-    } else {
-        hi |= (v << pos) & ((1ull << kHiBits) - 1);
-        lo |= v >> (kHiBits - pos);
-    }
-}
-
 __device__ __forceinline__ u64 get_bits(u64 hi, u64 lo, int pos, int b) {
     const u64 m = (1ull << b) - 1;
     if (pos + b <= kHiBits) return (hi >> pos) & m;
@@ -82,7 +71,7 @@ __device__ __forceinline__ u64 get_bits(u64 hi, u64 lo, int pos, int b) {
 // V = sum_j get(j) 2^(j b) (at most 124 bits), accumulated from the last
 // symbol with a 128-bit shift per symbol (no branch on where a symbol falls);
 // bits 0..59 of V go to hi under the length, bits 60..123 to lo.  This is the
-// layout put_bits / key_sym use.
+// layout key_sym reads.
 template <typename Get>
 __device__ __forceinline__ Key128 key_inline(Get get, u64 len, int b) {
     u64 vlo = 0, vhi = 0;  // V, 128 bits
