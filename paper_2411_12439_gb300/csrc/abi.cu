@@ -353,7 +353,9 @@ LevelHash level_hash(const lcg_ctx* ctx, u32 i) {
 
 // The planned rounds did not fit (or a graph capture had to be abandoned):
 // the build is redone round by round.
-struct Retry {};
+struct Retry {
+    bool levels = false;  // only the short rounds' levels did not: no reason for larger plans
+};
 
 void destroy_graph(lcg_ctx* ctx);
 
@@ -895,8 +897,11 @@ void next_input(lcg_ctx* ctx, RoundInput& in, RoundBufs& b) {
 // A round whose tile is the smallest (see round_tile) and that has at most
 // kTailSymbols symbols, and every round after it, run in two launches.  All
 // their buffers are parts of one allocation, sized by what a round can have at
-// most (n symbols in k strings: (n + k) / 2 phrases), so nothing is planned,
-// regrown or waited for; the levels of a fresh build share one allocation too.
+// most (n symbols in k strings: (n + k) / 2 phrases), so nothing is
+// regrown or waited for.  The levels of a fresh build share one allocation too, which
+// the grammar keeps: from kTailPlanned symbols on a plan makes it about as large as they
+// need (tail_levels), and where there is none it is replaced afterwards if they need
+// less (compact_levels).
 
 // (Where the slots of a table are limited the rounds that could need more run one by
 // one: theirs start within the limit.)
@@ -908,6 +913,14 @@ bool is_tail(const lcg_ctx* ctx, u64 n, const lcg_grammar* resident = nullptr) {
     const u64 most = ctx->tuning.table_slots_max;
     return n <= kTailSymbols && round_tile(ctx, n) == 1024 && (most == 0 || 3 * n <= most);
 }
+
+// Rules and symbols of a level.
+struct LevelSize {
+    u64 g, G;
+};
+// Below, the levels' arrays take what they can need at most (20 bytes a symbol over all
+// of them, 1 MB): a server's short requests, each of another make-up, are never redone.
+constexpr u64 kTailPlanned = 50000;
 
 // Offsets of the parts of one allocation.
 struct Parts {
@@ -922,8 +935,10 @@ struct Parts {
 // Enqueue round i and those after it (at most n_bound symbols in kk strings
 // enter it); returns how many there may be.  `in` becomes what follows the
 // last (nothing); cap[r]: the table slots of round r.
+// `planned`: what the arrays of a fresh build's levels are made for (those that it does
+// not name: for what they can have); a level that has more flags a capacity error.
 u32 tail_enqueue(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, u64 n_bound, u32 kk, bool against_resident,
-                 const DevStatus* ds_prev, u64* cap) {
+                 const DevStatus* ds_prev, u64* cap, const std::vector<LevelSize>& planned) {
     fail_if(ctx, i >= ctx->levels || i > kMaxRounds,
             LCG_ELEVELS, "hash family too short: needs more than " + std::to_string(ctx->levels) + " functions");
     const u32 most = std::min<u32>({kTailRounds, ctx->levels - i, kMaxRounds - i + 1});
@@ -932,6 +947,7 @@ u32 tail_enqueue(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, u64 n_boun
         u64 n, k, P, units, cap, ids, words;
         u64 sbm, first, tab, minpos;                                          // cleared parts
         u64 string_first, soff, sid, R_phr, R_sid, cnt, pfx, brk, T, F, crec, rank_of, rrec;
+        LevelSize lv;                                                         // the level's arrays
         u64 off, rhs, lvF;                                                    // in the levels' slab
     };
     std::vector<Size> z;
@@ -966,9 +982,12 @@ u32 tail_enqueue(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, u64 n_boun
         x.crec = plain.take(x.ids * claim_rec_bytes());
         x.rank_of = plain.take(x.ids * 4);
         x.rrec = plain.take(x.P * claim_rec_bytes());
-        x.off = slab.take((x.P + 1) * 8);
-        x.rhs = slab.take(n * 4);
-        x.lvF = slab.take(x.P * 4);
+        x.lv = LevelSize{x.P, n};
+        if (z.size() < planned.size())
+            x.lv = LevelSize{std::min(x.P, planned[z.size()].g), std::min(n, planned[z.size()].G)};
+        x.off = slab.take((x.lv.g + 1) * 8);
+        x.rhs = slab.take(x.lv.G * 4);
+        x.lvF = slab.take(x.lv.g * 4);
         chunks += rule_chunks(x.P);
         z.push_back(x);
         // the strings left have two symbols or more each
@@ -1008,8 +1027,8 @@ u32 tail_enqueue(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, u64 n_boun
             L.rhs_off = (u64*)(lv + x.off);
             L.rhs = (u32*)(lv + x.rhs);
             L.F = (u32*)(lv + x.lvF);
-            L.cap_g = x.P;
-            L.cap_G = x.n;
+            L.cap_g = x.lv.g;
+            L.cap_G = x.lv.G;
             L.shared_rules = L.shared_rhs = true;
             L.rvalid = false;
         }
@@ -1113,13 +1132,83 @@ u32 tail_enqueue(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, u64 n_boun
     return rounds;
 }
 
+// Copies of 32-bit columns, all of them in one launch.
+struct Copies {
+    std::vector<CopyCol> cols;
+    u64 blocks = 0;
+    // pad: a zero follows when n is odd
+    void add(void* dst, const void* src, u64 n, bool pad = false) {
+        if (n == 0) return;
+        cols.push_back(CopyCol{(u32*)dst, (const u32*)src, n, blocks, pad && (n & 1)});
+        blocks += copy_blocks(n);
+    }
+    void run(lcg_ctx* ctx, std::vector<void*>& temps) {
+        if (cols.empty()) return;
+        CopyCol* d = dalloc<CopyCol>(ctx, cols.size());
+        temps.push_back(d);
+        ck(ctx, cudaMemcpyAsync(d, cols.data(), cols.size() * sizeof(CopyCol), cudaMemcpyHostToDevice, ctx->st),
+           "columns");
+        ck(ctx, launch_copy_cols(d, (u32)cols.size(), blocks, ctx->st), "copy columns");
+        ctx->launches++;
+    }
+};
+
+// The levels from i on, all in the grammar's last slab: into one that holds what they
+// have, when that is less than half of it.  (Where there is no memory for it they stay.)
+void compact_levels(lcg_ctx* ctx, lcg_grammar* R, u32 i) {
+    if (R->slabs.empty()) return;
+    Parts have, need;
+    for (size_t l = i - 1; l < R->lv.size(); l++) {
+        const Level& L = R->lv[l];
+        if (!L.shared_rules || !L.shared_rhs) return;
+        have.take((L.cap_g + 1) * 8 + L.cap_G * 4 + L.cap_g * 4);
+        need.take((L.g + 1) * 8);
+        need.take(L.G * 4);
+        need.take(L.g * 4);
+    }
+    if (have.size < 2 * need.size + 65536) return;
+    void* p = nullptr;
+    if (alloc_async(ctx, &p, need.size) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    std::vector<void*> temps;
+    std::vector<Level> lv(R->lv.begin() + (i - 1), R->lv.end());
+    try {
+        Parts at;
+        Copies copies;
+        for (Level& L : lv) {
+            unsigned char* const off = (unsigned char*)p + at.take((L.g + 1) * 8);
+            unsigned char* const rhs = (unsigned char*)p + at.take(L.G * 4);
+            unsigned char* const F = (unsigned char*)p + at.take(L.g * 4);
+            copies.add(off, L.rhs_off, 2 * (L.g + 1));
+            copies.add(rhs, L.rhs, L.G);
+            copies.add(F, L.F, L.g);
+            L.rhs_off = (u64*)off;
+            L.rhs = (u32*)rhs;
+            L.F = (u32*)F;
+            L.cap_g = L.g;
+            L.cap_G = L.G;
+        }
+        copies.run(ctx, temps);
+    } catch (const Fail&) {
+        for (void* x : temps) dfree(ctx, x);
+        dfree(ctx, p);
+        return;
+    }
+    for (void* x : temps) dfree(ctx, x);
+    std::copy(lv.begin(), lv.end(), R->lv.begin() + (i - 1));
+    dfree(ctx, R->slabs.back());
+    R->slabs.back() = p;
+}
+
 // The short rounds of a build that is run round by round: one host
 // synchronisation after all of them.
 void tail_sync(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32& i, bool against_resident) {
     u64 cap[kMaxRounds + kTailRounds + 2] = {0};
     u64 n = in.n;
     u32 k = in.kk;
-    const u32 rounds = tail_enqueue(ctx, R, in, i, in.n, in.kk, against_resident, nullptr, cap);
+    const u32 rounds = tail_enqueue(ctx, R, in, i, in.n, in.kk, against_resident, nullptr, cap, {});
     std::vector<DevStatus> st(rounds);
     std::vector<RoundCounts> rc(rounds);
     fetch(ctx, {{st.data(), ctx->ds_arr + (i - 1), rounds * sizeof(DevStatus)},
@@ -1148,6 +1237,7 @@ void tail_sync(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32& i, bool agains
     }
     // levels that no round reached
     while (R->lv.size() > (size_t)(i + r - 1) && R->lv.back().g == 0) pop_level(ctx, R);
+    if (!against_resident) compact_levels(ctx, R, i);
     i += r;
     in.kk = k;
     in.n = n;
@@ -1293,6 +1383,7 @@ struct RoundPlan {
     u64 n_bound = 0, n_est = 0, n_alloc = 0, cap = 0, g_alloc = 0, G_alloc = 0, t_cap = 0;
     double P_est = 0, g_est = 0, G_est = 0;
     bool tail = false;  // this round and all after it run as the short rounds (n_alloc symbols at most)
+    std::vector<LevelSize> levels;  // of those rounds
 };
 
 // x rounded up to a step of 2^(1/4) (about 19 %): plans from slightly
@@ -1308,6 +1399,20 @@ u64 bucket(u64 x) {
     return 2 * b;
 }
 
+// What the arrays of the short rounds' levels from round r on are made for, as far as the
+// context has seen such levels: twice the estimates (times the plan slack) and room for
+// a few rules.  (What the rounds could have at most is far more, and a grammar keeps it:
+// 100 strings of 5 kB, all alike, held 10.0 MB so, now 0.26.)
+std::vector<LevelSize> tail_levels(const lcg_ctx* ctx, u32 r, double n_est) {
+    std::vector<LevelSize> v;
+    for (; r <= kMaxRounds && ctx->p_hint[r] > 0; r++) {
+        const double P = ctx->p_hint[r] * n_est, g = ctx->ratio_hint[r] * P, sl = 2.0 * ctx->plan_slack;
+        v.push_back(LevelSize{bucket((u64)(g * sl) + 512), bucket((u64)(ctx->glen_hint[r] * g * sl) + 2048)});
+        n_est = P + 64;
+    }
+    return v;
+}
+
 std::vector<RoundPlan> plan_rounds(lcg_ctx* ctx, u64 n1, u32 kk, u32 planned) {
     std::vector<RoundPlan> v(planned + 1);
     u64 n_bound = n1, n_est = n1;
@@ -1320,6 +1425,7 @@ std::vector<RoundPlan> plan_rounds(lcg_ctx* ctx, u64 n1, u32 kk, u32 planned) {
         p.n_alloc = (r == 1) ? n_bound : std::min<u64>(n_bound, v[r - 1].t_cap);
         p.tail = is_tail(ctx, p.n_alloc);
         if (p.tail) {
+            if (p.n_alloc >= kTailPlanned) p.levels = tail_levels(ctx, r, n_est);
             v.resize(r + 1);
             break;
         }
@@ -1352,6 +1458,7 @@ struct AsyncRounds {
     u32 planned = 0, kk = 0;  // rounds (with those of the tail), strings
     std::vector<RoundPlan> plan;
     std::vector<u64> g_base, G_base, cap;
+    u32 tail = 0;  // the first of the short rounds (0: none)
 };
 
 // Enqueue the planned rounds of a fresh build: every size comes from the plan;
@@ -1367,7 +1474,8 @@ void rounds_async_enqueue(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, AsyncRou
         const RoundPlan& p = ar.plan[r];
         if (p.tail) {
             const DevStatus* before = r > 1 ? ctx->ds_arr + (r - 2) : nullptr;
-            const u32 rounds = tail_enqueue(ctx, R, in, r, p.n_alloc, kk, false, before, ar.cap.data());
+            const u32 rounds = tail_enqueue(ctx, R, in, r, p.n_alloc, kk, false, before, ar.cap.data(), p.levels);
+            ar.tail = r;
             ar.planned = r - 1 + rounds;
             return;
         }
@@ -1411,7 +1519,7 @@ void rounds_async_enqueue(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, AsyncRou
 // After the enqueued rounds: read their statuses and counts (one host
 // synchronisation), set the levels' sizes and the build statistics.  Returns
 // 0, or -1 when a round did not fit (the build must then be redone round by
-// round); `i` becomes the first round not yet run, and `in` its input.
+// round; -2 when it was only the arrays of a short round's level); `i` becomes the first round not yet run, and `in` its input.
 int rounds_async_finish(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, const AsyncRounds& ar, u32& i) {
     const u32 planned = ar.planned;
     const u32 kk = ar.kk;
@@ -1420,7 +1528,11 @@ int rounds_async_finish(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, const Asyn
     fetch(ctx, {{st.data(), ctx->ds_arr, planned * sizeof(DevStatus)},
                 {rc.data(), ctx->rc_arr, planned * sizeof(RoundCounts)}});
     for (u32 r = 0; r < planned; r++) {
-        if (overfull(st[r], ar.cap[r + 1]) || st[r].error == kErrCapacity || st[r].error == kErrHalted) return -1;
+        if (overfull(st[r], ar.cap[r + 1]) || st[r].error == kErrHalted) return -1;
+        if (st[r].error == kErrCapacity) {
+            const Level& L = R->lv[r];
+            return ar.tail && r + 1 >= ar.tail && (st[r].claims > L.cap_g || st[r].claim_len > L.cap_G) ? -2 : -1;
+        }
         check_device_status(ctx, st[r]);
     }
     // rounds past the last active string (the data needed fewer rounds than
@@ -1529,7 +1641,14 @@ bool plan_covers(const std::vector<RoundPlan>& have, const std::vector<RoundPlan
     for (size_t r = 1; r < have.size(); r++) {
         const RoundPlan& h = have[r];
         const RoundPlan& n = need[r];
-        if (h.tail || n.tail) return h.tail && n.tail && h.n_alloc >= n.n_alloc;
+        if (h.tail || n.tail) {
+            if (!h.tail || !n.tail || h.n_alloc < n.n_alloc || h.levels.size() > n.levels.size()) return false;
+            // (a plan is for twice the estimates; levels that the plan at hand does not name
+            // have room for all they can have)
+            for (size_t l = 0; l < h.levels.size(); l++)
+                if (2 * h.levels[l].g < n.levels[l].g || 2 * h.levels[l].G < n.levels[l].G) return false;
+            return true;
+        }
         if (h.n_bound != n.n_bound || h.n_alloc < n.n_alloc || h.cap < n.cap || h.cap > 4 * n.cap ||
             h.g_alloc < n.g_alloc || h.G_alloc < n.G_alloc || h.t_cap < n.t_cap)
             return false;
@@ -1735,7 +1854,7 @@ lcg_grammar* build_with_graph(lcg_ctx* ctx, const unsigned char* d_in, const std
     }
     if (r < 0 || in.kk > 0) {  // did not fit, or more rounds are needed: run as launches
         free_grammar_now(G);
-        throw Retry{};
+        throw Retry{r == -2};
     }
     ctx->hint_rounds = ctx->stats.rounds;
     ctx->stats.kernel_launches = gb->launches;
@@ -1834,7 +1953,7 @@ void build_into(lcg_ctx* ctx, lcg_grammar* R, const uint8_t* data, const uint64_
             // a round outgrew its estimate: the caller starts again with synchronised rounds
             free_round_input(ctx, in);
             for (void* p : owned) dfree(ctx, p);
-            throw Retry{};
+            throw Retry{r == -2};
         }
     }
     double prev_ratio = 0.0, p_ratio = 0.35;
@@ -2711,8 +2830,8 @@ int lcg_build(lcg_ctx* ctx, const uint8_t* data, const uint64_t* offsets, uint32
         if (ok) {
             try {
                 G = build_with_graph(ctx, data + offsets[0], lens);
-            } catch (const Retry&) {
-                ctx->plan_slack = std::min(4.0, ctx->plan_slack * 1.6);
+            } catch (const Retry& r) {
+                if (!r.levels) ctx->plan_slack = std::min(4.0, ctx->plan_slack * 1.6);
                 G = nullptr;
                 kt_reset(ctx);
                 G = new_grammar(ctx);
@@ -2737,8 +2856,8 @@ int lcg_build(lcg_ctx* ctx, const uint8_t* data, const uint64_t* offsets, uint32
     try {
         build_into(ctx, G, data, offsets, k, data_on_device, false, true);
         if (ctx->stats.async_rounds > 0) ctx->plan_slack = std::max(1.0, ctx->plan_slack * 0.97);
-    } catch (const Retry&) {
-        ctx->plan_slack = std::min(4.0, ctx->plan_slack * 1.6);
+    } catch (const Retry& r) {
+        if (!r.levels) ctx->plan_slack = std::min(4.0, ctx->plan_slack * 1.6);
         // the rounds planned from the previous build did not fit: round by round
         sync(ctx);
         free_grammar_now(G);
@@ -3046,27 +3165,6 @@ int lcg_packed_size(const lcg_grammar* G, uint64_t* bytes) {
     *bytes = packed_bytes(G);
     return LCG_OK;
 }
-
-// Copies of 32-bit columns, all of them in one launch.
-struct Copies {
-    std::vector<CopyCol> cols;
-    u64 blocks = 0;
-    // pad: a zero follows when n is odd
-    void add(void* dst, const void* src, u64 n, bool pad = false) {
-        if (n == 0) return;
-        cols.push_back(CopyCol{(u32*)dst, (const u32*)src, n, blocks, pad && (n & 1)});
-        blocks += copy_blocks(n);
-    }
-    void run(lcg_ctx* ctx, std::vector<void*>& temps) {
-        if (cols.empty()) return;
-        CopyCol* d = dalloc<CopyCol>(ctx, cols.size());
-        temps.push_back(d);
-        ck(ctx, cudaMemcpyAsync(d, cols.data(), cols.size() * sizeof(CopyCol), cudaMemcpyHostToDevice, ctx->st),
-           "columns");
-        ck(ctx, launch_copy_cols(d, (u32)cols.size(), blocks, ctx->st), "copy columns");
-        ctx->launches++;
-    }
-};
 
 constexpr u64 kPackGather = 65536;
 

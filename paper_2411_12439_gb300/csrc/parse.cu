@@ -1525,8 +1525,9 @@ __global__ void k_rules(const RoundArgs a) { body_rules<T>(a); }
 // What bounds such rounds is latency: before, each took two cooperative
 // launches of its own with 3 and 4 grid barriers (55-95 us a round; a string of
 // 20 kB has 10 rounds and nothing else); now a round has two barriers and all
-// namings share four.  The sizes need no plan and cannot be outgrown: a round
-// of n symbols in k strings has at most (n + k) / 2 phrases.
+// namings share four.  Their buffers need no plan and cannot be outgrown: a round
+// of n symbols in k strings has at most (n + k) / 2 phrases.  (The levels' arrays, which
+// the grammar keeps, may be planned smaller.)
 // Why 524288: six builds of 12 MB into a growing grammar take 8.66 ms when the
 // short rounds begin at 131072 symbols, 8.27 at 262144, 7.94 at 524288 and 7.82 at
 // 1048576; a build of 8 x 1 MB 947, 948, 917 and 916 us; the larger builds do not
@@ -1915,7 +1916,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_naming_small(const __grid_con
         if (vload(&a.ds->error) || vload(&a.ds->overflow)) s_halt = 1;
         if (threadIdx.x == 0 && a.ds_prev && (vload(&a.ds_prev->error) || vload(&a.ds_prev->overflow))) s_halt = 1;
         if (g > a.r_cap || a.g_base + g > a.cap_g || a.G_base + *a.d_Gnew > a.cap_G) {
-            set_error(a.ds, kErrCapacity);  // not reached: the sizes are bounds
+            set_error(a.ds, kErrCapacity);  // a level that outgrew its plan
             s_halt = 1;
         }
         s_g[threadIdx.x] = g;

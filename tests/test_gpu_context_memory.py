@@ -26,3 +26,27 @@ def test_kept_after_a_build(hf, graph):
         ctx.build(data, off).free()
     ctx.set_graph(False)
     assert _pool_used(rt) - before <= n // 500
+
+
+@pytest.mark.parametrize("kind", ["copies", "dna", "bytes", "short"])
+def test_kept_by_a_grammar(hf, kind):
+    """A grammar's memory is what its arrays need, a few times over, not what the rounds of
+    its build could have needed."""
+    pytest.importorskip("torch")
+    import lcg_inputs as li
+    from paper_2411_12439_gb300 import Context
+    rng = np.random.default_rng(6)
+    one = li.random_dna(rng, 5_000)
+    coll = li.from_strings({"copies": [one] * 100, "dna": [li.random_dna(rng, 500_000)],
+                            "bytes": [rng.integers(0, 256, size=400_000, dtype=np.uint8)], "short": [one[:300]]}[kind])
+    rt = _cudart()
+    ctx = Context(hf, device=0)
+    for graph in (None, False, True):  # round by round, planned, a graph's
+        ctx.set_graph(bool(graph))
+        if graph is not None:
+            ctx.build(coll.data, coll.offsets).free()
+        before = _pool_used(rt)
+        g = ctx.build(coll.data, coll.offsets)
+        held = _pool_used(rt) - before
+        assert held <= 4 * g.packed_size() + 600_000, (graph, held, g.packed_size())
+        g.free()

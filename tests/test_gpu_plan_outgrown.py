@@ -69,3 +69,27 @@ def test_plan_of_unlike_collections(hf):
         g = ctx.build(coll.data, coll.offsets)
         assert O.grammars_equal(g.export(), O.build(coll, hf).export())
         g.free()
+
+
+@pytest.mark.parametrize("graph", [False, True])
+def test_levels_of_short_rounds_outgrow_their_plan(hf, graph):
+    """Copies of one string, then as many bytes of unlike ones: the levels of the short
+    rounds were planned for a hundredth of the rules."""
+    torch = pytest.importorskip("torch")
+    from paper_2411_12439_gb300 import Context
+    rng = np.random.default_rng(9)
+    one = li.random_dna(rng, 4_000)
+    copies = li.from_strings([one] * 100)
+    unlike = li.from_strings(np.split(li.random_dna(rng, 400_000), 100))
+    ctx = Context(hf, device=0)
+    ctx.set_graph(graph)
+    buf = torch.from_numpy(copies.data.copy()).cuda()
+    redone = []
+    for coll in (copies, copies, unlike, unlike, copies, unlike):
+        buf.copy_(torch.from_numpy(coll.data))
+        torch.cuda.synchronize()
+        g = ctx.build(buf, coll.offsets)
+        redone.append(ctx.last_build_stats()["redone"])
+        assert O.grammars_equal(g.export(), O.build(coll, hf).export())
+        g.free()
+    assert redone == [False, False, True, False, False, False]
