@@ -1371,6 +1371,7 @@ void round_sync(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, bool agains
     L.G += G_new;
     free_round(ctx, b);
     next_input(ctx, in, b);
+    in.prev_cap = std::min(in.prev_cap, st.aux[1]);  // (the numbers that were taken: keys as narrow as can be)
     in.n = rc.n_next;
     in.kk = (u32)rc.k_next;
     ctx->stats.rounds = i;

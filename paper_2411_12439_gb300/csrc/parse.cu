@@ -950,7 +950,8 @@ __device__ __forceinline__ void body_parse(const RoundArgs& a, u64 nunits) {
         pa.T_cap = a.T_cap;
         pa.retired = nr;
         pa.lh = a.lh;
-        pa.table = RoundTable{(Slot*)a.tab, a.tab_cap, a.minpos, (ClaimRec*)a.crec, a.id_cap, a.id_chunk, a.ds};
+        pa.table = RoundTable{(Slot*)a.tab, a.tab_cap, a.minpos, (ClaimRec*)a.crec, a.id_cap, a.id_chunk,
+                              kLive ? a.tab_cap : kMaxProbes, a.ds};  // (a short round's table is never too full)
         pa.rtab_cap = a.rtab_cap;
         pa.all = &a;
         pa.sym_w = (u32)a.sym_w;

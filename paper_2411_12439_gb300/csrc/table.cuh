@@ -201,6 +201,7 @@ struct RoundTable {
     ClaimRec* crec;  // claim -> key and fingerprint
     u64 id_cap;      // claim numbers that fit
     u32 id_chunk;    // claim numbers a block takes at a time
+    u64 max_probes;  // slots that a phrase tries before the table counts as too full
     DevStatus* ds;   // aux[1] (the counter of claim numbers), overflow, error
 };
 
@@ -306,7 +307,7 @@ __device__ __forceinline__ u64 table_resolve(const RoundTable& t, ClaimIds* ids,
     bool known_empty = home == kHomeEmpty;
     u64 res = kNoPub;
     bool done = !act;
-    const u64 limit = t.cap < kMaxProbes ? t.cap : kMaxProbes;
+    const u64 limit = t.cap < t.max_probes ? t.cap : t.max_probes;
     u64 probe = 0;
     for (u32 it = 1; !__all_sync(0xffffffffu, done); it++) {
         bool won = false;
@@ -378,7 +379,7 @@ __device__ u64 table_resolve_warp(const RoundTable& t, ClaimIds* ids, ClaimSum& 
     const u32 lane = threadIdx.x & 31;
     u64 s = key_home(k, t.cap);
     const Key128 empty{~0ull, ~0ull};
-    const u64 limit = t.cap < kMaxProbes ? t.cap : kMaxProbes;
+    const u64 limit = t.cap < t.max_probes ? t.cap : t.max_probes;
     for (u64 probe = 0; probe < limit; probe++) {
         Slot c{Key128{0, 0}, 0, 0};
         u64 mine = kNoPub;
