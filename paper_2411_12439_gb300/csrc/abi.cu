@@ -8,6 +8,7 @@
 #include <cstdio>
 #include <cstring>
 #include <initializer_list>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <string>
@@ -38,10 +39,31 @@ struct Level {
     bool shared_rules = false, shared_rhs = false;  // rhs_off and F, rhs: parts of one of the grammar's slabs
 };
 
+// A captured graph, kept by its context and by the grammar that its last launch wrote.
+// That grammar's memory is the graph's allocations, and it is freed before the graph is
+// destroyed: after a graph that was destroyed first, two later graphs were seen to be
+// given the same physical memory, and one's grammar overwrote the other's.
+struct GraphHold {
+    int device = 0;
+    cudaGraph_t graph = nullptr;
+    cudaGraphExec_t exec = nullptr;
+    GraphHold() = default;
+    GraphHold(const GraphHold&) = delete;
+    GraphHold& operator=(const GraphHold&) = delete;
+    ~GraphHold() {  // (nothing of it runs, or is allocated, any more)
+        if (exec) cudaGraphExecDestroy(exec);
+        if (graph) cudaGraphDestroy(graph);
+        // the graph's memory goes back to the device now, not when another graph would
+        // reuse it
+        if (graph) cudaDeviceGraphMemTrim(device);
+    }
+};
+
 }  // namespace
 
 struct lcg_grammar {
     int device = 0;
+    std::shared_ptr<GraphHold> hold;  // the graph whose launch wrote it
     lcg_ctx* owner = nullptr;  // the context that created it, while that context lives
     u64 tag = 0;
     u32* F0 = nullptr;  // 256 fingerprints of bytes (device)
@@ -544,6 +566,7 @@ void free_grammar_now(lcg_grammar* G) {
     for (void* p : G->slabs) release(p);
     release(G->c_level);
     release(G->c_rank);
+    if (G->hold.use_count() == 1) cudaStreamSynchronize(st);  // the graph goes with it, once all is freed
     delete G;
 }
 
@@ -1613,8 +1636,7 @@ struct GraphBuild {
     // round-1 offsets and ids, outside the graph
     u64* soff = nullptr;
     u32* sid = nullptr;
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t exec = nullptr;
+    std::shared_ptr<GraphHold> hold;
     lcg_grammar shape;  // host description of the grammar a launch writes
     AsyncRounds ar;
     u64 ctr_end = 0;    // tile counter after a launch
@@ -1661,8 +1683,6 @@ void destroy_graph(lcg_ctx* ctx) {
     GraphBuild* gb = ctx->graph;
     if (!gb) return;
     cudaStreamSynchronize(ctx->st);
-    if (gb->exec) cudaGraphExecDestroy(gb->exec);
-    if (gb->graph) cudaGraphDestroy(gb->graph);
     // the records of the last launch name the graph's events: they go with them
     ctx->krecs.erase(std::remove_if(ctx->krecs.begin(), ctx->krecs.end(),
                                     [](const lcg_ctx::KRec& r) { return r.graph; }),
@@ -1674,13 +1694,9 @@ void destroy_graph(lcg_ctx* ctx) {
     }
     if (gb->soff) cudaFreeAsync(gb->soff, ctx->st);
     if (gb->sid) cudaFreeAsync(gb->sid, ctx->st);
-    // a live grammar of the graph keeps its memory (freed with the grammar);
-    // the rest of the graph's memory goes back to the device now, not when
-    // another graph would reuse it
-    delete gb;
     ctx->graph = nullptr;
     cudaStreamSynchronize(ctx->st);
-    cudaDeviceGraphMemTrim(ctx->device);
+    delete gb;  // (and the graph, or with its live grammar)
 }
 
 void graph_grammar_freed(lcg_ctx* ctx, const lcg_grammar* G) {
@@ -1719,6 +1735,8 @@ void capture_graph(lcg_ctx* ctx, const unsigned char* d_in, const std::vector<u6
     gb->k = k;
     gb->lens = lens;
     gb->params = std::move(params);
+    gb->hold = std::make_shared<GraphHold>();
+    gb->hold->device = ctx->device;
     gb->n1 = n1;
     gb->soff = dalloc<u64>(ctx, k + 1);
     gb->sid = dalloc<u32>(ctx, k);
@@ -1771,7 +1789,7 @@ void capture_graph(lcg_ctx* ctx, const unsigned char* d_in, const std::vector<u6
         throw;
     }
     ctx->capturing = false;
-    const cudaError_t e = cudaStreamEndCapture(ctx->st, &gb->graph);
+    const cudaError_t e = cudaStreamEndCapture(ctx->st, &gb->hold->graph);
     gb->ctr_end = ctx->ctr_val;
     ctx->ctr_val = ctr_before;
     if (e != cudaSuccess) {
@@ -1787,7 +1805,7 @@ void capture_graph(lcg_ctx* ctx, const unsigned char* d_in, const std::vector<u6
         gb->krecs.back().graph = true;
     }
     ctx->krecs.resize(krec0);
-    const cudaError_t ei = cudaGraphInstantiate(&gb->exec, gb->graph, 0);
+    const cudaError_t ei = cudaGraphInstantiate(&gb->hold->exec, gb->hold->graph, 0);
     if (ei != cudaSuccess) {
         destroy_graph(ctx);
         ck(ctx, ei, "instantiate graph");
@@ -1824,7 +1842,7 @@ lcg_grammar* build_with_graph(lcg_ctx* ctx, const unsigned char* d_in, const std
     ck(ctx, cudaMemcpyAsync(gb->soff, soff_h.data(), (k + 1) * sizeof(u64), cudaMemcpyHostToDevice, ctx->st),
        "upload offsets");
     ck(ctx, cudaMemcpyAsync(gb->sid, sid_h.data(), k * sizeof(u32), cudaMemcpyHostToDevice, ctx->st), "upload ids");
-    cudaError_t el = cudaGraphLaunch(gb->exec, ctx->st);
+    cudaError_t el = cudaGraphLaunch(gb->hold->exec, ctx->st);
     if (el == cudaErrorMemoryAllocation) {
         // the graph has memory of its own beside the pool's: what earlier builds left in
         // the pool goes back to the device
@@ -1832,7 +1850,7 @@ lcg_grammar* build_with_graph(lcg_ctx* ctx, const unsigned char* d_in, const std
         sync(ctx);
         cudaMemPool_t pool;
         if (cudaDeviceGetDefaultMemPool(&pool, ctx->device) == cudaSuccess) cudaMemPoolTrimTo(pool, 0);
-        el = cudaGraphLaunch(gb->exec, ctx->st);
+        el = cudaGraphLaunch(gb->hold->exec, ctx->st);
     }
     ck(ctx, el, "graph launch");
     ctx->ctr_val = gb->ctr_end;
@@ -1841,6 +1859,7 @@ lcg_grammar* build_with_graph(lcg_ctx* ctx, const unsigned char* d_in, const std
     lcg_grammar* G = new lcg_grammar(gb->shape);
     G->owner = ctx;
     ctx->live.push_back(G);
+    G->hold = gb->hold;
     gb->live = G;
     RoundInput in{};
     in.n = gb->n1;
