@@ -1272,7 +1272,7 @@ void tail_sync(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32& i, bool agains
 // regrown and the parse rerun until it fits, and all later sizes are exact.
 // A round of up to kExactNext phrases gets room for as many as it can have (8 bytes
 // each) instead of waiting for their number: six builds of 12 MB into a growing
-// grammar 7.34 ms with 2^22, 7.22 with 2^24.
+// grammar 7.60 ms with 2^22, 7.51 with 2^24 (0.7 to 1.7 % in each of four pairs of runs).
 constexpr u64 kExactNext = 1ull << 24;  // phrases
 
 void round_sync(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, bool against_resident, double& prev_ratio,
@@ -1514,7 +1514,8 @@ void rounds_async_enqueue(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, AsyncRou
         // every id is under the claims that the round before may make
         if (r > 1) a.sym_w = rank_width(in.prev_cap);
         // (the phrases first: the pool may take a while over the table, the largest
-        // allocation, 0.4 ms for 0.5 GB in blocks that it has to piece together)
+        // allocation, 0.4 ms for 0.5 GB in blocks that it has to piece together; 32 x 2 MB
+        // of text 3.42 ms with the table first, 3.40 so in each of four pairs of runs)
         enqueue_phrases(ctx, a, p.n_est);
         alloc_table(ctx, b, in.symb, p.cap, p.g_alloc, kMaxRank + 1);
         set_table(a, b);
@@ -2995,11 +2996,11 @@ int lcg_selftest_wait_timeout(lcg_ctx* ctx) {
     ck(ctx, cudaSetDevice(ctx->device), "cudaSetDevice");
     kt_reset(ctx);
     reset_status(ctx);
-    // A scan of 8 tiles whose tile counter is read one ahead: the first block
+    // A scan of two tiles whose tile counter is read one ahead: the first block
     // takes tile 1 and waits for a tile 0 that no block takes.  Every block
-    // stays in bounds (tiles 1..8 of the 8 look-back slots sized below; tile 8
-    // returns at once), and the wait ends with kErrTimeout.
-    const u64 n = 16384;  // 8 tiles of the scan
+    // stays in bounds (tiles 1 and 2 of the three look-back slots sized below; tile
+    // 2 returns at once), and the wait ends with kErrTimeout.
+    const u64 n = 16384;  // two tiles of the scan
     const u64 tiles = scan2_tiles_for(n);
     ensure_lb(ctx, &ctx->lb2, &ctx->lb2_tiles, tiles + 1, scan2_lb_bytes(tiles + 1));
     u32* in = dalloc<u32>(ctx, n);
