@@ -146,7 +146,9 @@ int lcg_set_kernel_timing(lcg_ctx* ctx, int enable);
 /* Launch and sizing parameters of later builds (picked by an autotuner, e.g.
  * paper_2411_12439_gb300/autotune.py; the results do not depend on them):
  *   table_load          phrase-table slots per expected new rule is 1 / table_load
- *                       (0.3 .. 0.78; a table past 0.8 is regrown and the round rerun);
+ *                       (0.3 .. 0.78; a table is regrown and the round rerun when
+ *                       it fills past 0.8 to 0.9 of its slots, as the new rules fall
+ *                       on the blocks of the parse);
  *   parse_blocks_per_sm resident k_parse blocks per SM in the rounds over ranks, 0 =
  *                       as many as fit (a block of the byte round fills its SM);
  *   miss_flush          accepted (32 .. 256) and kept; it has no effect: every warp of

@@ -698,9 +698,9 @@ void alloc_round(lcg_ctx* ctx, RoundBufs& b, u64 n_bound, u32 kk, u64 t_cap) {
 // the numbers in ranges (a quarter of the claims that a block makes on
 // average, at least a warp's worth), of which each may leave all but one
 // unused.  All that may stay unused is a tenth of the slots at most (one number at a
-// time in the smallest tables), so a pass never fills more than 0.9 of them before it
-// runs out of numbers; whether more than 0.8 are full the host sees afterwards
-// (overfull).  `most`: ids that follow the resident ones and are below 2^31.
+// time in the smallest tables), so a pass that fills between 0.8 and 0.9 of the slots,
+// as the claims fall on the blocks, runs out of numbers.  (One that ends before it does
+// is as good as any, and not rerun for its load.)  `most`: ids that follow the resident ones and are below 2^31.
 void alloc_table(lcg_ctx* ctx, RoundBufs& b, int sym_bytes, u64 cap, u64 claims, u64 most) {
     b.cap = cap;
     claims = std::min(claims, cap - cap / 5);
@@ -719,10 +719,6 @@ void alloc_table(lcg_ctx* ctx, RoundBufs& b, int sym_bytes, u64 cap, u64 claims,
     ck(ctx, cudaMemsetAsync(b.tab, 0xFF, cap * slot_bytes(), ctx->st), "memset table");
     ck(ctx, cudaMemsetAsync(b.minpos, 0xFF, b.id_cap * sizeof(u64), ctx->st), "memset positions");
 }
-
-// Whether the pass has to be rerun with a larger table: it ran out of numbers or of
-// probes, or left the table past its load limit.
-bool overfull(const DevStatus& st, u64 cap) { return st.overflow != 0 || st.claims > cap - cap / 5; }
 
 void free_table(lcg_ctx* ctx, RoundBufs& b) {
     for (void* p : {(void*)b.tab, (void*)b.crec, (void*)b.minpos, (void*)b.rank_of}) dfree(ctx, p);
@@ -1343,21 +1339,23 @@ void round_sync(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, bool agains
     a.T_cap = b.Tcap;
     while (true) {
         fail_if(ctx, cap > kMaxRank + 1, LCG_ETABLE, "phrase table would exceed 2^31 slots");
-        // (a large table without a hint gets numbers for half its slots: they take
-        // more memory than the slots)
-        const u64 most = all || cap <= (1ull << 26) ? cap : std::max<u64>(cap / 2, (u64)g_hint);
+        // (a table of more than 2^28 slots, 8 GB, gets numbers for half of them without a
+        // hint: they take more memory than the slots.  With half from 2^26 slots on round 3
+        // of a first build of 4 x 3.1 Gbp, which fills 139 M slots to 0.795, was rerun with
+        // 555 M: in as much time, with twice the memory)
+        const u64 most = all || cap <= (1ull << 28) ? cap : std::max<u64>(cap / 2, (u64)g_hint);
         alloc_table(ctx, b, in.symb, cap, most, max_ids);
         set_table(a, b);
         enqueue_parse(ctx, a, n);
         fetch(ctx, {{&rc, a.rc, sizeof(rc)}, {&st, a.ds, sizeof(st)}});
         check_device_status(ctx, st);
-        if (!overfull(st, cap)) break;
+        if (!st.overflow) break;
         free_table(ctx, b);
         const bool ran_out = st.aux[1] >= b.id_cap;  // of numbers
         fail_if(ctx, ran_out && b.id_cap >= max_ids, LCG_EOVERFLOW, "level with 2^31 rules or more");
-        // a table with more room than numbers is tried with all of them first: the next
-        // larger one may be one too large (2^31 slots)
-        all = ran_out && b.id_cap < cap - cap / 5 && !all;
+        // where the next larger table would be one too large (2^31 slots) and this one has
+        // more room than numbers, it is tried with all of them
+        all = ran_out && b.id_cap < cap - cap / 5 && !all && cap * 4 > kMaxRank + 1;
         if (!all) cap *= 4;
         retries++;
         ck(ctx, cudaMemsetAsync(a.ds, 0, sizeof(DevStatus), ctx->st), "reset counters");
@@ -1555,7 +1553,7 @@ int rounds_async_finish(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, const Asyn
     fetch(ctx, {{st.data(), ctx->ds_arr, planned * sizeof(DevStatus)},
                 {rc.data(), ctx->rc_arr, planned * sizeof(RoundCounts)}});
     for (u32 r = 0; r < planned; r++) {
-        if (overfull(st[r], ar.cap[r + 1]) || st[r].error == kErrHalted) return -1;
+        if (st[r].overflow || st[r].error == kErrHalted) return -1;
         if (st[r].error == kErrCapacity) {
             const Level& L = R->lv[r];
             return ar.tail && r + 1 >= ar.tail && (st[r].claims > L.cap_g || st[r].claim_len > L.cap_G) ? -2 : -1;

@@ -1,6 +1,6 @@
-"""A phrase table that a round fills past 0.8 of its slots is regrown, however the claims
-fall on the blocks: rounds with a first table of 1.05 to 1.3 times their new rules, over
-bytes and over ranks, in tables of a few thousand slots and of millions."""
+"""A phrase table that a round would fill past 0.9 of its slots is regrown, however the
+claims fall on the blocks: rounds with a first table of 1.05 to 1.3 times their new
+rules, over bytes and over ranks, in tables of a few thousand slots and of millions."""
 import numpy as np
 import pytest
 
@@ -43,19 +43,20 @@ def test_tables_past_the_limit_are_regrown(hf, kind, room):
             g = ctx.build(coll.data, coll.offsets)
             rounds = ctx.last_build_stats()["per_round"]
             assert O.grammars_equal(g.export(), want)
-            assert rounds[i]["retries"] >= 1, (i, slots, rounds[i])
+            if room < 1.1:
+                assert rounds[i]["retries"] >= 1, (i, slots, rounds[i])
             for r in rounds:
-                assert r["g"] <= r["table_cap"] - r["table_cap"] // 5, r
+                assert r["g"] <= r["table_cap"] * 9 // 10, r
             g.free()
 
 
-def test_large_table_with_few_numbers(hf):
-    """A table of more than 2^26 slots gets numbers for half of them at first.  A round
+def test_largest_table_with_few_numbers(hf):
+    """A table of more than 2^28 slots gets numbers for half of them at first.  A round
     that claims more than those, and no more than the table may hold, is rerun with the
-    same table: a build whose next larger table would pass 2^31 slots is not refused."""
+    same table when the next larger one would pass 2^31 slots."""
     import torch
     from paper_2411_12439_gb300 import Context
-    n = 400_000_000
+    n = 3_300_000_000
     g = torch.Generator(device="cuda").manual_seed(1)
     data = torch.randint(0, 256, (n,), dtype=torch.uint8, device="cuda", generator=g)
     off = np.array([0, n], dtype=np.uint64)
@@ -63,10 +64,10 @@ def test_large_table_with_few_numbers(hf):
     ctx = Context(hf, device=0)
     first = ctx.build(data, off)
     rounds = ctx.last_build_stats()["per_round"]
-    i = int(np.argmax([r["g"] for r in rounds]))
-    slots = int(rounds[i]["g"] / 0.65) // 16 + 1  # reached by two steps of four
-    assert 16 * slots > 1 << 26
     first.free()
+    i = int(np.argmax([r["g"] for r in rounds]))
+    slots = max(int(rounds[i]["g"] / 0.65), (1 << 29) + 16) // 16 + 1  # reached by two steps of four
+    assert rounds[i]["g"] > 16 * slots // 2
     ctx = Context(hf, device=0)
     ctx.set_tuning(table_slots_max=slots)
     grammar = ctx.build(data, off)
@@ -74,5 +75,10 @@ def test_large_table_with_few_numbers(hf):
     assert [(r["g"], r["G"]) for r in again] == [(r["g"], r["G"]) for r in rounds]
     assert again[i]["table_cap"] == 16 * slots and again[i]["retries"] >= 3, again[i]
     out = torch.zeros(n, dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
     assert grammar.decompress(0, out) == n
     assert torch.equal(out, data)
+    grammar.free()
+    ctx.close()
+    del data, out
+    torch.cuda.empty_cache()
