@@ -167,7 +167,8 @@ int lcg_set_kernel_timing(lcg_ctx* ctx, int enable);
  *                       warps' worth of work with smaller ones);
  *   parse_tile_min      a round's tile is halved (down to 1024 positions) while the
  *                       round would have fewer than this many tiles per SM (0 .. 1024;
- *                       0 keeps every round at parse_tile).
+ *                       0 keeps every round at parse_tile, but for the last ones, of at
+ *                       most 1024 symbols, which have no tiles).
  * Defaults: 0.35, 0, 64, 0, 1, 4096, 16.  Out-of-range values give LCG_EINVAL. */
 typedef struct lcg_tuning {
     double table_load;

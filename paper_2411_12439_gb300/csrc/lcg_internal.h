@@ -164,6 +164,7 @@ constexpr u32 kParseWarps = 8;                 // warps of a block, a unit each
 // The short rounds at a build's end: one launch for their phrases and parses,
 // one for their naming.
 constexpr u64 kTailSymbols = 524288;  // of the first of them, at most
+constexpr u64 kSoloSymbols = 1024;    // of the rounds that one block takes in its shared memory
 constexpr u32 kTailRounds = 20;       // (each has at most half the symbols and a symbol per string)
 struct TailArgs {
     u32 rounds;

@@ -1570,10 +1570,9 @@ __device__ __forceinline__ u64 block_scan_small(Get get, u64 n, Put put) {
 // memory and the round's general steps each took about 25 us of round trips).
 // Phrases are compared by content in a small table, and numbered in the order
 // of their first occurrences, so a claim's number is its rank already.
-constexpr int kSoloSymbols = 1024;
-constexpr int kSoloWords = kSoloSymbols / 32;
-constexpr int kSoloStrings = kSoloSymbols / 2;                 // two symbols each, at least
-constexpr int kSoloPhrases = (kSoloSymbols + kSoloStrings) / 2;
+constexpr int kSoloWords = (int)kSoloSymbols / 32;
+constexpr int kSoloStrings = (int)kSoloSymbols / 2;                 // two symbols each, at least
+constexpr int kSoloPhrases = ((int)kSoloSymbols + kSoloStrings) / 2;
 constexpr int kSoloSlots = 2048;
 static_assert(kSoloWords == 32, "a warp takes a word per lane");
 
@@ -1848,7 +1847,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_parse_small(const __grid_c
         const RoundArgs& a = t.r[r];
         const u64 n = round_n(a);
         if (n == 0) break;
-        if (n <= (u64)kSoloSymbols) {
+        if (n <= kSoloSymbols) {
             if (blockIdx.x == 0) solo_rounds<kByte>(t, r);
             return;
         }
