@@ -1699,7 +1699,10 @@ void destroy_graph(lcg_ctx* ctx) {
     if (gb->sid) cudaFreeAsync(gb->sid, ctx->st);
     ctx->graph = nullptr;
     cudaStreamSynchronize(ctx->st);
+    const bool kept = gb->hold.use_count() > 1;
     delete gb;  // (and the graph, or with its live grammar)
+    // what the graph does not hold for that grammar goes back to the device now
+    if (kept) cudaDeviceGraphMemTrim(ctx->device);
 }
 
 void graph_grammar_freed(lcg_ctx* ctx, const lcg_grammar* G) {

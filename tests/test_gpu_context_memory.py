@@ -50,3 +50,40 @@ def test_kept_by_a_grammar(hf, kind):
         held = _pool_used(rt) - before
         assert held <= 4 * g.packed_size() + 600_000, (graph, held, g.packed_size())
         g.free()
+
+
+def test_replaced_graph_keeps_its_grammar_only(hf):
+    """A graph that goes while the grammar of its last launch is in use gives the memory
+    of its rounds back at once, and the rest with the grammar."""
+    torch = pytest.importorskip("torch")
+    from paper_2411_12439_gb300 import Context
+    import ctypes
+    rt = _cudart()
+
+    def reserved():  # by graphs, on the device
+        torch.cuda.synchronize()
+        x = ctypes.c_uint64()
+        attr_reserved_mem_current = 2  # cudaGraphMemAttrReservedMemCurrent
+        assert rt.cudaDeviceGetGraphMemAttribute(0, attr_reserved_mem_current, ctypes.byref(x)) == 0
+        return x.value
+
+    n = 64_000_000
+    g = torch.Generator(device="cuda").manual_seed(2)
+    data = torch.randint(0, 4, (n,), dtype=torch.uint8, device="cuda", generator=g)
+    off = np.array([0, n // 3, n], dtype=np.uint64)
+    torch.cuda.synchronize()
+    ctx = Context(hf, device=0)
+    ctx.build(data, off).free()
+    before = reserved()
+    ctx.set_graph(True)
+    grammar = ctx.build(data, off)
+    assert ctx.last_build_stats()["graph"] == 1
+    want = grammar.export_packed()
+    full = reserved() - before
+    ctx.set_graph(False)
+    held = reserved() - before
+    assert full > 2 * n and held < full // 2, (full, held)
+    ctx.build(data, off).free()
+    assert np.array_equal(np.asarray(grammar.export_packed()), np.asarray(want))
+    grammar.free()
+    assert reserved() <= before
