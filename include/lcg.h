@@ -250,7 +250,7 @@ int lcg_build(lcg_ctx* ctx, const uint8_t* data, const uint64_t* offsets, uint32
  * resident grammar keeps its rank, and new phrases are appended after the
  * resident rules of their level in first-occurrence order.  The result is
  * identical to lcg_merge(resident, lcg_build(T)).  `resident` is modified in
- * place; its C grows by k entries. */
+ * place; its C grows by k entries.  A call that fails leaves it as it was. */
 int lcg_build_into(lcg_ctx* ctx, lcg_grammar* resident, const uint8_t* data, const uint64_t* offsets,
                    uint32_t k, int data_on_device);
 
@@ -258,7 +258,8 @@ int lcg_build_into(lcg_ctx* ctx, lcg_grammar* resident, const uint8_t* data, con
  * Level by level, every rule of b whose right-hand side (rewritten into a's
  * ranks of the level below) is a rule of a maps to that rule; the others are
  * appended to a in b's rank order.  C_a becomes C_a . C_b.  Grammars built
- * with different hash families give LCG_EMISMATCH. */
+ * with different hash families give LCG_EMISMATCH.  A call that fails leaves a
+ * as it was. */
 int lcg_merge(lcg_ctx* ctx, lcg_grammar* a, const lcg_grammar* b);
 
 /* exp(C[j]) (Sec. 2.2).  Writes min(cap, |T_j|) bytes to `out` (device memory
