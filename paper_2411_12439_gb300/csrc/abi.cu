@@ -745,6 +745,14 @@ void free_round(lcg_ctx* ctx, RoundBufs& b) {
         dfree(ctx, p);
 }
 
+// Free all of a round's buffers, when the round fails: to be called by the caller of a
+// function that throws between its first allocation and next_input.
+void drop_round(lcg_ctx* ctx, RoundBufs& b) {
+    free_round(ctx, b);
+    for (void* p : {(void*)b.soff_next, (void*)b.sid_next, (void*)b.Tnext, (void*)b.Fnext, (void*)b.rank_of})
+        dfree(ctx, p);
+}
+
 // Bits that hold every rank below `count` (at least 1).
 int rank_width(u64 count) {
     int w = 1;
@@ -1019,7 +1027,8 @@ u32 tail_enqueue(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, u64 n_boun
     const u32 rounds = (u32)z.size();
     const u64 chunk_len = plain.take(chunks * 8);
     const u64 retired = plain.take((u64)ctx->sms * 8);
-    unsigned char* base = dalloc<unsigned char>(ctx, zero.size + ones.size + plain.size);
+    Temps fresh(ctx);  // (freed if a step below fails)
+    unsigned char* base = fresh.get<unsigned char>(zero.size + ones.size + plain.size);
     unsigned char *b0 = base, *b1 = base + zero.size, *b2 = b1 + ones.size;
     ck(ctx, cudaMemsetAsync(b0, 0, zero.size, ctx->st), "memset");
     ck(ctx, cudaMemsetAsync(b1, 0xFF, ones.size, ctx->st), "memset tables");
@@ -1146,7 +1155,7 @@ u32 tail_enqueue(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, u64 n_boun
     kt_end(ctx, h);
     ctx->launches += 2;
     free_round_input(ctx, in);
-    dfree(ctx, base);
+    fresh.drop(base);
     const u64 n = in.n;
     in = RoundInput{};
     in.n = n;
@@ -1268,7 +1277,8 @@ void tail_sync(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32& i, bool agains
             "hash family too short: needs more than " + std::to_string(ctx->levels) + " functions");
 }
 
-// One round with a host synchronisation after the parse: the table is
+// One round (b: its buffers, for the caller to free on failure) with a host
+// synchronisation after the parse: the table is
 // regrown and the parse rerun until it fits, and all later sizes are exact.
 // A round of up to kExactNext phrases gets room for as many as it can have (8 bytes
 // each) instead of waiting for their number: six builds of 12 MB into a growing
@@ -1276,7 +1286,7 @@ void tail_sync(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32& i, bool agains
 constexpr u64 kExactNext = 1ull << 24;  // phrases
 
 void round_sync(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, bool against_resident, double& prev_ratio,
-                double& p_ratio) {
+                double& p_ratio, RoundBufs& b) {
     fail_if(ctx, i >= ctx->levels || i > kMaxRounds,
             LCG_ELEVELS, "hash family too short: needs more than " + std::to_string(ctx->levels) + " functions");
     if (R->lv.size() < i) R->lv.emplace_back();
@@ -1284,7 +1294,6 @@ void round_sync(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, bool agains
     const u64 n = in.n;
     rs.n = n;
     rs.strings = in.kk;
-    RoundBufs b;
     alloc_round(ctx, b, n, in.kk, 0);
     Level& L = R->lv[i - 1];
     RoundArgs a = round_args(ctx, R, in, b, i);
@@ -1396,6 +1405,7 @@ void round_sync(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, u32 i, bool agains
     L.G += G_new;
     free_round(ctx, b);
     next_input(ctx, in, b);
+    b = RoundBufs{};
     in.prev_cap = std::min(in.prev_cap, st.aux[1]);  // (the numbers that were taken: keys as narrow as can be)
     in.n = rc.n_next;
     in.kk = (u32)rc.k_next;
@@ -1489,8 +1499,8 @@ struct AsyncRounds {
 
 // Enqueue the planned rounds of a fresh build: every size comes from the plan;
 // kernels read the actual sizes from the device and flag a round that
-// outgrows its buffers.
-void rounds_async_enqueue(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, AsyncRounds& ar) {
+// outgrows its buffers.  b: the round at hand, for the caller to free on failure.
+void rounds_async_enqueue(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, AsyncRounds& ar, RoundBufs& b) {
     const u32 kk = ar.kk;
     ar.planned = (u32)ar.plan.size() - 1;
     ar.g_base.assign(kMaxRounds + 1, 0);
@@ -1508,7 +1518,6 @@ void rounds_async_enqueue(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, AsyncRou
         ar.cap[r] = p.cap;
         if (R->lv.size() < r) R->lv.emplace_back();
         Level& L = R->lv[r - 1];
-        RoundBufs b;
         alloc_round(ctx, b, p.n_alloc, kk, p.t_cap);
         RoundArgs a = round_args(ctx, R, in, b, r);
         // a round stops early when the one before it failed
@@ -1540,6 +1549,17 @@ void rounds_async_enqueue(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, AsyncRou
         next_input(ctx, in, b);
         in.d_n = &a.rc->n_next;
         in.d_k = &a.rc->k_next;
+        b = RoundBufs{};  // (freed, or the next round's input)
+    }
+}
+
+void rounds_async_enqueue(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, AsyncRounds& ar) {
+    RoundBufs b;
+    try {
+        rounds_async_enqueue(ctx, R, in, ar, b);
+    } catch (...) {
+        drop_round(ctx, b);
+        throw;
     }
 }
 
@@ -1789,6 +1809,7 @@ void capture_graph(lcg_ctx* ctx, const unsigned char* d_in, const std::vector<u6
         cudaGraph_t g = nullptr;
         cudaStreamEndCapture(ctx->st, &g);
         if (g) cudaGraphDestroy(g);
+        cudaGetLastError();  // (frees of a capture that was abandoned)
         delete T;
         ctx->ctr_val = ctr_before;
         destroy_graph(ctx);
@@ -1888,6 +1909,21 @@ lcg_grammar* build_with_graph(lcg_ctx* ctx, const unsigned char* d_in, const std
     return G;
 }
 
+// All rounds of a build: planned ones if there is a plan, then round by round.
+void build_rounds(lcg_ctx* ctx, lcg_grammar* R, RoundInput& in, RoundBufs& b, bool against_resident, bool allow_async) {
+    u32 i = 1;
+    if (allow_async && !against_resident && ctx->hint_rounds > 0) {
+        const int r = rounds_async(ctx, R, in, i);
+        // a round outgrew its estimate: the caller starts again with synchronised rounds
+        if (r < 0) throw Retry{r == -2};
+    }
+    double prev_ratio = 0.0, p_ratio = 0.35;
+    while (in.kk > 0) {
+        if (is_tail(ctx, in.n, against_resident ? R : nullptr)) tail_sync(ctx, R, in, i, against_resident);
+        else round_sync(ctx, R, in, i++, against_resident, prev_ratio, p_ratio, b);
+    }
+}
+
 void build_into(lcg_ctx* ctx, lcg_grammar* R, const uint8_t* data, const uint64_t* off, uint32_t k, int on_dev,
                 bool against_resident, bool allow_async) {
     fail_if(ctx, k == 0 || off == nullptr || data == nullptr, LCG_EINVAL, "empty collection");
@@ -1909,16 +1945,14 @@ void build_into(lcg_ctx* ctx, lcg_grammar* R, const uint8_t* data, const uint64_
     ctx->stats = lcg_build_stats{};
     ctx->stats.input_bytes = off[k] - off[0];
     const u64 launches0 = ctx->launches;
-    std::vector<void*> owned;  // freed at the end
-    auto own = [&](void* p) { owned.push_back(p); return p; };
+    Temps owned(ctx);
 
     const u64 nbytes = off[k] - off[0];
     const unsigned char* d_in;
     if (on_dev) {
         d_in = data + off[0];
     } else {
-        unsigned char* p = dalloc<unsigned char>(ctx, nbytes);
-        own(p);
+        unsigned char* p = owned.get<unsigned char>(nbytes);
         ck(ctx, cudaMemcpyAsync(p, data + off[0], nbytes, cudaMemcpyHostToDevice, ctx->st), "copy input");
         d_in = p;
     }
@@ -1927,8 +1961,8 @@ void build_into(lcg_ctx* ctx, lcg_grammar* R, const uint8_t* data, const uint64_
     R->k += k;
 
     if (!lvl0_id.empty()) {
-        u64* dpos = (u64*)own(dalloc<u64>(ctx, lvl0_pos.size()));
-        u32* dids = (u32*)own(dalloc<u32>(ctx, lvl0_id.size()));
+        u64* dpos = owned.get<u64>(lvl0_pos.size());
+        u32* dids = owned.get<u32>(lvl0_id.size());
         ck(ctx, cudaMemcpyAsync(dpos, lvl0_pos.data(), lvl0_pos.size() * 8, cudaMemcpyHostToDevice, ctx->st), "copy");
         ck(ctx, cudaMemcpyAsync(dids, lvl0_id.data(), lvl0_id.size() * 4, cudaMemcpyHostToDevice, ctx->st), "copy");
         ck(ctx, launch_level0(d_in, dpos, dids, (u32)lvl0_id.size(), R->c_level, R->c_rank, ctx->st), "level0");
@@ -1938,7 +1972,6 @@ void build_into(lcg_ctx* ctx, lcg_grammar* R, const uint8_t* data, const uint64_
     u32 kk = (u32)act_id.size();
     if (kk == 0) {
         sync(ctx);
-        for (void* p : owned) dfree(ctx, p);
         ctx->stats.kernel_launches = ctx->launches - launches0;
         return;
     }
@@ -1946,15 +1979,16 @@ void build_into(lcg_ctx* ctx, lcg_grammar* R, const uint8_t* data, const uint64_
     std::vector<u64> soff_h(kk + 1, 0);
     for (u32 x = 0; x < kk; x++) soff_h[x + 1] = soff_h[x] + act_len[x];
     const u64 n1 = soff_h[kk];
-    u64* d_soff = dalloc<u64>(ctx, kk + 1);
-    u32* d_sid = dalloc<u32>(ctx, kk);
+    Temps first(ctx);  // the first round's input, until it is the rounds' to free
+    u64* d_soff = first.get<u64>(kk + 1);
+    u32* d_sid = first.get<u32>(kk);
     ck(ctx, cudaMemcpyAsync(d_soff, soff_h.data(), (kk + 1) * 8, cudaMemcpyHostToDevice, ctx->st), "copy soff");
     ck(ctx, cudaMemcpyAsync(d_sid, act_id.data(), kk * 4, cudaMemcpyHostToDevice, ctx->st), "copy sid");
     const void* S = d_in;
     void* S_owned = nullptr;
     if (!lvl0_id.empty()) {
-        unsigned char* g = dalloc<unsigned char>(ctx, n1);
-        u64* dsrc = (u64*)own(dalloc<u64>(ctx, kk));
+        unsigned char* g = first.get<unsigned char>(n1);
+        u64* dsrc = owned.get<u64>(kk);
         ck(ctx, cudaMemcpyAsync(dsrc, act_src.data(), kk * 8, cudaMemcpyHostToDevice, ctx->st), "copy");
         ck(ctx, launch_gather_strings(d_in, dsrc, d_soff, kk, g, ctx->st), "gather");
         ctx->launches++;
@@ -1972,25 +2006,18 @@ void build_into(lcg_ctx* ctx, lcg_grammar* R, const uint8_t* data, const uint64_
     in.sid = d_sid;
     ck(ctx, cudaMemsetAsync(ctx->ds_arr, 0, kMaxRounds * sizeof(DevStatus), ctx->st), "reset status");
     ck(ctx, cudaMemsetAsync(ctx->rc_arr, 0, kMaxRounds * sizeof(RoundCounts), ctx->st), "reset counts");
-    u32 i = 1;
-    if (allow_async && !against_resident && ctx->hint_rounds > 0) {
-        const int r = rounds_async(ctx, R, in, i);
-        if (r < 0) {
-            // a round outgrew its estimate: the caller starts again with synchronised rounds
-            free_round_input(ctx, in);
-            for (void* p : owned) dfree(ctx, p);
-            throw Retry{r == -2};
-        }
+    first.ptrs.clear();
+    RoundBufs b;  // of the round at hand
+    try {
+        build_rounds(ctx, R, in, b, against_resident, allow_async);
+        check_device_status(ctx, read_status(ctx));
+    } catch (...) {
+        drop_round(ctx, b);
+        free_round_input(ctx, in);
+        throw;
     }
-    double prev_ratio = 0.0, p_ratio = 0.35;
-    while (in.kk > 0) {
-        if (is_tail(ctx, in.n, against_resident ? R : nullptr)) tail_sync(ctx, R, in, i, against_resident);
-        else round_sync(ctx, R, in, i++, against_resident, prev_ratio, p_ratio);
-    }
-    check_device_status(ctx, read_status(ctx));
     ctx->hint_rounds = ctx->stats.rounds;
     free_round_input(ctx, in);
-    for (void* p : owned) dfree(ctx, p);
     ctx->stats.kernel_launches = ctx->launches - launches0;
 }
 

@@ -4,6 +4,8 @@ it as if nothing had been."""
 import numpy as np
 import pytest
 
+from test_zz_no_alloc import _cudart, _pool_used
+
 import lcg_inputs as li
 from oracle import oracle as O
 
@@ -60,3 +62,49 @@ def test_too_few_hash_functions():
     ctx.build_into(g, a.data, a.offsets)
     both = li.from_strings(2 * [a.string(j) for j in range(a.k)])
     assert O.grammars_equal(g.export(), O.build(both, hf).export())
+
+
+@pytest.mark.parametrize("n", [40_000, 700_000, 3_000_000])
+@pytest.mark.parametrize("mode", ["first", "planned", "graph", "resident"])
+def test_failed_builds_keep_no_memory(hf, n, mode):
+    """Every allocation of a build refused in turn: what the build had is given back."""
+    from paper_2411_12439_gb300 import Context, LCGError
+    a, b, _ = _collections(n)
+    rt = _cudart()
+    ctx = Context(hf, device=0)
+    g = ctx.build(a.data, a.offsets)
+    want = O.build(b, hf).export()
+    if mode in ("planned", "graph"):
+        ctx.build(b.data, b.offsets).free()
+    ctx.build_into(g, b.data, b.offsets)  # (what the context and the grammar keep)
+    before = g.export()
+    refused = 0
+    for nth in range(1, 400):
+        c = Context(hf, device=0) if mode == "first" else ctx
+        c.set_graph(mode == "graph")
+        used = []
+        # at first arrays of the resident grammar, the words of the scans (one more of
+        # them each time) or the upload buffer may grow, which are kept
+        for _ in range(6):
+            c.selftest_alloc_failure(nth)
+            try:
+                if mode == "resident":
+                    c.build_into(g, b.data, b.offsets)
+                else:
+                    h = c.build(b.data, b.offsets)
+                    assert O.grammars_equal(h.export(), want)
+                    h.free()
+                break
+            except LCGError as e:
+                assert e.code == LCG_ENOMEM, e
+            finally:
+                c.selftest_alloc_failure(0)
+            used.append(_pool_used(rt))
+            if mode == "resident":
+                assert O.grammars_equal(g.export(), before)
+        c.set_graph(False)
+        if len(used) < 6:
+            break
+        refused += 1
+        assert used[-1] == used[-2], (nth, used)
+    assert len(used) < 6 and refused >= 4
