@@ -122,6 +122,7 @@ struct lcg_ctx {
     int ktime = 0;  // 0 off, 1 every launch, 2 parse launches only
     bool capturing = false;              // the stream is being captured into a graph
     unsigned char* mail = nullptr;       // page-locked: what the host reads of a step (see fetch)
+    std::vector<std::shared_ptr<const void>> uploads;  // host arrays that copies may still read (see upload)
     unsigned char* upload = nullptr;     // host input of graph builds, at a fixed address
     u64 upload_cap = 0;
     struct KRec {
@@ -209,7 +210,20 @@ struct Temps {
     std::vector<void*> ptrs;
 };
 
-void sync(lcg_ctx* ctx) { ck(ctx, cudaStreamSynchronize(ctx->st), "stream synchronize"); }
+void sync(lcg_ctx* ctx) {
+    ck(ctx, cudaStreamSynchronize(ctx->st), "stream synchronize");
+    ctx->uploads.clear();
+}
+
+// Copies a host array to the device.  The context keeps it until it has waited for the
+// stream: where the device reads pageable memory directly, nothing says that the copy
+// is over when the call returns.
+template <typename T>
+void upload(lcg_ctx* ctx, T* dst, std::vector<T>&& src, const char* what) {
+    auto kept = std::make_shared<const std::vector<T>>(std::move(src));
+    ctx->uploads.push_back(kept);
+    ck(ctx, cudaMemcpyAsync(dst, kept->data(), kept->size() * sizeof(T), cudaMemcpyHostToDevice, ctx->st), what);
+}
 
 // ---- per-kernel timing: events around each launch when enabled -----------
 
@@ -496,8 +510,9 @@ void check_fingerprints(lcg_ctx* ctx, const lcg_grammar* G, std::vector<void*>& 
     if (lv.empty()) return;
     FpLevel* d = dalloc<FpLevel>(ctx, lv.size());
     temps.push_back(d);
-    ck(ctx, cudaMemcpyAsync(d, lv.data(), lv.size() * sizeof(FpLevel), cudaMemcpyHostToDevice, ctx->st), "levels");
-    ck(ctx, launch_check_fp(d, (u32)lv.size(), blocks, ctx->ds, ctx->st), "k_check_fp");
+    const u32 n = (u32)lv.size();
+    upload(ctx, d, std::move(lv), "levels");
+    ck(ctx, launch_check_fp(d, n, blocks, ctx->ds, ctx->st), "k_check_fp");
     ctx->launches++;
 }
 
@@ -1176,9 +1191,9 @@ struct Copies {
         if (cols.empty()) return;
         CopyCol* d = dalloc<CopyCol>(ctx, cols.size());
         temps.push_back(d);
-        ck(ctx, cudaMemcpyAsync(d, cols.data(), cols.size() * sizeof(CopyCol), cudaMemcpyHostToDevice, ctx->st),
-           "columns");
-        ck(ctx, launch_copy_cols(d, (u32)cols.size(), blocks, ctx->st), "copy columns");
+        const u32 n = (u32)cols.size();
+        upload(ctx, d, std::move(cols), "columns");
+        ck(ctx, launch_copy_cols(d, n, blocks, ctx->st), "copy columns");
         ctx->launches++;
     }
 };
