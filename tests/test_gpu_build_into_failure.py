@@ -1,6 +1,8 @@
 """A parse against a resident grammar that fails, for lack of memory at any of its
 allocations or of hash functions, leaves the grammar as it was, and the next one extends
 it as if nothing had been."""
+import gc
+
 import numpy as np
 import pytest
 
@@ -70,6 +72,7 @@ def test_failed_builds_keep_no_memory(hf, n, mode):
     """Every allocation of a build refused in turn: what the build had is given back."""
     from paper_2411_12439_gb300 import Context, LCGError
     a, b, _ = _collections(n)
+    gc.collect()  # (contexts of earlier tests go now, not between two reads of the pool)
     rt = _cudart()
     ctx = Context(hf, device=0)
     g = ctx.build(a.data, a.offsets)

@@ -1,5 +1,7 @@
 """What a context keeps between calls: words of the single-pass scans and of the breaks'
 look-ahead, a thousandth of the largest input, and nothing of a build's own."""
+import gc
+
 import numpy as np
 import pytest
 
@@ -18,6 +20,7 @@ def test_kept_after_a_build(hf, graph):
     g = torch.Generator(device="cuda").manual_seed(2)
     data = torch.randint(0, 4, (n,), dtype=torch.uint8, device="cuda", generator=g)
     off = np.array([0, n // 3, n], dtype=np.uint64)
+    gc.collect()  # (contexts of earlier tests go now, not between two reads of the pool)
     rt = _cudart()
     ctx = Context(hf, device=0)
     before = _pool_used(rt)
@@ -39,6 +42,7 @@ def test_kept_by_a_grammar(hf, kind):
     one = li.random_dna(rng, 5_000)
     coll = li.from_strings({"copies": [one] * 100, "dna": [li.random_dna(rng, 500_000)],
                             "bytes": [rng.integers(0, 256, size=400_000, dtype=np.uint8)], "short": [one[:300]]}[kind])
+    gc.collect()  # (contexts of earlier tests go now, not between two reads of the pool)
     rt = _cudart()
     ctx = Context(hf, device=0)
     for graph in (None, False, True):  # round by round, planned, a graph's
@@ -58,6 +62,7 @@ def test_replaced_graph_keeps_its_grammar_only(hf):
     torch = pytest.importorskip("torch")
     from paper_2411_12439_gb300 import Context
     import ctypes
+    gc.collect()  # (contexts of earlier tests go now, not between two reads of the pool)
     rt = _cudart()
 
     def reserved():  # by graphs, on the device

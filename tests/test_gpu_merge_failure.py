@@ -1,6 +1,8 @@
 """A merge that runs out of device memory, at each of its allocations in turn, leaves
 G_a as it was: its arrays, its packed and VByte forms, its strings.  The same merge
 afterwards equals the oracle's.  The allocation is refused on the host."""
+import gc
+
 import numpy as np
 import pytest
 
@@ -40,6 +42,7 @@ def test_every_allocation_of_a_merge(hf, kind):
     assert O.grammars_equal(back.export(), want)
     back.free()
     g.free()
+    gc.collect()  # (contexts of earlier tests go now, not between two reads of the pool)
     rt = _cudart()
     used = _pool_used(rt)
     refused = 0

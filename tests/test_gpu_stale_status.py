@@ -1,6 +1,8 @@
 """An error of one call does not carry over into the next: after a rejected VByte stream
 (and after a wait that ran out) a good grammar's strings, short and long, come back
 through both entry points, and an expansion that is refused leaves no memory behind."""
+import gc
+
 import numpy as np
 import pytest
 
@@ -58,6 +60,7 @@ def test_refused_expansion_returns_its_scratch(built, j):
     import torch
     from paper_2411_12439_gb300 import LCGError
     ctx, g, coll = built
+    gc.collect()  # (contexts of earlier tests go now, not between two reads of the pool)
     rt = _cudart()
     small = torch.zeros(coll.string(j).size - 1, dtype=torch.uint8, device="cuda")
     used = _pool_used(rt)
